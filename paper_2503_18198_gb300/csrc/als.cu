@@ -3,7 +3,7 @@
 // Per mode d (Gauss-Seidel over d = 0..N-1, Algorithm 1's mode loop):
 //   M      = spMTTKRP_d(Y)                                   (mttkrp.cu)
 //   V      = Hadamard over w != d of G_w,  G_w = Y_w^T Y_w    (R x R, FP64)
-//   L      = Cholesky(V) (FP64); W = V^{-1} = L^{-T} L^{-1}   (FP64, one block)
+//   W      = V^{-1} from V = L D L^T                          (FP64, als_tc.cuh)
 //   Z      = M W, accumulated in double-float (FP32 pairs)    (all SMs)
 //   lambda = column 2-norms of Z;  Y_d = Z / lambda stored as FP32 or BF16
 //   G_d    = Gram of the stored Y_d, exact FP32 products summed in
@@ -34,11 +34,13 @@ __global__ void gram_reduce_kernel(const double* __restrict__ part, int nblocks,
   gram_reduce_body(part, nblocks, R, G, err, blockIdx.x, gridDim.x);
 }
 
+// One column of W per block: least latency for one tensor.
 __global__ void __launch_bounds__(SYS_THREADS)
     system_kernel(const double* __restrict__ grams, int N, int d, int R,
-                  double* __restrict__ V, float* __restrict__ winv,
-                  unsigned char* __restrict__ wdig, int* __restrict__ err) {
-  system_col_body(grams, N, d, R, blockIdx.x, blockIdx.x + 1, V, winv, wdig, err);
+                  float* __restrict__ winv, unsigned char* __restrict__ wdig,
+                  int* __restrict__ err) {
+  __shared__ SystemSmem sm;
+  system_body(sm, grams, N, d, R, blockIdx.x, blockIdx.x + 1, winv, wdig, err);
 }
 
 template <int RPL, int LPR>
@@ -199,7 +201,6 @@ spm_status ensure_als_state(spmttkrp_plan_s* p) {
   const size_t RR = (size_t)R * R;
   SPM_TRY(plan_alloc(p, (void**)&A.gram, sizeof(double) * RR * p->N));
   SPM_TRY(plan_alloc(p, (void**)&A.gram_part, sizeof(double) * RR * A.gram_blocks));
-  SPM_TRY(plan_alloc(p, (void**)&A.chol, sizeof(double) * RR));
   SPM_TRY(plan_alloc(p, (void**)&A.winv, sizeof(float) * 2 * RR));
   SPM_TRY(plan_alloc(p, (void**)&A.colsq_part, sizeof(double) * R * A.gram_blocks));
   SPM_TRY(plan_alloc(p, (void**)&A.colmax_part, sizeof(float) * R * A.gram_blocks));
@@ -239,7 +240,7 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
     // previous mode's solve (the last reader of V^-1) before the overwrite.
     SPM_CUDA_TRY(cudaEventRecord(A.ev_fork, s));
     SPM_CUDA_TRY(cudaStreamWaitEvent(A.side, A.ev_fork, 0));
-    system_kernel<<<R, SYS_THREADS, 0, A.side>>>(A.gram, N, d, R, A.chol, A.winv, A.wdig,
+    system_kernel<<<R, SYS_THREADS, 0, A.side>>>(A.gram, N, d, R, A.winv, A.wdig,
                                                  p->dev_err);
     SPM_CUDA_TRY(cudaGetLastError());
     SPM_CUDA_TRY(cudaEventRecord(A.ev_join, A.side));
@@ -307,7 +308,6 @@ extern "C" spm_status spm_selftest_tc_rowpass(int R, int64_t I, const float* M, 
   };
   alloc((void**)&grams, sizeof(double) * 2 * RR);
   alloc((void**)&err, sizeof(int));
-  alloc((void**)&A.chol, sizeof(double) * RR);
   alloc((void**)&A.winv, sizeof(float) * 2 * RR);
   alloc((void**)&A.wdig, als_wdig_bytes(R));
   alloc((void**)&A.colsq_part, sizeof(double) * R * cap);
@@ -323,7 +323,7 @@ extern "C" spm_status spm_selftest_tc_rowpass(int R, int64_t I, const float* M, 
       SPM_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
       // V = the Hadamard product over the modes other than 0 of a two-mode "tensor": grams[1]
       SPM_CUDA_TRY(cudaMemcpyAsync(grams + RR, V, sizeof(double) * RR, cudaMemcpyDeviceToDevice, s));
-      system_kernel<<<R, SYS_THREADS, 0, s>>>(grams, 2, 0, R, A.chol, A.winv, A.wdig, err);
+      system_kernel<<<R, SYS_THREADS, 0, s>>>(grams, 2, 0, R, A.winv, A.wdig, err);
       const int nb = als_row_blocks(I, cap);
       SPM_TRY(launch_solve(R, nb, A, I, err, nullptr, s));
       const bool tcg = tc_gram_rank(R);
@@ -350,7 +350,7 @@ extern "C" spm_status spm_selftest_tc_rowpass(int R, int64_t I, const float* M, 
     st = run();
   }
   cudaStreamSynchronize(s);
-  for (void* p : {(void*)grams, (void*)err, (void*)A.chol, (void*)A.winv, (void*)A.wdig,
+  for (void* p : {(void*)grams, (void*)err, (void*)A.winv, (void*)A.wdig,
                   (void*)A.colsq_part, (void*)A.colmax_part, (void*)A.lambda_ws,
                   (void*)A.gram_part, (void*)A.inner_part})
     if (p) cudaFree(p);

@@ -8,7 +8,7 @@
 //    largest magnitude) and cut into SM_DIG integer digits of 7 bits,
 //    m_i = 2^e_i * sum_p k_p(i) 2^{-7(p+1)}, |k_p| <= 128;
 //  * each column c of W likewise into SW_DIG digits with scale 2^f_c (done
-//    once per mode by system_col_body, not per block).
+//    once per mode by system_body, not per block).
 // A digit is an integer of at most 8 bits, exact in BF16; a product of two
 // digits is at most 2^14, and a sum of at most SM_DIG * R such products stays
 // below 2^24, so the MMA accumulates it exactly in FP32.  Products of the
@@ -113,8 +113,43 @@ __device__ __forceinline__ void df_add(df& a, float x) {  // a += x (error-free 
   a.lo = __fadd_rn(a.lo, err);
 }
 
-// Threads of a system_col_body block.
-constexpr int SYS_THREADS = 128;
+// ---------------------------------------------------------------------------
+// The normal-equation system of one mode and columns of its inverse.
+//
+// V = the Hadamard product of the Grams of every mode but d (Sec. II-A5), FP64;
+// V = L D L^T (L unit lower triangular), X = L^{-1}, W = V^{-1} = X^T D^{-1} X.
+// L and X come out of one in-place elimination of the lower triangle T: step j
+// takes the pivot d_j = T(j, j) and, for every row i > j with l = T(i, j) / d_j,
+//   T(i, k) -= l T(k, j)  (j < k <= i, the Schur complement),
+//   T(i, k) -= l T(j, k)  (k < j, rows of X),   T(i, j) = -l,
+// so when step j is done row j + 1 holds X(j + 1, :).  A column of W is then
+// R dot products: no substitution chains.
+//
+// Bound: FP64 (2 fused multiply-adds per cycle and SM) and the chain pivot ->
+// reciprocal -> column -> next pivot, one per row.  So every entry of T lives
+// in a register of the thread that owns it for the whole elimination (entry e
+// of the triangle, row-major, belongs to thread e mod 256: the entries still
+// active at step j are a contiguous tail, spread evenly over the warps), the
+// pivot row and column go through shared memory once per step, and one warp
+// forms the reciprocal (a Newton step in place of an FP64 division).
+// One system, one column per block, alone on the GPU, R = 16 / 32 / 64: 12.3 /
+// 25.6 / 78 us (20 / 46 / 139 us for a Cholesky factor with triangle indices
+// recomputed in every step and two substitution chains of R steps per column);
+// 96 systems of R = 16 and 32 side by side 49 us (105 us).
+// ---------------------------------------------------------------------------
+constexpr int SYS_THREADS = 256;
+constexpr int SYS_RMAX = 64;
+constexpr int SYS_COLS = 16;  // most columns of W per block
+
+// Shared memory of a system block.
+struct SystemSmem {
+  double X[SYS_RMAX * (SYS_RMAX + 1)];  // X(k, c) at k (R | 1) + c
+  double W[SYS_COLS * SYS_RMAX];        // per column c: D^{-1} X(:, c), then W(:, c)
+  double piv[2][SYS_RMAX];              // step j: T(k, j) for k >= j, X(j, k) for k < j
+  double nl[SYS_RMAX];                  // step j: -T(i, j) / d_j for i > j
+  double rd[SYS_RMAX];                  // 1 / d_k
+  int bad;
+};
 
 // 2^k as a double for -1022 <= k <= 1023 (exact), else via scalbn.
 __device__ __forceinline__ double times_pow2(double x, int k) {
@@ -122,116 +157,162 @@ __device__ __forceinline__ double times_pow2(double x, int k) {
   return scalbn(x, k);
 }
 
-// Columns c0 .. c1-1 of W = V^{-1}, V the Hadamard product of the Grams of
-// every mode but d (Sec. II-A5), by one block (SYS_THREADS threads):
-//  * V in FP64 and its Cholesky factor L (right-looking, lower triangle; every
-//    block that solves columns of the same system computes the same L);
-//  * per column c, L y = e_c, then L^T w = y (one warp, FP64): w = W(:, c);
-//    warp k takes columns c0 + k, c0 + k + 4, ...
-// A column's arithmetic does not depend on which block or warp solves it:
-// one block per column (least latency, one tensor) and one block per system
-// (least work, many tensors at once) give the same bits.
-// w goes to V_out(:, c) (FP64), to winv as FP32 (hi, lo) pairs (W(s, c) at
-// s R + c and R R + s R + c), and, when wdig is non-null, into the digit tile
-// of the tensor-core solve: w is scaled by 2^-f_c (|w_s| < 2^f_c), rounded to
-// 49 fractional bits and recoded from the least significant end into SW_DIG
+// Reciprocal of a positive finite d in pieces that keep the chain behind it
+// short: d = m 2^(ex - 1023) with 1 <= m < 2, r0 = the FP32 reciprocal of m
+// (e = 1 - m r0 is below 2^-22) and the cubic Newton factor 1 + e + e^2, whose
+// error is e^3; x / d = (x r0 s) (1 + t) with t = e + e^2, s = 2^(1023 - ex).
+// Exponents at the ends of the range take the division.
+struct RecipPos {
+  double r0, t;  // 1 / d = r0 (1 + t)
+};
+__device__ __forceinline__ RecipPos recip_pos(double d) {
+  const int hi = __double2hiint(d), lo = __double2loint(d);
+  const int ex = hi >> 20;  // biased exponent
+  if (ex < 64 || ex > 1982) return {1.0 / d, 0.0};
+  const int mant = hi & 0xfffff;
+  float rf;  // in [0.5, 1]; widened by its bits below
+  asm("rcp.approx.ftz.f32 %0, %1;"
+      : "=f"(rf)
+      : "f"(__int_as_float(0x3f800000 | (mant << 3) | (int)((unsigned)lo >> 29))));
+  const int rb = __float_as_int(rf);
+  const int rh = (rb >> 3) + ((1023 - 127) << 20), rl = rb << 29;
+  const double e = fma(-__hiloint2double(mant | 0x3ff00000, lo), __hiloint2double(rh, rl), 1.0);
+  return {__hiloint2double(rh + ((1023 - ex) << 20), rl), fma(e, e, e)};
+}
+
+// Columns c0 .. c1-1 (at most SYS_COLS) of W by one block of SYS_THREADS
+// threads; NS >= R (R + 1) / 2 / SYS_THREADS entries of T per thread.  Every
+// block that takes columns of the same system computes the same L and X, and
+// an entry of W does not depend on which block or thread forms it, so any
+// split of the columns gives the same bits.
+// w = W(:, c) goes to winv as FP32 (hi, lo) pairs (W(s, c) at s R + c and
+// R R + s R + c), and, when wdig is non-null, into the digit tile of the
+// tensor-core solve: w is scaled by 2^-f_c (|w_s| < 2^f_c), rounded to 49
+// fractional bits and recoded from the least significant end into SW_DIG
 // balanced 7-bit digits (|k_q| <= 64 below the leading digit, |k_0| <= 128),
 // w_s 2^-f_c ~ sum_q k_q 2^{-7(q+1)}; digit q of w_s goes to row q R + c,
 // column s of a K-major (K = R) BF16 tile, f_c to the int array after it.
 // A pivot that is not positive and finite sets DEV_ERR_NUMERIC.
-__device__ __forceinline__ void system_col_body(const double* __restrict__ grams, int N, int d,
-                                                int R, int c0, int c1, double* __restrict__ V_out,
-                                                float* __restrict__ winv,
-                                                unsigned char* __restrict__ wdig,
-                                                int* __restrict__ err) {
-  __shared__ double S[64 * 64];
-  __shared__ double linv[64];  // 1 / L(j, j)
-  __shared__ double col[64];   // column j of L below the diagonal
-  __shared__ int bad;
+template <int NS>
+__device__ __forceinline__ void system_body_ns(SystemSmem& sm, const double* __restrict__ grams,
+                                               int N, int d, int R, int c0, int c1,
+                                               float* __restrict__ winv,
+                                               unsigned char* __restrict__ wdig,
+                                               int* __restrict__ err) {
   const int t = threadIdx.x;
-  if (t == 0) bad = *(volatile int*)err ? 1 : 0;
+  if (t == 0) sm.bad = *(volatile int*)err ? 1 : 0;
   __syncthreads();
-  if (bad) return;
-  const int RR = R * R;
-  for (int e = t; e < RR; e += SYS_THREADS) {
-    double v = 1.0;
-    for (int w = 0; w < N; ++w)
-      if (w != d) v = __dmul_rn(v, grams[(int64_t)w * RR + e]);
-    S[e] = v;
+  if (sm.bad) return;
+  const int RR = R * R, T = R * (R + 1) / 2;
+  int ei[NS], ek[NS], last[NS];  // row, column, last row of the warp's entries
+  double v[NS];
+#pragma unroll
+  for (int q = 0; q < NS; ++q) {
+    const int e = q * SYS_THREADS + t;  // e = i (i + 1) / 2 + k, k <= i
+    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    while (i * (i + 1) / 2 > e) --i;
+    while ((i + 1) * (i + 2) / 2 <= e) ++i;
+    ei[q] = e < T ? i : -1;
+    ek[q] = e < T ? e - i * (i + 1) / 2 : 0;
+    last[q] = __reduce_max_sync(SPM_FULL_MASK, ei[q]);
+    v[q] = 1.0;
   }
-  __syncthreads();
+  const int w0 = d == 0 ? 1 : 0;  // the first mode of the product (none: V = 1)
+  for (int w = w0; w < N; ++w)
+    if (w != d) {
+      double g[NS];
+#pragma unroll
+      for (int q = 0; q < NS; ++q)
+        g[q] = ei[q] >= 0 ? grams[(int64_t)w * RR + ei[q] * R + ek[q]] : 0.0;
+#pragma unroll
+      for (int q = 0; q < NS; ++q) v[q] = w == w0 ? g[q] : __dmul_rn(v[q], g[q]);
+    }
   for (int j = 0; j < R; ++j) {
-    if (t == 0) {
-      const double piv = S[j * R + j];
-      if (!(piv > 0.0) || !isfinite(piv)) {
-        bad = 1;
-      } else {
-        const double r = rsqrt(piv);
-        linv[j] = r;
-        S[j * R + j] = __dmul_rn(piv, r);
+    const int b = j & 1;
+#pragma unroll
+    for (int q = 0; q < NS; ++q)
+      if (ei[q] >= j && (ek[q] == j || ei[q] == j)) sm.piv[b][ek[q] == j ? ei[q] : ek[q]] = v[q];
+    __syncthreads();
+    if (t < 32) {
+      const double piv = sm.piv[b][j];
+      const int hi = __double2hiint(piv);
+      // positive and finite, by its bits
+      const bool good = hi >= 0 && hi < 0x7ff00000 && (hi | __double2loint(piv)) != 0;
+      const RecipPos r = good ? recip_pos(piv) : RecipPos{0.0, 0.0};
+      for (int i = j + 1 + t; i < R; i += 32) {
+        const double x = __dmul_rn(sm.piv[b][i], -r.r0);
+        sm.nl[i] = fma(x, r.t, x);
+      }
+      if (t == 0) {
+        sm.rd[j] = fma(r.r0, r.t, r.r0);
+        if (!good) sm.bad = 1;
       }
     }
     __syncthreads();
-    if (bad) break;
-    const double r = linv[j];
-    for (int i = j + 1 + t; i < R; i += SYS_THREADS) {
-      const double l = __dmul_rn(S[i * R + j], r);
-      col[i] = l;
-      S[i * R + j] = l;
+    if (sm.bad) break;
+    // Operands of every slot first (rows up to j: a zero multiplier; column j:
+    // -l = fma(-l, 1, 0)), then the multiply-adds of the slots that hold a row
+    // beyond j anywhere in the warp: no divergent branch, no slot waits for
+    // the one before it.
+    double l[NS], pv[NS];
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+      l[q] = ei[q] > j ? sm.nl[ei[q]] : 0.0;
+      pv[q] = ek[q] == j ? 1.0 : sm.piv[b][ek[q]];
+      if (ei[q] > j && ek[q] == j) v[q] = 0.0;
     }
-    __syncthreads();
-    // trailing lower triangle (rows and columns j+1 .. R-1), entry e of it
-    // row-major: row a, column b <= a
-    const int m = R - j - 1;
-    const int T = m * (m + 1) / 2;
-    for (int e = t; e < T; e += SYS_THREADS) {
-      int a = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-      while (a * (a + 1) / 2 > e) --a;
-      while ((a + 1) * (a + 2) / 2 <= e) ++a;
-      const int i = j + 1 + a, k = j + 1 + (e - a * (a + 1) / 2);
-      S[i * R + k] = fma(-col[i], col[k], S[i * R + k]);
-    }
-    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NS; ++q)
+      if (last[q] > j) v[q] = fma(l[q], pv[q], v[q]);
   }
-  if (bad) {
+  if (sm.bad) {
     if (t == 0) atomicOr(err, DEV_ERR_NUMERIC);
     return;
   }
-  // L^T into the strict upper triangle (S(i, k) = L(k, i), k > i) so that
-  // both substitutions read rows of S
-  for (int e = t; e < RR; e += SYS_THREADS) {
-    const int i = e / R, k = e % R;
-    if (k > i) S[e] = S[k * R + i];
+  const int LD = R | 1;
+#pragma unroll
+  for (int q = 0; q < NS; ++q)
+    if (ei[q] >= 0) sm.X[ei[q] * LD + ek[q]] = ei[q] == ek[q] ? 1.0 : v[q];
+  __syncthreads();
+  const int nc = c1 - c0;
+  for (int x = t; x < nc * R; x += SYS_THREADS) {
+    const int cc = x / R, k = x - cc * R;
+    sm.W[cc * SYS_RMAX + k] = k >= c0 + cc ? __dmul_rn(sm.X[k * LD + c0 + cc], sm.rd[k]) : 0.0;
+  }
+  __syncthreads();
+  // W(s, c) = sum over k >= max(s, c) of X(k, s) X(k, c) / d_k: four threads
+  // per entry (k mod 4), added by shuffles
+  constexpr int NW = SYS_COLS * SYS_RMAX * 4 / SYS_THREADS;  // rounds at most
+  double wv[NW];
+#pragma unroll
+  for (int p = 0; p < NW; ++p) {
+    const int x = p * (SYS_THREADS / 4) + (t >> 2);
+    if (p * (SYS_THREADS / 4) >= nc * R) break;
+    double a = 0.0;
+    if (x < nc * R) {
+      const int cc = x / R, s = x - cc * R;
+      for (int k = (max(s, c0 + cc) & ~3) + (t & 3); k < R; k += 4)
+        if (k >= s) a = fma(sm.X[k * LD + s], sm.W[cc * SYS_RMAX + k], a);
+    }
+    a += __shfl_xor_sync(SPM_FULL_MASK, a, 1);
+    a += __shfl_xor_sync(SPM_FULL_MASK, a, 2);
+    wv[p] = a;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int p = 0; p < NW; ++p) {
+    const int x = p * (SYS_THREADS / 4) + (t >> 2);
+    if (x < nc * R && (t & 3) == 0) sm.W[(x / R) * SYS_RMAX + x % R] = wv[p];
   }
   __syncthreads();
   const int l = t & 31;
-  for (int c = c0 + (t >> 5); c < c1; c += SYS_THREADS / 32) {
-    // lane l keeps entries l and l + 32 of the right-hand side / solution
-    double b0 = l == c ? 1.0 : 0.0, b1 = l + 32 == c ? 1.0 : 0.0;
-    for (int i = c; i < R; ++i) {  // L y = e_c (y_i = 0 for i < c)
-      const double yi = __dmul_rn(__shfl_sync(SPM_FULL_MASK, i < 32 ? b0 : b1, i & 31), linv[i]);
-      if (l > i && l < R) b0 = fma(-S[i * R + l], yi, b0);
-      if (l + 32 > i && l + 32 < R) b1 = fma(-S[i * R + l + 32], yi, b1);
-      if (l == (i & 31)) {
-        if (i < 32) b0 = yi;
-        else b1 = yi;
-      }
-    }
-    for (int i = R - 1; i >= 0; --i) {  // L^T w = y
-      const double wi = __dmul_rn(__shfl_sync(SPM_FULL_MASK, i < 32 ? b0 : b1, i & 31), linv[i]);
-      if (l < i) b0 = fma(-S[i * R + l], wi, b0);
-      if (l + 32 < i) b1 = fma(-S[i * R + l + 32], wi, b1);
-      if (l == (i & 31)) {
-        if (i < 32) b0 = wi;
-        else b1 = wi;
-      }
-    }
+  for (int cc = t >> 5; cc < nc; cc += SYS_THREADS / 32) {
+    const int c = c0 + cc;
     int fx = INT_MIN;  // exponent bound of the column
     for (int h = 0; h < 2; ++h) {
       const int s = l + 32 * h;
       if (s >= R) continue;
-      const double w = h ? b1 : b0;
-      V_out[s * R + c] = w;
+      const double w = sm.W[cc * SYS_RMAX + s];
       const float hi = (float)w;
       winv[s * R + c] = hi;
       winv[RR + s * R + c] = (float)__dsub_rn(w, (double)hi);
@@ -248,7 +329,7 @@ __device__ __forceinline__ void system_col_body(const double* __restrict__ grams
     for (int h = 0; h < 2; ++h) {
       const int s = l + 32 * h;
       if (s >= R) continue;
-      long long n = __double2ll_rn(times_pow2(h ? b1 : b0, 49 - fx));  // |n| <= 2^49
+      long long n = __double2ll_rn(times_pow2(sm.W[cc * SYS_RMAX + s], 49 - fx));  // |n| <= 2^49
 #pragma unroll
       for (int q = SW_DIG - 1; q >= 0; --q) {
         long long dg = n;
@@ -257,16 +338,25 @@ __device__ __forceinline__ void system_col_body(const double* __restrict__ grams
           n = (n - dg) >> 7;           // exact
         }
         *reinterpret_cast<__nv_bfloat16*>(wdig + tc::kmajor_offset(q * R + c, s, R)) =
-            __float2bfloat16_rn((float)dg);
+            __float2bfloat16_rn((float)(int)dg);
       }
     }
   }
 }
 
+__device__ __forceinline__ void system_body(SystemSmem& sm, const double* __restrict__ grams, int N,
+                                            int d, int R, int c0, int c1, float* __restrict__ winv,
+                                            unsigned char* __restrict__ wdig,
+                                            int* __restrict__ err) {
+  if (R <= 16) system_body_ns<1>(sm, grams, N, d, R, c0, c1, winv, wdig, err);
+  else if (R <= 32) system_body_ns<3>(sm, grams, N, d, R, c0, c1, winv, wdig, err);
+  else system_body_ns<9>(sm, grams, N, d, R, c0, c1, winv, wdig, err);
+}
+
 // Z = M W for rows tile vb, vb + nvb, ... (see the head of this file), with
 // the column sums of Z^2 and the column maxima of |Z| of those rows into
 // colsq_part / colmax_part (block vb's slots).  `wdig` is the mode's W digit
-// tile (system_col_body).
+// tile (system_body).
 template <int R>
 __device__ __forceinline__ void tc_solve_body(const float* __restrict__ M,
                                               const unsigned char* __restrict__ wdig, int64_t I,

@@ -42,12 +42,16 @@ __global__ void batch_fixup_kernel(const BatchTensor* __restrict__ bt, const int
   mttkrp_fixup_body(a.cta_part, a.cta_meta, b.kappa, b.R, b.M, tz.y, threadIdx.x & 31);
 }
 
-// One block per tensor: its system factored once, its columns by the warps.
+// Block (x, y): columns y SYS_COLS .. of tensor it[x]'s system (every block of
+// a tensor eliminates its own copy: with 16 columns a block, the dot products
+// of the columns weigh as much as the elimination).
 __global__ void __launch_bounds__(SYS_THREADS)
     batch_system_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it, int mode) {
+  __shared__ SystemSmem sm;
   const BatchTensor& b = bt[it[blockIdx.x].x];
-  if (!b.active) return;
-  system_col_body(b.gram, b.N, mode, b.R, 0, b.R, b.chol, b.winv, b.wdig, b.err);
+  const int c0 = blockIdx.y * SYS_COLS;
+  if (!b.active || c0 >= b.R) return;
+  system_body(sm, b.gram, b.N, mode, b.R, c0, min(b.R, c0 + SYS_COLS), b.winv, b.wdig, b.err);
 }
 
 __global__ void __launch_bounds__(ALS_THREADS)
@@ -248,7 +252,6 @@ spm_status batch_add(spm_batch_s* B, spmttkrp_plan_s* p, void* const* factors, d
   b.kclass = kc;
   b.gram = A.gram;
   b.gram_part = A.gram_part;
-  b.chol = A.chol;
   b.winv = A.winv;
   b.colsq_part = A.colsq_part;
   b.colmax_part = A.colmax_part;
@@ -457,7 +460,7 @@ spm_status batch_sweep(spm_batch_s* B, cudaStream_t s) {
       SPM_CUDA_TRY(cudaEventRecord(B->ev_fork, s));
       SPM_CUDA_TRY(cudaStreamWaitEvent(B->side, B->ev_fork, 0));
     }
-    batch_system_kernel<<<I.n_tens, SYS_THREADS, 0, ss>>>(B->bt, it + I.tens_off, d);
+    batch_system_kernel<<<dim3(I.n_tens, ceil_div(B->maxR, SYS_COLS)), SYS_THREADS, 0, ss>>>(B->bt, it + I.tens_off, d);
     SPM_CUDA_TRY(cudaGetLastError());
     if (fork) SPM_CUDA_TRY(cudaEventRecord(B->ev_join, B->side));
     SPM_TRY(batch_mttkrp(B, d, s));

@@ -34,7 +34,6 @@ struct BatchTensor {
   // ALS state of the tensor's plan
   double* gram;
   double* gram_part;
-  double* chol;
   float* winv;
   double* colsq_part;
   float* colmax_part;

@@ -43,7 +43,6 @@ struct spm_als_state {
   double* gram = nullptr;             // [N][R*R] Grams of the stored factors
   double* gram_part = nullptr;        // [gram_blocks][R*R] block partials
   int gram_blocks = 0;
-  double* chol = nullptr;             // R*R: Cholesky factor of V (lower)
   float* winv = nullptr;              // 2*R*R: V^{-1} as hi/lo float pairs
   double* colsq_part = nullptr;       // [gram_blocks][R] column sums of Z^2
   float* colmax_part = nullptr;       // [gram_blocks][R] column maxima of |Z|
