@@ -102,7 +102,7 @@ spm_status launch_gram(spmttkrp_plan_s* p, const void* Y, int64_t I, double* G, 
                        const uint32_t* mask) {
   const int R = p->R;
   spm_als_state& A = p->als;
-  const int nb = als_row_blocks(I, A.gram_blocks);
+  const int nb = gram_row_blocks(I, A.gram_blocks);
   const int64_t rpb = ceil_div<int64_t>(I, nb);
   const FT* y = static_cast<const FT*>(Y);
   switch (gram_tile(R)) {
@@ -230,7 +230,6 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
     }
     A.ready = true;
   }
-  const int nb_solve = A.gram_blocks;
   for (int d = 0; d < N; ++d) {
     const int64_t I = p->dims[d];
     // V, its Cholesky factor and V^-1 for mode d need the other modes'
@@ -246,7 +245,7 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
     SPM_CUDA_TRY(cudaEventRecord(A.ev_join, A.side));
     SPM_TRY(run_mttkrp(p, d, factors, A.M, s));
     SPM_CUDA_TRY(cudaStreamWaitEvent(s, A.ev_join, 0));
-    const int nb = als_row_blocks(I, nb_solve);
+    const int nb = solve_blocks(R, I, A.gram_blocks);
     // rows without nonzeros in mode d have a zero update: passes skip them
     const uint32_t* live = p->mode[d].empty_rows > 0 ? p->mode[d].rowmask : nullptr;
     SPM_TRY(launch_solve(R, nb, A, I, p->dev_err, live, s));
@@ -261,7 +260,7 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
       gram_reduce_kernel<<<std::max(1, std::min(1024, R * R / 8)), 256, 0, s>>>(
           A.gram_part, nin, R, A.gram + (size_t)d * R * R, p->dev_err);
     } else {
-      nin = als_row_blocks(I, nb_solve);
+      nin = als_row_blocks(I, A.gram_blocks);
       if (p->bf16)
         scale_kernel<__nv_bfloat16><<<nin, ALS_THREADS, 0, s>>>(
             A.Z, A.lambda_ws, I, R, static_cast<__nv_bfloat16*>(factors[d]), last ? A.M : nullptr,
@@ -324,7 +323,7 @@ extern "C" spm_status spm_selftest_tc_rowpass(int R, int64_t I, const float* M, 
       // V = the Hadamard product over the modes other than 0 of a two-mode "tensor": grams[1]
       SPM_CUDA_TRY(cudaMemcpyAsync(grams + RR, V, sizeof(double) * RR, cudaMemcpyDeviceToDevice, s));
       system_kernel<<<R, SYS_THREADS, 0, s>>>(grams, 2, 0, R, A.winv, A.wdig, err);
-      const int nb = als_row_blocks(I, cap);
+      const int nb = solve_blocks(R, I, cap);
       SPM_TRY(launch_solve(R, nb, A, I, err, nullptr, s));
       const bool tcg = tc_gram_rank(R);
       lambda_kernel<<<R, 32, 0, s>>>(A.colsq_part, A.colmax_part, nb, R, A.lambda_ws, err);

@@ -52,6 +52,12 @@ __host__ __device__ constexpr bool tc_solve_rank(int R) {
   return SPM_ALS_TC && (R == 16 || R == 32 || R == 64);
 }
 
+// Virtual blocks of the row solve over I rows: one tile of the tensor-core
+// solve each while the partial buffers last.
+inline int solve_blocks(int R, int64_t I, int cap) {
+  return tc_solve_rank(R) ? work_blocks(I, TC_ROWS, cap) : als_row_blocks(I, cap);
+}
+
 // Shapes of the solve's shared-memory tiles (bytes) for rank R.
 template <int R>
 struct TcSolveShape {

@@ -158,29 +158,56 @@ __global__ void __launch_bounds__(ALS_THREADS)
                  last ? b.M : nullptr, b.inner_part, b.err, tv.y, b.nb_scale[mode], b.live[mode]);
 }
 
-// Gram partials of factor `mode` (also used for the initial Grams).
+// Gram partials of factor `mode` on the CUDA cores.  `init`: of a new member's
+// factors, whose rows without nonzeros may hold anything.
 template <typename FT>
 __global__ void __launch_bounds__(ALS_THREADS)
-    batch_gram_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it, int mode) {
+    batch_gram_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it, int mode,
+                      bool init) {
   const int2 tv = it[blockIdx.x];
   const BatchTensor& b = bt[tv.x];
   if (!b.active) return;
   const FT* y = static_cast<const FT*>(b.fac[mode]);
   const int64_t I = b.dims[mode];
   const int64_t rpb = b.gram_rpb[mode];
+  const uint32_t* live = init ? nullptr : b.live[mode];
   switch (gram_tile(b.R)) {
-    case 1: gram_partial_body<FT, 1>(y, I, b.R, rpb, b.gram_part, tv.y, b.live[mode]); break;
-    case 2: gram_partial_body<FT, 2>(y, I, b.R, rpb, b.gram_part, tv.y, b.live[mode]); break;
-    default: gram_partial_body<FT, 4>(y, I, b.R, rpb, b.gram_part, tv.y, b.live[mode]); break;
+    case 1: gram_partial_body<FT, 1>(y, I, b.R, rpb, b.gram_part, tv.y, live); break;
+    case 2: gram_partial_body<FT, 2>(y, I, b.R, rpb, b.gram_part, tv.y, live); break;
+    default: gram_partial_body<FT, 4>(y, I, b.R, rpb, b.gram_part, tv.y, live); break;
   }
 }
 
-__global__ void batch_gram_reduce_kernel(const BatchTensor* __restrict__ bt,
-                                         const int2* __restrict__ it, int mode) {
+// Block (x, y): share y of the entries of tensor it[x]'s Gram.  The FP64
+// additions (R^2 per partial) spread over the SMs: with one block per tensor
+// they took 183 us for 96 tensors of R = 16 and 32 and 680 us for 10 tensors
+// up to R = 64; now 61 and 32 us.
+__global__ void __launch_bounds__(256)
+    batch_gram_reduce_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it,
+                             int mode, bool init) {
   const BatchTensor& b = bt[it[blockIdx.x].x];
   if (!b.active) return;
-  gram_reduce_body(b.gram_part, b.nb_gram[mode], b.R, b.gram + (int64_t)mode * b.R * b.R, b.err,
-                   0, 1);
+  gram_reduce_body(b.gram_part, init ? b.nb_init[mode] : b.nb_gram[mode], b.R,
+                   b.gram + (int64_t)mode * b.R * b.R, b.err, blockIdx.y, gridDim.y);
+}
+
+spm_status launch_batch_gram_reduce(const spm_batch_s* B, const int2* it, int n, int mode,
+                                    bool init, cudaStream_t s) {
+  // about four blocks per SM, of at least 32 entries each
+  const int shares = std::max(1, std::min(ceil_div(B->maxR * B->maxR, 32), ceil_div(4 * B->grid, n)));
+  batch_gram_reduce_kernel<<<dim3(n, shares), 256, 0, s>>>(B->bt, it, mode, init);
+  SPM_CUDA_TRY(cudaGetLastError());
+  return SPM_OK;
+}
+
+spm_status launch_batch_gram(const spm_batch_s* B, const int2* it, int n, int mode, bool init,
+                             cudaStream_t s) {
+  if (B->bf16 == 1)
+    batch_gram_kernel<__nv_bfloat16><<<n, ALS_THREADS, 0, s>>>(B->bt, it, mode, init);
+  else
+    batch_gram_kernel<float><<<n, ALS_THREADS, 0, s>>>(B->bt, it, mode, init);
+  SPM_CUDA_TRY(cudaGetLastError());
+  return SPM_OK;
 }
 
 // Fit after the tensor's last mode, then the convergence decision.
@@ -292,17 +319,16 @@ spm_status batch_add(spm_batch_s* B, spmttkrp_plan_s* p, void* const* factors, d
     a.nin = p->N - 1;
     a.nu = p->nu;
     // the single-tensor sweep's virtual block counts (identical sums)
-    b.nb_gram[d] = als_row_blocks(I, A.gram_blocks);
-    b.gram_rpb[d] = ceil_div<int64_t>(I, b.nb_gram[d]);
-    b.nb_solve[d] = als_row_blocks(I, A.gram_blocks);
+    b.nb_gram[d] = b.nb_init[d] = gram_row_blocks(I, A.gram_blocks);
+    b.gram_rpb[d] = ceil_div<int64_t>(I, b.nb_init[d]);
+    b.nb_solve[d] = solve_blocks(p->R, I, A.gram_blocks);
     b.nb_scale[d] = als_row_blocks(I, A.gram_blocks);
     if (tc_gram_rank(p->R))  // the tensor-core normalisation/Gram pass: its own split
       b.nb_gram[d] = b.nb_scale[d] = tc_gram_blocks(I, A.gram_blocks);
   }
-  for (int w = 0; w < p->N; ++w)
-    SPM_TRY(gram(p, factors[w], p->dims[w], A.gram + (size_t)w * p->R * p->R, s));
   B->plans.push_back(p);
   B->host.push_back(b);
+  B->fresh.push_back(1);
   B->bf16 = p->bf16 ? 1 : 0;
   B->dirty = true;
   return SPM_OK;
@@ -311,6 +337,7 @@ spm_status batch_add(spm_batch_s* B, spmttkrp_plan_s* p, void* const* factors, d
 void batch_remove(spm_batch_s* B, int t) {
   B->plans.erase(B->plans.begin() + t);
   B->host.erase(B->host.begin() + t);
+  B->fresh.erase(B->fresh.begin() + t);
   if (B->plans.empty()) B->bf16 = -1;
   B->dirty = true;
 }
@@ -395,6 +422,8 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
         return tc_gram_rank(R) && R == (16 << k) ? B->host[t].nb_scale[d] : 0;
       });
     per_tensor(&I.fit_off, &I.n_fit, [&](int t) { return d == B->plans[t]->N - 1 ? 1 : 0; });
+    per_tensor(&I.init_off, &I.n_init, [&](int t) { return B->fresh[t] ? B->host[t].nb_init[d] : 0; });
+    per_tensor(&I.initt_off, &I.n_initt, [&](int t) { return B->fresh[t] ? 1 : 0; });
   }
   SPM_TRY(grow(&B->bt, &B->bt_cap, std::max<size_t>(1, n)));
   SPM_TRY(grow(&B->items, &B->items_cap, std::max<size_t>(1, v.size())));
@@ -414,6 +443,14 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
     B->smem_set[kc] = B->mtt_smem[kc];
   }
   if (B->grid == 0) B->grid = std::max(1, sm_count());
+  // Grams of the new members' factors, all of a mode in one launch
+  for (int d = 0; d < B->maxN; ++d) {
+    const spm_batch_s::ModeItems& I = B->mi[d];
+    if (I.n_init == 0) continue;
+    SPM_TRY(launch_batch_gram(B, B->items + I.init_off, I.n_init, d, true, s));
+    SPM_TRY(launch_batch_gram_reduce(B, B->items + I.initt_off, I.n_initt, d, true, s));
+  }
+  std::fill(B->fresh.begin(), B->fresh.end(), 0);
   // the staged host vectors must outlive the asynchronous copies
   SPM_CUDA_TRY(cudaStreamSynchronize(s));
   B->dirty = false;
@@ -475,17 +512,12 @@ spm_status batch_sweep(spm_batch_s* B, cudaStream_t s) {
       else
         batch_scale_kernel<float><<<I.n_scale, ALS_THREADS, 0, s>>>(B->bt, it + I.scale_off, d);
     }
-    if (I.n_gram > 0) {
-      if (B->bf16 == 1)
-        batch_gram_kernel<__nv_bfloat16><<<I.n_gram, ALS_THREADS, 0, s>>>(B->bt, it + I.gram_off, d);
-      else
-        batch_gram_kernel<float><<<I.n_gram, ALS_THREADS, 0, s>>>(B->bt, it + I.gram_off, d);
-    }
+    if (I.n_gram > 0) SPM_TRY(launch_batch_gram(B, it + I.gram_off, I.n_gram, d, false, s));
     for (int k = 0; k < 2; ++k)
       if (I.n_tcg[k] > 0)
         SPM_TRY(launch_batch_tc_scale_gram(16 << k, B->bf16 == 1, B->bt, it + I.tcg_off[k],
                                            I.n_tcg[k], d, s));
-    batch_gram_reduce_kernel<<<I.n_tens, 256, 0, s>>>(B->bt, it + I.tens_off, d);
+    SPM_TRY(launch_batch_gram_reduce(B, it + I.tens_off, I.n_tens, d, false, s));
     if (I.n_fit > 0) batch_fit_kernel<<<I.n_fit, ALS_THREADS, 0, s>>>(B->bt, it + I.fit_off, d);
     SPM_CUDA_TRY(cudaGetLastError());
   }

@@ -12,6 +12,7 @@ struct spm_batch_s {
   int bf16 = -1;  // factor storage type of the members, -1 while empty
   std::vector<spmttkrp_plan_s*> plans;
   std::vector<spm::BatchTensor> host;  // descriptors; the device copy is newer after sweeps
+  std::vector<char> fresh;             // member's starting Grams still to be formed
   bool dirty = true;                   // host list changed since the last upload
   // Work-item tables of one mode, as offsets into `items`.
   struct ModeItems {
@@ -25,6 +26,8 @@ struct spm_batch_s {
     int tcg_off[2] = {}, n_tcg[2] = {};  // tensor-core normalisation + Gram, R = 16, 32
     int gram_off = 0, n_gram = 0;    // CUDA-core Gram partials
     int fit_off = 0, n_fit = 0;  // tensors whose last mode is this one
+    int init_off = 0, n_init = 0;    // (tensor, virtual block): Grams of new members' factors
+    int initt_off = 0, n_initt = 0;  // (tensor, 0): new members
   } mi[SPM_MAX_MODES];
   int maxN = 0;
   int maxR = 1;  // largest rank of the members (grid of the system launch)
@@ -47,9 +50,8 @@ struct spm_batch_s {
 namespace spm {
 
 // Add a tensor (its plan, device factors, and where its weights and fit go).
-// Computes the Grams of its factors on `s` (after pulling the members' state
-// if the device copy is current); the device tables are rebuilt by the next
-// batch_commit.  Factors must stay allocated while it is a member.
+// The device tables are rebuilt, and the Grams of its factors formed, by the
+// next batch_commit.  Factors must stay allocated while it is a member.
 // A resumed tensor starts with `start_sweeps` sweeps done and `prev_fit` as
 // the fit of its last sweep.
 spm_status batch_add(spm_batch_s* B, spmttkrp_plan_s* p, void* const* factors, double* lambda,

@@ -27,9 +27,10 @@ struct BatchTensor {
   uint32_t* rowmask[SPM_MAX_MODES];
   const uint32_t* live[SPM_MAX_MODES];  // rowmask when the mode has empty rows, else null
   int nb_gram[SPM_MAX_MODES];   // virtual blocks of the row passes per mode
+  int nb_init[SPM_MAX_MODES];   // and of the CUDA-core Gram of a stored factor
   int nb_solve[SPM_MAX_MODES];
   int nb_scale[SPM_MAX_MODES];
-  int64_t gram_rpb[SPM_MAX_MODES];  // rows per Gram block
+  int64_t gram_rpb[SPM_MAX_MODES];  // rows per block of that Gram
   int N, R, kappa, kclass;
   // ALS state of the tensor's plan
   double* gram;
