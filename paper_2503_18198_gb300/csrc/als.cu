@@ -193,8 +193,24 @@ spm_status ensure_als_state(spmttkrp_plan_s* p) {
   if (!A.side) SPM_CUDA_TRY(cudaStreamCreateWithFlags(&A.side, cudaStreamNonBlocking));
   if (!A.ev_fork) SPM_CUDA_TRY(cudaEventCreateWithFlags(&A.ev_fork, cudaEventDisableTiming));
   if (!A.ev_join) SPM_CUDA_TRY(cudaEventCreateWithFlags(&A.ev_join, cudaEventDisableTiming));
-  if (A.M) return SPM_OK;
   const int R = p->R;
+  if (p->bf16 && A.split_cap < p->kappa && mttkrp_split(p->nnz, p->kappa, p->nu, sm_count()) > 1) {
+    const size_t units = (size_t)p->kappa * p->nu;
+    if (A.split_cap) {  // repartitioned since: queued work may still use the old arrays
+      SPM_CUDA_TRY(cudaDeviceSynchronize());
+      SPM_TRY(plan_realloc(p, (void**)&A.upart, sizeof(float) * 2 * units * R));
+      SPM_TRY(plan_realloc(p, (void**)&A.urow, sizeof(int) * 2 * units));
+      SPM_TRY(plan_realloc(p, (void**)&A.pdone, sizeof(int) * (size_t)p->kappa));
+    } else {
+      SPM_TRY(plan_alloc(p, (void**)&A.upart, sizeof(float) * 2 * units * R));
+      SPM_TRY(plan_alloc(p, (void**)&A.urow, sizeof(int) * 2 * units));
+      SPM_TRY(plan_alloc(p, (void**)&A.pdone, sizeof(int) * (size_t)p->kappa));
+    }
+    SPM_CUDA_TRY(cudaMemsetAsync(A.pdone, 0, sizeof(int) * (size_t)p->kappa, A.side));
+    SPM_CUDA_TRY(cudaStreamSynchronize(A.side));
+    A.split_cap = p->kappa;
+  }
+  if (A.M) return SPM_OK;
   int64_t Imax = 1;
   for (int w = 0; w < p->N; ++w) Imax = std::max(Imax, p->dims[w]);
   A.gram_blocks = std::max(1, sm_count()) * 4;
@@ -243,7 +259,7 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
                                                  p->dev_err);
     SPM_CUDA_TRY(cudaGetLastError());
     SPM_CUDA_TRY(cudaEventRecord(A.ev_join, A.side));
-    SPM_TRY(run_mttkrp(p, d, factors, A.M, s));
+    SPM_TRY(run_mttkrp(p, d, factors, A.M, s, p->bf16));
     SPM_CUDA_TRY(cudaStreamWaitEvent(s, A.ev_join, 0));
     const int nb = solve_blocks(R, I, A.gram_blocks);
     // rows without nonzeros in mode d have a zero update: passes skip them

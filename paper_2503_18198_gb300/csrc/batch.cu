@@ -20,26 +20,32 @@ namespace {
 
 constexpr int64_t BATCH_ZERO_WORDS = 1 << 10;  // row-bitmap words per zero-fill item
 
-__global__ void batch_zero_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it,
-                                  int mode) {
-  const int2 tc = it[blockIdx.x];
-  const BatchTensor& b = bt[tc.x];
-  if (!b.active) return;
-  const int64_t words = (b.dims[mode] + 31) / 32;
-  const int64_t w0 = (int64_t)tc.y * BATCH_ZERO_WORDS;
-  const int64_t w1 = std::min<int64_t>(words, w0 + BATCH_ZERO_WORDS);
-  zero_empty_rows_body(b.rowmask[mode], b.dims[mode], b.R, b.M, w0 + threadIdx.x, w1, blockDim.x);
-}
-
-__global__ void batch_fixup_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it,
-                                   int nitems, int mode) {
+// Rows cut by block boundaries, for members with many of them: one warp per
+// (tensor, partition).
+__global__ void __launch_bounds__(256)
+    batch_fixup_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it, int nitems,
+                       int mode) {
   const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   if (i >= nitems) return;
   const int2 tz = it[i];
   const BatchTensor& b = bt[tz.x];
   if (!b.active) return;
   const MttkrpArgs& a = b.margs[mode];
-  mttkrp_fixup_body(a.cta_part, a.cta_meta, b.kappa, b.R, b.M, tz.y, threadIdx.x & 31);
+  mttkrp_fixup_body(a.cta_part, a.cta_meta, a.nblocks / (a.split > 1 ? a.split : 1), b.R, b.M, tz.y,
+                    threadIdx.x & 31);
+}
+
+// Outputs of members without nonzeros (they have no MTTKRP items).
+__global__ void __launch_bounds__(256)
+    batch_zero_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it, int mode) {
+  const int2 tc = it[blockIdx.x];
+  const BatchTensor& b = bt[tc.x];
+  if (!b.active) return;
+  const int64_t words = (b.dims[mode] + 31) / 32;
+  const int64_t w0 = (int64_t)tc.y * BATCH_ZERO_WORDS;
+  const int64_t w1 = std::min<int64_t>(words, w0 + BATCH_ZERO_WORDS);
+  zero_empty_rows_body(b.rowmask[mode], b.dims[mode], b.R, b.M, w0 + (threadIdx.x >> 5), w1,
+                       blockDim.x >> 5, threadIdx.x & 31);
 }
 
 // Block (x, y): columns y SYS_COLS .. of tensor it[x]'s system (every block of
@@ -275,7 +281,6 @@ spm_status batch_add(spm_batch_s* B, spmttkrp_plan_s* p, void* const* factors, d
   BatchTensor b{};
   b.N = p->N;
   b.R = p->R;
-  b.kappa = p->kappa;
   b.kclass = kc;
   b.gram = A.gram;
   b.gram_part = A.gram_part;
@@ -305,7 +310,6 @@ spm_status batch_add(spm_batch_s* B, spmttkrp_plan_s* p, void* const* factors, d
     MttkrpArgs& a = b.margs[d];
     a = MttkrpArgs{};
     a.rec = p->mode[d].rec;
-    a.woff = p->mode[d].woff;
     int m = 0;
     for (int w = 0; w < p->N; ++w)
       if (w != d) a.fac[m++] = b.fac[w];
@@ -317,7 +321,7 @@ spm_status batch_add(spm_batch_s* B, spmttkrp_plan_s* p, void* const* factors, d
     a.I = I;
     a.R = p->R;
     a.nin = p->N - 1;
-    a.nu = p->nu;
+    if (p->mode[d].empty_rows > 0) a.rowmask = p->mode[d].rowmask;
     // the single-tensor sweep's virtual block counts (identical sums)
     b.nb_gram[d] = b.nb_init[d] = gram_row_blocks(I, A.gram_blocks);
     b.gram_rpb[d] = ceil_div<int64_t>(I, b.nb_init[d]);
@@ -356,16 +360,22 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
   B->maxN = 0;
   B->maxR = 1;
   for (int kc = 0; kc < KC_NONE; ++kc) B->mtt_smem[kc] = 0;
+  const int queue_stride = KC_NONE + n;
+  SPM_TRY(grow(&B->queue, &B->queue_cap, (size_t)SPM_MAX_MODES * queue_stride));
   for (int t = 0; t < n; ++t) {
-    const spmttkrp_plan_s* p = B->plans[t];
+    spmttkrp_plan_s* p = B->plans[t];
     B->maxN = std::max(B->maxN, p->N);
+    SPM_TRY(ensure_als_state(p));  // sized for its present partitions
     B->maxR = std::max(B->maxR, p->R);
     // partitions may have changed since the tensor was added (autotuning)
-    B->host[t].kappa = p->kappa;
-    for (int d = 0; d < p->N; ++d) B->host[t].margs[d].woff = p->mode[d].woff;
     const int kc = B->host[t].kclass;
-    B->mtt_smem[kc] =
-        std::max(B->mtt_smem[kc], mttkrp_smem_bytes(p->R, record_int4s(p->N), p->nu, p->bf16 ? 2 : 4));
+    for (int d = 0; d < p->N; ++d) {
+      MttkrpArgs& a = B->host[t].margs[d];
+      mttkrp_set_shape(p, d, p->bf16, &a);
+      a.done = mttkrp_few_parts(a) ? B->queue + d * queue_stride + KC_NONE + t : nullptr;
+      B->mtt_smem[kc] =
+          std::max(B->mtt_smem[kc], mttkrp_smem_bytes(p->R, a.nu * std::max(1, a.split), BATCH_THREADS / 32));
+    }
   }
   std::vector<int2>& v = B->stage;
   v.clear();
@@ -377,16 +387,21 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
       for (int t = 0; t < n; ++t) {
         const spmttkrp_plan_s* p = B->plans[t];
         if (d < p->N && B->host[t].kclass == kc && p->nnz > 0)
-          for (int z = 0; z < p->kappa; ++z) v.push_back(make_int2(t, z));
+          for (int z = 0; z < B->host[t].margs[d].nblocks; ++z) v.push_back(make_int2(t, z));
       }
       I.n_mtt[kc] = (int)v.size() - I.mtt_off[kc];
     }
+    I.fix_off = (int)v.size();
+    for (int t = 0; t < n; ++t) {
+      const MttkrpArgs& a = B->host[t].margs[d];
+      if (d >= B->plans[t]->N || B->plans[t]->nnz == 0 || a.done) continue;
+      for (int z = 0; z < mttkrp_parts(a); ++z) v.push_back(make_int2(t, z));
+    }
+    I.n_fix = (int)v.size() - I.fix_off;
     I.zero_off = (int)v.size();
     for (int t = 0; t < n; ++t) {
       const spmttkrp_plan_s* p = B->plans[t];
-      // an empty tensor has no partition items: its row masks are all
-      // clear, so the zero-fill items cover its whole output
-      if (d < p->N && (p->nnz == 0 || p->mode[d].empty_rows > 0)) {
+      if (d < p->N && p->nnz == 0) {  // its row masks are all clear
         const int64_t chunks = ceil_div<int64_t>((p->dims[d] + 31) / 32, BATCH_ZERO_WORDS);
         for (int64_t c = 0; c < chunks; ++c) v.push_back(make_int2(t, (int)c));
       }
@@ -427,7 +442,6 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
   }
   SPM_TRY(grow(&B->bt, &B->bt_cap, std::max<size_t>(1, n)));
   SPM_TRY(grow(&B->items, &B->items_cap, std::max<size_t>(1, v.size())));
-  if (!B->queue) SPM_CUDA_TRY(cudaMalloc((void**)&B->queue, sizeof(int) * SPM_MAX_MODES * KC_NONE));
   if (n > 0)
     SPM_CUDA_TRY(cudaMemcpyAsync(B->bt, B->host.data(), sizeof(BatchTensor) * n,
                                  cudaMemcpyHostToDevice, s));
@@ -460,23 +474,22 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
 spm_status batch_mttkrp(spm_batch_s* B, int d, cudaStream_t s) {
   const spm_batch_s::ModeItems& I = B->mi[d];
   if (I.n_zero > 0) batch_zero_kernel<<<I.n_zero, 256, 0, s>>>(B->bt, B->items + I.zero_off, d);
-  int* q = B->queue + d * KC_NONE;
-  SPM_CUDA_TRY(cudaMemsetAsync(q, 0, sizeof(int) * KC_NONE, s));
+  // the item counters of the classes and the finished-block counters of the members
+  const int stride = KC_NONE + (int)B->host.size();
+  int* q = B->queue + d * stride;
+  SPM_CUDA_TRY(cudaMemsetAsync(q, 0, sizeof(int) * stride, s));
   for (int kc = 0; kc < KC_NONE; ++kc) {
     const int n = I.n_mtt[kc];
     if (n == 0) continue;
-    const int grid = std::min(B->grid, n);
+    const int grid = std::min(2 * B->grid, n);
     const int2* it = B->items + I.mtt_off[kc];
     SPM_TRY(B->bf16 == 1
                 ? launch_batch_mttkrp_bf16(kc, B->bt, it, n, q + kc, d, grid, B->mtt_smem[kc], s)
                 : launch_batch_mttkrp_f32(kc, B->bt, it, n, q + kc, d, grid, B->mtt_smem[kc], s));
   }
-  for (int kc = 0; kc < KC_NONE; ++kc) {
-    const int n = I.n_mtt[kc];
-    if (n == 0) continue;
-    batch_fixup_kernel<<<(int)ceil_div<int64_t>((int64_t)n * 32, 256), 256, 0, s>>>(
-        B->bt, B->items + I.mtt_off[kc], n, d);
-  }
+  if (I.n_fix > 0)
+    batch_fixup_kernel<<<(int)ceil_div<int64_t>((int64_t)I.n_fix * 32, 256), 256, 0, s>>>(
+        B->bt, B->items + I.fix_off, I.n_fix, d);
   SPM_CUDA_TRY(cudaGetLastError());
   return SPM_OK;
 }

@@ -17,8 +17,9 @@ struct spm_batch_s {
   // Work-item tables of one mode, as offsets into `items`.
   struct ModeItems {
     int mtt_off[spm::KC_NONE] = {};
-    int n_mtt[spm::KC_NONE] = {};  // (tensor, partition) per (N, R) class
-    int zero_off = 0, n_zero = 0;  // (tensor, element chunk)
+    int n_mtt[spm::KC_NONE] = {};  // (tensor, block) per (N, R) class
+    int fix_off = 0, n_fix = 0;    // (tensor, partition) with boundary rows to add
+    int zero_off = 0, n_zero = 0;  // (empty tensor, bitmap chunk)
     int tens_off = 0, n_tens = 0;  // (tensor, 0): tensors that have this mode
     int solve_off = 0, n_solve = 0;  // (tensor, virtual block), CUDA-core solve ranks
     int tcs_off[3] = {}, n_tcs[3] = {};  // the same for the tensor-core solve, R = 16, 32, 64
@@ -36,8 +37,10 @@ struct spm_batch_s {
   size_t bt_cap = 0;
   int2* items = nullptr;
   size_t items_cap = 0;
-  int* queue = nullptr;  // work-queue counters, one per (mode, class)
-  int grid = 0;          // persistent blocks of an MTTKRP launch
+  int* queue = nullptr;  // per mode: work-queue counters of the classes, then the
+                         // finished-block counters of the members
+  size_t queue_cap = 0;
+  int grid = 0;          // SMs
   size_t mtt_smem[spm::KC_NONE] = {};
   size_t smem_set[spm::KC_NONE] = {};  // dynamic shared memory the attribute allows
   std::vector<int2> stage;
@@ -69,8 +72,8 @@ spm_status batch_pull(spm_batch_s* B, cudaStream_t s);
 // changed (stream-ordered on `s`; may allocate, so not under graph capture).
 spm_status batch_commit(spm_batch_s* B, cudaStream_t s);
 
-// The spMTTKRP of mode d for every member (zero-fill, persistent launches per
-// class, fix-up), output in each member's ALS M buffer.
+// The spMTTKRP of mode d for every member (one persistent launch per class),
+// output in each member's ALS M buffer.
 spm_status batch_mttkrp(spm_batch_s* B, int d, cudaStream_t s);
 
 // One CP-ALS sweep of every active member (launches only once committed).

@@ -14,11 +14,11 @@ spm_status launch_class(const BatchTensor* bt, const int2* items, int nitems, in
   if (grid == 0) {
     // configuration only (at batch creation, outside any stream capture)
     SPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int carve = (int)std::min<size_t>(100, (smem + 4096) * 100 / (228 * 1024) + 1);
+    const int carve = (int)std::min<size_t>(100, (2 * smem + 6144) * 100 / (228 * 1024) + 1);
     SPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve));
     return SPM_OK;
   }
-  fn<<<grid, MT_THREADS, smem, s>>>(bt, items, nitems, queue, mode);
+  fn<<<grid, BATCH_THREADS, smem, s>>>(bt, items, nitems, queue, mode);
   SPM_CUDA_TRY(cudaGetLastError());
   return SPM_OK;
 }

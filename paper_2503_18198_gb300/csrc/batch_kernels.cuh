@@ -5,11 +5,11 @@
 // its arithmetic and summation order are exactly those of a single-tensor
 // sweep: a tensor's result does not depend on which other tensors share the
 // batch.  What changes is the launch structure:
-//  * spMTTKRP: one persistent launch per mode; blocks take (tensor,
-//    partition) items from a global work queue and run the partition body of
+//  * spMTTKRP: one persistent launch per mode and (N, R) class; blocks take
+//    (tensor, block) items from a global work queue and run the block body of
 //    the single-tensor kernel on them (the per-job work queue);
-//  * fix-up, empty-row zeroing and the ALS passes: one launch per step whose
-//    blocks map to (tensor, virtual block) items.
+//  * the ALS passes: one launch per step whose blocks map to (tensor, virtual
+//    block) items.
 // Converged tensors (fit change below the tolerance, or the sweep limit) are
 // marked inactive on the device and skipped, so a CUDA graph of one sweep can
 // be replayed without host round trips.
@@ -31,7 +31,7 @@ struct BatchTensor {
   int nb_solve[SPM_MAX_MODES];
   int nb_scale[SPM_MAX_MODES];
   int64_t gram_rpb[SPM_MAX_MODES];  // rows per block of that Gram
-  int N, R, kappa, kclass;
+  int N, R, kclass;
   // ALS state of the tensor's plan
   double* gram;
   double* gram_part;
@@ -79,17 +79,23 @@ struct BatchClass {
   static constexpr int RI = N <= 3 ? 1 : 2;  // 16-byte words per record
 };
 
-// Persistent spMTTKRP over the (tensor, partition) items of one mode and one
+// Threads of a persistent block: two blocks per SM, so that one's start and
+// merge overlap the other's gathers (a tensor's items may hold as few as 1024
+// nonzeros).
+constexpr int BATCH_THREADS = 512;
+
+// Persistent spMTTKRP over the (tensor, block) items of one mode and one
 // (N, R) class: blocks take items from a work queue in order.  One kernel per
 // class keeps each instantiation's register allocation that of the
 // single-tensor kernel.
 template <typename FT, int KC>
-__global__ void __launch_bounds__(MT_THREADS, 1)
+__global__ void __launch_bounds__(BATCH_THREADS, 2)
     mttkrp_batch_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ items,
                         int nitems, int* __restrict__ queue, int mode) {
   using C = BatchClass<KC>;
   // the lane layout the single-tensor kernel picks for this (type, rank)
   constexpr int V = (sizeof(FT) == 2 && C::N == 3 && C::R <= 32) ? 4 : 16 / (int)sizeof(FT);
+  constexpr bool PLAN = sizeof(FT) == 2;  // BF16 decompositions sum in plan order
   __shared__ int item;
   for (;;) {
     if (threadIdx.x == 0) item = atomicAdd(queue, 1);
@@ -99,7 +105,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1)
     if (i >= nitems) return;
     const int2 tz = items[i];
     const BatchTensor& b = bt[tz.x];
-    if (b.active) mttkrp_partition<C::RI, C::N - 1, FT, V, C::R / V, 1>(b.margs[mode], tz.y);
+    if (b.active) mttkrp_partition<C::RI, C::N - 1, FT, V, C::R / V, 1, false, PLAN>(b.margs[mode], tz.y);
     __syncthreads();
     // a bounded wait that gave up may leave a copy in flight into this
     // block's ring: take no further partition into it

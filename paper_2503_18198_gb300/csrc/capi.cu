@@ -186,11 +186,12 @@ spm_status spmttkrp_plan(spmttkrp_plan_t* out, int nmodes, const int64_t* dims, 
   p->policy = policy;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
 
-  spm_status st = plan_alloc(p, (void**)&p->dev_err, sizeof(int));
+  const int nb = boundary_blocks(nnz, kappa, sm_count());
+  spm_status st = plan_alloc(p, (void**)&p->dev_err, 2 * sizeof(int));
   if (st == SPM_OK) st = plan_alloc(p, (void**)&p->normX2, sizeof(double));
-  if (st == SPM_OK) st = plan_alloc(p, (void**)&p->cta_part, sizeof(float) * 2 * (size_t)kappa * rank);
-  if (st == SPM_OK) st = plan_alloc(p, (void**)&p->cta_meta, sizeof(int) * 4 * (size_t)kappa);
-  if (st == SPM_OK && cudaMemsetAsync(p->dev_err, 0, sizeof(int), s) != cudaSuccess) st = SPM_ERR_CUDA;
+  if (st == SPM_OK) st = plan_alloc(p, (void**)&p->cta_part, sizeof(float) * 2 * (size_t)nb * rank);
+  if (st == SPM_OK) st = plan_alloc(p, (void**)&p->cta_meta, sizeof(int) * 4 * (size_t)nb);
+  if (st == SPM_OK && cudaMemsetAsync(p->dev_err, 0, 2 * sizeof(int), s) != cudaSuccess) st = SPM_ERR_CUDA;
   if (st == SPM_OK) st = build_copies(p, idx, vals, s);
   if (st != SPM_OK) {
     cudaStreamSynchronize(s);
@@ -260,7 +261,8 @@ spm_status spmttkrp_plan_bytes_estimate(int nmodes, const int64_t* dims, int64_t
   if (fibre && (nmodes != 3 || fibre_slots(rank) == 0)) return SPM_ERR_UNSUPPORTED;
   size_t tr = 0;
   plan_bytes_estimate(nmodes, dims, nnz, rank, kappa, true, (flags & SPM_PLAN_LEAN) != 0, resident,
-                      &tr, fibre, (int)((flags & SPM_POLICY_MASK) >> 4));
+                      &tr, fibre, (int)((flags & SPM_POLICY_MASK) >> 4),
+                      (flags & SPM_FACTOR_MASK) == SPM_FACTOR_BF16);
   if (transient) *transient = tr;
   return SPM_OK;
 }
@@ -417,7 +419,9 @@ spm_status spmttkrp_plan_status(spmttkrp_plan_t plan, void* stream) {
   int h = 0;
   SPM_CUDA_TRY(cudaMemcpyAsync(&h, plan->dev_err, sizeof(int), cudaMemcpyDeviceToHost, s));
   SPM_CUDA_TRY(cudaStreamSynchronize(s));
-  SPM_CUDA_TRY(cudaMemsetAsync(plan->dev_err, 0, sizeof(int), s));
+  SPM_CUDA_TRY(cudaMemsetAsync(plan->dev_err, 0, 2 * sizeof(int), s));
+  if (plan->als.pdone)  // a batch that gave up leaves partitions unfinished
+    SPM_CUDA_TRY(cudaMemsetAsync(plan->als.pdone, 0, sizeof(int) * plan->als.split_cap, s));
   if (h & DEV_ERR_NUMERIC) return SPM_ERR_NUMERIC;
   if (h & DEV_ERR_TIMEOUT) return SPM_ERR_TIMEOUT;
   return SPM_OK;

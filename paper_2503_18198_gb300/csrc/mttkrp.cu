@@ -1,6 +1,7 @@
-// mttkrp.cu -- launch sequence of one spMTTKRP along mode d (Algorithm 1's
-// body for one mode): [clear output if Scheme 1] -> mttkrp kernel over the
-// kappa partitions -> fix-up of rows that straddle partitions (Scheme 2).
+// mttkrp.cu -- launch of one spMTTKRP along mode d (Algorithm 1's body for one
+// mode): one kernel over the copy's blocks, which also zeroes the rows without
+// nonzeros and adds the rows cut by block boundaries.  Fibre copies take
+// separate zeroing and fix-up launches, Scheme 1 copies a cleared output.
 #include <algorithm>
 
 #include "mttkrp_kernel.cuh"
@@ -14,6 +15,9 @@ MttkrpKernelFn pick_mttkrp_bf16_a(int nin, int R);
 MttkrpKernelFn pick_mttkrp_bf16_b(int nin, int R);
 MttkrpKernelFn pick_mttkrp_f32_c(int R);
 MttkrpKernelFn pick_mttkrp_bf16_c(int R);
+MttkrpKernelFn pick_mttkrp_bf16_plan_a(int nin, int R);
+MttkrpKernelFn pick_mttkrp_bf16_plan_b(int nin, int R);
+MttkrpKernelFn pick_mttkrp_bf16_plan_lean(int nin, int R);
 MttkrpKernelFn pick_mttkrp_f32_lean(int nin, int R);
 MttkrpKernelFn pick_mttkrp_bf16_lean(int nin, int R);
 
@@ -29,24 +33,24 @@ MttkrpKernelFn pick_mttkrp(bool bf16, int nin, int R) {
 namespace {
 
 // Rows without nonzeros (bit clear in `mask`) are written as zeros.
-__global__ void zero_empty_rows_kernel(const uint32_t* __restrict__ mask, int64_t I, int R,
-                                       float* __restrict__ out) {
-  zero_empty_rows_body(mask, I, R, out, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
-                       (I + 31) / 32, (int64_t)gridDim.x * blockDim.x);
+__global__ void __launch_bounds__(256)
+    zero_empty_rows_kernel(const uint32_t* __restrict__ mask, int64_t I, int R,
+                           float* __restrict__ out) {
+  zero_empty_rows_body(mask, I, R, out, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                       (I + 31) / 32, (int)(gridDim.x * (blockDim.x >> 5)), threadIdx.x & 31);
 }
 
-// One warp per partition z (see mttkrp_fixup_body).
+// One warp per block z of the MTTKRP (see mttkrp_fixup_body).
 __global__ void __launch_bounds__(256)
-    mttkrp_fixup_kernel(const float* __restrict__ cta_part, const int* __restrict__ cta_meta,
-                        int kappa, int R, float* __restrict__ out) {
+    mttkrp_fixup_kernel(const float* cta_part, const int* cta_meta, int nblocks, int R,
+                        float* __restrict__ out) {
   const int z = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-  if (z < kappa) mttkrp_fixup_body(cta_part, cta_meta, kappa, R, out, z, threadIdx.x & 31);
+  if (z < nblocks) mttkrp_fixup_body(cta_part, cta_meta, nblocks, R, out, z, threadIdx.x & 31);
 }
 
 }  // namespace
 
-// Launch the partition fix-up on given boundary partials (used by callers
-// that keep those partials outside a plan).
+// Launch the boundary fix-up on given partials (no finished-block counter).
 spm_status launch_mttkrp_fixup(const float* cta_part, const int* cta_meta, int kappa, int R,
                                float* out, cudaStream_t s) {
   if (kappa <= 1) return SPM_OK;
@@ -57,8 +61,30 @@ spm_status launch_mttkrp_fixup(const float* cta_part, const int* cta_meta, int k
   return SPM_OK;
 }
 
+void mttkrp_set_shape(const spmttkrp_plan_s* p, int d, bool plan_order, MttkrpArgs* a) {
+  const spm_mode_copy& c = p->mode[d];
+  a->words = 4 * record_int4s(p->N);
+  a->nplan = p->kappa * p->nu;
+  a->woff = c.woff;
+  if (!plan_order) {
+    a->split = 0;
+    a->nu = c.nx;
+    a->nblocks = c.kx;
+    return;
+  }
+  a->split = 1;
+  if (p->als.split_cap >= p->kappa && c.scheme != 1) {
+    a->split = mttkrp_split(p->nnz, p->kappa, p->nu, sm_count());
+    a->upart = p->als.upart;
+    a->urow = p->als.urow;
+    a->pdone = p->als.pdone;
+  }
+  a->nu = p->nu / a->split;
+  a->nblocks = p->kappa * a->split;
+}
+
 spm_status run_mttkrp(spmttkrp_plan_s* p, int mode, const void* const* factors, float* out,
-                      cudaStream_t s) {
+                      cudaStream_t s, bool plan_order) {
   if (!p || mode < 0 || mode >= p->N || !factors || !out) return SPM_ERR_INVALID_ARG;
   const int R = p->R;
   const spm_mode_copy& c = p->mode[mode];
@@ -67,7 +93,6 @@ spm_status run_mttkrp(spmttkrp_plan_s* p, int mode, const void* const* factors, 
   a.rec = lean ? p->mode[0].rec : c.rec;
   a.src = c.src;
   a.fmode = mode;
-  a.woff = c.woff;
   int m = 0;
   for (int w = 0; w < p->N; ++w) {
     if (w == mode) continue;
@@ -82,7 +107,7 @@ spm_status run_mttkrp(spmttkrp_plan_s* p, int mode, const void* const* factors, 
   a.I = p->dims[mode];
   a.R = R;
   a.nin = p->N - 1;
-  a.nu = p->nu;
+  mttkrp_set_shape(p, mode, plan_order, &a);
   a.err = p->dev_err;
   a.wait_limit = p->wait_limit;
   const size_t out_bytes = sizeof(float) * (size_t)a.I * (size_t)R;
@@ -90,36 +115,45 @@ spm_status run_mttkrp(spmttkrp_plan_s* p, int mode, const void* const* factors, 
     SPM_CUDA_TRY(cudaMemsetAsync(out, 0, out_bytes, s));
     return SPM_OK;
   }
-  if (c.scheme == 1) {
-    SPM_CUDA_TRY(cudaMemsetAsync(out, 0, out_bytes, s));
-  } else if (c.empty_rows > 0) {
-    const int64_t words = (a.I + 31) / 32;
-    const int blocks = (int)std::min<int64_t>(ceil_div<int64_t>(words, 256), 152 * 8);
-    zero_empty_rows_kernel<<<blocks, 256, 0, s>>>(c.rowmask, a.I, R, out);
-    SPM_CUDA_TRY(cudaGetLastError());
-  }
   if (c.fstream) {
+    if (c.empty_rows > 0) {
+      const int blocks = (int)std::min<int64_t>(ceil_div<int64_t>((a.I + 31) / 32, 8), 152 * 8);
+      zero_empty_rows_kernel<<<blocks, 256, 0, s>>>(c.rowmask, a.I, R, out);
+      SPM_CUDA_TRY(cudaGetLastError());
+    }
     SPM_TRY(launch_mttkrp_fibre(p, mode, factors, out, s));
+    return launch_mttkrp_fixup(p->cta_part, p->cta_meta, p->kappa, R, out, s);
+  }
+  if (c.scheme == 1) {  // no row spans two partitions
+    SPM_CUDA_TRY(cudaMemsetAsync(out, 0, out_bytes, s));
   } else {
-    MttkrpKernelFn fn = lean ? (p->bf16 ? pick_mttkrp_bf16_lean(p->N - 1, R)
-                                        : pick_mttkrp_f32_lean(p->N - 1, R))
-                             : pick_mttkrp(p->bf16, p->N - 1, R);
-    if (!fn) return SPM_ERR_UNSUPPORTED;
-    const size_t smem = mttkrp_smem_bytes(R, record_int4s(p->N), p->nu, p->bf16 ? 2 : 4);
-    SPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // Smallest shared-memory carve-out that fits: the rest of the unified
-    // array is L1 for the gathered factor rows.
-    const int carve = (int)std::min<size_t>(100, (smem + 4096) * 100 / (228 * 1024) + 1);
-    SPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve));
-    fn<<<p->kappa, MT_THREADS, smem, s>>>(a);
-    SPM_CUDA_TRY(cudaGetLastError());
+    if (mttkrp_few_parts(a)) a.done = p->dev_err + 1;
+    if (c.empty_rows > 0) a.rowmask = c.rowmask;
   }
-  if (c.scheme != 1 && p->kappa > 1) {
-    const int threads = 256;
-    const int blocks = (int)ceil_div<int64_t>((int64_t)p->kappa * 32, threads);
-    mttkrp_fixup_kernel<<<blocks, threads, 0, s>>>(p->cta_part, p->cta_meta, p->kappa, R, out);
-    SPM_CUDA_TRY(cudaGetLastError());
-  }
+  const int nin = p->N - 1;
+  MttkrpKernelFn fn;
+  if (a.split > 0)  // BF16 (run_mttkrp's plan order)
+    fn = lean ? pick_mttkrp_bf16_plan_lean(nin, R)
+              : (nin <= 2 ? pick_mttkrp_bf16_plan_a(nin, R) : pick_mttkrp_bf16_plan_b(nin, R));
+  else if (lean)
+    fn = p->bf16 ? pick_mttkrp_bf16_lean(nin, R) : pick_mttkrp_f32_lean(nin, R);
+  else
+    fn = pick_mttkrp(p->bf16, nin, R);
+  if (!fn) return SPM_ERR_UNSUPPORTED;
+  // a block that is full of short units leaves room for a second one
+  const int warps = a.split > 1 || (a.split == 1 && p->nnz / p->kappa < 4096) ? 16
+                    : a.split == 1 ? 32 : mttkrp_warps(a.nu);
+  const size_t smem = mttkrp_smem_bytes(R, a.split > 1 ? p->nu : a.nu, warps);
+  SPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // Smallest shared-memory carve-out that fits the resident blocks: the rest
+  // of the unified array is L1 for the gathered factor rows.
+  const size_t used = (smem + 2048) * (warps == 32 ? 1 : 2);
+  const int carve = (int)std::min<size_t>(100, (used + 2048) * 100 / (228 * 1024) + 1);
+  SPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve));
+  fn<<<a.nblocks, warps * 32, smem, s>>>(a);
+  SPM_CUDA_TRY(cudaGetLastError());
+  if (c.scheme != 1 && !a.done)
+    return launch_mttkrp_fixup(p->cta_part, p->cta_meta, mttkrp_parts(a), R, out, s);
   return SPM_OK;
 }
 

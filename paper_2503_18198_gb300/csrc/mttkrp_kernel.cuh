@@ -4,11 +4,13 @@
 //   M_d(c_d, r) = sum over nonzeros of val * prod_{w != d} Y_w(c_w, r).
 //
 // How (GB300 design, not the paper's block layout):
-//  * One thread block per partition B_{d,z} (Algorithm 1's parallel loop),
-//    1024 threads as in the paper's R x P = 32 x 32 block.  The partition is
-//    cut by the plan into NU contiguous work units; the block's 32 warps take
-//    units from a shared-memory counter, so a warp that drew cheap units
-//    takes more (dynamic balance inside the block, fixed merge order).
+//  * A copy is run by a number of blocks and of contiguous work units per
+//    block that the plan chooses for its size (mttkrp_shape): large copies one
+//    block of 32 warps per partition B_{d,z} (Algorithm 1's parallel loop) and
+//    up to 128 units each, small ones fewer and smaller blocks.  A block's
+//    warps take units from a shared-memory counter, so a warp that drew cheap
+//    units takes more (dynamic balance inside the block); sums are merged in
+//    an order that depends on the units only, not on the warps.
 //  * A warp streams its unit of the copy through a 3-stage ring of small
 //    shared-memory tiles filled by 1-D bulk copies (cp.async.bulk on the TMA
 //    engine, completion on an mbarrier).  Tiles are small so that most of
@@ -24,14 +26,13 @@
 //    combined with a segmented shuffle scan and finished rows are stored
 //    once.  Partial rows never round-trip through global memory (the paper's
 //    point about intermediate values, Sec. I).
-//  * Rows cut by a unit boundary are merged by the block with a segmented
-//    scan over the units' boundary partials in shared memory (the paper's
-//    Local_Update); rows cut by a partition boundary (equal-nnz or balanced
-//    policies) leave one partial per block in a small workspace that a fix-up
-//    kernel adds in partition order (the paper's Global_Update, made
-//    deterministic).
-//  * Rows with no nonzero are zeroed by a separate pass over a plan-time
-//    bitmap of non-empty rows.
+//  * Rows cut by a unit boundary are merged by the block from the units'
+//    boundary partials in shared memory (the paper's Local_Update); rows cut
+//    by a block boundary leave one partial per block in a small workspace that a
+//    fix-up kernel (with few blocks: the block finishing last) adds in block
+//    order (the paper's Global_Update, made deterministic).
+//  * Rows with no nonzero are zeroed by the warps that run out of units, from
+//    a plan-time bitmap of non-empty rows.
 #pragma once
 
 #include <type_traits>
@@ -55,6 +56,7 @@ constexpr int MT_THREADS = MT_WARPS * 32;
 #define SPM_MT_TILE 64
 #endif
 constexpr int MT_STAGES = SPM_MT_STAGES;
+constexpr int MT_MAX_UNITS = 128;  // most units of a block
 constexpr int MT_TILE_RECS = SPM_MT_TILE;  // 16-byte records per stage tile (per warp);
                                            // a tile of 32-byte records holds half as many
 
@@ -62,11 +64,14 @@ struct MttkrpArgs {
   const int4* rec;        // copy records (lean copy: the mode-0 copy's)
   const int32_t* src;     // lean copy: position in the mode-0 copy of each copy position
   int fmode;              // lean copy: the output mode (its index is word fmode of a record)
-  const int64_t* woff;    // work-unit offsets [kappa * nu + 1]
+  const int64_t* woff;    // the plan's work-unit offsets [nplan + 1]
   const void* fac[SPM_MAX_MODES - 1];  // input factors in record order
   float* out;             // I_d x R
-  float* cta_part;        // [kappa][2][R] boundary partials
-  int* cta_meta;          // [kappa][4] (first row, last row, flags, 0)
+  float* cta_part;        // [nblocks][2][R] boundary partials
+  int* cta_meta;          // [nblocks][4] (first row, last row, flags, 0)
+  int* done;              // few blocks: those finished so far, zero between runs; the last one
+                          // adds the rows cut by block boundaries (null: the caller launches that)
+  const uint32_t* rowmask;  // bit i set: row i has a nonzero; other rows are zeroed (null: none)
   int* err;               // sticky device error flags
   const int* guard;       // if non-null and non-zero when the block starts, the block
                           // writes no output (a failed input check of the same call)
@@ -76,15 +81,34 @@ struct MttkrpArgs {
   int64_t I;              // rows of the output
   int R;                  // rank (runtime; equals the template rank when exact)
   int nin;                // number of input modes (N - 1)
-  int nu;                 // work units per partition
+  int words;              // 32-bit words per record
+  int nu;                 // work units per block
+  int nblocks;            // blocks (and items of a batch) of this copy
+  // PLAN kernels: the sums take the tree that the plan's partitions define (unit
+  // partials merged per partition by a segmented scan), whatever the number of
+  // blocks that share a partition; the others sum in any order (split = 0, see
+  // mttkrp_shape).  Two kernels: with both merges in one the record loop of the
+  // 4-mode BF16 kernel lost registers (30M nonzeros, R = 64: 695 -> 720 us).
+  int split;              // blocks per partition in plan order (then nu * split units each)
+  float* upart;           // split > 1: [nplan][2][R] unit boundary partials
+  int* urow;              // split > 1: [nplan][2] their rows
+  int* pdone;             // split > 1: [nblocks / split] finished blocks, zero between runs
+  int nplan;              // work units of the plan
 };
+
+// Pieces whose boundary rows are added at the end of a run, and whether the
+// block that finishes last does it.  It saves a launch (4 blocks: 10.5 against
+// 12.3 us per product), but one block pays the load latencies of all pieces:
+// for 293 blocks 24.6 us against 16.4 us with the fix-up kernel.
+inline int mttkrp_parts(const MttkrpArgs& a) { return a.nblocks / (a.split > 1 ? a.split : 1); }
+inline bool mttkrp_few_parts(const MttkrpArgs& a) { return mttkrp_parts(a) <= 32; }
 
 // cta_meta flags
 enum : int {
   META_PART0 = 1,        // cta_part[z][0] holds the first row's partial
   META_PART1 = 2,        // cta_part[z][1] holds the last row's partial
-  META_SHARED_PREV = 4,  // first row continues from the previous partition
-  META_SHARED_NEXT = 8,  // last row continues into the next partition
+  META_SHARED_PREV = 4,  // first row continues from the previous block
+  META_SHARED_NEXT = 8,  // last row continues into the next block
   META_EMPTY = 16,
 };
 
@@ -107,11 +131,9 @@ enum : int {
 // barriers, and two boundary partials (+ row ids) per work unit.  A stage
 // tile has the same bytes for either record size; the factor type does not
 // enter.
-inline size_t mttkrp_smem_bytes(int R, int RI, int nu, int fsize) {
-  (void)RI;
-  (void)fsize;
-  return (size_t)MT_WARPS * MT_STAGES * MT_TILE_RECS * 16 +
-         (size_t)MT_WARPS * MT_STAGES * sizeof(uint64_t) + (size_t)2 * nu * R * sizeof(float) +
+inline size_t mttkrp_smem_bytes(int R, int nu, int warps) {
+  return (size_t)warps * MT_STAGES * MT_TILE_RECS * 16 +
+         (size_t)warps * MT_STAGES * sizeof(uint64_t) + (size_t)2 * nu * R * sizeof(float) +
          (size_t)2 * nu * sizeof(int);
 }
 
@@ -222,13 +244,345 @@ __device__ __forceinline__ void store_vec(float* row_ptr, int R, int r0, const f
   }
 }
 
+// Boundary fix-up for block z, one warp (lane = its lane): if z holds
+// the start of a row that continues into later blocks (its last-row partial),
+// add the first-row partials of the following blocks in block order and store
+// the row.  The partials were written by other SMs, in the same launch when the
+// last block runs this: they are read from L2.
+__device__ __forceinline__ void mttkrp_fixup_body(const float* cta_part,
+                                                  const int* cta_meta, int nblocks,
+                                                  int R, float* __restrict__ out, int z, int lane) {
+  const int4 m = __ldcg(reinterpret_cast<const int4*>(cta_meta) + z);
+  if (!(m.z & META_PART1)) return;
+  const int row = m.y;
+  float s[8];
+  const float* p1 = cta_part + (int64_t)(2 * z + 1) * R;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int r = lane + 32 * j;
+    s[j] = r < R ? __ldcg(p1 + r) : 0.f;
+  }
+  // The blocks after z that continue `row`, in order; their metadata and
+  // partials are loaded FQ at a time ahead of the (ordered) additions, so a
+  // head row cut into many blocks does not pay one load latency each.
+  constexpr int FQ = 4;
+  bool more = true;
+  for (int q0 = z + 1; q0 < nblocks && more; q0 += FQ) {
+    int4 mq[FQ];
+    float pq[FQ][8];
+#pragma unroll
+    for (int k = 0; k < FQ; ++k) {
+      const int q = q0 + k;
+      mq[k] = q < nblocks ? __ldcg(reinterpret_cast<const int4*>(cta_meta) + q) : make_int4(-1, -1, 0, 0);
+      const float* p0 = cta_part + (int64_t)(2 * (q < nblocks ? q : z)) * R;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int r = lane + 32 * j;
+        pq[k][j] = r < R ? __ldcg(p0 + r) : 0.f;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < FQ; ++k) {
+      if (!more || q0 + k >= nblocks) {
+        more = false;
+        continue;
+      }
+      const int fq = mq[k].z;
+      if (fq & META_EMPTY) continue;
+      if (mq[k].x != row) {
+        more = false;
+        continue;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int r = lane + 32 * j;
+        if (r < R) s[j] += pq[k][j];
+      }
+      if (!(mq[k].y == row && (fq & META_SHARED_NEXT))) more = false;
+    }
+  }
+  float* dst = out + (int64_t)row * R;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int r = lane + 32 * j;
+    if (r < R) dst[r] = s[j];
+  }
+}
+
+// Whether this block is the last of n to get here (every thread must call it);
+// what the others wrote before is then visible, read past L1.  The counter is
+// left at zero.
+__device__ __forceinline__ bool block_is_last(int* counter, int n, int* flag) {
+  __syncthreads();  // the block's writes are done
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const int last = atomicAdd(counter, 1) == n - 1;
+    if (last) {
+      *counter = 0;
+      __threadfence();
+    }
+    *flag = last;
+  }
+  __syncthreads();
+  return *flag != 0;
+}
+
+// Rows of an I x R output whose bit in `mask` is clear are zeroed, for the
+// bitmap words w0, w0 + wstep, ... below w1 (word w covers rows 32w ..
+// 32w+31), by one warp: the lanes side by side along a row.
+__device__ __forceinline__ void zero_empty_rows_body(const uint32_t* __restrict__ mask, int64_t I,
+                                                     int R, float* __restrict__ out, int64_t w0,
+                                                     int64_t w1, int wstep, int lane) {
+  for (int64_t wb = w0; wb < w1; wb += 32 * (int64_t)wstep) {
+    // 32 of the words at once, one per lane
+    const int64_t wl = wb + (int64_t)lane * wstep;
+    const uint32_t mine = wl < w1 ? ~__ldg(&mask[wl]) : 0u;
+    uint32_t some = __ballot_sync(SPM_FULL_MASK, mine != 0u);
+    while (some) {
+      const int l = __ffs(some) - 1;
+      some &= some - 1;
+      uint32_t clear = __shfl_sync(SPM_FULL_MASK, mine, l);
+      const int64_t w = wb + (int64_t)l * wstep;
+      while (clear) {
+        const int b = __ffs(clear) - 1;
+        clear &= clear - 1;
+        const int64_t row = w * 32 + b;
+        if (row >= I) break;
+        float* dst = out + row * R;
+        if ((R & 3) == 0) {
+          for (int c = 4 * lane; c < R; c += 128)
+            *reinterpret_cast<float4*>(dst + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+        } else {
+          for (int c = lane; c < R; c += 32) dst[c] = 0.f;
+        }
+      }
+    }
+  }
+}
+
+// First copy position of unit j of the nblocks * nu units of a run: j / (nblocks
+// * nu) of the way through the plan's nplan units, inside one by its length.
+__device__ __forceinline__ int64_t mttkrp_unit_begin(const MttkrpArgs& a, unsigned j) {
+  const unsigned nrun = (unsigned)a.nblocks * (unsigned)a.nu, nplan = (unsigned)a.nplan;
+  if (nrun == nplan) return __ldg(a.woff + j);
+  const uint64_t x = (uint64_t)j * nplan;
+  const unsigned u = (unsigned)(x / nrun), rem = (unsigned)(x - (uint64_t)u * nrun);
+  const int64_t b = __ldg(a.woff + u);
+  return rem ? b + (__ldg(a.woff + u + 1) - b) * (int64_t)rem / (int64_t)nrun : b;
+}
+
+// Inclusive segmented scan of the NE x R entries, one (entry, rank) each for up
+// to EPT entries e0, e0 + step, ... of rank r per thread.
+template <int EPT>
+__device__ __forceinline__ void merge_scan(float* part, const int* prow, int NE, int R, int e0,
+                                           int step, int r) {
+  for (int d = 1; d < NE; d <<= 1) {
+    float tmp[EPT];
+    int any = 0;
+#pragma unroll
+    for (int k = 0; k < EPT; ++k) {
+      const int e = e0 + k * step;
+      tmp[k] = 0.f;
+      if (e >= d && e < NE && prow[e - d] == prow[e]) {
+        tmp[k] = part[(e - d) * R + r];
+        any = 1;
+      }
+    }
+    if (!__syncthreads_or(any)) break;
+#pragma unroll
+    for (int k = 0; k < EPT; ++k) {
+      const int e = e0 + k * step;
+      if (e < NE) part[e * R + r] += tmp[k];
+    }
+    __syncthreads();
+  }
+}
+
+// Output row of copy position k.
+__device__ __forceinline__ int mttkrp_row_at(const MttkrpArgs& a, int64_t k) {
+  const int* w = reinterpret_cast<const int*>(a.rec);
+  return a.src ? __ldg(w + (int64_t)__ldg(a.src + k) * a.words + a.fmode) : __ldg(w + k * a.words);
+}
+
+// The end of a block's run, by every thread: zero its share of the rows without
+// nonzeros, merge its units' boundary partials, and, with few blocks, add the
+// rows cut by block boundaries in the block that finishes last.  `part` holds
+// the partials of the units and then their rows; ubeg the units' positions;
+// sh[0], sh[1] are scratch; sh[2], sh[3] the rows of the records before and
+// after the block's (on their way by cp.async; plan order with several blocks
+// per partition and lean copies load them here); sh[4] a flag that a wait gave
+// up; sh[5] scratch; sh[6] the block z; sh[7] whether it was told to store
+// nothing.  The entries' rows are sorted: entries without a partial hold zeros
+// and, in any order, a neighbour's row (plan order: see there).
+template <bool PLAN>
+__device__ __forceinline__ void mttkrp_finish(const MttkrpArgs& a, float* part, int* sh,
+                                                  const int64_t* ubeg) {
+  const int z = sh[6];
+  const int R = a.R, NU = a.nu;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  int* prow = reinterpret_cast<int*>(part + (size_t)2 * NU * R);  // [2 * NU]
+  const unsigned j0 = (unsigned)z * (unsigned)NU;
+  // the partition (in plan order: of a.split blocks) whose boundary rows this merge leaves
+  const int split = PLAN && a.split > 1 ? a.split : 1;
+  const int zp = z / split, nparts = a.nblocks / split;
+  int64_t K0 = ubeg[0], K1 = ubeg[NU];
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (a.src && threadIdx.x < 2) {
+    const int64_t k = threadIdx.x ? K1 : K0 - 1;
+    sh[2 + threadIdx.x] = k >= 0 && k < a.nnz ? mttkrp_row_at(a, k) : -1;
+  }
+  // this block's share of the rows without nonzeros
+  if (a.rowmask && !sh[7]) {
+    const int64_t words = (a.I + 31) / 32;
+    zero_empty_rows_body(a.rowmask, a.I, R, a.out, words * z / a.nblocks + warp,
+                         words * (z + 1) / a.nblocks, nwarps, lane);
+  }
+  __syncthreads();
+
+  // ---- merge of the unit-boundary partials ----------------------------------
+  // Entries e = 2u (first row of unit u) and 2u+1 (its distinct last row) in
+  // copy order; every run of equal rows is one group.
+  int NE = 2 * NU;
+  if (PLAN && split > 1) {
+    // a partition shared by blocks: its merge is the last block's
+    float* gp = a.upart + (int64_t)j0 * 2 * R;
+    int* gr = a.urow + (int64_t)j0 * 2;
+    for (int x = threadIdx.x; x < NE * R; x += blockDim.x) gp[x] = part[x];
+    for (int e = threadIdx.x; e < NE; e += blockDim.x) gr[e] = prow[e];
+    if (!block_is_last(&a.pdone[zp], split, &sh[5])) return;
+    K0 = mttkrp_unit_begin(a, (unsigned)(zp * split) * NU);
+    K1 = mttkrp_unit_begin(a, (unsigned)((zp + 1) * split) * NU);
+    if (threadIdx.x < 2) {
+      const int64_t k = threadIdx.x ? K1 : K0 - 1;
+      sh[2 + threadIdx.x] = k >= 0 && k < a.nnz ? mttkrp_row_at(a, k) : -1;
+    }
+    NE *= split;
+    prow = reinterpret_cast<int*>(part + (size_t)NE * R);
+    gp = a.upart + (int64_t)zp * NE * R;
+    gr = a.urow + (int64_t)zp * NE;
+    for (int x = threadIdx.x; x < NE * R; x += blockDim.x) part[x] = __ldcg(gp + x);
+    for (int e = threadIdx.x; e < NE; e += blockDim.x) prow[e] = __ldcg(gr + e);
+    // another block of the partition may have given up
+    if (threadIdx.x == 0 && (*(volatile int*)a.err & DEV_ERR_TIMEOUT)) sh[4] = 1;
+    __syncthreads();
+  }
+  int* meta = a.cta_meta + 4 * zp;
+  if (K1 == K0 || sh[4]) {
+    if (threadIdx.x == 0) { meta[0] = -1; meta[1] = -1; meta[2] = META_EMPTY; meta[3] = 0; }
+  } else {
+    const int estep = blockDim.x / R, r = threadIdx.x % R;
+    const int eq = threadIdx.x < estep * R ? threadIdx.x / R : NE;  // none for a leftover thread
+    // Plan order: rows of missing entries = that of the last real entry before
+    // (-1 before any), by a running maximum.
+    if constexpr (PLAN) {
+      if (warp == 0) {
+        int m = -1;
+        const int per = (NE + 31) / 32;
+        const int e0 = lane * per;
+        for (int e = e0; e < e0 + per && e < NE; ++e) m = max(m, prow[e]);
+        int incl = m;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(SPM_FULL_MASK, incl, o);
+          if (lane >= o) incl = max(incl, t);
+        }
+        int run = __shfl_up_sync(SPM_FULL_MASK, incl, 1);
+        if (lane == 0) run = -1;
+        for (int e = e0; e < e0 + per && e < NE; ++e) {
+          const int row = prow[e];
+          if (run < 0 && row >= 0) sh[0] = row;  // the partition's first row
+          run = max(run, row);
+          prow[e] = run;
+        }
+      }
+      __syncthreads();
+    }
+    const int F = PLAN ? sh[0] : prow[0], L = prow[NE - 1];
+    const bool shared_prev = K0 > 0 && sh[2] == F;
+    const bool shared_next = K1 < a.nnz && sh[3] == L;
+    float* part0 = a.cta_part + (int64_t)(2 * zp) * R;
+    float* part1 = part0 + R;
+    auto row_dst = [&](int row) -> float* {
+      if (row == F && shared_prev) return part0;
+      if (row == L && shared_next) return part1;
+      return a.out + (int64_t)row * R;
+    };
+    if constexpr (PLAN) {
+      // inclusive segmented scan (Hillis-Steele), as many rounds as the longest
+      // group takes: each group's total ends on its last entry
+      if (estep * 9 >= NE) merge_scan<9>(part, prow, NE, R, eq, estep, r);
+      else merge_scan<18>(part, prow, NE, R, eq, estep, r);  // 512 threads, R <= 64
+      for (int e = eq; e < NE; e += estep) {
+        const int row = prow[e];
+        if (row < 0 || (e + 1 < NE && prow[e + 1] == row)) continue;
+        row_dst(row)[r] = part[e * R + r];
+      }
+    } else {
+      // Any order: a thread adds the runs inside 8 entries of one rank; a run
+      // that leaves its 8 is added up from its pieces, each kept at the first
+      // entry of its 8 (or where the run begins).  (A scan over all entries, 2
+      // log2(NE) barriers, was most of the time of a block with few nonzeros
+      // and 3% of the largest.)
+      constexpr int C = 8;
+      for (int c0 = eq * C; c0 < NE; c0 += estep * C) {
+        int rw[C];
+        float v[C];
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+          rw[i] = c0 + i < NE ? prow[c0 + i] : -2;
+          v[i] = c0 + i < NE ? part[(c0 + i) * R + r] : 0.f;
+        }
+        const int next = c0 + C < NE ? prow[c0 + C] : -1, prev = c0 > 0 ? prow[c0 - 1] : -1;
+#pragma unroll
+        for (int i = C - 1; i > 0; --i)
+          if (rw[i] == rw[i - 1]) v[i - 1] += v[i];
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+          if (rw[i] < 0 || (i > 0 && rw[i] == rw[i - 1])) continue;  // a run begins in these 8 here
+          if ((i == 0 && rw[0] == prev) || rw[i] == next) part[(c0 + i) * R + r] = v[i];
+          else row_dst(rw[i])[r] = v[i];
+        }
+      }
+      __syncthreads();
+      for (int c0 = eq * C; c0 + C < NE; c0 += estep * C) {
+        const int next = prow[c0 + C];
+        int b = c0 + C - 1;  // first entry, among these 8, of a run that leaves them
+        if (prow[b] != next) continue;
+        while (b > c0 && prow[b - 1] == next) --b;
+        if (b == c0 && c0 > 0 && prow[c0 - 1] == next) continue;  // it began before
+        float s = part[b * R + r];
+        for (int q = c0 + C; q < NE && prow[q] == next; q += 4 * C) {
+          float v[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int p = q + i * C;
+            v[i] = p < NE && prow[p] == next ? part[p * R + r] : 0.f;
+          }
+          s += (v[0] + v[1]) + (v[2] + v[3]);
+        }
+        row_dst(next)[r] = s;
+      }
+    }
+    if (threadIdx.x == 0) {
+      int flags = (shared_prev ? META_SHARED_PREV : 0) | (shared_next ? META_SHARED_NEXT : 0);
+      if (shared_prev) flags |= META_PART0;
+      if (shared_next && !(F == L && shared_prev)) flags |= META_PART1;
+      meta[0] = F; meta[1] = L; meta[2] = flags; meta[3] = 0;
+    }
+  }
+  // ---- rows cut by partition boundaries: the block that finishes last -------
+  if (!a.done || nparts == 1 || !block_is_last(a.done, nparts, &sh[5])) return;
+  for (int q = warp; q < nparts; q += nwarps)
+    mttkrp_fixup_body(a.cta_part, a.cta_meta, nparts, R, a.out, q, lane);
+}
+
 // NIN > 0: exactly NIN input modes.  NIN == 0: runtime a.nin (six or more
 // modes); the first two input modes are batched, further ones are fetched
 // when the step is computed.
 //
-// mttkrp_partition processes partition z of one mode copy with the whole
-// thread block (every thread must call it); it is the body of the
-// single-tensor kernel and of the batched persistent kernel.
+// mttkrp_partition processes block z of one mode copy with the whole thread
+// block (every thread must call it; any number of warps); it is the body of
+// the single-tensor kernel and of the batched persistent kernel.
 // Words of a mode-0 record rearranged into the mode-d order: word d moves to
 // the front, words 0..d-1 one place back (the other modes stay ascending).
 template <int W>
@@ -243,7 +597,7 @@ __device__ __forceinline__ void rotate_to_front(int (&w)[W], int d) {
   w[0] = cd;
 }
 
-template <int RI, int NIN, typename FT, int VEC, int LPN, int CPL, bool LEAN = false>
+template <int RI, int NIN, typename FT, int VEC, int LPN, int CPL, bool LEAN = false, bool PLAN = false>
 __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int z) {
   using S = Slice<FT, VEC>;
   constexpr int RAWN = S::RAWN;
@@ -265,21 +619,21 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
 #endif
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int next_unit;
-  __shared__ int aborted;  // some warp gave up on a record copy: no merge, no stores
+  __shared__ int64_t ubeg[MT_MAX_UNITS + 1];  // copy positions at which the block's units begin
+  __shared__ int edge[8];    // see mttkrp_finish
+  int& aborted = edge[4];    // some warp gave up on a record copy: no merge, no stores
 
   const int R = a.R;
   const int NU = a.nu;
   const int nin = NIN > 0 ? NIN : a.nin;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int slot = lane / LPN, sub = lane % LPN;
-  const int64_t* uoff = a.woff + (int64_t)z * NU;
-  const int64_t K0 = uoff[0], K1 = uoff[NU];
-
+  const int nwarps = blockDim.x >> 5;
   unsigned char* stages = smem + (size_t)warp * MT_STAGES * tile_bytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)MT_WARPS * MT_STAGES * tile_bytes) +
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)nwarps * MT_STAGES * tile_bytes) +
                    warp * MT_STAGES;
-  float* part = reinterpret_cast<float*>(smem + (size_t)MT_WARPS * MT_STAGES * tile_bytes +
-                                         (size_t)MT_WARPS * MT_STAGES * sizeof(uint64_t));
+  float* part = reinterpret_cast<float*>(smem + (size_t)nwarps * MT_STAGES * tile_bytes +
+                                         (size_t)nwarps * MT_STAGES * sizeof(uint64_t));
   int* prow = reinterpret_cast<int*>(part + (size_t)2 * NU * R);  // [2 * NU]
 
   auto row_at = [&](int64_t k) -> int {
@@ -314,16 +668,31 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
     for (int st = 0; st < MT_STAGES; ++st) mbar_init(&bars[st], 1);
     fence_mbar_init();
   }
+  for (int u = threadIdx.x; u <= NU; u += blockDim.x)
+    ubeg[u] = mttkrp_unit_begin(a, (unsigned)z * (unsigned)NU + u);
   if (threadIdx.x == 0) {
-    next_unit = MT_WARPS;
+    next_unit = nwarps;
     aborted = (a.guard && *(volatile const int*)a.guard) ? 1 : 0;
+    edge[6] = z;
+    edge[7] = aborted;
   }
   __syncthreads();
+  if constexpr (!LEAN) {
+    // rows of the records before and after the block's, for the merge
+    if (threadIdx.x < 2 && (!PLAN || a.split <= 1)) {
+      const int64_t k = threadIdx.x ? ubeg[NU] : ubeg[0] - 1;
+      if (k >= 0 && k < a.nnz)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(&edge[2 + threadIdx.x])),
+                     "l"(a.rec + k * RI)
+                     : "memory");
+      else
+        edge[2 + threadIdx.x] = -1;
+    }
+  }
   const uint32_t wait_polls = a.wait_limit == 0u ? (1u << 24) : (a.wait_limit == ~0u ? 0u : a.wait_limit);
 
   int seq_issued = 0;    // ring sequence: tiles issued by this warp so far
   bool timeout = false;
-  const bool skip = aborted != 0;  // guard set: no unit is taken, no copy issued
 
   auto slot_reduce = [&](float (&x)[CPL][VEC]) {
 #pragma unroll
@@ -334,8 +703,8 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
         for (int e = 0; e < VEC; ++e) x[c][e] += __shfl_xor_sync(SPM_FULL_MASK, x[c][e], o);
   };
 
-  for (int u = warp; u < NU && !timeout && !skip;) {
-    const int64_t k0 = uoff[u], k1 = uoff[u + 1];
+  for (int u = edge[7] ? NU : warp; u < NU && !timeout;) {  // guard set: no unit, no copy
+    const int64_t k0 = ubeg[u], k1 = ubeg[u + 1];
     const int lenw = (int)(k1 - k0);
     float* pf = part + (size_t)(2 * u) * R;
     float* pl = pf + R;
@@ -821,14 +1190,17 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
         for (int r = lane; r < R; r += 32) pl[r] = 0.f;
       if (lane == 0) {
         prow[2 * u] = first_row;
-        prow[2 * u + 1] = distinct_last ? cur : -1;
+        prow[2 * u + 1] = distinct_last ? cur : (PLAN ? -1 : first_row);
       }
       seq_issued = seq0 + ntiles;
     } else {
       for (int r = lane; r < 2 * R; r += 32) pf[r] = 0.f;
       if (lane == 0) {
-        prow[2 * u] = -1;
-        prow[2 * u + 1] = -1;
+        // any order: the row of the next record of the block (else of the last)
+        int row = -1;
+        if (!PLAN && ubeg[NU] > ubeg[0]) row = row_at(k0 < ubeg[NU] ? k0 : k0 - 1);
+        prow[2 * u] = row;
+        prow[2 * u + 1] = row;
       }
     }
     int nu_next = 0;
@@ -839,174 +1211,12 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
 #pragma unroll
     for (int st = 0; st < MT_STAGES; ++st) mbar_inval(&bars[st]);
   }
-  __syncthreads();
-
-  // ---- block merge of the unit-boundary partials ---------------------------
-  // Entries e = 2u (first row of unit u) and 2u+1 (its distinct last row) in
-  // copy order.  Missing entries take the row of the entry before them with a
-  // zero value, so rows stay sorted and every run of equal rows is one group.
-  // An inclusive segmented scan (Hillis-Steele, fixed order) leaves each
-  // group's total on its last entry.
-  int* meta = a.cta_meta + 4 * z;
-  const int64_t len = K1 - K0;
-  if (len == 0 || aborted) {
-    if (threadIdx.x == 0) { meta[0] = -1; meta[1] = -1; meta[2] = META_EMPTY; meta[3] = 0; }
-    return;
-  }
-  const int NE = 2 * NU;  // <= 256
-  // rows of missing entries (value already zero): running maximum of the
-  // entries so far, i.e. the row of the last real entry (-1 before any)
-  if (warp == 0) {
-    int m = -1;
-    const int per = (NE + 31) / 32;
-    const int e0 = lane * per;
-    for (int e = e0; e < e0 + per && e < NE; ++e) m = max(m, prow[e]);
-    int incl = m;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(SPM_FULL_MASK, incl, o);
-      if (lane >= o) incl = max(incl, t);
-    }
-    int run = __shfl_up_sync(SPM_FULL_MASK, incl, 1);
-    if (lane == 0) run = -1;
-    for (int e = e0; e < e0 + per && e < NE; ++e) {
-      run = max(run, prow[e]);
-      prow[e] = run;
-    }
-  }
-  __syncthreads();
-  // inclusive segmented scan of the partials, rows as segment keys
-  // NE * R <= 8192 for every rank (units per partition = clamp(4096/R, 16, 128))
-  constexpr int MERGE_PER_THREAD = (8192 + MT_THREADS - 1) / MT_THREADS;
-  for (int d = 1; d < NE; d <<= 1) {
-    float tmp[MERGE_PER_THREAD];
-    int cnt = 0;
-    for (int x = threadIdx.x; x < NE * R && cnt < MERGE_PER_THREAD; x += MT_THREADS, ++cnt) {
-      const int e = x / R;
-      tmp[cnt] = (e >= d && prow[e - d] == prow[e]) ? part[x - d * R] : 0.f;
-    }
-    __syncthreads();
-    cnt = 0;
-    for (int x = threadIdx.x; x < NE * R && cnt < MERGE_PER_THREAD; x += MT_THREADS, ++cnt)
-      part[x] += tmp[cnt];
-    __syncthreads();
-  }
-  // each group's last entry holds the group total
-  const int F = row_at(K0);
-  const int L = row_at(K1 - 1);
-  const bool shared_prev = K0 > 0 && row_at(K0 - 1) == F;
-  const bool shared_next = K1 < a.nnz && row_at(K1) == L;
-  float* part0 = a.cta_part + (int64_t)(2 * z) * R;
-  float* part1 = part0 + R;
-  for (int x = threadIdx.x; x < NE * R; x += MT_THREADS) {
-    const int e = x / R, r = x % R;
-    const int row = prow[e];
-    if (row < 0 || (e + 1 < NE && prow[e + 1] == row)) continue;
-    float* dst;
-    if (row == F && shared_prev) dst = part0;
-    else if (row == L && shared_next) dst = part1;
-    else dst = a.out + (int64_t)row * R;
-    dst[r] = part[x];
-  }
-  if (threadIdx.x == 0) {
-    int flags = (shared_prev ? META_SHARED_PREV : 0) | (shared_next ? META_SHARED_NEXT : 0);
-    if (shared_prev) flags |= META_PART0;
-    if (shared_next && !(F == L && shared_prev)) flags |= META_PART1;
-    meta[0] = F; meta[1] = L; meta[2] = flags; meta[3] = 0;
-  }
+  mttkrp_finish<PLAN>(a, part, edge, ubeg);
 }
 
-// Partition fix-up for partition z, one warp (lane = its lane): if z holds
-// the start of a row that continues into later partitions (its last-row
-// partial), add the first-row partials of the following partitions in
-// partition order and store the row.
-__device__ __forceinline__ void mttkrp_fixup_body(const float* __restrict__ cta_part,
-                                                  const int* __restrict__ cta_meta, int kappa,
-                                                  int R, float* __restrict__ out, int z, int lane) {
-  const int* m = cta_meta + 4 * z;
-  if (!(m[2] & META_PART1)) return;
-  const int row = m[1];
-  float s[8];
-  const float* p1 = cta_part + (int64_t)(2 * z + 1) * R;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int r = lane + 32 * j;
-    s[j] = r < R ? p1[r] : 0.f;
-  }
-  // The partitions after z that continue `row`, in order; their metadata and
-  // partials are loaded FQ at a time ahead of the (ordered) additions, so a
-  // head row cut into many partitions does not pay one load latency each.
-  constexpr int FQ = 4;
-  bool more = true;
-  for (int q0 = z + 1; q0 < kappa && more; q0 += FQ) {
-    int4 mq[FQ];
-    float pq[FQ][8];
-#pragma unroll
-    for (int k = 0; k < FQ; ++k) {
-      const int q = q0 + k;
-      mq[k] = q < kappa ? *reinterpret_cast<const int4*>(cta_meta + 4 * q) : make_int4(-1, -1, 0, 0);
-      const float* p0 = cta_part + (int64_t)(2 * (q < kappa ? q : z)) * R;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int r = lane + 32 * j;
-        pq[k][j] = r < R ? p0[r] : 0.f;
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < FQ; ++k) {
-      if (!more || q0 + k >= kappa) {
-        more = false;
-        continue;
-      }
-      const int fq = mq[k].z;
-      if (fq & META_EMPTY) continue;
-      if (mq[k].x != row) {
-        more = false;
-        continue;
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int r = lane + 32 * j;
-        if (r < R) s[j] += pq[k][j];
-      }
-      if (!(mq[k].y == row && (fq & META_SHARED_NEXT))) more = false;
-    }
-  }
-  float* dst = out + (int64_t)row * R;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int r = lane + 32 * j;
-    if (r < R) dst[r] = s[j];
-  }
-}
-
-// Rows of an I x R output whose bit in `mask` is clear are zeroed, for the
-// bitmap words [w0, w1) (word w covers rows 32w .. 32w+31), one word per
-// thread stepping by wstep.  Full words cost one load; an empty row is
-// cleared with 16-byte stores when R allows.
-__device__ __forceinline__ void zero_empty_rows_body(const uint32_t* __restrict__ mask, int64_t I,
-                                                     int R, float* __restrict__ out, int64_t w0,
-                                                     int64_t w1, int64_t wstep) {
-  for (int64_t w = w0; w < w1; w += wstep) {
-    uint32_t clear = ~__ldg(&mask[w]);
-    while (clear) {
-      const int b = __ffs(clear) - 1;
-      clear &= clear - 1;
-      const int64_t row = w * 32 + b;
-      if (row >= I) break;
-      float* dst = out + row * R;
-      if ((R & 3) == 0) {
-        for (int c = 0; c < R; c += 4) *reinterpret_cast<float4*>(dst + c) = make_float4(0.f, 0.f, 0.f, 0.f);
-      } else {
-        for (int c = 0; c < R; ++c) dst[c] = 0.f;
-      }
-    }
-  }
-}
-
-template <int RI, int NIN, typename FT, int VEC, int LPN, int CPL, bool LEAN = false>
-__global__ void __launch_bounds__(MT_THREADS, 1) mttkrp_kernel(const MttkrpArgs a) {
-  mttkrp_partition<RI, NIN, FT, VEC, LPN, CPL, LEAN>(a, blockIdx.x);
+template <int RI, int NIN, typename FT, int VEC, int LPN, int CPL, bool LEAN = false, bool PLAN = false>
+__global__ void __launch_bounds__(MT_THREADS, 1) mttkrp_kernel(const __grid_constant__ MttkrpArgs a) {
+  mttkrp_partition<RI, NIN, FT, VEC, LPN, CPL, LEAN, PLAN>(a, blockIdx.x);
 }
 
 }  // namespace spm

@@ -166,10 +166,13 @@ extern "C" spm_status spmttkrp_run_noalloc(int nmodes, const int64_t* dims, int6
   a.R = rank;
   a.nin = nmodes - 1;
   a.nu = nu;
+  a.nblocks = kappa;
+  a.words = 4 * record_int4s(nmodes);
+  a.nplan = (int)P;
   a.err = err;    // read back by spmttkrp_noalloc_status
   a.guard = err;  // set by the record check: the blocks store nothing
   MttkrpKernelFn fn = pick_mttkrp(bf16, nmodes - 1, rank);
-  const size_t smem = mttkrp_smem_bytes(rank, record_int4s(nmodes), nu, bf16 ? 2 : 4);
+  const size_t smem = mttkrp_smem_bytes(rank, nu, MT_WARPS);
   SPM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   fn<<<kappa, MT_THREADS, smem, s>>>(a);
   SPM_CUDA_TRY(cudaGetLastError());

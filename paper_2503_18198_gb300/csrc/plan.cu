@@ -564,6 +564,13 @@ __global__ void popc_kernel(const uint32_t* __restrict__ mask, int64_t words,
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, c);
 }
 
+int resolved_scheme(int policy, int64_t dim, int kappa) {
+  if (policy == (int)(SPM_POLICY_SCHEME2 >> 4)) return 2;
+  if (policy == (int)(SPM_POLICY_SCHEME1 >> 4)) return 1;
+  if (policy == (int)(SPM_POLICY_ADAPTIVE >> 4)) return dim >= kappa ? 1 : 2;
+  return 0;
+}
+
 int grid_for(int64_t n, int threads) {
   const int64_t b = ceil_div<int64_t>(n > 0 ? n : 1, threads);
   return (int)std::min<int64_t>(b, 152 * 32);
@@ -757,14 +764,11 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
   // ---- partitions (Sec. III-B) and work units
   const int units = p->nu;
   const int64_t P = (int64_t)p->kappa * units;
+  for (int d = 0; d < N; ++d) p->mode[d].scheme = resolved_scheme(p->policy, p->dims[d], p->kappa);
+  if (st == SPM_OK) plan_shapes(p);
   for (int d = 0; d < N && st == SPM_OK; ++d) {
     spm_mode_copy& c = p->mode[d];
-    int scheme = 0;
-    if (p->policy == (int)(SPM_POLICY_SCHEME2 >> 4)) scheme = 2;
-    if (p->policy == (int)(SPM_POLICY_SCHEME1 >> 4)) scheme = 1;
-    if (p->policy == (int)(SPM_POLICY_ADAPTIVE >> 4)) scheme = p->dims[d] >= p->kappa ? 1 : 2;
-    c.scheme = scheme;
-    if (scheme != 1 || n == 0) {
+    if (c.scheme != 1 || n == 0) {
       int64_t stride = 0;
       const int* rows = n > 0 ? copy_rows(p, d, reinterpret_cast<int*>(k64b), &stride, s) : nullptr;
       partition_copy(p, d, rows, stride, sc.hist, sc.dtot, reinterpret_cast<uint32_t*>(va), s);
@@ -848,8 +852,19 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
 
 }  // namespace
 
+void plan_shapes(spmttkrp_plan_s* p) {
+  const int sms = sm_count();
+  for (int d = 0; d < p->N; ++d) {
+    spm_mode_copy& c = p->mode[d];
+    const MttkrpShape x = mttkrp_shape(c.scheme, p->nnz, p->kappa, p->nu, sms);
+    c.kx = x.kx;
+    c.nx = x.nx;
+  }
+}
+
 void plan_bytes_estimate(int N, const int64_t* dims, int64_t nnz, int R, int kappa, bool als,
-                         bool lean, size_t* resident, size_t* transient, bool fibre, int policy) {
+                         bool lean, size_t* resident, size_t* transient, bool fibre, int policy,
+                         bool bf16) {
   // mirrors the plan_alloc calls of spmttkrp_plan, build_copies and
   // ensure_als_state (each allocation of 0 bytes counts 16)
   const int RI = record_int4s(N);
@@ -857,8 +872,9 @@ void plan_bytes_estimate(int N, const int64_t* dims, int64_t nnz, int R, int kap
   const int64_t nn = nnz > 0 ? nnz : 1;
   int64_t Imax = 1;
   for (int w = 0; w < N; ++w) Imax = std::max(Imax, dims[w]);
-  size_t b = sizeof(int) + sizeof(double);  // dev_err, normX2
-  b += sizeof(float) * 2 * (size_t)kappa * R + sizeof(int) * 4 * (size_t)kappa;
+  const size_t nb = (size_t)boundary_blocks(nnz, kappa, sm_count());
+  size_t b = 2 * sizeof(int) + sizeof(double);  // dev_err, normX2
+  b += sizeof(float) * 2 * nb * R + sizeof(int) * 4 * nb;
   b += sizeof(double) * NORM_BLOCKS;
   for (int d = 0; d < N; ++d) {
     if (lean && d > 0) {
@@ -883,6 +899,8 @@ void plan_bytes_estimate(int N, const int64_t* dims, int64_t nnz, int R, int kap
     b += sizeof(float) * 2 * RR + sizeof(double) * R * gb * 2 + sizeof(double) * 2 * R;
     b += sizeof(float) * R * gb + als_wdig_bytes(R);  // column maxima of Z, W digit tiles
     b += sizeof(float) * (size_t)Imax * R * 2;
+    if (bf16 && mttkrp_split(nnz, kappa, nu, sm_count()) > 1)
+      b += (sizeof(float) * R + sizeof(int)) * 2 * (size_t)kappa * nu + sizeof(int) * (size_t)kappa;
   }
   *resident = b;
   // stream-ordered scratch of the build (keys, payloads, histograms)
@@ -910,11 +928,13 @@ spm_status plan_repartition(spmttkrp_plan_s* p, int kappa, cudaStream_t s) {
       SPM_TRY(plan_realloc(p, (void**)&p->mode[d].woff,
                            sizeof(int64_t) * ((size_t)kappa * p->nu + 1)));
     }
-    SPM_TRY(plan_realloc(p, (void**)&p->cta_part, sizeof(float) * 2 * (size_t)kappa * p->R));
-    SPM_TRY(plan_realloc(p, (void**)&p->cta_meta, sizeof(int) * 4 * (size_t)kappa));
+    const size_t nb = (size_t)boundary_blocks(p->nnz, kappa, sm_count());
+    SPM_TRY(plan_realloc(p, (void**)&p->cta_part, sizeof(float) * 2 * nb * p->R));
+    SPM_TRY(plan_realloc(p, (void**)&p->cta_meta, sizeof(int) * 4 * nb));
     p->kappa_cap = kappa;
   }
   p->kappa = kappa;
+  plan_shapes(p);
   const int64_t n = p->nnz;
   const int64_t nn = n > 0 ? n : 1;
   uint32_t *hist = nullptr, *dtot = nullptr, *before = nullptr;

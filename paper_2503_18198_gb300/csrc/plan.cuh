@@ -25,6 +25,7 @@ struct spm_mode_copy {
   int32_t* src = nullptr;    // lean copy: position in copy 0 of each copy position
   int64_t* off = nullptr;    // device int64[kappa+1] partition offsets
   int64_t* woff = nullptr;   // device int64[kappa*nu+1] work-unit offsets
+  int kx = 0, nx = 0;        // thread blocks and units per block with which the kernel runs it
   uint32_t* rowmask = nullptr;  // bit i set: output row i has a nonzero
   int64_t empty_rows = 0;    // rows without nonzeros
   int scheme = 0;            // 0 cost-balanced, 1 or 2 (Sec. III-B)
@@ -51,6 +52,12 @@ struct spm_als_state {
   double* lambda_ws = nullptr;        // R
   float* M = nullptr;                 // Imax*R MTTKRP output
   float* Z = nullptr;                 // Imax*R unnormalised update
+  // plan-order MTTKRP with several blocks per partition: unit boundary partials
+  // [kappa*nu][2][R], their rows, finished blocks per partition (else null)
+  float* upart = nullptr;
+  int* urow = nullptr;
+  int* pdone = nullptr;
+  int split_cap = 0;  // partitions those hold
   // the normal-equation systems of mode d depend only on the other modes'
   // Grams, so they are formed on a side stream while the MTTKRP of mode d runs
   cudaStream_t side = nullptr;
@@ -73,10 +80,11 @@ struct spmttkrp_plan_s {
   int policy = 0;  // SPM_POLICY_* >> 4
   spm_mode_copy mode[SPM_MAX_MODES];
   // MTTKRP workspace: per-partition boundary-row partial sums.
-  float* cta_part = nullptr;   // [kappa][2][R]
-  int* cta_meta = nullptr;     // [kappa][4]
+  float* cta_part = nullptr;   // [boundary_blocks][2][R]
+  int* cta_meta = nullptr;     // [boundary_blocks][4]
   // Device scalars.
-  int* dev_err = nullptr;      // sticky error flags (spm::DEV_ERR_*)
+  int* dev_err = nullptr;      // [0] sticky error flags (spm::DEV_ERR_*), [1] finished blocks
+                               // of the running MTTKRP (zero between runs)
   double* normX2 = nullptr;    // |X|_F^2 (duplicates summed)
   double* norm_part = nullptr; // partials for normX2
   spm_als_state als;
@@ -91,8 +99,8 @@ struct spmttkrp_plan_s {
   // set ~0u so the first wait gives up at once)
   uint32_t wait_limit = 0;
   // allocation bookkeeping
-  void* allocs[64] = {};
-  size_t alloc_bytes[64] = {};
+  void* allocs[96] = {};
+  size_t alloc_bytes[96] = {};
   int nallocs = 0;
 };
 
@@ -127,7 +135,55 @@ inline int fibre_slots(int R) {
 // (transient scratch), for the given shape.
 void plan_bytes_estimate(int N, const int64_t* dims, int64_t nnz, int R, int kappa, bool als,
                          bool lean, size_t* resident, size_t* transient, bool fibre = false,
-                         int policy = 0);
+                         int policy = 0, bool bf16 = false);
+
+// Thread blocks and work units per block with which a record copy of nnz
+// nonzeros is run.  The partitions B_{d,z} that the caller sees (kappa, nu)
+// are kept where they are large enough to fill a block of 32 warps; otherwise
+// the copy is cut for the device:
+//  * a block per 1024 nonzeros up to two per SM.  One tensor of 4,096
+//    nonzeros on the default 304 partitions of 128 units ran 31 us per mode
+//    (cold caches), 300,000 nonzeros 50 us; in this shape 14 and 11 us;
+//  * units of at least 128 nonzeros (two record tiles), 16 to nu per block.
+// The kernel reads its unit boundaries off the plan's: unit j of kx * nx begins
+// j / (kx * nx) of the way through the plan's units, inside one by its length.
+// Scheme 1 keeps its partitions: their rows are not in order across them.
+struct MttkrpShape {
+  int kx, nx;
+};
+inline int mttkrp_fine_blocks(int64_t nnz, int sms) {
+  const int64_t b = (nnz + 1023) / 1024;
+  return (int)(b < 1 ? 1 : b > 2 * sms ? 2 * sms : b);
+}
+inline MttkrpShape mttkrp_shape(int scheme, int64_t nnz, int kappa, int nu, int sms) {
+  if (scheme == 1) return {kappa, nu};
+  const int fine = mttkrp_fine_blocks(nnz, sms);
+  const int kx = kappa >= fine && nnz / kappa >= 4096 ? kappa : fine;
+  int nx = 16;
+  while (2 * nx <= nu && nnz / kx >= (int64_t)nx * 256) nx *= 2;
+  return {kx, nx};
+}
+// Blocks per partition of a run in plan order (BF16 CP-ALS, see run_mttkrp): a
+// partition's units are shared by up to nu / 16 blocks (16 warps take one each)
+// while there are fewer than two blocks per SM and 1024 nonzeros for each.
+inline int mttkrp_split(int64_t nnz, int kappa, int nu, int sms) {
+  int s = 1;
+  while (32 * s <= nu && nu % (2 * s) == 0 && kappa * s < 2 * sms && nnz / kappa >= 2048 * (int64_t)s) s *= 2;
+  return s;
+}
+
+// Warps of a block: short unit lists leave half of the SM to a second block,
+// whose start and merge overlap the first one's gathers.
+inline int mttkrp_warps(int nx) { return nx >= 32 ? 32 : 16; }
+
+// Blocks for which boundary partials are held.
+inline int boundary_blocks(int64_t nnz, int kappa, int sms) {
+  const int fine = mttkrp_fine_blocks(nnz, sms);
+  return kappa > fine ? kappa : fine;
+}
+
+// Set every copy's kx and nx from the plan's kappa.
+void plan_shapes(spmttkrp_plan_s* p);
 
 // P2 again for a new partition count (cost-balanced and Scheme 2 policies).
 spm_status plan_repartition(spmttkrp_plan_s* p, int kappa, cudaStream_t s);
@@ -137,8 +193,16 @@ spm_status build_copies(spmttkrp_plan_s* p, const int32_t* const* idx,
                         const float* vals, cudaStream_t s);
 
 // P3 + P4: one MTTKRP launch sequence for mode d (mttkrp.cu).
+// plan_order (BF16 factors, R <= 64): sum in the order that the plan's
+// partitions define, whatever the launch shape.  A decomposition with BF16 factors asks for it: each update is
+// rounded to 8 bits, so one flipped last bit of M becomes another factor, and a
+// result would depend on how the device is filled.
 spm_status run_mttkrp(spmttkrp_plan_s* p, int mode, const void* const* factors,
-                      float* out, cudaStream_t s);
+                      float* out, cudaStream_t s, bool plan_order = false);
+
+// The launch shape and plan-order fields of `a` for mode d of plan p.
+struct MttkrpArgs;
+void mttkrp_set_shape(const spmttkrp_plan_s* p, int d, bool plan_order, MttkrpArgs* a);
 
 // P6: one CP-ALS sweep (als.cu).
 spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda,
