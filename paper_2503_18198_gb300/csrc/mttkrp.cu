@@ -24,7 +24,28 @@ MttkrpKernelFn pick_mttkrp_bf16_lean(int nin, int R);
 spm_status launch_mttkrp_fibre(spmttkrp_plan_s* p, int mode, const void* const* factors,
                                float* out, cudaStream_t s);  // mttkrp_fibre.cu
 
+MttkrpKernelFn pick_mttkrp_f32_between3(int R);
+MttkrpKernelFn pick_mttkrp_f32_between4(int R);
+MttkrpKernelFn pick_mttkrp_f32_between5(int R);
+MttkrpKernelFn pick_mttkrp_bf16_between3(int R);
+MttkrpKernelFn pick_mttkrp_bf16_between4(int R);
+MttkrpKernelFn pick_mttkrp_bf16_between5(int R);
+
+// 3 to 5 modes and a rank without a fast shape: the shape between, or null.
+static MttkrpKernelFn pick_mttkrp_between(bool bf16, int nin, int R) {
+  const int W = bf16 ? 8 : 4, l = R / W;
+  const bool fast = (R % W == 0 && l <= 64 && (l & (l - 1)) == 0) || (bf16 && nin == 2 && R == 4);
+  if (fast) return nullptr;
+  switch (nin) {
+    case 2: return bf16 ? pick_mttkrp_bf16_between3(R) : pick_mttkrp_f32_between3(R);
+    case 3: return bf16 ? pick_mttkrp_bf16_between4(R) : pick_mttkrp_f32_between4(R);
+    case 4: return bf16 ? pick_mttkrp_bf16_between5(R) : pick_mttkrp_f32_between5(R);
+    default: return nullptr;
+  }
+}
+
 MttkrpKernelFn pick_mttkrp(bool bf16, int nin, int R) {
+  if (MttkrpKernelFn fn = pick_mttkrp_between(bf16, nin, R)) return fn;
   if (nin == 4) return bf16 ? pick_mttkrp_bf16_c(R) : pick_mttkrp_f32_c(R);
   if (bf16) return nin <= 2 ? pick_mttkrp_bf16_a(nin, R) : pick_mttkrp_bf16_b(nin, R);
   return nin <= 2 ? pick_mttkrp_f32_a(nin, R) : pick_mttkrp_f32_b(nin, R);

@@ -1,0 +1,6 @@
+// BF16-factor MTTKRP instantiations for ranks between the fast shapes, 3 modes.
+#include "mttkrp_inst.cuh"
+
+namespace spm {
+MttkrpKernelFn pick_mttkrp_bf16_between3(int R) { return pick_mttkrp_between_t<__nv_bfloat16, 2>(R); }
+}  // namespace spm

@@ -1,0 +1,6 @@
+// F32-factor MTTKRP instantiations for ranks between the fast shapes, 4 modes.
+#include "mttkrp_inst.cuh"
+
+namespace spm {
+MttkrpKernelFn pick_mttkrp_f32_between4(int R) { return pick_mttkrp_between_t<float, 3>(R); }
+}  // namespace spm

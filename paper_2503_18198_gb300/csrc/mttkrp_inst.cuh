@@ -13,8 +13,41 @@ using MttkrpKernelFn = void (*)(const MttkrpArgs);
 #define SPM_MT_NARROW 0
 #endif
 
+// Ranks between the fast shapes: VEC ranks per lane (a divisor of R that keeps
+// every lane's load aligned), the lanes padded to a power of two and masked, so
+// that a warp step still holds 32 / LPN nonzeros.  Odd ranks take one rank per
+// lane.  (2M nonzeros, R = 24, FP32, three modes: 652 us with one nonzero per
+// step and eight chunks of 32 ranks, 158 us so; R = 10, 48, 100 with 3 modes: 253,
+// 280, 335 us per mode against 43, 72, 112.)
+template <typename FT, int NIN>
+MttkrpKernelFn pick_mttkrp_between_t(int R) {
+  constexpr int RI = record_int4s(NIN + 1);
+  if constexpr (sizeof(FT) == 2) {
+    if (R % 8 == 0 && R > 32) {
+      if (R <= 64) return &mttkrp_kernel<RI, NIN, FT, 8, 8, 1, false, false, true>;
+      if (R <= 128) return &mttkrp_kernel<RI, NIN, FT, 8, 16, 1, false, false, true>;
+      return &mttkrp_kernel<RI, NIN, FT, 8, 32, 1, false, false, true>;
+    }
+  }
+  if (R % 4 == 0 && R <= 128) {
+    if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 4, 8, 1, false, false, true>;
+    if (R <= 64) return &mttkrp_kernel<RI, NIN, FT, 4, 16, 1, false, false, true>;
+    return &mttkrp_kernel<RI, NIN, FT, 4, 32, 1, false, false, true>;
+  }
+  if (R % 2 == 0 && R <= 64) {
+    if (R <= 16) return &mttkrp_kernel<RI, NIN, FT, 2, 8, 1, false, false, true>;
+    if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 2, 16, 1, false, false, true>;
+    return &mttkrp_kernel<RI, NIN, FT, 2, 32, 1, false, false, true>;
+  }
+  if (R <= 16) return &mttkrp_kernel<RI, NIN, FT, 1, 16, 1>;
+  if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 1, 32, 1>;
+  if (R <= 64) return &mttkrp_kernel<RI, NIN, FT, 1, 32, 2>;
+  return nullptr;
+}
+
 // Fast shapes: the rank is VEC * LPN * CPL with one 16-byte load per lane
-// and chunk.  Anything else uses the scalar variant (one nonzero per step).
+// and chunk.  Anything else uses the scalar variant (one nonzero per step)
+// unless pick_mttkrp_between_t has a shape for it.
 template <typename FT, int NIN, bool LEAN = false, bool PLAN = false>
 MttkrpKernelFn pick_mttkrp_t(int R) {
   constexpr int RI = record_int4s(NIN > 0 ? NIN + 1 : SPM_MAX_MODES);
@@ -56,6 +89,10 @@ MttkrpKernelFn pick_mttkrp_t(int R) {
         default: break;
       }
     }
+  }
+  if constexpr (PLAN) {  // the scalar variant's order with the chunks that R fills
+    if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 1, 32, 1, LEAN, PLAN>;
+    return &mttkrp_kernel<RI, NIN, FT, 1, 32, 2, LEAN, PLAN>;
   }
   return &mttkrp_kernel<RI, NIN, FT, 1, 32, 8, LEAN, PLAN>;
 }

@@ -204,6 +204,34 @@ struct Slice<__nv_bfloat16, 4> {
   }
 };
 
+// Two ranks per lane, for even ranks that are no multiple of 4.
+template <>
+struct Slice<float, 2> {
+  static constexpr int RAWN = 2;
+  static __device__ __forceinline__ void load(const void* base, int64_t row, int R, int r0,
+                                              uint32_t* raw) {
+    const uint2 x = __ldg(reinterpret_cast<const uint2*>(static_cast<const float*>(base) + row * R + r0));
+    raw[0] = x.x; raw[1] = x.y;
+  }
+  static __device__ __forceinline__ void cvt(const uint32_t* raw, float* f) {
+    f[0] = __uint_as_float(raw[0]);
+    f[1] = __uint_as_float(raw[1]);
+  }
+};
+
+template <>
+struct Slice<__nv_bfloat16, 2> {
+  static constexpr int RAWN = 1;
+  static __device__ __forceinline__ void load(const void* base, int64_t row, int R, int r0,
+                                              uint32_t* raw) {
+    raw[0] = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const __nv_bfloat16*>(base) + row * R + r0));
+  }
+  static __device__ __forceinline__ void cvt(const uint32_t* raw, float* f) {
+    f[0] = __uint_as_float(raw[0] << 16);
+    f[1] = __uint_as_float(raw[0] & 0xFFFF0000u);
+  }
+};
+
 template <>
 struct Slice<float, 1> {
   static constexpr int RAWN = 1;
@@ -597,7 +625,8 @@ __device__ __forceinline__ void rotate_to_front(int (&w)[W], int d) {
   w[0] = cd;
 }
 
-template <int RI, int NIN, typename FT, int VEC, int LPN, int CPL, bool LEAN = false, bool PLAN = false>
+template <int RI, int NIN, typename FT, int VEC, int LPN, int CPL, bool LEAN = false, bool PLAN = false,
+          bool MASK = false>
 __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int z) {
   using S = Slice<FT, VEC>;
   constexpr int RAWN = S::RAWN;
@@ -644,6 +673,11 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
       return __ldg(&a.rec[k * RI].x);
   };
   auto rank0 = [&](int c) -> int { return (c * LPN + sub) * VEC; };
+  // MASK: R < VEC * LPN is a multiple of VEC; the lanes beyond it repeat the
+  // last lane's ranks and store nothing.
+  static_assert(!MASK || (CPL == 1 && !LEAN && !PLAN), "masked ranks: one chunk");
+  const bool store_lane = !MASK || rank0(0) < R;
+  auto load_rank = [&](int c) -> int { return MASK ? min(rank0(c), R - VEC) : rank0(c); };
   // Vector path with the rank fixed at compile time (R == VEC * LPN * CPL):
   // full steps are processed without per-step predication, gathers address
   // rows with a constant stride from per-lane base pointers.
@@ -656,12 +690,15 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
   constexpr bool P32 = std::is_same<FT, float>::value;
   constexpr bool PAIRS = FAST && ((P32 && SPM_MT_PAIRS && LANE_BYTES == 16) ||
                                   (!P32 && SPM_MT_PAIRS_BF16));
+  // elements between rows, in units of a lane's load (the rank is a compile-
+  // time constant unless lanes are masked)
   constexpr int RT = VEC * LPN * CPL;
+  const unsigned rstride = MASK ? (unsigned)R / VEC : (unsigned)(RT / VEC);
   constexpr int NINF = NIN > 0 ? NIN : 1;
   const LdT* facb[NINF];
 #pragma unroll
   for (int m = 0; m < NINF; ++m)
-    facb[m] = reinterpret_cast<const LdT*>(static_cast<const FT*>(a.fac[m]) + sub * VEC);
+    facb[m] = reinterpret_cast<const LdT*>(static_cast<const FT*>(a.fac[m]) + load_rank(0));
 
   if (lane == 0) {
 #pragma unroll
@@ -751,7 +788,8 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
       auto put_row = [&](int row, const float (&x)[CPL][VEC]) {
         float* dst = row == first_row ? pf : a.out + (int64_t)row * R;
 #pragma unroll
-        for (int c = 0; c < CPL; ++c) store_vec<VEC>(dst, R, rank0(c), x[c]);
+        for (int c = 0; c < CPL; ++c)
+          if (store_lane) store_vec<VEC>(dst, R, rank0(c), x[c]);
       };
 
       // Fold one step's contributions v (rows `row`, empty slots already on
@@ -890,7 +928,7 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
 #pragma unroll
                 for (int c = 0; c < CPL; ++c) {
                   const LdT* src =
-                      facb[m] + (size_t)(uint32_t)w[uu][1 + m] * (RT * sizeof(FT) / sizeof(LdT)) + c * LPN;
+                      facb[m] + (size_t)(uint32_t)w[uu][1 + m] * rstride + c * LPN;
                   if constexpr (P32) {
                     const ulonglong2 x = ld_nc_v2_u64(src);
                     y[uu][m][c][0] = x.x;
@@ -1000,7 +1038,7 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
                   if (m == 0 && !fresh0[uu]) continue;  // taken from the previous step below
 #endif
                   const LdT* src = facb[m] +
-                                   (size_t)(uint32_t)w[uu][1 + m] * (RT * sizeof(FT) / sizeof(LdT)) +
+                                   (size_t)(uint32_t)w[uu][1 + m] * rstride +
                                    c * LPN;
                   if constexpr (LANE_BYTES == 16) {
 #if SPM_L2_HINTS
@@ -1118,7 +1156,7 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
                 for (int i = 0; i < RAWN; ++i) y[uu][m][c][i] = 0u;
               if (valid[uu] && m < nin) {
 #pragma unroll
-                for (int c = 0; c < CPL; ++c) S::load(a.fac[m], w[uu][1 + m], R, rank0(c), y[uu][m][c]);
+                for (int c = 0; c < CPL; ++c) S::load(a.fac[m], w[uu][1 + m], R, load_rank(c), y[uu][m][c]);
               }
             }
 #pragma unroll
@@ -1153,7 +1191,7 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
                   for (int qq = 1; qq < W; ++qq)
                     if (qq == 1 + m) idx = w[uu][qq];
                   uint32_t raw[RAWN];
-                  if (valid[uu]) S::load(a.fac[m], idx, R, rank0(c), raw);
+                  if (valid[uu]) S::load(a.fac[m], idx, R, load_rank(c), raw);
                   else raw[0] = 0u;
                   S::cvt(raw, f);
 #pragma unroll
@@ -1184,7 +1222,8 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
       if (slot == 0) {
         float* dst = distinct_last ? pl : pf;
 #pragma unroll
-        for (int c = 0; c < CPL; ++c) store_vec<VEC>(dst, R, rank0(c), acc[c]);
+        for (int c = 0; c < CPL; ++c)
+          if (store_lane) store_vec<VEC>(dst, R, rank0(c), acc[c]);
       }
       if (!distinct_last)
         for (int r = lane; r < R; r += 32) pl[r] = 0.f;
@@ -1214,9 +1253,10 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
   mttkrp_finish<PLAN>(a, part, edge, ubeg);
 }
 
-template <int RI, int NIN, typename FT, int VEC, int LPN, int CPL, bool LEAN = false, bool PLAN = false>
+template <int RI, int NIN, typename FT, int VEC, int LPN, int CPL, bool LEAN = false, bool PLAN = false,
+          bool MASK = false>
 __global__ void __launch_bounds__(MT_THREADS, 1) mttkrp_kernel(const __grid_constant__ MttkrpArgs a) {
-  mttkrp_partition<RI, NIN, FT, VEC, LPN, CPL, LEAN, PLAN>(a, blockIdx.x);
+  mttkrp_partition<RI, NIN, FT, VEC, LPN, CPL, LEAN, PLAN, MASK>(a, blockIdx.x);
 }
 
 }  // namespace spm

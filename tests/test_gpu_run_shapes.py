@@ -70,3 +70,27 @@ def test_bf16_sweep_with_shared_partitions(R, kappa):
         torch.cuda.synchronize()
         for d in range(3):
             assert np.array_equal(fac2[d].float().cpu().numpy(), fac[d])
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("R", [1, 2, 6, 10, 12, 17, 22, 23, 28, 33, 36, 40, 48, 62, 63, 66, 72, 100,
+                               124, 136, 248])
+@pytest.mark.parametrize("dims", [(61, 47, 33), (40, 23, 11, 7), (19, 13, 11, 5, 3)])
+def test_ranks_between_the_fast_shapes(dims, R, dtype):
+    nnz = 3001
+    g = np.random.default_rng(R)
+    idx = [(n * g.random(nnz) ** 2).astype(np.int32) for n in dims]
+    vals = g.random(nnz).astype(np.float32)
+    Y = [torch.as_tensor(f).to(dtype) for f in synth.factors(dims, R, seed=R)]
+    flags = spm.SPM_FACTOR_BF16 if dtype == torch.bfloat16 else 0
+    plan = spm.spmttkrp_plan(dims, [torch.as_tensor(c).cuda() for c in idx],
+                             torch.as_tensor(vals).cuda(), R, flags)
+    fac = [f.cuda() for f in Y]
+    for d in range(len(dims)):
+        # guard rows: nothing beyond the output is written
+        buf = torch.full((dims[d] + 8, R), 7.0, device="cuda")
+        lo = 4 if R % 4 == 0 else 0  # the output starts on a 16-byte boundary
+        out = buf[lo:lo + dims[d]]
+        spm.spmttkrp_run(plan, d, fac, out)
+        assert torch.all(buf[:lo] == 7.0) and torch.all(buf[lo + dims[d]:] == 7.0)
+        check_mode_elementwise(out.cpu().numpy(), dims, idx, vals, [f.float().numpy() for f in Y], d)
