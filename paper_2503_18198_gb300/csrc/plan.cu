@@ -6,15 +6,19 @@
 //
 // Ordering used for copy d: (c_d, then c_w for w != d in ascending w, then the
 // input position), i.e. a stable sort.  It is built with a device LSD radix
-// sort:
+// sort whose digits are slices of one coordinate, at most 10 bits each (a
+// 20-bit coordinate: two passes):
 //   * copy 0: the full lexicographic key (c_0, c_1, ..., c_{N-1}) packed into
 //     64-bit words (several words, least significant first, when the index
-//     bits exceed 64), 8-bit digits, stable passes, payload = input position;
-//   * copy d >= 1: a stable sort of copy 0 by c_d alone.  Among nonzeros with
-//     equal c_d, copy 0's order is lexicographic on the remaining modes in
-//     ascending order, which is exactly the tie-break of copy d.
+//     bits exceed 64), payload = input position; the records are decoded from
+//     the sorted keys, only the values are gathered;
+//   * copy d >= 1: a stable sort of copy 0 by c_d alone, its keys read from
+//     copy 0's records in the first pass.  Among nonzeros with equal c_d, copy
+//     0's order is lexicographic on the remaining modes in ascending order,
+//     which is exactly the tie-break of copy d.
 // Records of copy d hold [c_d, other indices ascending, value bits, padding].
 #include <algorithm>
+#include <utility>
 #include <vector>
 
 #include "plan.cuh"
@@ -22,38 +26,42 @@
 namespace spm {
 namespace {
 
-constexpr int RS_WARPS = 8;
-constexpr int RS_THREADS = RS_WARPS * 32;  // == RS_BINS (used by the scan)
+constexpr int RS_WARPS = 16;
+constexpr int RS_THREADS = RS_WARPS * 32;
 constexpr int RS_ITEMS = 16;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
-constexpr int RS_BINS = 256;
+constexpr int RS_BITS = 10;  // widest digit
+constexpr int RS_BINS = 1 << RS_BITS;
 
 struct IdxPtrs {
   const int32_t* p[SPM_MAX_MODES];
 };
 
 // ---------------------------------------------------------------------------
-// LSD radix sort of (key, int32 payload) pairs, 8 bits per pass, stable.
+// LSD radix sort of (key, int32 payload) pairs, up to 10 bits per pass, stable.
+// A pass is bound by memory: keys read for the tile histograms, pairs read and
+// written by the scatter.  The scatter ranks its tile of 8192 in registers and
+// writes it out from shared memory in digit order, so that the 8 or more pairs
+// of a digit leave as one run.  50M pairs of 64-bit keys, 10 bits: 630 us a
+// pass (8 bits straight from registers: 990 us); 32-bit keys 530 (800).
 // ---------------------------------------------------------------------------
 
 template <typename K>
 __global__ void __launch_bounds__(RS_THREADS)
-    rs_hist_kernel(const K* __restrict__ keys, int64_t n, int shift,
-                   uint32_t* __restrict__ hist, int nblocks) {
+    rs_hist_kernel(const K* __restrict__ keys, int64_t stride, int64_t n, int shift, int width,
+                   uint32_t* __restrict__ hist, int ntiles) {
   __shared__ uint32_t cnt[RS_BINS];
-  cnt[threadIdx.x] = 0;
+  const int bins = 1 << width;
+  for (int b = threadIdx.x; b < bins; b += RS_THREADS) cnt[b] = 0;
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t wbase = (int64_t)blockIdx.x * RS_TILE + (int64_t)warp * (32 * RS_ITEMS);
-#pragma unroll 4
+  const int64_t base = (int64_t)blockIdx.x * RS_TILE + threadIdx.x;
+#pragma unroll
   for (int i = 0; i < RS_ITEMS; ++i) {
-    const int64_t k = wbase + i * 32 + lane;
-    const unsigned d = k < n ? (unsigned)((keys[k] >> shift) & (RS_BINS - 1)) : RS_BINS;
-    const unsigned peers = __match_any_sync(SPM_FULL_MASK, d);
-    if (d < RS_BINS && (__ffs(peers) - 1) == lane) atomicAdd(&cnt[d], (uint32_t)__popc(peers));
+    const int64_t k = base + i * RS_THREADS;
+    if (k < n) atomicAdd(&cnt[(unsigned)(keys[k * stride] >> shift) & (bins - 1)], 1u);
   }
   __syncthreads();
-  hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = cnt[threadIdx.x];
+  for (int b = threadIdx.x; b < bins; b += RS_THREADS) hist[(int64_t)b * ntiles + blockIdx.x] = cnt[b];
 }
 
 // One block per digit: exclusive scan of hist[d][0..nblocks) in place and the
@@ -98,73 +106,141 @@ __global__ void __launch_bounds__(1024)
 }
 
 template <typename K>
-__global__ void __launch_bounds__(RS_THREADS)
-    rs_scatter_kernel(const K* __restrict__ keys_in, const int32_t* __restrict__ vals_in,
-                      K* __restrict__ keys_out, int32_t* __restrict__ vals_out, int64_t n,
-                      int shift, const uint32_t* __restrict__ hist, const uint32_t* __restrict__ dtot,
-                      int nblocks) {
-  __shared__ uint32_t wcnt[RS_WARPS][RS_BINS];
-  __shared__ uint32_t gbase[RS_BINS];
-  __shared__ uint32_t wsum[RS_WARPS];
+struct ScatterSmem {
+  K keys[RS_TILE];                       // the tile in digit order, then its payloads
+  unsigned short wcnt[RS_WARPS][RS_BINS];  // per warp and digit: count, then first place in the tile
+  uint32_t gbase[RS_BINS];               // global place of a digit's run minus its place in the tile
+};
+
+// Exclusive block scan of one value per thread.
+__device__ __forceinline__ uint32_t rs_block_exclusive(uint32_t v, uint32_t* wsum) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int t = threadIdx.x; t < RS_WARPS * RS_BINS; t += RS_THREADS) (&wcnt[0][0])[t] = 0;
-  {
-    // gbase[d] = sum_{d' < d} dtot[d'] + hist[d][block]   (block exclusive scan)
-    const uint32_t v = dtot[threadIdx.x];
-    uint32_t x = v;
+  uint32_t x = v;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t y = __shfl_up_sync(SPM_FULL_MASK, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[warp] = x;
-    __syncthreads();
-    uint32_t pre = 0;
-    for (int w = 0; w < warp; ++w) pre += wsum[w];
-    gbase[threadIdx.x] = pre + x - v + hist[(int64_t)threadIdx.x * nblocks + blockIdx.x];
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(SPM_FULL_MASK, x, o);
+    if (lane >= o) x += y;
   }
   __syncthreads();
-  K key[RS_ITEMS];
-  int32_t val[RS_ITEMS];
-  uint32_t lrank[RS_ITEMS];
+  if (lane == 31) wsum[warp] = x;
+  __syncthreads();
+  uint32_t pre = 0;
+#pragma unroll
+  for (int w = 0; w < RS_WARPS; ++w) pre += w < warp ? wsum[w] : 0u;
+  return pre + x - v;
+}
+
+// One tile: pairs (keys[k * stride], vals ? vals[k] : k) to their places by
+// digit.  hist: the tile histograms scanned along the tiles, dtot the digit
+// totals (both null: the only tile).  keys_out may be null.
+template <typename K>
+__global__ void __launch_bounds__(RS_THREADS, 2)
+    rs_scatter_kernel(const K* __restrict__ keys_in, int64_t stride,
+                      const int32_t* __restrict__ vals_in, K* __restrict__ keys_out,
+                      int32_t* __restrict__ vals_out, int64_t n, int shift, int width,
+                      const uint32_t* __restrict__ hist, const uint32_t* __restrict__ dtot,
+                      int ntiles) {
+  extern __shared__ __align__(16) unsigned char smem_rs[];
+  ScatterSmem<K>& sm = *reinterpret_cast<ScatterSmem<K>*>(smem_rs);
+  __shared__ uint32_t wsum[RS_WARPS];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const unsigned bins = 1u << width;
+  for (unsigned x = t; x < RS_WARPS * RS_BINS / 2; x += RS_THREADS)
+    reinterpret_cast<uint32_t*>(&sm.wcnt[0][0])[x] = 0;
+  __syncthreads();
   const unsigned lt = (1u << lane) - 1u;
-  const int64_t wbase = (int64_t)blockIdx.x * RS_TILE + (int64_t)warp * (32 * RS_ITEMS);
+  const int64_t tbase = (int64_t)blockIdx.x * RS_TILE;
+  const int64_t wbase = tbase + (int64_t)warp * (32 * RS_ITEMS) + lane;
+  const int nv = (int)(n - tbase < RS_TILE ? n - tbase : RS_TILE);
+  // rank of each pair among its warp's pairs of the same digit so far; places
+  // past the end take the last digit and end up past the tile's last pair
+  K key[RS_ITEMS];
+  uint32_t rk[RS_ITEMS / 2];  // two 16-bit places per word
 #pragma unroll
   for (int i = 0; i < RS_ITEMS; ++i) {
-    const int64_t k = wbase + i * 32 + lane;
-    const bool valid = k < n;
-    key[i] = valid ? keys_in[k] : K(0);
-    val[i] = valid ? vals_in[k] : 0;
-    const unsigned d = valid ? (unsigned)((key[i] >> shift) & (RS_BINS - 1)) : RS_BINS;
-    const unsigned peers = __match_any_sync(SPM_FULL_MASK, d);
-    const uint32_t r = __popc(peers & lt);
-    uint32_t b = 0;
-    if (valid) b = wcnt[warp][d];
+    const int64_t k = wbase + i * 32;
+    key[i] = k < n ? keys_in[k * stride] : ~K(0);
+  }
+#pragma unroll
+  for (int i = 0; i < RS_ITEMS; ++i) {
+    const unsigned d = (unsigned)(key[i] >> shift) & (bins - 1);
+    unsigned peers = SPM_FULL_MASK;
+#pragma unroll
+    for (int b = 0; b < RS_BITS; ++b) {
+      const bool bit = (d >> b) & 1u;
+      const unsigned with = __ballot_sync(SPM_FULL_MASK, bit);
+      peers &= bit ? with : ~with;
+    }
+    const unsigned r = __popc(peers & lt);
+    const unsigned before = sm.wcnt[warp][d];
     __syncwarp();
-    lrank[i] = b + r;
-    if (valid && r == 0) wcnt[warp][d] = b + __popc(peers);
+    if (r == 0) sm.wcnt[warp][d] = (unsigned short)(before + __popc(peers));
     __syncwarp();
+    if (i & 1) rk[i / 2] |= (before + r) << 16;
+    else rk[i / 2] = before + r;
   }
   __syncthreads();
-  {
-    uint32_t run = 0;
+  // digits 2t and 2t + 1: counts of the warps before, then of the digits before
+  unsigned c0 = 0, c1 = 0;
+  const unsigned b0 = 2 * t, b1 = 2 * t + 1;
+  if (b0 < bins) {
 #pragma unroll
     for (int w = 0; w < RS_WARPS; ++w) {
-      const uint32_t c = wcnt[w][threadIdx.x];
-      wcnt[w][threadIdx.x] = run;
-      run += c;
+      const uint32_t c = *reinterpret_cast<const uint32_t*>(&sm.wcnt[w][b0]);
+      *reinterpret_cast<uint32_t*>(&sm.wcnt[w][b0]) = c0 | (c1 << 16);
+      c0 += c & 0xffffu;
+      c1 += c >> 16;
     }
+  }
+  const uint32_t lo = rs_block_exclusive(c0 + c1, wsum);
+  uint32_t go = 0, t0 = 0;
+  if (hist) {
+    t0 = b0 < bins ? dtot[b0] : 0u;
+    const uint32_t t1 = b1 < bins ? dtot[b1] : 0u;
+    go = rs_block_exclusive(t0 + t1, wsum);
+  }
+  if (b0 < bins) {
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) {
+      const uint32_t c = *reinterpret_cast<const uint32_t*>(&sm.wcnt[w][b0]);
+      *reinterpret_cast<uint32_t*>(&sm.wcnt[w][b0]) =
+          ((c & 0xffffu) + lo) | (((c >> 16) + lo + c0) << 16);
+    }
+    sm.gbase[b0] = hist ? go + hist[(int64_t)b0 * ntiles + blockIdx.x] - lo : 0u;
+    if (b1 < bins)
+      sm.gbase[b1] = hist ? go + t0 + hist[(int64_t)b1 * ntiles + blockIdx.x] - (lo + c0) : 0u;
   }
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < RS_ITEMS; ++i) {
-    const int64_t k = wbase + i * 32 + lane;
-    if (k < n) {
-      const unsigned d = (unsigned)((key[i] >> shift) & (RS_BINS - 1));
-      const uint32_t pos = gbase[d] + wcnt[warp][d] + lrank[i];
-      keys_out[pos] = key[i];
-      vals_out[pos] = val[i];
+    const unsigned d = (unsigned)(key[i] >> shift) & (bins - 1);
+    const unsigned pos = sm.wcnt[warp][d] + ((rk[i / 2] >> (16 * (i & 1))) & 0xffffu);
+    sm.keys[pos] = key[i];
+    rk[i / 2] = (i & 1) ? (rk[i / 2] & 0xffffu) | (pos << 16) : (rk[i / 2] & 0xffff0000u) | pos;
+  }
+  __syncthreads();
+  uint32_t g[RS_ITEMS];
+#pragma unroll
+  for (int i = 0; i < RS_ITEMS; ++i) {
+    const int x = t + i * RS_THREADS;
+    if (x < nv) {
+      const K k = sm.keys[x];
+      g[i] = sm.gbase[(unsigned)(k >> shift) & (bins - 1)] + x;
+      if (keys_out) keys_out[g[i]] = k;
     }
+  }
+  __syncthreads();
+  int32_t* sv = reinterpret_cast<int32_t*>(sm.keys);
+#pragma unroll
+  for (int i = 0; i < RS_ITEMS; ++i) {
+    const int64_t k = wbase + i * 32;
+    if (k < n) sv[(rk[i / 2] >> (16 * (i & 1))) & 0xffffu] = vals_in ? vals_in[k] : (int32_t)k;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < RS_ITEMS; ++i) {
+    const int x = t + i * RS_THREADS;
+    if (x < nv) vals_out[g[i]] = sv[x];
   }
 }
 
@@ -173,19 +249,43 @@ struct SortScratch {
   uint32_t* dtot = nullptr;
 };
 
-// Sorts (keys, vals) by the low `bits` bits of the keys, stably.  The result
-// ends in (keys, vals) (buffers are swapped internally as needed).
+// One stable pass by digit (key >> shift) & (2^width - 1).
+template <typename K>
+spm_status radix_pass(const K* keys, int64_t stride, const int32_t* vals, K* keys_out,
+                      int32_t* vals_out, int64_t n, int shift, int width, const SortScratch& sc,
+                      cudaStream_t s) {
+  const int ntiles = (int)ceil_div<int64_t>(n, RS_TILE);
+  constexpr int smem = (int)sizeof(ScatterSmem<K>);
+  SPM_CUDA_TRY(cudaFuncSetAttribute(rs_scatter_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  if (ntiles > 1) {
+    rs_hist_kernel<K><<<ntiles, RS_THREADS, 0, s>>>(keys, stride, n, shift, width, sc.hist, ntiles);
+    const int st = std::min(1024, (ntiles + 31) / 32 * 32);
+    rs_scan_rows_kernel<<<1 << width, st, 0, s>>>(sc.hist, ntiles, sc.dtot);
+  }
+  rs_scatter_kernel<K><<<ntiles, RS_THREADS, smem, s>>>(
+      keys, stride, vals, keys_out, vals_out, n, shift, width, ntiles > 1 ? sc.hist : nullptr,
+      ntiles > 1 ? sc.dtot : nullptr, ntiles);
+  SPM_CUDA_TRY(cudaGetLastError());
+  return SPM_OK;
+}
+
+// Digits of a field of `bits` bits: count and width of each (the last may reach
+// past the field: the bits there are zero or belong to what is sorted later).
+inline int digit_count(int bits) { return ceil_div(bits, RS_BITS); }
+inline int digit_width(int bits) { return bits > 0 ? ceil_div(bits, digit_count(bits)) : 0; }
+
+// Sorts (keys, vals) by the `bits` bits of the keys from `shift` on, stably.
+// The result ends in (keys, vals) (buffers are swapped internally as needed).
+// vals_iota: the payloads of the first pass are the positions.
 template <typename K>
 spm_status radix_sort_pairs(K*& keys, int32_t*& vals, K*& keys_alt, int32_t*& vals_alt,
-                            int64_t n, int bits, const SortScratch& sc, cudaStream_t s) {
-  if (n <= 1 || bits <= 0) return SPM_OK;
-  const int nblocks = (int)ceil_div<int64_t>(n, RS_TILE);
-  for (int shift = 0; shift < bits; shift += 8) {
-    rs_hist_kernel<K><<<nblocks, RS_THREADS, 0, s>>>(keys, n, shift, sc.hist, nblocks);
-    rs_scan_rows_kernel<<<RS_BINS, 1024, 0, s>>>(sc.hist, nblocks, sc.dtot);
-    rs_scatter_kernel<K><<<nblocks, RS_THREADS, 0, s>>>(keys, vals, keys_alt, vals_alt, n, shift,
-                                                        sc.hist, sc.dtot, nblocks);
-    SPM_CUDA_TRY(cudaGetLastError());
+                            int64_t n, int bits, bool vals_iota, const SortScratch& sc,
+                            cudaStream_t s) {
+  const int nd = digit_count(bits), w = digit_width(bits);
+  for (int p = 0; p < nd; ++p) {
+    const int wp = std::min(w, bits - p * w);
+    SPM_TRY(radix_pass<K>(keys, 1, vals_iota && p == 0 ? nullptr : vals, keys_alt, vals_alt, n,
+                          p * w, wp, sc, s));
     std::swap(keys, keys_alt);
     std::swap(vals, vals_alt);
   }
@@ -196,32 +296,31 @@ spm_status radix_sort_pairs(K*& keys, int32_t*& vals, K*& keys_alt, int32_t*& va
 // Small element-wise kernels.
 // ---------------------------------------------------------------------------
 
-__global__ void validate_kernel(IdxPtrs idx, int nmodes, const int64_t* __restrict__ dims,
-                                int64_t n, int* __restrict__ err) {
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    bool bad = false;
-    for (int w = 0; w < nmodes; ++w) {
-      const int32_t c = idx.p[w][k];
-      bad |= (c < 0) || ((int64_t)c >= dims[w]);
-    }
-    if (bad) atomicOr(err, DEV_ERR_INDEX);
-  }
-}
-
-__global__ void iota_kernel(int32_t* __restrict__ a, int64_t n) {
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    a[k] = (int32_t)k;
-}
-
-// key[k] = packed (c_lo, ..., c_hi) of input position perm[k] (identity if
-// perm == nullptr); mode w occupies bits [shift[w], shift[w] + bits[w]).
+// Every index against its dimension, and (key non-null) the packed key of each
+// nonzero: mode w from bit spec.shift[w] on, for w in [spec.lo, spec.hi].
 struct PackSpec {
   int lo, hi;
   int shift[SPM_MAX_MODES];
 };
+__global__ void validate_pack_kernel(IdxPtrs idx, int nmodes, const int64_t* __restrict__ dims,
+                                     int64_t n, PackSpec spec, unsigned long long* __restrict__ key,
+                                     int* __restrict__ err) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    bool bad = false;
+    unsigned long long v = 0;
+    for (int w = 0; w < nmodes; ++w) {
+      const int32_t c = idx.p[w][k];
+      bad |= (c < 0) || ((int64_t)c >= dims[w]);
+      if (w >= spec.lo && w <= spec.hi) v |= (unsigned long long)(uint32_t)c << spec.shift[w];
+    }
+    if (key) key[k] = v;
+    if (bad) atomicOr(err, DEV_ERR_INDEX);
+  }
+}
 
+// key[k] = packed (c_lo, ..., c_hi) of input position perm[k] (identity if
+// perm == nullptr).
 __global__ void pack_keys_kernel(IdxPtrs idx, PackSpec spec, const int32_t* __restrict__ perm,
                                  int64_t n, unsigned long long* __restrict__ key) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
@@ -258,15 +357,49 @@ __global__ void records_from_input_kernel(IdxPtrs idx, const float* __restrict__
   }
 }
 
-// key[k] = word `d` of the copy-0 record k (that is c_d in copy-0 order).
+// Copy-0 records from the sorted packed keys (all modes in one word) and the
+// gathered values, with the block partials of |X|^2: repeated cells are
+// adjacent and summed before squaring, by the first of them.
+struct UnpackSpec {
+  int shift[SPM_MAX_MODES];
+  unsigned mask[SPM_MAX_MODES];
+};
 template <int RI>
-__global__ void key_from_records_kernel(const int4* __restrict__ rec, int d, int64_t n,
-                                        uint32_t* __restrict__ key) {
+__global__ void __launch_bounds__(256)
+    records_from_keys_kernel(const unsigned long long* __restrict__ key, UnpackSpec spec,
+                             const float* __restrict__ vals, const int32_t* __restrict__ perm,
+                             int nmodes, int64_t n, int4* __restrict__ rec,
+                             double* __restrict__ part) {
+  __shared__ double sh[256];
+  double acc = 0.0;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
-    const int* w = reinterpret_cast<const int*>(rec + k * RI);
-    key[k] = (uint32_t)w[d];
+    const unsigned long long v = key[k];
+    const float x = __ldg(vals + perm[k]);
+    int words[4 * RI];
+#pragma unroll
+    for (int j = 0; j < 4 * RI; ++j) {
+      words[j] = 0;
+      if (j < SPM_MAX_MODES && j < nmodes)
+        words[j] = (int)((unsigned)(v >> spec.shift[j]) & spec.mask[j]);
+      else if (j == nmodes)
+        words[j] = __float_as_int(x);
+    }
+#pragma unroll
+    for (int q = 0; q < RI; ++q)
+      rec[k * RI + q] = make_int4(words[4 * q], words[4 * q + 1], words[4 * q + 2], words[4 * q + 3]);
+    if (k > 0 && key[k - 1] == v) continue;
+    double cell = (double)x;
+    for (int64_t q = k + 1; q < n && key[q] == v; ++q) cell += (double)__ldg(vals + perm[q]);
+    acc = fma(cell, cell, acc);
   }
+  sh[threadIdx.x] = acc;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
 // Copy-d record k from copy-0 record rel[k]: rotate c_d to the front,
@@ -433,12 +566,13 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
+// One warp, fixed order.
 __global__ void sum_partials_kernel(const double* __restrict__ part, int n, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s += part[i];
-    *out = s;
-  }
+  double s = 0.0;
+  for (int i = threadIdx.x; i < n; i += 32) s += part[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(SPM_FULL_MASK, s, o);
+  if (threadIdx.x == 0) *out = s;
 }
 
 // ---- work units -----------------------------------------------------------
@@ -459,78 +593,114 @@ __global__ void units_from_partitions_kernel(const int64_t* __restrict__ off, in
   }
 }
 
-__global__ void partitions_from_units_kernel(const int64_t* __restrict__ woff, int kappa, int units,
-                                             int64_t* __restrict__ off) {
-  for (int z = blockIdx.x * blockDim.x + threadIdx.x; z <= kappa; z += gridDim.x * blockDim.x)
-    off[z] = woff[(int64_t)z * units];
-}
-
-// Row starts per tile of RS_TILE copy positions.  The row of copy position k
-// is rows[k * stride] (a copy's records, or a gathered key array).
-__global__ void __launch_bounds__(RS_THREADS)
-    head_count_kernel(const int* __restrict__ rows, int64_t stride, int64_t n,
-                      uint32_t* __restrict__ bsum) {
-  __shared__ uint32_t red[RS_THREADS];
-  const int64_t base = (int64_t)blockIdx.x * RS_TILE + (int64_t)threadIdx.x * RS_ITEMS;
-  uint32_t c = 0;
-  for (int i = 0; i < RS_ITEMS; ++i) {
-    const int64_t k = base + i;
-    if (k < n) c += (k == 0 || rows[k * stride] != rows[(k - 1) * stride]) ? 1u : 0u;
-  }
-  red[threadIdx.x] = c;
-  __syncthreads();
-  for (int o = RS_THREADS / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) bsum[blockIdx.x] = red[0];
-}
-
-// heads_before[k] = number of row starts at positions < k (bsum scanned).
-__global__ void __launch_bounds__(RS_THREADS)
-    head_prefix_kernel(const int* __restrict__ rows, int64_t stride, int64_t n,
-                       const uint32_t* __restrict__ bexcl, uint32_t* __restrict__ before) {
-  __shared__ uint32_t sc[RS_THREADS];
-  const int64_t base = (int64_t)blockIdx.x * RS_TILE + (int64_t)threadIdx.x * RS_ITEMS;
-  uint32_t c = 0;
-  for (int i = 0; i < RS_ITEMS; ++i) {
-    const int64_t k = base + i;
-    if (k < n) c += (k == 0 || rows[k * stride] != rows[(k - 1) * stride]) ? 1u : 0u;
-  }
-  sc[threadIdx.x] = c;
-  __syncthreads();
-  for (int o = 1; o < RS_THREADS; o <<= 1) {  // inclusive Hillis-Steele scan
-    const uint32_t t = threadIdx.x >= o ? sc[threadIdx.x - o] : 0u;
-    __syncthreads();
-    sc[threadIdx.x] += t;
-    __syncthreads();
-  }
-  uint32_t run = bexcl[blockIdx.x] + sc[threadIdx.x] - c;
-  for (int i = 0; i < RS_ITEMS; ++i) {
-    const int64_t k = base + i;
-    if (k < n) {
-      before[k] = run;
-      run += (k == 0 || rows[k * stride] != rows[(k - 1) * stride]) ? 1u : 0u;
+// Row starts per segment of SEG copy positions (one warp each), and the bitmap
+// of non-empty output rows (mask non-null).  The row of copy position k is
+// rows[k * stride] (a copy's records, or its sorted keys).
+constexpr int SEG = 512;
+__global__ void __launch_bounds__(256)
+    row_heads_kernel(const int* __restrict__ rows, int64_t stride, int64_t n, int64_t nseg,
+                     uint32_t* __restrict__ cnt, uint32_t* __restrict__ mask) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < nseg;
+       g += (int64_t)gridDim.x * (blockDim.x >> 5)) {
+    const int64_t base = g * SEG;
+    int r[SEG / 32];
+#pragma unroll
+    for (int i = 0; i < SEG / 32; ++i) {
+      const int64_t k = base + i * 32 + lane;
+      r[i] = k < n ? rows[k * stride] : -1;
     }
+    int last = base > 0 ? rows[(base - 1) * stride] : -1;  // the row before the chunk
+    uint32_t c = 0;
+#pragma unroll
+    for (int i = 0; i < SEG / 32; ++i) {
+      int prev = __shfl_up_sync(SPM_FULL_MASK, r[i], 1);
+      if (lane == 0) prev = last;
+      last = __shfl_sync(SPM_FULL_MASK, r[i], 31);
+      const bool head = r[i] >= 0 && r[i] != prev;
+      c += __popc(__ballot_sync(SPM_FULL_MASK, head));
+      if (head && mask) atomicOr(&mask[r[i] >> 5], 1u << (r[i] & 31));
+    }
+    if (lane == 0) cnt[g] = c;
+  }
+}
+
+// Exclusive scan of cnt[0 .. n) in place, total to *total (one block).
+__global__ void __launch_bounds__(1024)
+    seg_scan_kernel(uint32_t* __restrict__ cnt, int64_t n, uint32_t* __restrict__ total) {
+  __shared__ uint32_t wsum[32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int64_t per = (n + 1023) / 1024;
+  const int64_t b = t * per, e = b + per < n ? b + per : n;
+  uint32_t v = 0;
+#pragma unroll 4
+  for (int64_t i = b; i < e; ++i) v += cnt[i];
+  uint32_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(SPM_FULL_MASK, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[warp] = x;
+  __syncthreads();
+  uint32_t pre = 0;
+  for (int w = 0; w < warp; ++w) pre += wsum[w];
+  uint32_t run = pre + x - v;
+  if (t == 1023) *total = run + v;
+  for (int64_t i = b; i < e; ++i) {
+    const uint32_t c = cnt[i];
+    cnt[i] = run;
+    run += c;
   }
 }
 
 // woff[j] = min{k in [0, n] : C(k) * P >= j * C(n)},
-// C(k) = k + row_cost * before[k], C(n) = n + row_cost * total_heads.
-__global__ void balanced_units_kernel(const uint32_t* __restrict__ before,
-                                      const uint32_t* __restrict__ total_heads, int64_t n,
-                                      int64_t P, int row_cost, int64_t* __restrict__ woff) {
-  const int64_t Ct = n + (int64_t)row_cost * (int64_t)(*total_heads);
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= P;
-       j += (int64_t)gridDim.x * blockDim.x) {
+// C(k) = k + row_cost * (row starts before k), C(n) = n + row_cost * heads;
+// off[z] = woff[z * units].  One warp per unit: a binary search over the
+// segments, then the row starts inside one.
+__global__ void __launch_bounds__(256)
+    balanced_units_kernel(const int* __restrict__ rows, int64_t stride, int64_t n,
+                          const uint32_t* __restrict__ seg, int64_t nseg,
+                          const uint32_t* __restrict__ heads, int64_t P, int units, int row_cost,
+                          int64_t* __restrict__ woff, int64_t* __restrict__ off) {
+  const int lane = threadIdx.x & 31;
+  const int64_t Ct = n + (int64_t)row_cost * (int64_t)(*heads);
+  for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j <= P;
+       j += (int64_t)gridDim.x * (blockDim.x >> 5)) {
     const int64_t target = j * Ct;  // compare C(k) * P >= target
-    int64_t lo = 0, hi = n;         // C(n) * P >= target always holds
-    while (lo < hi) {
+    // last segment that starts below the target (none: position 0)
+    int64_t lo = -1, hi = nseg;
+    while (hi - lo > 1) {
       const int64_t mid = lo + (hi - lo) / 2;
-      const int64_t C = mid + (int64_t)row_cost * (int64_t)before[mid];
-      if (C * P >= target) hi = mid; else lo = mid + 1;
+      const int64_t C = mid * SEG + (int64_t)row_cost * (int64_t)seg[mid];
+      if (C * P < target) lo = mid; else hi = mid;
     }
-    woff[j] = lo;
+    int64_t res = 0;
+    if (lo >= 0) {
+      const int64_t base = lo * SEG;
+      res = base + SEG < n ? base + SEG : n;
+      int64_t before = seg[lo];
+      int last = base > 0 ? rows[(base - 1) * stride] : -1;
+      for (int i = 0; i < SEG / 32; ++i) {
+        const int64_t k = base + i * 32 + lane;
+        const int r = k < n ? rows[k * stride] : -1;
+        int prev = __shfl_up_sync(SPM_FULL_MASK, r, 1);
+        if (lane == 0) prev = last;
+        last = __shfl_sync(SPM_FULL_MASK, r, 31);
+        const unsigned hb = __ballot_sync(SPM_FULL_MASK, r >= 0 && r != prev);
+        const int64_t C = k + (int64_t)row_cost * (before + __popc(hb & ((1u << lane) - 1u)));
+        const unsigned ok = __ballot_sync(SPM_FULL_MASK, k <= n && C * P >= target);
+        if (ok) {
+          res = base + i * 32 + (__ffs(ok) - 1);
+          break;
+        }
+        before += __popc(hb);
+      }
+    }
+    if (lane == 0) {
+      woff[j] = res;
+      if (j % units == 0) off[j / units] = res;
+    }
   }
 }
 
@@ -555,8 +725,8 @@ __global__ void gather_rows_kernel(const int* __restrict__ rec0, int64_t words, 
 }
 
 __global__ void popc_kernel(const uint32_t* __restrict__ mask, int64_t words,
-                            unsigned long long* __restrict__ count) {
-  unsigned long long c = 0;
+                            unsigned* __restrict__ count) {
+  unsigned c = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words;
        i += (int64_t)gridDim.x * blockDim.x)
     c += __popc(mask[i]);
@@ -602,10 +772,11 @@ const int* copy_rows(spmttkrp_plan_s* p, int d, int* scratch, int64_t* stride, c
 // P2 for a copy under the cost-balanced policy (scheme 0) or Scheme 2, and
 // for an empty tensor under any policy: partition offsets off[0..kappa] and
 // work-unit offsets woff[0..kappa*nu].  rows/stride: the copy's rows in copy
-// order.  Scratch: hist >= ceil(nnz/RS_TILE) words, dtot >= 1 word,
-// before >= nnz words.
-void partition_copy(spmttkrp_plan_s* p, int d, const int* rows, int64_t stride, uint32_t* hist,
-                    uint32_t* dtot, uint32_t* before, cudaStream_t s) {
+// order.  Scheme 0 leaves the number of distinct rows in *heads and, with
+// `mask`, sets the (cleared) bitmap of non-empty rows.  Scratch: seg >=
+// ceil(nnz/SEG) words.
+void partition_copy(spmttkrp_plan_s* p, int d, const int* rows, int64_t stride, uint32_t* seg,
+                    uint32_t* heads, uint32_t* mask, cudaStream_t s) {
   const int T = 256;
   const int64_t n = p->nnz;
   const int units = p->nu;
@@ -613,14 +784,11 @@ void partition_copy(spmttkrp_plan_s* p, int d, const int* rows, int64_t stride, 
   spm_mode_copy& c = p->mode[d];
   if (c.scheme == 0 && n > 0) {
     // cost-balanced work units over the copy order
-    const int nb = (int)ceil_div<int64_t>(n, RS_TILE);
-    head_count_kernel<<<nb, RS_THREADS, 0, s>>>(rows, stride, n, hist);
-    rs_scan_rows_kernel<<<1, 1024, 0, s>>>(hist, nb, dtot);
-    head_prefix_kernel<<<nb, RS_THREADS, 0, s>>>(rows, stride, n, hist, before);
-    balanced_units_kernel<<<grid_for(P + 1, T), T, 0, s>>>(before, dtot, n, P, SPM_ROW_COST,
-                                                          c.woff);
-    partitions_from_units_kernel<<<grid_for(p->kappa + 1, T), T, 0, s>>>(c.woff, p->kappa,
-                                                                        units, c.off);
+    const int64_t nseg = ceil_div<int64_t>(n, SEG);
+    row_heads_kernel<<<grid_for(nseg * 32, T), T, 0, s>>>(rows, stride, n, nseg, seg, mask);
+    seg_scan_kernel<<<1, 1024, 0, s>>>(seg, nseg, heads);
+    balanced_units_kernel<<<grid_for((P + 1) * 32, T), T, 0, s>>>(
+        rows, stride, n, seg, nseg, heads, P, units, SPM_ROW_COST, c.woff, c.off);
     return;
   }
   equal_offsets_kernel<<<grid_for(p->kappa + 1, T), T, 0, s>>>(n, p->kappa, c.off);
@@ -640,6 +808,56 @@ int64_t sort_capacity(int N, const int64_t* dims, int64_t nn, int policy, int ka
   return std::max(nn, rows);
 }
 
+// Transient device memory of a build: one stream-ordered allocation.
+struct BuildScratch {
+  void* base = nullptr;
+  unsigned long long *ka = nullptr, *kb = nullptr;  // keys
+  int32_t *va = nullptr, *vb = nullptr;             // payloads
+  SortScratch sort;
+  int64_t* dims = nullptr;
+  unsigned* count = nullptr;  // non-empty rows per mode
+  // Bytes for `cap` keys; the pieces are laid out when `p` is non-null.
+  static size_t layout(int64_t cap, unsigned char* p, BuildScratch* b) {
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+      unsigned char* q = p ? p + at : nullptr;
+      at += (bytes + 255) & ~(size_t)255;
+      return q;
+    };
+    unsigned char* q[7];
+    q[0] = take(sizeof(unsigned long long) * (size_t)cap);
+    q[1] = take(sizeof(unsigned long long) * (size_t)cap);
+    q[2] = take(sizeof(int32_t) * (size_t)cap);
+    q[3] = take(sizeof(int32_t) * (size_t)cap);
+    q[4] = take(sizeof(uint32_t) * RS_BINS * (size_t)ceil_div<int64_t>(cap, RS_TILE));
+    q[5] = take(sizeof(uint32_t) * RS_BINS);
+    q[6] = take(sizeof(int64_t) * SPM_MAX_MODES + sizeof(unsigned) * SPM_MAX_MODES);
+    if (b) {
+      b->base = p;
+      b->ka = reinterpret_cast<unsigned long long*>(q[0]);
+      b->kb = reinterpret_cast<unsigned long long*>(q[1]);
+      b->va = reinterpret_cast<int32_t*>(q[2]);
+      b->vb = reinterpret_cast<int32_t*>(q[3]);
+      b->sort.hist = reinterpret_cast<uint32_t*>(q[4]);
+      b->sort.dtot = reinterpret_cast<uint32_t*>(q[5]);
+      b->dims = reinterpret_cast<int64_t*>(q[6]);
+      b->count = reinterpret_cast<unsigned*>(b->dims + SPM_MAX_MODES);
+    }
+    return at;
+  }
+  spm_status alloc(int64_t cap, cudaStream_t s) {
+    void* p = nullptr;
+    SPM_CUDA_TRY(cudaMallocAsync(&p, layout(cap, nullptr, nullptr), s));
+    layout(cap, static_cast<unsigned char*>(p), this);
+    return SPM_OK;
+  }
+  spm_status release(cudaStream_t s) {
+    SPM_CUDA_TRY(cudaFreeAsync(base, s));
+    base = nullptr;
+    return SPM_OK;
+  }
+};
+
 template <int RI>
 spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, const float* vals,
                           cudaStream_t s) {
@@ -650,27 +868,48 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
   const int T = 256;
   const int G = grid_for(n, T);
 
-  // scratch (stream-ordered, freed at the end)
-  unsigned long long *k64a = nullptr, *k64b = nullptr;
-  int32_t *va = nullptr, *vb = nullptr;
-  SortScratch sc;
-  int64_t* d_dims = nullptr;
+  // scratch (one stream-ordered allocation, freed at the end)
   const int64_t nn = n > 0 ? n : 1;
   // the keys, payloads and histograms hold nnz entries, or I_d entries where
   // Scheme 1 sorts the rows of a mode by degree
   const int64_t cap = sort_capacity(N, p->dims, nn, p->policy, p->kappa);
-  const int nblocks_max = (int)ceil_div<int64_t>(cap, RS_TILE);
-  SPM_CUDA_TRY(cudaMallocAsync((void**)&k64a, sizeof(unsigned long long) * cap, s));
-  SPM_CUDA_TRY(cudaMallocAsync((void**)&k64b, sizeof(unsigned long long) * cap, s));
-  SPM_CUDA_TRY(cudaMallocAsync((void**)&va, sizeof(int32_t) * cap, s));
-  SPM_CUDA_TRY(cudaMallocAsync((void**)&vb, sizeof(int32_t) * cap, s));
-  SPM_CUDA_TRY(cudaMallocAsync((void**)&sc.hist, sizeof(uint32_t) * RS_BINS * (size_t)nblocks_max, s));
-  SPM_CUDA_TRY(cudaMallocAsync((void**)&sc.dtot, sizeof(uint32_t) * RS_BINS, s));
-  SPM_CUDA_TRY(cudaMallocAsync((void**)&d_dims, sizeof(int64_t) * SPM_MAX_MODES, s));
-  SPM_CUDA_TRY(cudaMemcpyAsync(d_dims, p->dims, sizeof(int64_t) * N, cudaMemcpyHostToDevice, s));
+  BuildScratch b;
+  SPM_TRY(b.alloc(cap, s));
+  const SortScratch& sc = b.sort;
+  SPM_CUDA_TRY(cudaMemcpyAsync(b.dims, p->dims, sizeof(int64_t) * N, cudaMemcpyHostToDevice, s));
 
-  // Validation: every index within its dimension.
-  if (n > 0) validate_kernel<<<G, T, 0, s>>>(idx, N, d_dims, n, p->dev_err);
+  // modes grouped into <=64-bit key words from the last mode backwards
+  int bits[SPM_MAX_MODES];
+  for (int w = 0; w < N; ++w) bits[w] = bits_for(p->dims[w]);
+  struct Group { int lo, hi; };
+  std::vector<Group> groups;
+  {
+    int hi = N - 1, acc = 0;
+    for (int w = N - 1; w >= 0; --w) {
+      if (acc + bits[w] > 64) {
+        groups.push_back({w + 1, hi});
+        hi = w;
+        acc = 0;
+      }
+      acc += bits[w];
+    }
+    groups.push_back({0, hi});
+  }
+  auto spec_of = [&](const Group& g) {
+    PackSpec spec{};
+    spec.lo = g.lo;
+    spec.hi = g.hi;
+    int sh = 0;
+    for (int w = g.hi; w >= g.lo; --w) {
+      spec.shift[w] = sh;
+      sh += bits[w];
+    }
+    return spec;
+  };
+
+  // Validation: every index within its dimension; and the keys of the first sort.
+  if (n > 0)
+    validate_pack_kernel<<<G, T, 0, s>>>(idx, N, b.dims, n, spec_of(groups[0]), b.ka, p->dev_err);
   int herr = 0;
   SPM_CUDA_TRY(cudaMemcpyAsync(&herr, p->dev_err, sizeof(int), cudaMemcpyDeviceToHost, s));
   SPM_CUDA_TRY(cudaStreamSynchronize(s));
@@ -696,82 +935,102 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
                       sizeof(uint32_t) * (size_t)((p->dims[d] + 31) / 32));
   }
 
+  for (int d = 0; d < N; ++d) p->mode[d].scheme = resolved_scheme(p->policy, p->dims[d], p->kappa);
+  plan_shapes(p);
+  const int units = p->nu;
+  const int64_t P = (int64_t)p->kappa * units;
+  if (st == SPM_OK) {
+    SPM_CUDA_TRY(cudaMemsetAsync(b.count, 0, sizeof(unsigned) * SPM_MAX_MODES, s));
+    for (int d = 0; d < N; ++d)
+      SPM_CUDA_TRY(cudaMemsetAsync(p->mode[d].rowmask, 0,
+                                   sizeof(uint32_t) * (size_t)((p->dims[d] + 31) / 32), s));
+  }
+
   if (st == SPM_OK && n > 0) {
     // ---- copy 0: full lexicographic order, least significant key word first.
-    int bits[SPM_MAX_MODES];
-    for (int w = 0; w < N; ++w) bits[w] = bits_for(p->dims[w]);
-    // group modes into <=64-bit words from the last mode backwards
-    struct Group { int lo, hi, nbits; };
-    std::vector<Group> groups;
-    {
-      int hi = N - 1, acc = 0, lo = N - 1;
-      for (int w = N - 1; w >= 0; --w) {
-        if (acc + bits[w] > 64) {
-          groups.push_back({w + 1, hi, acc});
-          hi = w;
-          acc = 0;
-        }
-        acc += bits[w];
-        lo = w;
-      }
-      groups.push_back({lo, hi, acc});
-    }
-    // perm in va (identity), keys in k64a
-    iota_kernel<<<G, T, 0, s>>>(va, n);
-    unsigned long long *ka = k64a, *kb = k64b;
-    int32_t *pa = va, *pb = vb;
-    for (const Group& g : groups) {  // least significant group first
-      PackSpec spec{};
-      spec.lo = g.lo;
-      spec.hi = g.hi;
-      int sh = 0;
+    spm_mode_copy& c0 = p->mode[0];
+    unsigned long long *ka = b.ka, *kb = b.kb;
+    const int32_t* pa = nullptr;  // null: input positions in order
+    int32_t* free_perm[2] = {b.va, b.vb};
+    for (size_t q = 0; q < groups.size() && st == SPM_OK; ++q) {  // least significant group first
+      const Group& g = groups[q];
+      const PackSpec spec = spec_of(g);
+      if (q > 0) pack_keys_kernel<<<G, T, 0, s>>>(idx, spec, pa, n, ka);
+      std::vector<std::pair<int, int>> passes;  // (shift, width)
       for (int w = g.hi; w >= g.lo; --w) {
-        spec.shift[w] = sh;
-        sh += bits[w];
+        const int wd = digit_width(bits[w]);
+        for (int x = 0; x < bits[w]; x += wd)
+          passes.push_back({spec.shift[w] + x, std::min(wd, bits[w] - x)});
       }
-      pack_keys_kernel<<<G, T, 0, s>>>(idx, spec, pa, n, ka);
-      st = radix_sort_pairs<unsigned long long>(ka, pa, kb, pb, n, g.nbits, sc, s);
-      if (st != SPM_OK) break;
+      if (passes.empty() && q + 1 == groups.size()) passes.push_back({0, 1});  // writes the order
+      for (size_t x = 0; x < passes.size() && st == SPM_OK; ++x) {
+        const bool last = q + 1 == groups.size() && x + 1 == passes.size();
+        int32_t* out = last ? c0.perm : free_perm[0];
+        st = radix_pass<unsigned long long>(ka, 1, pa, kb, out, n, passes[x].first,
+                                            passes[x].second, sc, s);
+        std::swap(ka, kb);
+        std::swap(free_perm[0], free_perm[1]);
+        pa = out;
+      }
     }
     if (st == SPM_OK) {
-      spm_mode_copy& c0 = p->mode[0];
-      SPM_CUDA_TRY(cudaMemcpyAsync(c0.perm, pa, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
-      records_from_input_kernel<RI><<<G, T, 0, s>>>(idx, vals, c0.perm, N, n, c0.rec);
-      // |X|^2 (duplicates summed) from copy 0
-      norm_partial_kernel<RI><<<NORM_BLOCKS, 256, 0, s>>>(c0.rec, N, n, p->norm_part);
+      if (groups.size() == 1) {
+        UnpackSpec u{};
+        const PackSpec spec = spec_of(groups[0]);
+        for (int w = 0; w < N; ++w) {
+          u.shift[w] = bits[w] ? spec.shift[w] : 0;
+          u.mask[w] = bits[w] ? (unsigned)((1ull << bits[w]) - 1) : 0u;
+        }
+        records_from_keys_kernel<RI><<<NORM_BLOCKS, 256, 0, s>>>(ka, u, vals, c0.perm, N, n, c0.rec,
+                                                               p->norm_part);
+      } else {
+        records_from_input_kernel<RI><<<G, T, 0, s>>>(idx, vals, c0.perm, N, n, c0.rec);
+        // |X|^2 (duplicates summed) from copy 0
+        norm_partial_kernel<RI><<<NORM_BLOCKS, 256, 0, s>>>(c0.rec, N, n, p->norm_part);
+      }
       sum_partials_kernel<<<1, 32, 0, s>>>(p->norm_part, NORM_BLOCKS, p->normX2);
-    }
-    // ---- copies d >= 1: stable sort of copy 0 by c_d.
-    for (int d = 1; d < N && st == SPM_OK; ++d) {
-      uint32_t* ka32 = reinterpret_cast<uint32_t*>(k64a);
-      uint32_t* kb32 = reinterpret_cast<uint32_t*>(k64b);
-      int32_t *ra = va, *rb = vb;
-      key_from_records_kernel<RI><<<G, T, 0, s>>>(p->mode[0].rec, d, n, ka32);
-      iota_kernel<<<G, T, 0, s>>>(ra, n);
-      st = radix_sort_pairs<uint32_t>(ka32, ra, kb32, rb, n, bits[d], sc, s);
-      if (st != SPM_OK) break;
-      if (p->lean)
-        SPM_CUDA_TRY(cudaMemcpyAsync(p->mode[d].src, ra, sizeof(int32_t) * n,
-                                     cudaMemcpyDeviceToDevice, s));
-      else
-        records_from_copy0_kernel<RI><<<G, T, 0, s>>>(p->mode[0].rec, p->mode[0].perm, ra, N, d,
-                                                       n, p->mode[d].rec, p->mode[d].perm);
     }
   } else if (st == SPM_OK) {
     SPM_CUDA_TRY(cudaMemsetAsync(p->normX2, 0, sizeof(double), s));
   }
 
-  // ---- partitions (Sec. III-B) and work units
-  const int units = p->nu;
-  const int64_t P = (int64_t)p->kappa * units;
-  for (int d = 0; d < N; ++d) p->mode[d].scheme = resolved_scheme(p->policy, p->dims[d], p->kappa);
-  if (st == SPM_OK) plan_shapes(p);
-  for (int d = 0; d < N && st == SPM_OK; ++d) {
+  // ---- copies d >= 1 (stable sort of copy 0 by c_d), then each copy's
+  // partitions (Sec. III-B), work units and bitmap of non-empty rows; copy 0
+  // last, because Scheme 1 reorders it
+  for (int x = 1; x <= N && st == SPM_OK; ++x) {
+    const int d = x % N;
     spm_mode_copy& c = p->mode[d];
+    const int* rows = n > 0 ? reinterpret_cast<const int*>(p->mode[0].rec) : nullptr;
+    int64_t stride = 4 * RI;
+    if (d > 0 && n > 0) {
+      uint32_t *ko = reinterpret_cast<uint32_t*>(b.kb), *kf = reinterpret_cast<uint32_t*>(b.ka);
+      const uint32_t* ki = reinterpret_cast<const uint32_t*>(rows) + d;
+      const int32_t* ri = nullptr;
+      int32_t *ro = b.va, *rf = b.vb;
+      const int nb = std::max(1, bits[d]), wd = digit_width(nb);
+      for (int bit = 0; bit < nb && st == SPM_OK; bit += wd) {
+        int32_t* out = p->lean && bit + wd >= nb ? c.src : ro;
+        st = radix_pass<uint32_t>(ki, bit == 0 ? stride : 1, ri, ko, out, n, bit,
+                                  std::min(wd, nb - bit), sc, s);
+        ki = ko;
+        ri = out;
+        std::swap(ko, kf);
+        std::swap(ro, rf);
+      }
+      if (st != SPM_OK) break;
+      if (!p->lean)
+        records_from_copy0_kernel<RI><<<G, T, 0, s>>>(p->mode[0].rec, p->mode[0].perm, ri, N, d, n,
+                                                       c.rec, c.perm);
+      rows = reinterpret_cast<const int*>(ki);
+      stride = 1;
+    }
     if (c.scheme != 1 || n == 0) {
-      int64_t stride = 0;
-      const int* rows = n > 0 ? copy_rows(p, d, reinterpret_cast<int*>(k64b), &stride, s) : nullptr;
-      partition_copy(p, d, rows, stride, sc.hist, sc.dtot, reinterpret_cast<uint32_t*>(va), s);
+      partition_copy(p, d, rows, stride, sc.hist, b.count + d, c.rowmask, s);
+      if (c.scheme != 0 && n > 0) {
+        row_mask_kernel<<<G, T, 0, s>>>(rows, stride, n, c.rowmask);
+        const int64_t words = (p->dims[d] + 31) / 32;
+        popc_kernel<<<grid_for(words, T), T, 0, s>>>(c.rowmask, words, b.count + d);
+      }
       continue;
     }
     // Scheme 1: degree-ordered cyclic deal of the rows, copy ordered by partition.
@@ -787,19 +1046,19 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
     SPM_CUDA_TRY(cudaMemsetAsync(deg, 0, sizeof(int32_t) * I, s));
     row_degree_kernel<RI><<<G, T, 0, s>>>(c.rec, n, deg);
     {
-      unsigned long long *ka = k64a, *kb = k64b;
-      int32_t *ra = va, *rb = vb;
+      unsigned long long *ka = b.ka, *kb = b.kb;
+      int32_t *ra = b.va, *rb = b.vb;
       row_order_key_kernel<<<grid_for(I, T), T, 0, s>>>(deg, I, ka, ra);
-      st = radix_sort_pairs<unsigned long long>(ka, ra, kb, rb, I, 64, sc, s);
+      st = radix_sort_pairs<unsigned long long>(ka, ra, kb, rb, I, 64, false, sc, s);
       if (st == SPM_OK) deal_rows_kernel<<<grid_for(I, T), T, 0, s>>>(ra, deg, I, p->kappa, part);
     }
     if (st == SPM_OK) {
-      uint32_t* ka32 = reinterpret_cast<uint32_t*>(k64a);
-      uint32_t* kb32 = reinterpret_cast<uint32_t*>(k64b);
-      int32_t *ra = va, *rb = vb;
+      uint32_t* ka32 = reinterpret_cast<uint32_t*>(b.ka);
+      uint32_t* kb32 = reinterpret_cast<uint32_t*>(b.kb);
+      int32_t *ra = b.va, *rb = b.vb;
       part_key_kernel<RI><<<G, T, 0, s>>>(c.rec, part, n, ka32);
-      iota_kernel<<<G, T, 0, s>>>(ra, n);
-      st = radix_sort_pairs<uint32_t>(ka32, ra, kb32, rb, n, bits_for(p->kappa), sc, s);
+      st = radix_sort_pairs<uint32_t>(ka32, ra, kb32, rb, n, std::max(1, bits_for(p->kappa)), true,
+                                      sc, s);
       if (st == SPM_OK) {
         reorder_copy_kernel<RI><<<G, T, 0, s>>>(c.rec, c.perm, ra, n, rec_tmp, perm_tmp);
         SPM_CUDA_TRY(cudaMemcpyAsync(c.rec, rec_tmp, sizeof(int4) * RI * (size_t)n,
@@ -810,6 +1069,9 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
                                                                           c.off);
         units_from_partitions_kernel<<<grid_for(P + 1, T), T, 0, s>>>(c.off, p->kappa, units,
                                                                       c.woff);
+        row_mask_kernel<<<G, T, 0, s>>>(reinterpret_cast<const int*>(c.rec), 4 * RI, n, c.rowmask);
+        const int64_t words = (I + 31) / 32;
+        popc_kernel<<<grid_for(words, T), T, 0, s>>>(c.rowmask, words, b.count + d);
       }
     }
     SPM_CUDA_TRY(cudaFreeAsync(deg, s));
@@ -817,34 +1079,12 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
     SPM_CUDA_TRY(cudaFreeAsync(rec_tmp, s));
     SPM_CUDA_TRY(cudaFreeAsync(perm_tmp, s));
   }
-  // ---- non-empty row bitmaps (rows without nonzeros are zeroed per run)
-  unsigned long long* d_cnt = nullptr;
-  unsigned long long h_cnt[SPM_MAX_MODES] = {};
-  if (st == SPM_OK) {
-    SPM_CUDA_TRY(cudaMallocAsync((void**)&d_cnt, sizeof(unsigned long long) * SPM_MAX_MODES, s));
-    SPM_CUDA_TRY(cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long) * SPM_MAX_MODES, s));
-    for (int d = 0; d < N; ++d) {
-      const int64_t words = (p->dims[d] + 31) / 32;
-      SPM_CUDA_TRY(cudaMemsetAsync(p->mode[d].rowmask, 0, sizeof(uint32_t) * words, s));
-      if (n > 0) {
-        int64_t stride = 0;
-        const int* rows = copy_rows(p, d, reinterpret_cast<int*>(k64b), &stride, s);
-        row_mask_kernel<<<G, T, 0, s>>>(rows, stride, n, p->mode[d].rowmask);
-      }
-      popc_kernel<<<grid_for(words, T), T, 0, s>>>(p->mode[d].rowmask, words, d_cnt + d);
-    }
-    SPM_CUDA_TRY(cudaMemcpyAsync(h_cnt, d_cnt, sizeof(unsigned long long) * SPM_MAX_MODES,
+  unsigned h_cnt[SPM_MAX_MODES] = {};
+  if (st == SPM_OK)
+    SPM_CUDA_TRY(cudaMemcpyAsync(h_cnt, b.count, sizeof(unsigned) * SPM_MAX_MODES,
                                  cudaMemcpyDeviceToHost, s));
-    SPM_CUDA_TRY(cudaFreeAsync(d_cnt, s));
-  }
   SPM_CUDA_TRY(cudaGetLastError());
-  SPM_CUDA_TRY(cudaFreeAsync(k64a, s));
-  SPM_CUDA_TRY(cudaFreeAsync(k64b, s));
-  SPM_CUDA_TRY(cudaFreeAsync(va, s));
-  SPM_CUDA_TRY(cudaFreeAsync(vb, s));
-  SPM_CUDA_TRY(cudaFreeAsync(sc.hist, s));
-  SPM_CUDA_TRY(cudaFreeAsync(sc.dtot, s));
-  SPM_CUDA_TRY(cudaFreeAsync(d_dims, s));
+  SPM_TRY(b.release(s));
   SPM_CUDA_TRY(cudaStreamSynchronize(s));
   for (int d = 0; d < N; ++d) p->mode[d].empty_rows = p->dims[d] - (int64_t)h_cnt[d];
   return st;
@@ -905,10 +1145,7 @@ void plan_bytes_estimate(int N, const int64_t* dims, int64_t nnz, int R, int kap
   *resident = b;
   // stream-ordered scratch of the build (keys, payloads, histograms)
   const int64_t cap = sort_capacity(N, dims, nn, policy, kappa);
-  *transient = sizeof(unsigned long long) * 2 * (size_t)cap + sizeof(int32_t) * 2 * (size_t)cap +
-               sizeof(uint32_t) * RS_BINS * (size_t)ceil_div<int64_t>(cap, RS_TILE) +
-               sizeof(uint32_t) * RS_BINS + sizeof(int64_t) * SPM_MAX_MODES +
-               sizeof(unsigned long long) * SPM_MAX_MODES;
+  *transient = BuildScratch::layout(cap, nullptr, nullptr);
   if (fibre)  // the record copies live until every fibre stream is built
     *transient = std::max<size_t>(*transient, (sizeof(int4) * RI + 256) * (size_t)nn * N +
                                                   sizeof(int32_t) * (size_t)nn);
@@ -937,21 +1174,18 @@ spm_status plan_repartition(spmttkrp_plan_s* p, int kappa, cudaStream_t s) {
   plan_shapes(p);
   const int64_t n = p->nnz;
   const int64_t nn = n > 0 ? n : 1;
-  uint32_t *hist = nullptr, *dtot = nullptr, *before = nullptr;
+  uint32_t *seg = nullptr, *heads = nullptr;
   int* rows_tmp = nullptr;
-  SPM_CUDA_TRY(cudaMallocAsync((void**)&hist, sizeof(uint32_t) * ceil_div<int64_t>(nn, RS_TILE), s));
-  SPM_CUDA_TRY(cudaMallocAsync((void**)&dtot, sizeof(uint32_t), s));
-  SPM_CUDA_TRY(cudaMallocAsync((void**)&before, sizeof(uint32_t) * nn, s));
+  SPM_CUDA_TRY(cudaMallocAsync((void**)&seg, sizeof(uint32_t) * (ceil_div<int64_t>(nn, SEG) + 1), s));
+  heads = seg + ceil_div<int64_t>(nn, SEG);
   if (p->lean) SPM_CUDA_TRY(cudaMallocAsync((void**)&rows_tmp, sizeof(int) * nn, s));
   for (int d = 0; d < p->N; ++d) {
     int64_t stride = 0;
     const int* rows = n > 0 ? copy_rows(p, d, rows_tmp, &stride, s) : nullptr;
-    partition_copy(p, d, rows, stride, hist, dtot, before, s);
+    partition_copy(p, d, rows, stride, seg, heads, nullptr, s);
   }
   SPM_CUDA_TRY(cudaGetLastError());
-  SPM_CUDA_TRY(cudaFreeAsync(hist, s));
-  SPM_CUDA_TRY(cudaFreeAsync(dtot, s));
-  SPM_CUDA_TRY(cudaFreeAsync(before, s));
+  SPM_CUDA_TRY(cudaFreeAsync(seg, s));
   if (rows_tmp) SPM_CUDA_TRY(cudaFreeAsync(rows_tmp, s));
   return SPM_OK;
 }
