@@ -28,8 +28,17 @@ namespace {
 
 constexpr int RS_WARPS = 16;
 constexpr int RS_THREADS = RS_WARPS * 32;
-constexpr int RS_ITEMS = 16;
-constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
+// Pairs per thread of a tile: 16, or 4 while that leaves few tiles (up to 2^20
+// pairs: a tile's chain of ranks is short and there are four times the blocks).
+constexpr int RS_ITEMS = 16, RS_ITEMS_SMALL = 4;
+constexpr int64_t RS_SMALL = 1 << 20;
+inline int rs_tile(int64_t n) { return RS_THREADS * (n <= RS_SMALL ? RS_ITEMS_SMALL : RS_ITEMS); }
+// Tiles of n pairs, and the most of any count up to cap.
+inline int64_t rs_tiles(int64_t n) { return (n + rs_tile(n) - 1) / rs_tile(n); }
+inline int64_t rs_tiles_cap(int64_t cap) {
+  const int64_t small = rs_tiles(cap < RS_SMALL ? cap : RS_SMALL);
+  return rs_tiles(cap) > small ? rs_tiles(cap) : small;
+}
 constexpr int RS_BITS = 10;  // widest digit
 constexpr int RS_BINS = 1 << RS_BITS;
 
@@ -46,7 +55,7 @@ struct IdxPtrs {
 // pass (8 bits straight from registers: 990 us); 32-bit keys 530 (800).
 // ---------------------------------------------------------------------------
 
-template <typename K>
+template <typename K, int ITEMS>
 __global__ void __launch_bounds__(RS_THREADS)
     rs_hist_kernel(const K* __restrict__ keys, int64_t stride, int64_t n, int shift, int width,
                    uint32_t* __restrict__ hist, int ntiles) {
@@ -54,12 +63,16 @@ __global__ void __launch_bounds__(RS_THREADS)
   const int bins = 1 << width;
   for (int b = threadIdx.x; b < bins; b += RS_THREADS) cnt[b] = 0;
   __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * RS_TILE + threadIdx.x;
+  const int64_t base = (int64_t)blockIdx.x * (RS_THREADS * ITEMS) + threadIdx.x;
+  K key[ITEMS];
 #pragma unroll
-  for (int i = 0; i < RS_ITEMS; ++i) {
+  for (int i = 0; i < ITEMS; ++i) {
     const int64_t k = base + i * RS_THREADS;
-    if (k < n) atomicAdd(&cnt[(unsigned)(keys[k * stride] >> shift) & (bins - 1)], 1u);
+    key[i] = k < n ? keys[k * stride] : K(0);
   }
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i)
+    if (base + i * RS_THREADS < n) atomicAdd(&cnt[(unsigned)(key[i] >> shift) & (bins - 1)], 1u);
   __syncthreads();
   for (int b = threadIdx.x; b < bins; b += RS_THREADS) hist[(int64_t)b * ntiles + blockIdx.x] = cnt[b];
 }
@@ -105,9 +118,9 @@ __global__ void __launch_bounds__(1024)
   if (threadIdx.x == 0) dtot[blockIdx.x] = carry;
 }
 
-template <typename K>
+template <typename K, int ITEMS>
 struct ScatterSmem {
-  K keys[RS_TILE];                       // the tile in digit order, then its payloads
+  K keys[RS_THREADS * ITEMS];                       // the tile in digit order, then its payloads
   unsigned short wcnt[RS_WARPS][RS_BINS];  // per warp and digit: count, then first place in the tile
   uint32_t gbase[RS_BINS];               // global place of a digit's run minus its place in the tile
 };
@@ -133,7 +146,7 @@ __device__ __forceinline__ uint32_t rs_block_exclusive(uint32_t v, uint32_t* wsu
 // One tile: pairs (keys[k * stride], vals ? vals[k] : k) to their places by
 // digit.  hist: the tile histograms scanned along the tiles, dtot the digit
 // totals (both null: the only tile).  keys_out may be null.
-template <typename K>
+template <typename K, int ITEMS>
 __global__ void __launch_bounds__(RS_THREADS, 2)
     rs_scatter_kernel(const K* __restrict__ keys_in, int64_t stride,
                       const int32_t* __restrict__ vals_in, K* __restrict__ keys_out,
@@ -141,7 +154,8 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
                       const uint32_t* __restrict__ hist, const uint32_t* __restrict__ dtot,
                       int ntiles) {
   extern __shared__ __align__(16) unsigned char smem_rs[];
-  ScatterSmem<K>& sm = *reinterpret_cast<ScatterSmem<K>*>(smem_rs);
+  constexpr int TILE = RS_THREADS * ITEMS;
+  ScatterSmem<K, ITEMS>& sm = *reinterpret_cast<ScatterSmem<K, ITEMS>*>(smem_rs);
   __shared__ uint32_t wsum[RS_WARPS];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const unsigned bins = 1u << width;
@@ -149,20 +163,20 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
     reinterpret_cast<uint32_t*>(&sm.wcnt[0][0])[x] = 0;
   __syncthreads();
   const unsigned lt = (1u << lane) - 1u;
-  const int64_t tbase = (int64_t)blockIdx.x * RS_TILE;
-  const int64_t wbase = tbase + (int64_t)warp * (32 * RS_ITEMS) + lane;
-  const int nv = (int)(n - tbase < RS_TILE ? n - tbase : RS_TILE);
+  const int64_t tbase = (int64_t)blockIdx.x * TILE;
+  const int64_t wbase = tbase + (int64_t)warp * (32 * ITEMS) + lane;
+  const int nv = (int)(n - tbase < TILE ? n - tbase : TILE);
   // rank of each pair among its warp's pairs of the same digit so far; places
   // past the end take the last digit and end up past the tile's last pair
-  K key[RS_ITEMS];
-  uint32_t rk[RS_ITEMS / 2];  // two 16-bit places per word
+  K key[ITEMS];
+  uint32_t rk[ITEMS / 2];  // two 16-bit places per word
 #pragma unroll
-  for (int i = 0; i < RS_ITEMS; ++i) {
+  for (int i = 0; i < ITEMS; ++i) {
     const int64_t k = wbase + i * 32;
     key[i] = k < n ? keys_in[k * stride] : ~K(0);
   }
 #pragma unroll
-  for (int i = 0; i < RS_ITEMS; ++i) {
+  for (int i = 0; i < ITEMS; ++i) {
     const unsigned d = (unsigned)(key[i] >> shift) & (bins - 1);
     unsigned peers = SPM_FULL_MASK;
 #pragma unroll
@@ -212,16 +226,16 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
   }
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < RS_ITEMS; ++i) {
+  for (int i = 0; i < ITEMS; ++i) {
     const unsigned d = (unsigned)(key[i] >> shift) & (bins - 1);
     const unsigned pos = sm.wcnt[warp][d] + ((rk[i / 2] >> (16 * (i & 1))) & 0xffffu);
     sm.keys[pos] = key[i];
     rk[i / 2] = (i & 1) ? (rk[i / 2] & 0xffffu) | (pos << 16) : (rk[i / 2] & 0xffff0000u) | pos;
   }
   __syncthreads();
-  uint32_t g[RS_ITEMS];
+  uint32_t g[ITEMS];
 #pragma unroll
-  for (int i = 0; i < RS_ITEMS; ++i) {
+  for (int i = 0; i < ITEMS; ++i) {
     const int x = t + i * RS_THREADS;
     if (x < nv) {
       const K k = sm.keys[x];
@@ -232,13 +246,13 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
   __syncthreads();
   int32_t* sv = reinterpret_cast<int32_t*>(sm.keys);
 #pragma unroll
-  for (int i = 0; i < RS_ITEMS; ++i) {
+  for (int i = 0; i < ITEMS; ++i) {
     const int64_t k = wbase + i * 32;
     if (k < n) sv[(rk[i / 2] >> (16 * (i & 1))) & 0xffffu] = vals_in ? vals_in[k] : (int32_t)k;
   }
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < RS_ITEMS; ++i) {
+  for (int i = 0; i < ITEMS; ++i) {
     const int x = t + i * RS_THREADS;
     if (x < nv) vals_out[g[i]] = sv[x];
   }
@@ -249,24 +263,36 @@ struct SortScratch {
   uint32_t* dtot = nullptr;
 };
 
+template <typename K, int ITEMS>
+spm_status radix_pass_t(const K* keys, int64_t stride, const int32_t* vals, K* keys_out,
+                        int32_t* vals_out, int64_t n, int shift, int width, const SortScratch& sc,
+                        cudaStream_t s) {
+  const int ntiles = (int)ceil_div<int64_t>(n, RS_THREADS * ITEMS);
+  constexpr int smem = (int)sizeof(ScatterSmem<K, ITEMS>);
+  SPM_CUDA_TRY(cudaFuncSetAttribute(rs_scatter_kernel<K, ITEMS>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  if (ntiles > 1) {
+    rs_hist_kernel<K, ITEMS><<<ntiles, RS_THREADS, 0, s>>>(keys, stride, n, shift, width, sc.hist,
+                                                          ntiles);
+    const int st = std::min(1024, (ntiles + 31) / 32 * 32);
+    rs_scan_rows_kernel<<<1 << width, st, 0, s>>>(sc.hist, ntiles, sc.dtot);
+  }
+  rs_scatter_kernel<K, ITEMS><<<ntiles, RS_THREADS, smem, s>>>(
+      keys, stride, vals, keys_out, vals_out, n, shift, width, ntiles > 1 ? sc.hist : nullptr,
+      ntiles > 1 ? sc.dtot : nullptr, ntiles);
+  SPM_CUDA_TRY(cudaGetLastError());
+  return SPM_OK;
+}
+
 // One stable pass by digit (key >> shift) & (2^width - 1).
 template <typename K>
 spm_status radix_pass(const K* keys, int64_t stride, const int32_t* vals, K* keys_out,
                       int32_t* vals_out, int64_t n, int shift, int width, const SortScratch& sc,
                       cudaStream_t s) {
-  const int ntiles = (int)ceil_div<int64_t>(n, RS_TILE);
-  constexpr int smem = (int)sizeof(ScatterSmem<K>);
-  SPM_CUDA_TRY(cudaFuncSetAttribute(rs_scatter_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  if (ntiles > 1) {
-    rs_hist_kernel<K><<<ntiles, RS_THREADS, 0, s>>>(keys, stride, n, shift, width, sc.hist, ntiles);
-    const int st = std::min(1024, (ntiles + 31) / 32 * 32);
-    rs_scan_rows_kernel<<<1 << width, st, 0, s>>>(sc.hist, ntiles, sc.dtot);
-  }
-  rs_scatter_kernel<K><<<ntiles, RS_THREADS, smem, s>>>(
-      keys, stride, vals, keys_out, vals_out, n, shift, width, ntiles > 1 ? sc.hist : nullptr,
-      ntiles > 1 ? sc.dtot : nullptr, ntiles);
-  SPM_CUDA_TRY(cudaGetLastError());
-  return SPM_OK;
+  return n <= RS_SMALL ? radix_pass_t<K, RS_ITEMS_SMALL>(keys, stride, vals, keys_out, vals_out, n,
+                                                        shift, width, sc, s)
+                       : radix_pass_t<K, RS_ITEMS>(keys, stride, vals, keys_out, vals_out, n, shift,
+                                                   width, sc, s);
 }
 
 // Digits of a field of `bits` bits: count and width of each (the last may reach
@@ -625,39 +651,59 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// Exclusive scan of cnt[0 .. n) in place, total to *total (one block).
+// Exclusive scan of cnt[0 .. n) in place, total to *total (one block, 4096
+// entries a round; cnt is 16-byte aligned).
 __global__ void __launch_bounds__(1024)
     seg_scan_kernel(uint32_t* __restrict__ cnt, int64_t n, uint32_t* __restrict__ total) {
   __shared__ uint32_t wsum[32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int64_t per = (n + 1023) / 1024;
-  const int64_t b = t * per, e = b + per < n ? b + per : n;
-  uint32_t v = 0;
-#pragma unroll 4
-  for (int64_t i = b; i < e; ++i) v += cnt[i];
-  uint32_t x = v;
+  uint32_t carry = 0;
+  auto load = [&](int64_t b) -> uint4 {
+    if (b + 4 <= n) return *reinterpret_cast<const uint4*>(cnt + b);
+    return make_uint4(b < n ? cnt[b] : 0u, b + 1 < n ? cnt[b + 1] : 0u, b + 2 < n ? cnt[b + 2] : 0u, 0u);
+  };
+  uint4 v = load(4 * t);
+  for (int64_t base = 0; base < n; base += 4096) {
+    const int64_t b = base + 4 * t;
+    const uint4 ahead = load(b + 4096);
+    const uint32_t own = v.x + v.y + v.z + v.w;
+    uint32_t x = own;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(SPM_FULL_MASK, x, o);
-    if (lane >= o) x += y;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(SPM_FULL_MASK, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[warp] = x;
+    __syncthreads();
+    uint32_t y = wsum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t z = __shfl_up_sync(SPM_FULL_MASK, y, o);
+      if (lane >= o) y += z;
+    }
+    const uint32_t all = __shfl_sync(SPM_FULL_MASK, y, 31);
+    const uint32_t pre = __shfl_sync(SPM_FULL_MASK, y, warp > 0 ? warp - 1 : 0);
+    const uint32_t e0 = carry + (warp > 0 ? pre : 0u) + x - own;
+    const uint4 o = make_uint4(e0, e0 + v.x, e0 + v.x + v.y, e0 + v.x + v.y + v.z);
+    if (b + 4 <= n) {
+      *reinterpret_cast<uint4*>(cnt + b) = o;
+    } else {
+      if (b < n) cnt[b] = o.x;
+      if (b + 1 < n) cnt[b + 1] = o.y;
+      if (b + 2 < n) cnt[b + 2] = o.z;
+    }
+    carry += all;
+    v = ahead;
+    __syncthreads();
   }
-  if (lane == 31) wsum[warp] = x;
-  __syncthreads();
-  uint32_t pre = 0;
-  for (int w = 0; w < warp; ++w) pre += wsum[w];
-  uint32_t run = pre + x - v;
-  if (t == 1023) *total = run + v;
-  for (int64_t i = b; i < e; ++i) {
-    const uint32_t c = cnt[i];
-    cnt[i] = run;
-    run += c;
-  }
+  if (t == 0) *total = carry;
 }
 
 // woff[j] = min{k in [0, n] : C(k) * P >= j * C(n)},
 // C(k) = k + row_cost * (row starts before k), C(n) = n + row_cost * heads;
 // off[z] = woff[z * units].  One warp per unit: a binary search over the
-// segments, then the row starts inside one.
+// segments, then the row starts inside one.  For copies of many nonzeros per
+// unit (50M: 78 us); see units_by_position_kernel.
 __global__ void __launch_bounds__(256)
     balanced_units_kernel(const int* __restrict__ rows, int64_t stride, int64_t n,
                           const uint32_t* __restrict__ seg, int64_t nseg,
@@ -680,14 +726,20 @@ __global__ void __launch_bounds__(256)
       const int64_t base = lo * SEG;
       res = base + SEG < n ? base + SEG : n;
       int64_t before = seg[lo];
-      int last = base > 0 ? rows[(base - 1) * stride] : -1;
+      int r[SEG / 32];
+#pragma unroll
       for (int i = 0; i < SEG / 32; ++i) {
         const int64_t k = base + i * 32 + lane;
-        const int r = k < n ? rows[k * stride] : -1;
-        int prev = __shfl_up_sync(SPM_FULL_MASK, r, 1);
+        r[i] = k < n ? rows[k * stride] : -1;
+      }
+      int last = base > 0 ? rows[(base - 1) * stride] : -1;
+#pragma unroll
+      for (int i = 0; i < SEG / 32; ++i) {
+        const int64_t k = base + i * 32 + lane;
+        int prev = __shfl_up_sync(SPM_FULL_MASK, r[i], 1);
         if (lane == 0) prev = last;
-        last = __shfl_sync(SPM_FULL_MASK, r, 31);
-        const unsigned hb = __ballot_sync(SPM_FULL_MASK, r >= 0 && r != prev);
+        last = __shfl_sync(SPM_FULL_MASK, r[i], 31);
+        const unsigned hb = __ballot_sync(SPM_FULL_MASK, r[i] >= 0 && r[i] != prev);
         const int64_t C = k + (int64_t)row_cost * (before + __popc(hb & ((1u << lane) - 1u)));
         const unsigned ok = __ballot_sync(SPM_FULL_MASK, k <= n && C * P >= target);
         if (ok) {
@@ -700,6 +752,75 @@ __global__ void __launch_bounds__(256)
     if (lane == 0) {
       woff[j] = res;
       if (j % units == 0) off[j / units] = res;
+    }
+  }
+}
+
+// The same from the side of the positions, for few nonzeros per unit: position
+// k is the first with C(k) * P >= j * C(n) for the units
+// floor(C(k - 1) P / C(n)) < j <= floor(C(k) P / C(n)).  One warp per 32
+// positions, which counts the row starts before them in its segment (30,000
+// nonzeros, 38,912 units: 51 us by search, 47 us with a warp per segment and
+// its 16 chains of 64-bit divisions, 6 us so).
+__global__ void __launch_bounds__(256)
+    units_by_position_kernel(const int* __restrict__ rows, int64_t stride, int64_t n,
+                             const uint32_t* __restrict__ seg, int64_t nseg,
+                             const uint32_t* __restrict__ heads, int64_t P, int units, int row_cost,
+                             int64_t* __restrict__ woff, int64_t* __restrict__ off) {
+  const int lane = threadIdx.x & 31;
+  const int64_t Ct = n + (int64_t)row_cost * (int64_t)(*heads);
+  // positions 0 .. n: position n closes the copy
+  for (int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q * 32 <= n;
+       q += (int64_t)gridDim.x * (blockDim.x >> 5)) {
+    const int64_t g = q / (SEG / 32), base = g * SEG;
+    const int chunk = (int)(q % (SEG / 32));
+    int r[SEG / 32];
+#pragma unroll
+    for (int i = 0; i < SEG / 32; ++i) {
+      const int64_t k = base + i * 32 + lane;
+      r[i] = i <= chunk && k < n ? rows[k * stride] : -1;
+    }
+    int last = base > 0 ? rows[(base - 1) * stride] : -1;
+    int64_t before = g < nseg ? seg[g] : *heads;
+    bool prev_head = false;  // whether position 32 q - 1 starts a row
+    if (chunk == 0 && base > 0) prev_head = base == 1 || rows[(base - 2) * stride] != last;
+    unsigned hb = 0;
+#pragma unroll
+    for (int i = 0; i < SEG / 32; ++i) {
+      if (i <= chunk) {
+        int prev = __shfl_up_sync(SPM_FULL_MASK, r[i], 1);
+        if (lane == 0) prev = last;
+        last = __shfl_sync(SPM_FULL_MASK, r[i], 31);
+        hb = __ballot_sync(SPM_FULL_MASK, r[i] >= 0 && r[i] != prev);
+        if (i < chunk) {
+          before += __popc(hb);
+          prev_head = hb >> 31;
+        }
+      }
+    }
+    const int64_t k = q * 32 + lane;
+    const int64_t C = k + (int64_t)row_cost * (before + __popc(hb & ((1u << lane) - 1u)));
+    const int j1 = k <= n ? (int)(C * P / Ct) : (int)P;
+    int j0 = __shfl_up_sync(SPM_FULL_MASK, j1, 1);
+    if (lane == 0)
+      j0 = q == 0 ? -1
+                  : (int)((k - 1 + (int64_t)row_cost * (before - (prev_head ? 1 : 0))) * P / Ct);
+    const int cnt = k <= n ? j1 - j0 : 0;
+    if (cnt > 0 && cnt <= 4) {
+      for (int j = j0 + 1; j <= j1; ++j) {
+        woff[j] = k;
+        if (j % units == 0) off[j / units] = k;
+      }
+    }
+    unsigned many = __ballot_sync(SPM_FULL_MASK, cnt > 4);
+    while (many) {
+      const int l = __ffs(many) - 1;
+      many &= many - 1;
+      const int a = __shfl_sync(SPM_FULL_MASK, j0, l), e = __shfl_sync(SPM_FULL_MASK, j1, l);
+      for (int j = a + 1 + lane; j <= e; j += 32) {
+        woff[j] = q * 32 + l;
+        if (j % units == 0) off[j / units] = q * 32 + l;
+      }
     }
   }
 }
@@ -787,8 +908,12 @@ void partition_copy(spmttkrp_plan_s* p, int d, const int* rows, int64_t stride, 
     const int64_t nseg = ceil_div<int64_t>(n, SEG);
     row_heads_kernel<<<grid_for(nseg * 32, T), T, 0, s>>>(rows, stride, n, nseg, seg, mask);
     seg_scan_kernel<<<1, 1024, 0, s>>>(seg, nseg, heads);
-    balanced_units_kernel<<<grid_for((P + 1) * 32, T), T, 0, s>>>(
-        rows, stride, n, seg, nseg, heads, P, units, SPM_ROW_COST, c.woff, c.off);
+    if (n < 16 * P)
+      units_by_position_kernel<<<grid_for(n + 32, T), T, 0, s>>>(
+          rows, stride, n, seg, nseg, heads, P, units, SPM_ROW_COST, c.woff, c.off);
+    else
+      balanced_units_kernel<<<grid_for((P + 1) * 32, T), T, 0, s>>>(
+          rows, stride, n, seg, nseg, heads, P, units, SPM_ROW_COST, c.woff, c.off);
     return;
   }
   equal_offsets_kernel<<<grid_for(p->kappa + 1, T), T, 0, s>>>(n, p->kappa, c.off);
@@ -829,7 +954,7 @@ struct BuildScratch {
     q[1] = take(sizeof(unsigned long long) * (size_t)cap);
     q[2] = take(sizeof(int32_t) * (size_t)cap);
     q[3] = take(sizeof(int32_t) * (size_t)cap);
-    q[4] = take(sizeof(uint32_t) * RS_BINS * (size_t)ceil_div<int64_t>(cap, RS_TILE));
+    q[4] = take(sizeof(uint32_t) * RS_BINS * (size_t)rs_tiles_cap(cap));
     q[5] = take(sizeof(uint32_t) * RS_BINS);
     q[6] = take(sizeof(int64_t) * SPM_MAX_MODES + sizeof(unsigned) * SPM_MAX_MODES);
     if (b) {
