@@ -239,16 +239,12 @@ spm_status grow(T** buf, size_t* cap, size_t need) {
   if (need <= *cap) return SPM_OK;
   const size_t n = std::max(need, *cap + *cap / 2);
   if (*buf) {
-    cudaFree(*buf);  // synchronises the device: queued work is done with it
+    cudaDeviceSynchronize();  // queued work is done with it
+    dev_free(*buf, sizeof(T) * *cap);
     *buf = nullptr;
     *cap = 0;
   }
-  cudaError_t e = cudaMalloc((void**)buf, sizeof(T) * n);
-  if (e != cudaSuccess) {
-    (void)cudaGetLastError();
-    *buf = nullptr;
-    return e == cudaErrorMemoryAllocation ? SPM_ERR_OOM : SPM_ERR_CUDA;
-  }
+  SPM_TRY(dev_alloc((void**)buf, sizeof(T) * n));
   *cap = n;
   return SPM_OK;
 }
@@ -540,9 +536,9 @@ spm_status batch_sweep(spm_batch_s* B, cudaStream_t s) {
 void batch_free(spm_batch_s* B) {
   if (!B) return;
   cudaDeviceSynchronize();
-  if (B->bt) cudaFree(B->bt);
-  if (B->items) cudaFree(B->items);
-  if (B->queue) cudaFree(B->queue);
+  dev_free(B->bt, sizeof(BatchTensor) * B->bt_cap);
+  dev_free(B->items, sizeof(int2) * B->items_cap);
+  dev_free(B->queue, sizeof(int) * B->queue_cap);
   if (B->ev_fork) cudaEventDestroy(B->ev_fork);
   if (B->ev_join) cudaEventDestroy(B->ev_join);
   if (B->side) cudaStreamDestroy(B->side);

@@ -13,12 +13,7 @@ spm_status plan_alloc(spmttkrp_plan_s* p, void** ptr, size_t bytes) {
   if (p->nallocs >= (int)(sizeof(p->allocs) / sizeof(p->allocs[0]))) return SPM_ERR_OOM;
   if (alloc_fault_due()) return SPM_ERR_OOM;  // injected by spm_inject_alloc_failure
   if (bytes == 0) bytes = 16;
-  cudaError_t e = cudaMalloc(ptr, bytes);
-  if (e != cudaSuccess) {
-    (void)cudaGetLastError();
-    *ptr = nullptr;
-    return e == cudaErrorMemoryAllocation ? SPM_ERR_OOM : SPM_ERR_CUDA;
-  }
+  SPM_TRY(dev_alloc(ptr, bytes));
   p->alloc_bytes[p->nallocs] = bytes;
   p->allocs[p->nallocs++] = *ptr;
   p->bytes += bytes;
@@ -31,12 +26,9 @@ spm_status plan_realloc(spmttkrp_plan_s* p, void** ptr, size_t bytes) {
   if (i == p->nallocs) return SPM_ERR_INVALID_ARG;
   if (bytes == 0) bytes = 16;
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, bytes);
-  if (e != cudaSuccess) {
-    (void)cudaGetLastError();
-    return e == cudaErrorMemoryAllocation ? SPM_ERR_OOM : SPM_ERR_CUDA;
-  }
-  cudaFree(*ptr);
+  SPM_TRY(dev_alloc(&q, bytes));
+  cudaDeviceSynchronize();
+  dev_free(*ptr, p->alloc_bytes[i]);
   p->bytes = p->bytes - p->alloc_bytes[i] + bytes;
   p->allocs[i] = q;
   p->alloc_bytes[i] = bytes;
@@ -48,7 +40,8 @@ void plan_free(spmttkrp_plan_s* p, void** ptr) {
   int i = 0;
   while (i < p->nallocs && p->allocs[i] != *ptr) ++i;
   if (i == p->nallocs) return;
-  cudaFree(*ptr);
+  cudaDeviceSynchronize();
+  dev_free(*ptr, p->alloc_bytes[i]);
   p->bytes -= p->alloc_bytes[i];
   for (int j = i + 1; j < p->nallocs; ++j) {
     p->allocs[j - 1] = p->allocs[j];
@@ -87,7 +80,7 @@ void free_plan(spmttkrp_plan_s* p) {
   if (p->als.ev_fork) cudaEventDestroy(p->als.ev_fork);
   if (p->als.ev_join) cudaEventDestroy(p->als.ev_join);
   if (p->als.side) cudaStreamDestroy(p->als.side);
-  for (int i = 0; i < p->nallocs; ++i) cudaFree(p->allocs[i]);
+  for (int i = 0; i < p->nallocs; ++i) dev_free(p->allocs[i], p->alloc_bytes[i]);
   (void)cudaGetLastError();
   delete p;
 }
@@ -194,7 +187,7 @@ spm_status spmttkrp_plan(spmttkrp_plan_t* out, int nmodes, const int64_t* dims, 
   if (st == SPM_OK && cudaMemsetAsync(p->dev_err, 0, 2 * sizeof(int), s) != cudaSuccess) st = SPM_ERR_CUDA;
   if (st == SPM_OK) st = build_copies(p, idx, vals, s);
   if (st != SPM_OK) {
-    cudaStreamSynchronize(s);
+    cudaDeviceSynchronize();
     (void)cudaGetLastError();
     free_plan(p);
     return st;

@@ -328,8 +328,11 @@ struct PackSpec {
   int lo, hi;
   int shift[SPM_MAX_MODES];
 };
-__global__ void validate_pack_kernel(IdxPtrs idx, int nmodes, const int64_t* __restrict__ dims,
-                                     int64_t n, PackSpec spec, unsigned long long* __restrict__ key,
+struct DimLimits {
+  uint32_t d[SPM_MAX_MODES];  // dims, each below 2^31
+};
+__global__ void validate_pack_kernel(IdxPtrs idx, int nmodes, DimLimits dims, int64_t n,
+                                     PackSpec spec, unsigned long long* __restrict__ key,
                                      int* __restrict__ err) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
@@ -337,7 +340,7 @@ __global__ void validate_pack_kernel(IdxPtrs idx, int nmodes, const int64_t* __r
     unsigned long long v = 0;
     for (int w = 0; w < nmodes; ++w) {
       const int32_t c = idx.p[w][k];
-      bad |= (c < 0) || ((int64_t)c >= dims[w]);
+      bad |= (uint32_t)c >= dims.d[w];  // negative indices too
       if (w >= spec.lo && w <= spec.hi) v |= (unsigned long long)(uint32_t)c << spec.shift[w];
     }
     if (key) key[k] = v;
@@ -933,13 +936,12 @@ int64_t sort_capacity(int N, const int64_t* dims, int64_t nn, int policy, int ka
   return std::max(nn, rows);
 }
 
-// Transient device memory of a build: one stream-ordered allocation.
+// Transient device memory of a build: one allocation.
 struct BuildScratch {
   void* base = nullptr;
   unsigned long long *ka = nullptr, *kb = nullptr;  // keys
   int32_t *va = nullptr, *vb = nullptr;             // payloads
   SortScratch sort;
-  int64_t* dims = nullptr;
   unsigned* count = nullptr;  // non-empty rows per mode
   // Bytes for `cap` keys; the pieces are laid out when `p` is non-null.
   static size_t layout(int64_t cap, unsigned char* p, BuildScratch* b) {
@@ -956,7 +958,7 @@ struct BuildScratch {
     q[3] = take(sizeof(int32_t) * (size_t)cap);
     q[4] = take(sizeof(uint32_t) * RS_BINS * (size_t)rs_tiles_cap(cap));
     q[5] = take(sizeof(uint32_t) * RS_BINS);
-    q[6] = take(sizeof(int64_t) * SPM_MAX_MODES + sizeof(unsigned) * SPM_MAX_MODES);
+    q[6] = take(sizeof(unsigned) * SPM_MAX_MODES);
     if (b) {
       b->base = p;
       b->ka = reinterpret_cast<unsigned long long*>(q[0]);
@@ -965,22 +967,23 @@ struct BuildScratch {
       b->vb = reinterpret_cast<int32_t*>(q[3]);
       b->sort.hist = reinterpret_cast<uint32_t*>(q[4]);
       b->sort.dtot = reinterpret_cast<uint32_t*>(q[5]);
-      b->dims = reinterpret_cast<int64_t*>(q[6]);
-      b->count = reinterpret_cast<unsigned*>(b->dims + SPM_MAX_MODES);
+      b->count = reinterpret_cast<unsigned*>(q[6]);
     }
     return at;
   }
-  spm_status alloc(int64_t cap, cudaStream_t s) {
+  size_t bytes = 0;
+  spm_status alloc(int64_t cap) {
     void* p = nullptr;
-    SPM_CUDA_TRY(cudaMallocAsync(&p, layout(cap, nullptr, nullptr), s));
+    bytes = layout(cap, nullptr, nullptr);
+    SPM_TRY(dev_alloc(&p, bytes));
     layout(cap, static_cast<unsigned char*>(p), this);
     return SPM_OK;
   }
-  spm_status release(cudaStream_t s) {
-    SPM_CUDA_TRY(cudaFreeAsync(base, s));
-    base = nullptr;
-    return SPM_OK;
-  }
+  // Freed by the owner's scope, after the build's stream is drained.
+  BuildScratch() = default;
+  BuildScratch(const BuildScratch&) = delete;
+  BuildScratch& operator=(const BuildScratch&) = delete;
+  ~BuildScratch() { dev_free(base, bytes); }
 };
 
 template <int RI>
@@ -993,15 +996,17 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
   const int T = 256;
   const int G = grid_for(n, T);
 
-  // scratch (one stream-ordered allocation, freed at the end)
   const int64_t nn = n > 0 ? n : 1;
   // the keys, payloads and histograms hold nnz entries, or I_d entries where
   // Scheme 1 sorts the rows of a mode by degree
   const int64_t cap = sort_capacity(N, p->dims, nn, p->policy, p->kappa);
   BuildScratch b;
-  SPM_TRY(b.alloc(cap, s));
+  struct Drain {  // runs before the scratch is freed, on every way out
+    cudaStream_t s;
+    ~Drain() { cudaStreamSynchronize(s); }
+  } drain{s};
+  SPM_TRY(b.alloc(cap));
   const SortScratch& sc = b.sort;
-  SPM_CUDA_TRY(cudaMemcpyAsync(b.dims, p->dims, sizeof(int64_t) * N, cudaMemcpyHostToDevice, s));
 
   // modes grouped into <=64-bit key words from the last mode backwards
   int bits[SPM_MAX_MODES];
@@ -1033,8 +1038,11 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
   };
 
   // Validation: every index within its dimension; and the keys of the first sort.
-  if (n > 0)
-    validate_pack_kernel<<<G, T, 0, s>>>(idx, N, b.dims, n, spec_of(groups[0]), b.ka, p->dev_err);
+  if (n > 0) {
+    DimLimits lim{};
+    for (int w = 0; w < N; ++w) lim.d[w] = (uint32_t)p->dims[w];
+    validate_pack_kernel<<<G, T, 0, s>>>(idx, N, lim, n, spec_of(groups[0]), b.ka, p->dev_err);
+  }
   int herr = 0;
   SPM_CUDA_TRY(cudaMemcpyAsync(&herr, p->dev_err, sizeof(int), cudaMemcpyDeviceToHost, s));
   SPM_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1209,7 +1217,6 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
     SPM_CUDA_TRY(cudaMemcpyAsync(h_cnt, b.count, sizeof(unsigned) * SPM_MAX_MODES,
                                  cudaMemcpyDeviceToHost, s));
   SPM_CUDA_TRY(cudaGetLastError());
-  SPM_TRY(b.release(s));
   SPM_CUDA_TRY(cudaStreamSynchronize(s));
   for (int d = 0; d < N; ++d) p->mode[d].empty_rows = p->dims[d] - (int64_t)h_cnt[d];
   return st;

@@ -106,6 +106,11 @@ struct spmttkrp_plan_s {
 
 namespace spm {
 
+// Device memory (dev_alloc.cu).  dev_free: with the size it was allocated with,
+// once no queued work uses it.
+spm_status dev_alloc(void** ptr, size_t bytes);
+void dev_free(void* ptr, size_t bytes);
+
 // Allocation owned by the plan (recorded for destroy and for plan_bytes).
 spm_status plan_alloc(spmttkrp_plan_s* p, void** ptr, size_t bytes);
 

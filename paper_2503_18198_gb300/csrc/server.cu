@@ -95,15 +95,20 @@ void release_plan(spm_server_s* S, Job* j) {
   }
 }
 
+size_t one_factor_bytes(const spm_server_s* S, const Job* j, int w) {
+  return ((S->flags & SPM_FACTOR_MASK) == SPM_FACTOR_BF16 ? 2 : 4) * (size_t)j->dims[w] * j->R;
+}
+
 void release_all(spm_server_s* S, Job* j) {
   release_plan(S, j);
+  if (j->fac[0] || j->lamfit) cudaDeviceSynchronize();  // queued work is done with them
   for (int w = 0; w < SPM_MAX_MODES; ++w)
     if (j->fac[w]) {
-      cudaFree(j->fac[w]);
+      dev_free(j->fac[w], one_factor_bytes(S, j, w));
       j->fac[w] = nullptr;
     }
   if (j->lamfit) {
-    cudaFree(j->lamfit);
+    dev_free(j->lamfit, sizeof(double) * (j->R + 1));
     j->lamfit = nullptr;
   }
   S->used -= std::min(S->used, j->held);
@@ -128,11 +133,8 @@ spm_status admit(spm_server_s* S, Job* j) {
   const bool bf16 = (S->flags & SPM_FACTOR_MASK) == SPM_FACTOR_BF16;
   for (int w = 0; w < j->N; ++w) {
     const int64_t n = j->dims[w] * j->R;
-    const size_t bytes = (bf16 ? 2 : 4) * (size_t)n;
-    if (cudaMalloc(&j->fac[w], bytes) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return SPM_ERR_OOM;
-    }
+    const size_t bytes = one_factor_bytes(S, j, w);
+    SPM_TRY(dev_alloc(&j->fac[w], bytes));
     S->used += bytes;
     j->held += bytes;
     if (bf16)
@@ -141,10 +143,7 @@ spm_status admit(spm_server_s* S, Job* j) {
     else
       SPM_CUDA_TRY(cudaMemcpyAsync(j->fac[w], j->init[w], bytes, cudaMemcpyDeviceToDevice, s));
   }
-  if (cudaMalloc((void**)&j->lamfit, sizeof(double) * (j->R + 1)) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return SPM_ERR_OOM;
-  }
+  SPM_TRY(dev_alloc((void**)&j->lamfit, sizeof(double) * (j->R + 1)));
   S->used += sizeof(double) * (j->R + 1);
   j->held += sizeof(double) * (j->R + 1);
   SPM_CUDA_TRY(cudaGetLastError());
