@@ -209,7 +209,21 @@ __device__ __forceinline__ void gram_reduce_body(const double* __restrict__ part
     double v[GR_ENTRIES];
 #pragma unroll
     for (int k = 0; k < GR_ENTRIES; ++k) v[k] = 0.0;
-    for (int b = lane; b < nblocks; b += 32) {
+    // the loads of four partials ahead of the (ordered) additions
+    int b = lane;
+    for (; b + 96 < nblocks; b += 128) {
+      double x[4][GR_ENTRIES];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int k = 0; k < GR_ENTRIES; ++k)
+          x[u][k] = e + k < RR ? part[(int64_t)(b + 32 * u) * RR + e + k] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int k = 0; k < GR_ENTRIES; ++k) v[k] += x[u][k];
+    }
+    for (; b < nblocks; b += 32) {
       const double* pb = part + (int64_t)b * RR + e;
 #pragma unroll
       for (int k = 0; k < GR_ENTRIES; ++k)

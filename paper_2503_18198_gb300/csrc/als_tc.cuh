@@ -131,29 +131,64 @@ __device__ __forceinline__ void df_add(df& a, float x) {  // a += x (error-free 
 // so when step j is done row j + 1 holds X(j + 1, :).  A column of W is then
 // R dot products: no substitution chains.
 //
-// Bound: FP64 (2 fused multiply-adds per cycle and SM) and the chain pivot ->
-// reciprocal -> column -> next pivot, one per row.  So every entry of T lives
-// in a register of the thread that owns it for the whole elimination (entry e
-// of the triangle, row-major, belongs to thread e mod 256: the entries still
-// active at step j are a contiguous tail, spread evenly over the warps), the
-// pivot row and column go through shared memory once per step, and one warp
-// forms the reciprocal (a Newton step in place of an FP64 division).
-// One system, one column per block, alone on the GPU, R = 16 / 32 / 64: 12.3 /
-// 25.6 / 78 us (20 / 46 / 139 us for a Cholesky factor with triangle indices
-// recomputed in every step and two substitution chains of R steps per column);
-// 96 systems of R = 16 and 32 side by side 49 us (105 us).
+// Every entry of T lives in a register of the thread that owns it for the whole
+// elimination (entry e of the triangle, row-major, belongs to thread e mod 256:
+// the entries still active at step j are a contiguous tail, spread evenly over
+// the warps), the pivot row and column go through shared memory once per step,
+// and one warp forms the reciprocal.
+//
+// Bound: the chain pivot -> reciprocal -> column -> next pivot, and in FP64 its
+// throughput (2 fused multiply-adds per cycle and SM, 64 cycles each).  So the
+// elimination and the dot products run in double-float (FP32 pairs, 2^-46) on
+// V scaled by powers of two to a diagonal in [1, 4), and each column then takes
+// one step of iterative refinement: its residual e_c - V w in FP64 (R^2
+// multiply-adds), the correction X^T D^{-1} X r in FP32.  That leaves an error
+// below that of an FP64 factorisation while cond(V) is moderate: it is taken
+// when every pivot is at least 2^-16 and trace(V^{-1}) of the scaled system at
+// most 2^12, which bounds cond(V) by 2^12 * 4 R (the error of the pairs,
+// 2^-46 cond, times the error of the FP32 correction, 2^-24 cond, is then below
+// 2^-53 cond * R); otherwise the same elimination runs in FP64, which also
+// decides whether V is positive definite.  Rows solved with it are as far from
+// extended precision as with an FP64 Cholesky factor for cond(V) = 3 .. 1e8 at
+// R = 16, 32, 64 (rms 2.5e-8, the FP32 rounding of Z; the splitting's 2^-34 is
+// the rest): tests/test_gpu_system.py.
+// One system, one column per block, alone on the GPU, R = 16 / 32 / 64: 11.5 /
+// 18.5 / 51 us (the same elimination in FP64 12.3 / 25.6 / 78 us; before it, a
+// Cholesky factor and two substitution chains per column, 20 / 46 / 139 us).
 // ---------------------------------------------------------------------------
 constexpr int SYS_THREADS = 256;
 constexpr int SYS_RMAX = 64;
-constexpr int SYS_COLS = 16;  // most columns of W per block
+constexpr int SYS_COLS = 8;  // most columns of W per block
+constexpr int SYS_TRI = SYS_RMAX * (SYS_RMAX + 1) / 2;
 
 // Shared memory of a system block.
 struct SystemSmem {
-  double X[SYS_RMAX * (SYS_RMAX + 1)];  // X(k, c) at k (R | 1) + c
-  double W[SYS_COLS * SYS_RMAX];        // per column c: D^{-1} X(:, c), then W(:, c)
-  double piv[2][SYS_RMAX];              // step j: T(k, j) for k >= j, X(j, k) for k < j
-  double nl[SYS_RMAX];                  // step j: -T(i, j) / d_j for i > j
-  double rd[SYS_RMAX];                  // 1 / d_k
+  union {
+    double X[SYS_RMAX * (SYS_RMAX + 1)];  // FP64: X(k, c) at k (R | 1) + c
+    struct {                              // pairs: lower triangles, entry i (i + 1) / 2 + k
+      double A[SYS_TRI];                  // V scaled
+      float2 XF[SYS_TRI];                 // X as (hi, lo)
+    };
+  };
+  double W[SYS_COLS * SYS_RMAX];          // per column c: D^{-1} X(:, c) (FP64), then W(:, c)
+  union {
+    float2 y[SYS_COLS * SYS_RMAX];        // pairs: D^{-1} X(:, c)
+    float ru[2][SYS_COLS * SYS_RMAX];     // then the residual and D^{-1} X r
+  };
+  union {                                 // step j: T(k, j) for k >= j, X(j, k) for k < j
+    double piv[2][SYS_RMAX];
+    float2 pivf[2][SYS_RMAX];
+  };
+  union {                                 // step j: -T(i, j) / d_j for i > j
+    double nl[SYS_RMAX];
+    float2 nlf[SYS_RMAX];
+  };
+  union {                                 // 1 / d_k
+    double rd[SYS_RMAX];
+    float2 rdf[SYS_RMAX];
+  };
+  int ex[SYS_RMAX];                       // row i of V is scaled by 2^-ex[i]
+  float red[SYS_THREADS / 32];
   int bad;
 };
 
@@ -186,18 +221,64 @@ __device__ __forceinline__ RecipPos recip_pos(double d) {
   return {__hiloint2double(rh + ((1023 - ex) << 20), rl), fma(e, e, e)};
 }
 
+// W(:, c0 .. c0 + nc - 1) out of shared memory: w = W(:, c) goes to winv as FP32
+// (hi, lo) pairs (W(s, c) at s R + c and R R + s R + c), or, when wdig is
+// non-null, into the digit tile of the tensor-core solve: w is scaled by 2^-f_c
+// (|w_s| < 2^f_c), rounded to 49 fractional bits and recoded from the least
+// significant end into SW_DIG balanced 7-bit digits (|k_q| <= 64 below the
+// leading digit, |k_0| <= 128), w_s 2^-f_c ~ sum_q k_q 2^{-7(q+1)}; digit q of
+// w_s goes to row q R + c, column s of a K-major (K = R) BF16 tile, f_c to the
+// int array after it.
+__device__ __forceinline__ void system_store(const SystemSmem& sm, int R, int c0, int nc,
+                                             float* __restrict__ winv,
+                                             unsigned char* __restrict__ wdig) {
+  const int t = threadIdx.x, RR = R * R;
+  const int l = t & 31;
+  for (int cc = t >> 5; cc < nc; cc += SYS_THREADS / 32) {
+    const int c = c0 + cc;
+    int fx = INT_MIN;  // exponent bound of the column
+    for (int h = 0; h < 2; ++h) {
+      const int s = l + 32 * h;
+      if (s >= R) continue;
+      const double w = sm.W[cc * SYS_RMAX + s];
+      if (!wdig) {
+        const float hi = (float)w;
+        winv[s * R + c] = hi;
+        winv[RR + s * R + c] = (float)__dsub_rn(w, (double)hi);
+      }
+      const unsigned long long bits = __double_as_longlong(w) & 0x7FFFFFFFFFFFFFFFull;
+      if (bits != 0) {
+        const int be = (int)(bits >> 52);
+        fx = max(fx, be == 0 ? -1021 : be - 1022);  // |w| < 2^(be - 1022)
+      }
+    }
+    if (!wdig) continue;
+    fx = __reduce_max_sync(SPM_FULL_MASK, fx);
+    if (fx == INT_MIN) fx = 0;
+    if (l == 0) reinterpret_cast<int*>(wdig + SW_DIG * RR * 2)[c] = fx;
+    for (int h = 0; h < 2; ++h) {
+      const int s = l + 32 * h;
+      if (s >= R) continue;
+      long long n = __double2ll_rn(times_pow2(sm.W[cc * SYS_RMAX + s], 49 - fx));  // |n| <= 2^49
+#pragma unroll
+      for (int q = SW_DIG - 1; q >= 0; --q) {
+        long long dg = n;
+        if (q > 0) {
+          dg = ((n + 64) & 127) - 64;  // balanced remainder mod 128
+          n = (n - dg) >> 7;           // exact
+        }
+        *reinterpret_cast<__nv_bfloat16*>(wdig + tc::kmajor_offset(q * R + c, s, R)) =
+            __float2bfloat16_rn((float)(int)dg);
+      }
+    }
+  }
+}
+
 // Columns c0 .. c1-1 (at most SYS_COLS) of W by one block of SYS_THREADS
 // threads; NS >= R (R + 1) / 2 / SYS_THREADS entries of T per thread.  Every
 // block that takes columns of the same system computes the same L and X, and
 // an entry of W does not depend on which block or thread forms it, so any
 // split of the columns gives the same bits.
-// w = W(:, c) goes to winv as FP32 (hi, lo) pairs (W(s, c) at s R + c and
-// R R + s R + c), and, when wdig is non-null, into the digit tile of the
-// tensor-core solve: w is scaled by 2^-f_c (|w_s| < 2^f_c), rounded to 49
-// fractional bits and recoded from the least significant end into SW_DIG
-// balanced 7-bit digits (|k_q| <= 64 below the leading digit, |k_0| <= 128),
-// w_s 2^-f_c ~ sum_q k_q 2^{-7(q+1)}; digit q of w_s goes to row q R + c,
-// column s of a K-major (K = R) BF16 tile, f_c to the int array after it.
 // A pivot that is not positive and finite sets DEV_ERR_NUMERIC.
 template <int NS>
 __device__ __forceinline__ void system_body_ns(SystemSmem& sm, const double* __restrict__ grams,
@@ -311,52 +392,257 @@ __device__ __forceinline__ void system_body_ns(SystemSmem& sm, const double* __r
     if (x < nc * R && (t & 3) == 0) sm.W[(x / R) * SYS_RMAX + x % R] = wv[p];
   }
   __syncthreads();
-  const int l = t & 31;
-  for (int cc = t >> 5; cc < nc; cc += SYS_THREADS / 32) {
-    const int c = c0 + cc;
-    int fx = INT_MIN;  // exponent bound of the column
-    for (int h = 0; h < 2; ++h) {
-      const int s = l + 32 * h;
-      if (s >= R) continue;
-      const double w = sm.W[cc * SYS_RMAX + s];
-      const float hi = (float)w;
-      winv[s * R + c] = hi;
-      winv[RR + s * R + c] = (float)__dsub_rn(w, (double)hi);
-      const unsigned long long bits = __double_as_longlong(w) & 0x7FFFFFFFFFFFFFFFull;
-      if (bits != 0) {
-        const int be = (int)(bits >> 52);
-        fx = max(fx, be == 0 ? -1021 : be - 1022);  // |w| < 2^(be - 1022)
-      }
-    }
-    if (!wdig) continue;
-    fx = __reduce_max_sync(SPM_FULL_MASK, fx);
-    if (fx == INT_MIN) fx = 0;
-    if (l == 0) reinterpret_cast<int*>(wdig + SW_DIG * RR * 2)[c] = fx;
-    for (int h = 0; h < 2; ++h) {
-      const int s = l + 32 * h;
-      if (s >= R) continue;
-      long long n = __double2ll_rn(times_pow2(sm.W[cc * SYS_RMAX + s], 49 - fx));  // |n| <= 2^49
+  system_store(sm, R, c0, nc, winv, wdig);
+}
+
+// ---- the same in double-float with refinement ----
+__device__ __forceinline__ float2 ff_norm(float h, float l) {  // |h| >= |l|
+  const float s = __fadd_rn(h, l);
+  return make_float2(s, __fsub_rn(l, __fsub_rn(s, h)));
+}
+__device__ __forceinline__ float2 ff_mul(float2 a, float2 b) {
+  const float p = __fmul_rn(a.x, b.x);
+  float e = fmaf(a.x, b.x, -p);
+  e = fmaf(a.x, b.y, e);
+  e = fmaf(a.y, b.x, e);
+  return ff_norm(p, e);
+}
+__device__ __forceinline__ float2 ff_add(float2 a, float2 b) {
+  const float s = __fadd_rn(a.x, b.x);
+  const float bb = __fsub_rn(s, a.x);
+  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
+  return ff_norm(s, __fadd_rn(e, __fadd_rn(a.y, b.y)));
+}
+__device__ __forceinline__ float2 ff_fma(float2 a, float2 b, float2 c) {  // a b + c
+  const float p = __fmul_rn(a.x, b.x);
+  float e = fmaf(a.x, b.x, -p);
+  e = fmaf(a.x, b.y, e);
+  e = fmaf(a.y, b.x, e);
+  const float s = __fadd_rn(c.x, p);
+  const float bb = __fsub_rn(s, c.x);
+  const float t = __fadd_rn(__fsub_rn(c.x, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+  return ff_norm(s, __fadd_rn(t, __fadd_rn(c.y, e)));
+}
+
+// Columns c0 .. c1-1 of W; false (nothing written) when V is not well enough
+// conditioned for it.  Every block of a system takes the same decision.
+template <int NS>
+__device__ __forceinline__ bool system_pairs_ns(SystemSmem& sm, const double* __restrict__ grams,
+                                                int N, int d, int R, int c0, int c1,
+                                                float* __restrict__ winv,
+                                                unsigned char* __restrict__ wdig) {
+  constexpr int QG = NS % 3 == 0 ? 3 : 1;
+  const int t = threadIdx.x, lane = t & 31;
+  const int RR = R * R, T = R * (R + 1) / 2;
+  int ei[NS], ek[NS], last[NS];  // last: the warp's entries' last row, so far
+  float2 v[NS];
+  if (t == 0) sm.bad = 0;
+  {
+    double a[NS];
 #pragma unroll
-      for (int q = SW_DIG - 1; q >= 0; --q) {
-        long long dg = n;
-        if (q > 0) {
-          dg = ((n + 64) & 127) - 64;  // balanced remainder mod 128
-          n = (n - dg) >> 7;           // exact
-        }
-        *reinterpret_cast<__nv_bfloat16*>(wdig + tc::kmajor_offset(q * R + c, s, R)) =
-            __float2bfloat16_rn((float)(int)dg);
+    for (int q = 0; q < NS; ++q) {
+      const int e = q * SYS_THREADS + t;  // e = i (i + 1) / 2 + k, k <= i
+      int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+      while (i * (i + 1) / 2 > e) --i;
+      while ((i + 1) * (i + 2) / 2 <= e) ++i;
+      ei[q] = e < T ? i : -1;
+      ek[q] = e < T ? e - i * (i + 1) / 2 : 0;
+      last[q] = __reduce_max_sync(SPM_FULL_MASK, ei[q]);
+      if (q > 0) last[q] = max(last[q], last[q - 1]);  // past the triangle
+      a[q] = 1.0;
+    }
+    const int w0 = d == 0 ? 1 : 0;  // the first mode of the product (none: V = 1)
+    for (int w = w0; w < N; ++w)
+      if (w != d) {
+        double g[NS];
+#pragma unroll
+        for (int q = 0; q < NS; ++q)
+          g[q] = ei[q] >= 0 ? grams[(int64_t)w * RR + ei[q] * R + ek[q]] : 0.0;
+#pragma unroll
+        for (int q = 0; q < NS; ++q) a[q] = w == w0 ? g[q] : __dmul_rn(a[q], g[q]);
+      }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NS; ++q)
+      if (ei[q] >= 0 && ei[q] == ek[q]) {
+        const int hi = __double2hiint(a[q]);
+        const int ex = (hi >> 20) - 1023;
+        if (hi < 0 || ex < -900 || ex > 900) sm.bad = 1;
+        sm.ex[ei[q]] = ex >> 1;
+      }
+    __syncthreads();
+    if (sm.bad) return false;
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+      v[q] = make_float2(0.f, 0.f);
+      if (ei[q] >= 0) {
+        const double x = times_pow2(a[q], -(sm.ex[ei[q]] + sm.ex[ek[q]]));
+        sm.A[q * SYS_THREADS + t] = x;
+        v[q].x = (float)x;
+        v[q].y = (float)__dsub_rn(x, (double)v[q].x);
       }
     }
   }
+  for (int j = 0; j < R; ++j) {
+    const int b = j & 1;
+#pragma unroll
+    for (int q = 0; q < NS; ++q)
+      if (ei[q] >= j && (ek[q] == j || ei[q] == j)) sm.pivf[b][ek[q] == j ? ei[q] : ek[q]] = v[q];
+    __syncthreads();
+    if (t < 32) {
+      const float2 p = sm.pivf[b][j];
+      const bool good = p.x >= 1.52587890625e-5f && p.x <= 16.f;  // 2^-16; false for NaN
+      float r0;
+      asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(good ? p.x : 1.f));
+      float e = fmaf(-p.x, r0, 1.f);
+      e = fmaf(-p.y, r0, e);
+      const float2 r = ff_norm(r0, __fmul_rn(r0, fmaf(e, e, e)));
+      const float2 nr = make_float2(-r.x, -r.y);
+      for (int i = j + 1 + t; i < R; i += 32) sm.nlf[i] = ff_mul(sm.pivf[b][i], nr);
+      if (t == 0) {
+        sm.rdf[j] = r;
+        if (!good) sm.bad = 1;
+      }
+    }
+    __syncthreads();
+    if (sm.bad) break;
+    // Three slots at a time while the warp has a row beyond j in them; rows up
+    // to j: a zero multiplier; column j: -l = fma(-l, 1, 0).
+#pragma unroll
+    for (int q0 = 0; q0 < NS; q0 += QG) {
+      if (last[q0 + QG - 1] <= j) continue;
+      float2 l[QG], pv[QG];
+#pragma unroll
+      for (int u = 0; u < QG; ++u) {
+        const int q = q0 + u;
+        const float2 z = make_float2(0.f, 0.f);
+        l[u] = ei[q] > j ? sm.nlf[ei[q]] : z;
+        pv[u] = ek[q] == j ? make_float2(1.f, 0.f) : sm.pivf[b][ek[q]];
+        if (ei[q] > j && ek[q] == j) v[q] = z;
+      }
+#pragma unroll
+      for (int u = 0; u < QG; ++u) v[q0 + u] = ff_fma(l[u], pv[u], v[q0 + u]);
+    }
+  }
+  if (sm.bad) return false;
+  // X, and trace(W) = sum of X(k, c)^2 / d_k, summed in a fixed order
+  float tr = 0.f;
+#pragma unroll
+  for (int q = 0; q < NS; ++q)
+    if (ei[q] >= 0) {
+      const float2 x = ei[q] == ek[q] ? make_float2(1.f, 0.f) : v[q];
+      sm.XF[q * SYS_THREADS + t] = x;
+      tr = fmaf(__fmul_rn(x.x, x.x), sm.rdf[ei[q]].x, tr);
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(SPM_FULL_MASK, tr, o);
+  if (lane == 0) sm.red[t >> 5] = tr;
+  __syncthreads();
+  float trace = 0.f;
+#pragma unroll
+  for (int w = 0; w < SYS_THREADS / 32; ++w) trace += sm.red[w];
+  if (!(trace <= 4096.f)) return false;
+  auto X = [&](int k, int c) -> float2 { return sm.XF[k * (k + 1) / 2 + c]; };
+  const int nc = c1 - c0;
+  const unsigned rinv = (65535u + R) / R;  // x / R = x rinv >> 16 for x < 1024
+  for (int x = t; x < nc * R; x += SYS_THREADS) {
+    const int cc = (int)((unsigned)x * rinv >> 16), k = x - cc * R;
+    sm.y[cc * SYS_RMAX + k] = k >= c0 + cc ? ff_mul(X(k, c0 + cc), sm.rdf[k]) : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  // every sum below: four threads per entry (index mod 4), added by shuffles
+  const int sub = t & 3, ntask = nc * R, step = SYS_THREADS / 4;
+  // w = X^T (D^{-1} X(:, c))
+  for (int x0 = 0; x0 < ntask; x0 += step) {
+    const int x = x0 + (t >> 2);
+    float2 a = make_float2(0.f, 0.f);
+    int cc = 0, s = 0;
+    if (x < ntask) {
+      cc = (int)((unsigned)x * rinv >> 16);
+      s = x - cc * R;
+      for (int k = (max(s, c0 + cc) & ~3) + sub; k < R; k += 4)
+        if (k >= s) a = ff_fma(X(k, s), sm.y[cc * SYS_RMAX + k], a);
+    }
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1)
+      a = ff_add(a, make_float2(__shfl_xor_sync(SPM_FULL_MASK, a.x, o),
+                                __shfl_xor_sync(SPM_FULL_MASK, a.y, o)));
+    if (x < ntask && sub == 0) sm.W[cc * SYS_RMAX + s] = __dadd_rn((double)a.x, (double)a.y);
+  }
+  __syncthreads();
+  // r = e_c - V w in FP64
+  for (int x0 = 0; x0 < ntask; x0 += step) {
+    const int x = x0 + (t >> 2);
+    double a = 0.0;
+    int cc = 0, i = 0;
+    if (x < ntask) {
+      cc = (int)((unsigned)x * rinv >> 16);
+      i = x - cc * R;
+      if (sub == 0 && i == c0 + cc) a = -1.0;
+      for (int k = sub; k < R; k += 4)
+        a = fma(k <= i ? sm.A[i * (i + 1) / 2 + k] : sm.A[k * (k + 1) / 2 + i],
+                sm.W[cc * SYS_RMAX + k], a);
+    }
+    a += __shfl_xor_sync(SPM_FULL_MASK, a, 1);
+    a += __shfl_xor_sync(SPM_FULL_MASK, a, 2);
+    if (x < ntask && sub == 0) sm.ru[0][cc * SYS_RMAX + i] = -(float)a;
+  }
+  __syncthreads();
+  // D^{-1} X r
+  for (int x0 = 0; x0 < ntask; x0 += step) {
+    const int x = x0 + (t >> 2);
+    float a = 0.f;
+    int cc = 0, k = 0;
+    if (x < ntask) {
+      cc = (int)((unsigned)x * rinv >> 16);
+      k = x - cc * R;
+      for (int i = sub; i <= k; i += 4) a = fmaf(X(k, i).x, sm.ru[0][cc * SYS_RMAX + i], a);
+    }
+    a += __shfl_xor_sync(SPM_FULL_MASK, a, 1);
+    a += __shfl_xor_sync(SPM_FULL_MASK, a, 2);
+    if (x < ntask && sub == 0) sm.ru[1][cc * SYS_RMAX + k] = __fmul_rn(a, sm.rdf[k].x);
+  }
+  __syncthreads();
+  // w += X^T of that; the scaling undone
+  for (int x0 = 0; x0 < ntask; x0 += step) {
+    const int x = x0 + (t >> 2);
+    float a = 0.f;
+    int cc = 0, s = 0;
+    if (x < ntask) {
+      cc = (int)((unsigned)x * rinv >> 16);
+      s = x - cc * R;
+      for (int k = (s & ~3) + sub; k < R; k += 4)
+        if (k >= s) a = fmaf(X(k, s).x, sm.ru[1][cc * SYS_RMAX + k], a);
+    }
+    a += __shfl_xor_sync(SPM_FULL_MASK, a, 1);
+    a += __shfl_xor_sync(SPM_FULL_MASK, a, 2);
+    if (x < ntask && sub == 0)
+      sm.W[cc * SYS_RMAX + s] = times_pow2(__dadd_rn(sm.W[cc * SYS_RMAX + s], (double)a),
+                                           -(sm.ex[s] + sm.ex[c0 + cc]));
+  }
+  __syncthreads();
+  system_store(sm, R, c0, nc, winv, wdig);
+  return true;
+}
+
+template <int NS>
+__device__ __forceinline__ void system_body_n(SystemSmem& sm, const double* __restrict__ grams, int N,
+                                              int d, int R, int c0, int c1, float* __restrict__ winv,
+                                              unsigned char* __restrict__ wdig,
+                                              int* __restrict__ err) {
+  if (__syncthreads_or(threadIdx.x == 0 && *(volatile int*)err)) return;
+  if (system_pairs_ns<NS>(sm, grams, N, d, R, c0, c1, winv, wdig)) return;
+  __syncthreads();  // shared memory is reused
+  system_body_ns<NS>(sm, grams, N, d, R, c0, c1, winv, wdig, err);
 }
 
 __device__ __forceinline__ void system_body(SystemSmem& sm, const double* __restrict__ grams, int N,
                                             int d, int R, int c0, int c1, float* __restrict__ winv,
                                             unsigned char* __restrict__ wdig,
                                             int* __restrict__ err) {
-  if (R <= 16) system_body_ns<1>(sm, grams, N, d, R, c0, c1, winv, wdig, err);
-  else if (R <= 32) system_body_ns<3>(sm, grams, N, d, R, c0, c1, winv, wdig, err);
-  else system_body_ns<9>(sm, grams, N, d, R, c0, c1, winv, wdig, err);
+  if (R <= 16) system_body_n<1>(sm, grams, N, d, R, c0, c1, winv, wdig, err);
+  else if (R <= 32) system_body_n<3>(sm, grams, N, d, R, c0, c1, winv, wdig, err);
+  else system_body_n<9>(sm, grams, N, d, R, c0, c1, winv, wdig, err);
 }
 
 // Z = M W for rows tile vb, vb + nvb, ... (see the head of this file), with

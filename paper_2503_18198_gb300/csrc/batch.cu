@@ -49,8 +49,7 @@ __global__ void __launch_bounds__(256)
 }
 
 // Block (x, y): columns y SYS_COLS .. of tensor it[x]'s system (every block of
-// a tensor eliminates its own copy: with 16 columns a block, the dot products
-// of the columns weigh as much as the elimination).
+// a tensor eliminates its own copy).
 __global__ void __launch_bounds__(SYS_THREADS)
     batch_system_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it, int mode) {
   __shared__ SystemSmem sm;
