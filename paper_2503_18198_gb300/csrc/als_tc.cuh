@@ -111,6 +111,41 @@ __device__ __forceinline__ uint32_t pack_bf16_int(float a, float b) {
   return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
 }
 
+// ---- pairs of FP32 values in one instruction (f32x2): the same roundings as
+// the scalar operations, half the issue slots, which bound the row passes
+// (solve of 567,000 rows of R = 32: 86 -> 73 us, normalisation and Gram 97 ->
+// 90 us, on average over the modes of the scale workload).
+__device__ __forceinline__ uint64_t f2_const(float x) { return f2_pack(x, x); }
+__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {  // a - b, rounded once
+  return f2_fma(b, f2_const(-1.f), a);
+}
+// round_int of both
+__device__ __forceinline__ uint64_t f2_round_int(uint64_t y) {
+  return f2_add(f2_add(y, f2_const(12582912.f)), f2_const(-12582912.f));
+}
+__device__ __forceinline__ uint32_t f2_pack_bf16_int(uint64_t k) {
+  return __byte_perm((uint32_t)k, (uint32_t)(k >> 32), 0x7632);
+}
+struct df2 {  // two double-floats
+  uint64_t hi, lo;
+};
+__device__ __forceinline__ void df2_add(df2& a, uint64_t x) {  // a += x (error-free two-sum)
+  const uint64_t s = f2_add(a.hi, x);
+  const uint64_t bb = f2_sub(s, a.hi);
+  const uint64_t err = f2_add(f2_sub(a.hi, f2_sub(s, bb)), f2_sub(x, bb));
+  a.hi = s;
+  a.lo = f2_add(a.lo, err);
+}
+__device__ __forceinline__ void df2_add_square(df2& a, uint64_t z) {  // a += z z
+  const uint64_t p = f2_mul(z, z);
+  const uint64_t e = f2_fma(z, z, f2_mul(p, f2_const(-1.f)));
+  const uint64_t s = f2_add(a.hi, p);
+  const uint64_t bb = f2_sub(s, a.hi);
+  const uint64_t err = f2_add(f2_sub(a.hi, f2_sub(s, bb)), f2_sub(p, bb));
+  a.hi = s;
+  a.lo = f2_add(a.lo, f2_add(err, e));
+}
+
 __device__ __forceinline__ void df_add(df& a, float x) {  // a += x (error-free two-sum)
   const float s = __fadd_rn(a.hi, x);
   const float bb = __fsub_rn(s, a.hi);
@@ -704,7 +739,7 @@ __device__ __forceinline__ void tc_solve_body(const float* __restrict__ M,
     if (vb < ntiles) { fetch(vb, 0); fetched = 1; }
   }
   ok = mbar_wait_bounded(&bars[3], 0u);
-  df sq = {0.f, 0.f};  // column (t % R) sum of Z^2 over this block's rows
+  df2 sq = {0ull, 0ull};  // column (t % R) sums of Z^2 over this block's rows, two at a time
   float mx = 0.f;      // and max |Z|
   int it = 0;
   if (__syncthreads_and(ok))
@@ -735,31 +770,39 @@ __device__ __forceinline__ void tc_solve_body(const float* __restrict__ M,
 #pragma unroll
       for (int g = 0; g < H / 8; ++g) {
         const int gg = (g + rl) % (H / 8);
-        float x[8];
+        uint64_t x[4];
         if (in) {
           const float4 a = *reinterpret_cast<const float4*>(mr + gg * 8);
           const float4 b = *reinterpret_cast<const float4*>(mr + gg * 8 + 4);
-          x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
-          x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) x[j] = fast ? __fmul_rn(x[j], inv) : ldexpf(x[j], -e_row);
+          if (fast) {
+            const uint64_t iv = f2_const(inv);
+            x[0] = f2_mul(f2_pack(a.x, a.y), iv);
+            x[1] = f2_mul(f2_pack(a.z, a.w), iv);
+            x[2] = f2_mul(f2_pack(b.x, b.y), iv);
+            x[3] = f2_mul(f2_pack(b.z, b.w), iv);
+          } else {
+            x[0] = f2_pack(ldexpf(a.x, -e_row), ldexpf(a.y, -e_row));
+            x[1] = f2_pack(ldexpf(a.z, -e_row), ldexpf(a.w, -e_row));
+            x[2] = f2_pack(ldexpf(b.x, -e_row), ldexpf(b.y, -e_row));
+            x[3] = f2_pack(ldexpf(b.z, -e_row), ldexpf(b.w, -e_row));
+          }
         } else {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) x[j] = 0.f;
+          for (int j = 0; j < 4; ++j) x[j] = 0ull;
         }
         // digit p of each value: rint of the remainder scaled by 2^7 (exact steps)
 #pragma unroll
         for (int p = 0; p < SM_DIG; ++p) {
-          float k[8];
+          uint32_t k[4];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float y = __fmul_rn(x[j], 128.f);
-            k[j] = round_int(y);
-            x[j] = __fsub_rn(y, k[j]);
+          for (int j = 0; j < 4; ++j) {
+            const uint64_t y = f2_mul(x[j], f2_const(128.f));
+            const uint64_t kk = f2_round_int(y);
+            x[j] = f2_sub(y, kk);
+            k[j] = f2_pack_bf16_int(kk);
           }
           *reinterpret_cast<uint4*>(sA + tc::kmajor_offset(rl, p * R + half * H + gg * 8, S::KA)) =
-              make_uint4(pack_bf16_int(k[0], k[1]), pack_bf16_int(k[2], k[3]),
-                         pack_bf16_int(k[4], k[5]), pack_bf16_int(k[6], k[7]));
+              make_uint4(k[0], k[1], k[2], k[3]);
         }
       }
       fence_proxy_async_smem();  // digits visible to the tensor core
@@ -800,37 +843,48 @@ __device__ __forceinline__ void tc_solve_body(const float* __restrict__ M,
         for (int L = 0; L <= TC_LMAX; ++L) tc::ld8(lane_addr + (uint32_t)(L * R + c0), v[L]);
         tc::wait_ld();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          float h = __uint_as_float(v[TC_LMAX][j]);
+        for (int j = 0; j < 8; j += 2) {
+          auto lev = [&](int L) -> uint64_t {
+            return f2_pack(__uint_as_float(v[L][j]), __uint_as_float(v[L][j + 1]));
+          };
+          const uint64_t w7 = f2_const(0.0078125f);
+          uint64_t h = lev(TC_LMAX);
 #pragma unroll
-          for (int L = TC_LMAX - 1; L >= 2; --L) h = fmaf(h, 0.0078125f, __uint_as_float(v[L][j]));
-          df z = {__uint_as_float(v[1][j]), 0.f};
-          df_add(z, __fmul_rn(h, 0.0078125f));
-          z.hi = __fmul_rn(z.hi, 0.0078125f);
-          z.lo = __fmul_rn(z.lo, 0.0078125f);
-          df_add(z, __uint_as_float(v[0][j]));
-          const int k = e_row + fexp[c0 + j] - 14;
-          float zf;
-          if (k >= -126 && k <= 127) {
-            const float sc = pow2f(k);
-            zf = __fadd_rn(__fmul_rn(z.hi, sc), __fmul_rn(z.lo, sc));
+          for (int L = TC_LMAX - 1; L >= 2; --L) h = f2_fma(h, w7, lev(L));
+          df2 z = {lev(1), 0ull};
+          df2_add(z, f2_mul(h, w7));
+          z.hi = f2_mul(z.hi, w7);
+          z.lo = f2_mul(z.lo, w7);
+          df2_add(z, lev(0));
+          const int k0 = e_row + fexp[c0 + j] - 14, k1 = e_row + fexp[c0 + j + 1] - 14;
+          float z0, z1;
+          if (min(k0, k1) >= -126 && max(k0, k1) <= 127) {
+            const uint64_t sc = f2_pack(pow2f(k0), pow2f(k1));
+            f2_unpack(f2_add(f2_mul(z.hi, sc), f2_mul(z.lo, sc)), z0, z1);
           } else {
-            zf = __fadd_rn(ldexpf(z.hi, k), ldexpf(z.lo, k));
+            float h0, h1, l0, l1;
+            f2_unpack(z.hi, h0, h1);
+            f2_unpack(z.lo, l0, l1);
+            z0 = __fadd_rn(ldexpf(h0, k0), ldexpf(l0, k0));
+            z1 = __fadd_rn(ldexpf(h1, k1), ldexpf(l1, k1));
           }
-          sZ[rl * S::ZS_STRIDE + c0 + j] = zf;
+          sZ[rl * S::ZS_STRIDE + c0 + j] = z0;
+          sZ[rl * S::ZS_STRIDE + c0 + j + 1] = z1;
         }
       }
       tc::fence_before_sync();
       __syncthreads();
-      // column sums of Z^2 and maxima of |Z| (fixed order: rows of the tile
-      // in turn), and the tile of Z out (rows with nonzeros only)
+      // column sums of Z^2 and maxima of |Z| (fixed order), and the tile of Z
+      // out (rows with nonzeros only)
       {
         constexpr int PER = TC_THREADS / R;  // threads per column
+        static_assert(TC_ROWS % (2 * PER) == 0, "rows in pairs");
         const int c = t % R, g = t / R;
-        for (int rr = g; rr < TC_ROWS; rr += PER) {
-          const float zz = sZ[rr * S::ZS_STRIDE + c];
-          df_add_prod(sq, zz, zz);
-          mx = fmaxf(mx, fabsf(zz));
+#pragma unroll 4
+        for (int rr = g; rr < TC_ROWS; rr += 2 * PER) {
+          const float za = sZ[rr * S::ZS_STRIDE + c], zb = sZ[(rr + PER) * S::ZS_STRIDE + c];
+          df2_add_square(sq, f2_pack(za, zb));
+          mx = fmaxf(mx, fmaxf(fabsf(za), fabsf(zb)));
         }
       }
       for (int x = t; x < TC_ROWS * R / 4; x += TC_THREADS) {
@@ -855,7 +909,12 @@ __device__ __forceinline__ void tc_solve_body(const float* __restrict__ M,
     }
     __syncthreads();
   }
-  red[t] = df_value(sq);
+  {
+    df sa, sb;
+    f2_unpack(sq.hi, sa.hi, sb.hi);
+    f2_unpack(sq.lo, sa.lo, sb.lo);
+    red[t] = __dadd_rn(df_value(sa), df_value(sb));
+  }
   redm[t] = mx;
   tc::fence_before_sync();
   __syncthreads();
@@ -979,9 +1038,9 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
   if (t == 0)
     for (; fetched < nloc && fetched < GT_STAGES; ++fetched) fetch(fetched);
 
-  df acc[R];  // digit row t of D folded over q: acc(s) = sum_q 2^-7q D(t, qR + s)
+  df2 acc[R / 2];  // digit row t of D folded over q: acc(s) = sum_q 2^-7q D(t, qR + s)
 #pragma unroll
-  for (int s = 0; s < R; ++s) acc[s] = {0.f, 0.f};
+  for (int s = 0; s < R / 2; ++s) acc[s] = {0ull, 0ull};
   df inn = {0.f, 0.f};
   bool ok = true;
   int j = 0, committed = 0;
@@ -998,7 +1057,7 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
       // rows row0 + k0 .. + 7 share one word of the mask (row0 + k0 is a multiple of 8)
       const uint32_t live8 =
           mask ? (__ldg(&mask[(row0 + k0) >> 5]) >> ((row0 + k0) & 31)) & 0xFFu : 0xFFu;
-      float x[8];
+      float y8[8];
 #pragma unroll
       for (int jj = 0; jj < 8; ++jj) {
         const int64_t row = row0 + k0 + jj;
@@ -1011,20 +1070,25 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
           y = load_f<FT>(&ys, 0);
           if (M && lv) df_add_prod(inn, M[row * R + r], y);
         }
-        x[jj] = gfast ? __fmul_rn(y, gs) : ldexpf(y, -g);
+        y8[jj] = y;
       }
+      uint64_t x[4];
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj)
+        x[jj] = gfast ? f2_mul(f2_pack(y8[2 * jj], y8[2 * jj + 1]), f2_const(gs))
+                      : f2_pack(ldexpf(y8[2 * jj], -g), ldexpf(y8[2 * jj + 1], -g));
 #pragma unroll
       for (int p = 0; p < S::NDIG; ++p) {
-        float k[8];
+        uint32_t k[4];
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-          const float yy = __fmul_rn(x[jj], 128.f);
-          k[jj] = round_int(yy);
-          x[jj] = __fsub_rn(yy, k[jj]);
+        for (int jj = 0; jj < 4; ++jj) {
+          const uint64_t yy = f2_mul(x[jj], f2_const(128.f));
+          const uint64_t kk = f2_round_int(yy);
+          x[jj] = f2_sub(yy, kk);
+          k[jj] = f2_pack_bf16_int(kk);
         }
         *reinterpret_cast<uint4*>(A + tc::kmajor_offset(p * R + r, k0, GT_ROWS)) =
-            make_uint4(pack_bf16_int(k[0], k[1]), pack_bf16_int(k[2], k[3]),
-                       pack_bf16_int(k[4], k[5]), pack_bf16_int(k[6], k[7]));
+            make_uint4(k[0], k[1], k[2], k[3]);
       }
     }
     fence_proxy_async_smem();  // digits visible to the tensor core
@@ -1055,9 +1119,11 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
 #pragma unroll
           for (int c8 = 0; c8 < R / 8; ++c8) tc::ld8(lane_addr + (uint32_t)(q * R + c8 * 8), v[c8]);
           tc::wait_ld();
-          const float wq = pow2f(-7 * q);
+          const uint64_t wq = f2_const(pow2f(-7 * q));
 #pragma unroll
-          for (int s = 0; s < R; ++s) df_add(acc[s], __fmul_rn(__uint_as_float(v[s / 8][s % 8]), wq));
+          for (int s = 0; s < R; s += 2)
+            df2_add(acc[s / 2], f2_mul(f2_pack(__uint_as_float(v[s / 8][s % 8]),
+                                               __uint_as_float(v[s / 8][s % 8 + 1])), wq));
         }
       }
       tc::fence_before_sync();
@@ -1083,7 +1149,13 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
   double* red = reinterpret_cast<double*>(sA);
   if (t < 128)
 #pragma unroll
-    for (int s = 0; s < R; ++s) red[t * R + s] = times_pow2(df_value(acc[s]), -7 * (t / R));
+    for (int s = 0; s < R; s += 2) {
+      df a, b;
+      f2_unpack(acc[s / 2].hi, a.hi, b.hi);
+      f2_unpack(acc[s / 2].lo, a.lo, b.lo);
+      red[t * R + s] = times_pow2(df_value(a), -7 * (t / R));
+      red[t * R + s + 1] = times_pow2(df_value(b), -7 * (t / R));
+    }
   red_in[t] = df_value(inn);
   __syncthreads();
   if (ok) {
