@@ -26,7 +26,8 @@ template <typename FT, int GT>
 __global__ void __launch_bounds__(ALS_THREADS)
     gram_partial_kernel(const FT* __restrict__ Y, int64_t I, int R, int64_t rows_per_block,
                         double* __restrict__ part, const uint32_t* __restrict__ mask) {
-  gram_partial_body<FT, GT>(Y, I, R, rows_per_block, part, blockIdx.x, mask);
+  __shared__ GramSmem<GT> sm;
+  gram_partial_body<FT, GT>(sm, Y, I, R, rows_per_block, part, blockIdx.x, mask);
 }
 
 __global__ void gram_reduce_kernel(const double* __restrict__ part, int nblocks, int R,

@@ -115,59 +115,161 @@ __device__ __forceinline__ __nv_bfloat16 store_cvt<__nv_bfloat16>(float x) {
 }
 
 // ---------------------------------------------------------------------------
-// Gram partials: block b sums rows [i0, i1) of Y.  Only the lower triangle
-// r >= s is accumulated (G is symmetric): thread t owns entries
-// e = t, t + 256, ... of the R(R+1)/2 triangle entries in row-major order,
-// and mirrors them when it stores.  Requires R <= 16 * GT.
+// Gram partials: block vb sums rows [i0, i1) of Y in double-float.  Only the
+// lower triangle s <= r is accumulated (G is symmetric), in register tiles of
+// BR x 4 entries: a thread reads BR + 4 values of a row from shared memory for
+// BR x 4 products, and GROUPS threads share a tile of entries, each taking
+// every GROUPS-th row.  The next rows' loads are in flight meanwhile.  Bound:
+// FP32 arithmetic, 10 operations per entry and row.  (One entry per thread and
+// product, two shared loads each, no prefetch: 318 us for 567,000 rows of R =
+// 32, 37 us for 30,000 of R = 64 at the longest; so
+// 159 and 26 us.)
+// Requires R <= 16 * GT.
 // ---------------------------------------------------------------------------
+template <int GT>
+struct GramShape {
+  static constexpr int RMAX = 16 * GT;
+  static constexpr int BR = GT == 4 ? 8 : 4;           // rows of a register tile
+  static constexpr int NB = RMAX / BR;
+  // tiles (rb, sb) with sb * 4 <= rb * BR + BR - 1
+  static constexpr int TILES = BR == 4 ? NB * (NB + 1) / 2 : NB * (NB + 1);
+  static constexpr int GROUPS = ALS_THREADS / TILES;
+  static constexpr int LD = RMAX + 4;                  // row stride of the staged tile
+  static constexpr int PF = GRAM_TILE_ROWS * RMAX / ALS_THREADS;  // staged values per thread
+};
+// Shared memory of a Gram block: the staged rows, then the merged sums.
+template <int GT>
+struct GramSmem {
+  union {
+    float tile[GRAM_TILE_ROWS * GramShape<GT>::LD];
+    float2 sum[(GramShape<GT>::GROUPS + 1) / 2][GramShape<GT>::BR * 4][GramShape<GT>::TILES];
+  };
+};
+
 template <typename FT, int GT>
-__device__ __forceinline__ void gram_partial_body(const FT* __restrict__ Y, int64_t I, int R,
-                                                  int64_t rows_per_block, double* __restrict__ part,
-                                                  int vb, const uint32_t* __restrict__ mask) {
-  constexpr int RMAX = 16 * GT;
-  constexpr int EPT = (RMAX * (RMAX + 1) / 2 + ALS_THREADS - 1) / ALS_THREADS;  // entries per thread
-  __shared__ float tile[GRAM_TILE_ROWS][RMAX + 1];
-  __shared__ int live[GRAM_TILE_ROWS];
+__device__ __forceinline__ void gram_partial_body(GramSmem<GT>& sm, const FT* __restrict__ Y, int64_t I,
+                                                  int R, int64_t rows_per_block,
+                                                  double* __restrict__ part, int vb,
+                                                  const uint32_t* __restrict__ mask) {
+  using S = GramShape<GT>;
+  constexpr int RMAX = S::RMAX, BR = S::BR;
   const int64_t i0 = (int64_t)vb * rows_per_block;
   const int64_t i1 = std::min<int64_t>(I, i0 + rows_per_block);
-  const int T = R * (R + 1) / 2;
-  int er[EPT], es[EPT];
-  df acc[EPT];
-#pragma unroll
-  for (int k = 0; k < EPT; ++k) {
-    const int e = threadIdx.x + k * ALS_THREADS;
-    int r = 0;
-    while ((r + 1) * (r + 2) / 2 <= e) ++r;  // e = r (r + 1) / 2 + s, s <= r
-    er[k] = e < T ? r : 0;
-    es[k] = e < T ? e - r * (r + 1) / 2 : 0;
-    acc[k] = {0.f, 0.f};
+  const int t = threadIdx.x;
+  const int grp = t / S::TILES;
+  int rb = 0, sb = t % S::TILES;
+  if constexpr (BR == 4) {
+    while (sb > rb) sb -= ++rb;  // row rb of the triangle of tiles has rb + 1
+  } else {
+    while (sb > 2 * rb + 1) sb -= 2 * (++rb);  // 2 rb + 2
   }
+  const bool active = grp < S::GROUPS;
+  uint64_t hi[BR][2], lo[BR][2];
+#pragma unroll
+  for (int a = 0; a < BR; ++a) hi[a][0] = hi[a][1] = lo[a][0] = lo[a][1] = 0ull;
+  float pf[S::PF];
+  auto fetch = [&](int64_t t0) {
+#pragma unroll
+    for (int k = 0; k < S::PF; ++k) {
+      const int e = t + k * ALS_THREADS, cc = e % RMAX;
+      const int64_t row = t0 + e / RMAX;
+      pf[k] = row < i1 && cc < R && row_live(mask, row) ? load_f<FT>(Y, row * R + cc) : 0.f;
+    }
+  };
+  const uint64_t neg = f2_pack(-1.f, -1.f);
+  auto sub2 = [&](uint64_t a, uint64_t b) { return f2_fma(b, neg, a); };
+  fetch(i0);
   for (int64_t t0 = i0; t0 < i1; t0 += GRAM_TILE_ROWS) {
     const int nrow = (int)std::min<int64_t>(GRAM_TILE_ROWS, i1 - t0);
     __syncthreads();
-    if (threadIdx.x < GRAM_TILE_ROWS)
-      live[threadIdx.x] = threadIdx.x < nrow && row_live(mask, t0 + threadIdx.x);
-    __syncthreads();
-    for (int e = threadIdx.x; e < GRAM_TILE_ROWS * RMAX; e += ALS_THREADS) {
-      const int rr = e / RMAX, cc = e % RMAX;
-      tile[rr][cc] = (live[rr] && cc < R) ? load_f<FT>(Y, (t0 + rr) * R + cc) : 0.f;
-    }
-    __syncthreads();
-    for (int rr = 0; rr < nrow; ++rr) {
-      if (!live[rr]) continue;
 #pragma unroll
-      for (int k = 0; k < EPT; ++k) df_add_prod(acc[k], tile[rr][er[k]], tile[rr][es[k]]);
+    for (int k = 0; k < S::PF; ++k) {
+      const int e = t + k * ALS_THREADS;
+      sm.tile[(e / RMAX) * S::LD + e % RMAX] = pf[k];
     }
+    __syncthreads();
+    if (t0 + GRAM_TILE_ROWS < i1) fetch(t0 + GRAM_TILE_ROWS);
+    if (active)
+      for (int rr = grp; rr < nrow; rr += S::GROUPS) {
+        const float* row = sm.tile + rr * S::LD;
+        float a[BR];
+#pragma unroll
+        for (int k = 0; k < BR / 4; ++k) {
+          const float4 x = *reinterpret_cast<const float4*>(row + rb * BR + 4 * k);
+          a[4 * k] = x.x; a[4 * k + 1] = x.y; a[4 * k + 2] = x.z; a[4 * k + 3] = x.w;
+        }
+        const float4 bv = *reinterpret_cast<const float4*>(row + sb * 4);
+        const uint64_t b[2] = {f2_pack(bv.x, bv.y), f2_pack(bv.z, bv.w)};
+#pragma unroll
+        for (int k = 0; k < BR; ++k) {
+          const uint64_t aa = f2_pack(a[k], a[k]);
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {  // error-free product and sum, two entries at a time
+            const uint64_t p = f2_mul(aa, b[q]);
+            const uint64_t e = f2_fma(aa, b[q], f2_mul(p, neg));
+            const uint64_t s = f2_add(hi[k][q], p);
+            const uint64_t bb = sub2(s, hi[k][q]);
+            const uint64_t err = f2_add(sub2(hi[k][q], sub2(s, bb)), sub2(p, bb));
+            hi[k][q] = s;
+            lo[k][q] = f2_add(lo[k][q], f2_add(err, e));
+          }
+        }
+      }
   }
-  double* out = part + (int64_t)vb * R * R;
+  // The groups' sums, pairwise: the upper half hands its sums to the lower.
+  const int tl = t % S::TILES;
+  for (int n = S::GROUPS; n > 1; n = (n + 1) / 2) {
+    const int h = (n + 1) / 2;
+    __syncthreads();
+    if (active && grp >= h && grp < n)
 #pragma unroll
-  for (int k = 0; k < EPT; ++k) {
-    const int e = threadIdx.x + k * ALS_THREADS;
-    if (e < T) {
-      const double v = df_value(acc[k]);
-      out[er[k] * R + es[k]] = v;
-      out[es[k] * R + er[k]] = v;
-    }
+      for (int k = 0; k < BR; ++k)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          float2 x, y;
+          f2_unpack(hi[k][q], x.x, y.x);
+          f2_unpack(lo[k][q], x.y, y.y);
+          sm.sum[grp - h][4 * k + 2 * q][tl] = x;
+          sm.sum[grp - h][4 * k + 2 * q + 1][tl] = y;
+        }
+    __syncthreads();
+    if (grp + h < n)
+#pragma unroll
+      for (int k = 0; k < BR; ++k)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const float2 x = sm.sum[grp][4 * k + 2 * q][tl];
+          const float2 y = sm.sum[grp][4 * k + 2 * q + 1][tl];
+          const uint64_t p = f2_pack(x.x, y.x);
+          const uint64_t s = f2_add(hi[k][q], p);
+          const uint64_t bb = sub2(s, hi[k][q]);
+          const uint64_t err = f2_add(sub2(hi[k][q], sub2(s, bb)), sub2(p, bb));
+          hi[k][q] = s;
+          lo[k][q] = f2_add(lo[k][q], f2_add(err, f2_pack(x.y, y.y)));
+        }
+  }
+  __syncthreads();
+  if (grp == 0)
+#pragma unroll
+    for (int k = 0; k < BR; ++k)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        float2 x, y;
+        f2_unpack(hi[k][q], x.x, y.x);
+        f2_unpack(lo[k][q], x.y, y.y);
+        sm.sum[0][4 * k + 2 * q][tl] = x;
+        sm.sum[0][4 * k + 2 * q + 1][tl] = y;
+      }
+  __syncthreads();
+  double* out = part + (int64_t)vb * R * R;
+  for (int e = t; e < R * R; e += ALS_THREADS) {
+    const int r = e / R, s = e - r * R;
+    if (s > r) continue;
+    const int b = r / BR, first = BR == 4 ? b * (b + 1) / 2 : b * (b + 1);
+    const float2 v = sm.sum[0][(r % BR) * 4 + s % 4][first + s / 4];
+    const double x = __dadd_rn((double)v.x, (double)v.y);
+    out[e] = x;
+    out[s * R + r] = x;
   }
 }
 

@@ -164,11 +164,19 @@ __global__ void __launch_bounds__(ALS_THREADS)
 }
 
 // Gram partials of factor `mode` on the CUDA cores.  `init`: of a new member's
-// factors, whose rows without nonzeros may hold anything.
-template <typename FT>
-__global__ void __launch_bounds__(ALS_THREADS)
+// factors, whose rows without nonzeros may hold anything.  GTMAX: of the
+// batch's longest rank, as the body of R > 32 needs twice the registers
+// (starting Grams of 96 tensors of R = 16 and 32: 201 us with every body in
+// one kernel, 136 us without).
+template <typename FT, int GTMAX>
+__global__ void __launch_bounds__(ALS_THREADS, GTMAX < 4 ? 4 : 2)
     batch_gram_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it, int mode,
                       bool init) {
+  __shared__ union {
+    GramSmem<1> g1;
+    GramSmem<GTMAX < 2 ? GTMAX : 2> g2;
+    GramSmem<GTMAX> g4;
+  } sm;
   const int2 tv = it[blockIdx.x];
   const BatchTensor& b = bt[tv.x];
   if (!b.active) return;
@@ -176,11 +184,18 @@ __global__ void __launch_bounds__(ALS_THREADS)
   const int64_t I = b.dims[mode];
   const int64_t rpb = b.gram_rpb[mode];
   const uint32_t* live = init ? nullptr : b.live[mode];
-  switch (gram_tile(b.R)) {
-    case 1: gram_partial_body<FT, 1>(y, I, b.R, rpb, b.gram_part, tv.y, live); break;
-    case 2: gram_partial_body<FT, 2>(y, I, b.R, rpb, b.gram_part, tv.y, live); break;
-    default: gram_partial_body<FT, 4>(y, I, b.R, rpb, b.gram_part, tv.y, live); break;
+  const int gt = gram_tile(b.R);
+  if (gt == 1) {
+    gram_partial_body<FT, 1>(sm.g1, y, I, b.R, rpb, b.gram_part, tv.y, live);
+    return;
   }
+  if constexpr (GTMAX >= 2)
+    if (gt == 2) {
+      gram_partial_body<FT, 2>(sm.g2, y, I, b.R, rpb, b.gram_part, tv.y, live);
+      return;
+    }
+  if constexpr (GTMAX >= 4)
+    gram_partial_body<FT, 4>(sm.g4, y, I, b.R, rpb, b.gram_part, tv.y, live);
 }
 
 // Block (x, y): share y of the entries of tensor it[x]'s Gram.  The FP64
@@ -207,10 +222,18 @@ spm_status launch_batch_gram_reduce(const spm_batch_s* B, const int2* it, int n,
 
 spm_status launch_batch_gram(const spm_batch_s* B, const int2* it, int n, int mode, bool init,
                              cudaStream_t s) {
+  auto go = [&](auto ft) {
+    using FT = decltype(ft);
+    switch (gram_tile(B->maxR)) {
+      case 1: batch_gram_kernel<FT, 1><<<n, ALS_THREADS, 0, s>>>(B->bt, it, mode, init); break;
+      case 2: batch_gram_kernel<FT, 2><<<n, ALS_THREADS, 0, s>>>(B->bt, it, mode, init); break;
+      default: batch_gram_kernel<FT, 4><<<n, ALS_THREADS, 0, s>>>(B->bt, it, mode, init); break;
+    }
+  };
   if (B->bf16 == 1)
-    batch_gram_kernel<__nv_bfloat16><<<n, ALS_THREADS, 0, s>>>(B->bt, it, mode, init);
+    go(__nv_bfloat16{});
   else
-    batch_gram_kernel<float><<<n, ALS_THREADS, 0, s>>>(B->bt, it, mode, init);
+    go(0.f);
   SPM_CUDA_TRY(cudaGetLastError());
   return SPM_OK;
 }
