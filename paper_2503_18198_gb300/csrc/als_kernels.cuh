@@ -50,6 +50,13 @@ __device__ __forceinline__ void df_add_prod2(df& acc, float a, float bh, float b
   acc.hi = s;
   acc.lo = __fadd_rn(acc.lo, __fadd_rn(err, e));
 }
+__device__ __forceinline__ void df_add(df& a, float x) {  // a += x (error-free two-sum)
+  const float s = __fadd_rn(a.hi, x);
+  const float bb = __fsub_rn(s, a.hi);
+  const float err = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(x, bb));
+  a.hi = s;
+  a.lo = __fadd_rn(a.lo, err);
+}
 __device__ __forceinline__ double df_value(const df& a) { return __dadd_rn((double)a.hi, (double)a.lo); }
 
 // Sum of x[0], x[stride], ..., x[(n-1) stride] by one warp in a fixed order:
@@ -267,75 +274,100 @@ __device__ __forceinline__ void gram_partial_body(GramSmem<GT>& sm, const FT* __
     if (s > r) continue;
     const int b = r / BR, first = BR == 4 ? b * (b + 1) / 2 : b * (b + 1);
     const float2 v = sm.sum[0][(r % BR) * 4 + s % 4][first + s / 4];
-    const double x = __dadd_rn((double)v.x, (double)v.y);
-    out[e] = x;
-    out[s * R + r] = x;
+    out[e] = __dadd_rn((double)v.x, (double)v.y);
   }
 }
 
-// G = sum over blocks of the partials (FP64, fixed order).  Up to
-// ALS_SERIAL_PARTIALS partials one thread sums an entry in block order;
-// beyond that one warp does (lane-strided sums, then warp_sum_strided's
-// shuffle tree, lane 0's value kept).  Virtual block vb of nvb takes its
-// share of the entries, GR_ENTRIES at a time side by side so that their
-// loads are in flight together; an entry's order of addition does not
-// depend on the launch shape.
+// G = sum over blocks of the partials (FP64, fixed order), from their lower
+// triangles.  Up to ALS_SERIAL_PARTIALS partials one thread sums an entry in
+// block order; beyond, one warp sums a group of GR_ENTRIES neighbouring
+// entries, lane l the partials l, l + 32, ..., and the lanes' sums meet in a
+// butterfly in which each step halves the entries a lane still carries.  Warps
+// are dealt to the blocks in turn, so every SM has some.  Bound: latency of
+// the loads (8, or 4 x GR_ENTRIES, in flight) and FP64 issue.  (All R^2 entries, every lane
+// through every butterfly step: 63 us for 96 tensors of R = 16 and 32, 17.6 us
+// for 304 partials of R = 64; now 28 and 10.9 us.)  An entry's order of
+// addition does not depend on the launch shape.
 constexpr int GR_ENTRIES = 4;
 __device__ __forceinline__ void gram_reduce_body(const double* __restrict__ part, int nblocks,
                                                  int R, double* __restrict__ G,
                                                  const int* __restrict__ err, int vb, int nvb) {
   if (warp_err(err)) return;
-  const int RR = R * R;
+  const int64_t RR = (int64_t)R * R;
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int gw = (threadIdx.x >> 5) * nvb + vb;  // this warp among the launch's
   if (nblocks <= ALS_SERIAL_PARTIALS) {
-    // thread t takes entries e, e + step, ..., GR_ENTRIES of them at a time
-    const int step = nvb * blockDim.x;
-    for (int e = vb * blockDim.x + threadIdx.x; e < RR; e += GR_ENTRIES * step) {
-      double v[GR_ENTRIES];
+    for (int i = gw * 32 + lane; i < R * (R + 1) / 2; i += nvb * nw * 32) {
+      // entry i of the triangle: row r starts at r (r + 1) / 2
+      int r = (int)((sqrtf(1.f + 8.f * (float)i) - 1.f) * 0.5f);
+      while ((r + 1) * (r + 2) / 2 <= i) ++r;
+      while (r * (r + 1) / 2 > i) --r;
+      const int s = i - r * (r + 1) / 2, e = r * R + s;
+      double v = 0.0;
+      int b = 0;
+      for (; b + 7 < nblocks; b += 8) {
+        double x[8];
 #pragma unroll
-      for (int k = 0; k < GR_ENTRIES; ++k) v[k] = 0.0;
-#pragma unroll 4
-      for (int b = 0; b < nblocks; ++b) {
-        const double* pb = part + (int64_t)b * RR + e;
+        for (int u = 0; u < 8; ++u) x[u] = part[(b + u) * RR + e];
 #pragma unroll
-        for (int k = 0; k < GR_ENTRIES; ++k)
-          if (e + k * step < RR) v[k] += pb[k * step];
+        for (int u = 0; u < 8; ++u) v += x[u];
       }
-#pragma unroll
-      for (int k = 0; k < GR_ENTRIES; ++k)
-        if (e + k * step < RR) G[e + k * step] = v[k];
+      for (; b < nblocks; ++b) v += part[b * RR + e];
+      G[e] = v;
+      G[s * R + r] = v;
     }
     return;
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int e = (vb * nw + warp) * GR_ENTRIES; e < RR; e += nvb * nw * GR_ENTRIES) {
+  static_assert(GR_ENTRIES == 4, "row r has r / 4 + 1 groups; two halving steps");
+  const int groups = 2 * (R / 4) * (R / 4 + 1) + (R % 4) * (R / 4 + 1);
+  for (int q = gw; q < groups; q += nvb * nw) {
+    // group q of the triangle: rows 4 m .. 4 m + 3 start at 2 m (m + 1)
+    int m = (int)((sqrtf(1.f + 2.f * (float)q) - 1.f) * 0.5f);
+    while (2 * (m + 1) * (m + 2) <= q) ++m;
+    while (2 * m * (m + 1) > q) --m;
+    const int rem = q - 2 * m * (m + 1);
+    const int r = 4 * m + rem / (m + 1), s0 = rem % (m + 1) * GR_ENTRIES;
+    const double* p0 = part + r * R + s0;
+    const int have = min(GR_ENTRIES, r + 1 - s0);
     double v[GR_ENTRIES];
 #pragma unroll
     for (int k = 0; k < GR_ENTRIES; ++k) v[k] = 0.0;
-    // the loads of four partials ahead of the (ordered) additions
     int b = lane;
     for (; b + 96 < nblocks; b += 128) {
       double x[4][GR_ENTRIES];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int k = 0; k < GR_ENTRIES; ++k)
-          x[u][k] = e + k < RR ? part[(int64_t)(b + 32 * u) * RR + e + k] : 0.0;
+        for (int k = 0; k < GR_ENTRIES; ++k) x[u][k] = k < have ? p0[(b + 32 * u) * RR + k] : 0.0;
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int k = 0; k < GR_ENTRIES; ++k) v[k] += x[u][k];
     }
     for (; b < nblocks; b += 32) {
-      const double* pb = part + (int64_t)b * RR + e;
+      double x[GR_ENTRIES];
 #pragma unroll
-      for (int k = 0; k < GR_ENTRIES; ++k)
-        if (e + k < RR) v[k] += pb[k];
+      for (int k = 0; k < GR_ENTRIES; ++k) x[k] = k < have ? p0[b * RR + k] : 0.0;
+#pragma unroll
+      for (int k = 0; k < GR_ENTRIES; ++k) v[k] += x[k];
+    }
+    const bool up16 = lane & 16, up8 = lane & 8;
+    double a[2], c[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      a[k] = up16 ? v[2 + k] : v[k];
+      c[k] = up16 ? v[k] : v[2 + k];
     }
 #pragma unroll
-    for (int k = 0; k < GR_ENTRIES; ++k) {
+    for (int k = 0; k < 2; ++k) a[k] += __shfl_xor_sync(SPM_FULL_MASK, c[k], 16);
+    double w = up8 ? a[1] : a[0];
+    w += __shfl_xor_sync(SPM_FULL_MASK, up8 ? a[0] : a[1], 8);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(SPM_FULL_MASK, v[k], o);
-      if (lane == 0 && e + k < RR) G[e + k] = v[k];
+    for (int o = 4; o > 0; o >>= 1) w += __shfl_xor_sync(SPM_FULL_MASK, w, o);
+    const int k = (up16 ? 2 : 0) + (up8 ? 1 : 0);
+    if ((lane & 7) == 0 && k < have) {
+      G[r * R + s0 + k] = w;
+      G[(s0 + k) * R + r] = w;
     }
   }
 }

@@ -99,30 +99,22 @@ __device__ __forceinline__ int scale_expf(float amax) {
   return e;
 }
 
-// rint(y) for abs(y) <= 2^22 by the 1.5 * 2^23 shift (round half to even, like
-// rintf; two adds on the FMA pipe instead of the conversion pipe).
-__device__ __forceinline__ float round_int(float y) {
-  return __fsub_rn(__fadd_rn(y, 12582912.f), 12582912.f);
-}
-
-// Two integer-valued floats of magnitude <= 256 as a BF16 pair (lo = a): their
-// low 16 bits are zero, so the BF16 value is the high half, exactly.
-__device__ __forceinline__ uint32_t pack_bf16_int(float a, float b) {
-  return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
-}
-
 // ---- pairs of FP32 values in one instruction (f32x2): the same roundings as
 // the scalar operations, half the issue slots, which bound the row passes
 // (solve of 567,000 rows of R = 32: 86 -> 73 us, normalisation and Gram 97 ->
-// 90 us, on average over the modes of the scale workload).
+// 90 us, on average over the modes of the scale workload; then see
+// tc_scale_gram_body's last sums).
 __device__ __forceinline__ uint64_t f2_const(float x) { return f2_pack(x, x); }
 __device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {  // a - b, rounded once
   return f2_fma(b, f2_const(-1.f), a);
 }
-// round_int of both
+// rint of both for abs <= 2^22 by the 1.5 * 2^23 shift (round half to even, like
+// rintf; two adds on the FMA pipe instead of the conversion pipe).
 __device__ __forceinline__ uint64_t f2_round_int(uint64_t y) {
   return f2_add(f2_add(y, f2_const(12582912.f)), f2_const(-12582912.f));
 }
+// Two integer-valued floats of magnitude <= 256 as a BF16 pair (lo = a): their
+// low 16 bits are zero, so the BF16 value is the high half, exactly.
 __device__ __forceinline__ uint32_t f2_pack_bf16_int(uint64_t k) {
   return __byte_perm((uint32_t)k, (uint32_t)(k >> 32), 0x7632);
 }
@@ -146,13 +138,6 @@ __device__ __forceinline__ void df2_add_square(df2& a, uint64_t z) {  // a += z 
   a.lo = f2_add(a.lo, f2_add(err, e));
 }
 
-__device__ __forceinline__ void df_add(df& a, float x) {  // a += x (error-free two-sum)
-  const float s = __fadd_rn(a.hi, x);
-  const float bb = __fsub_rn(s, a.hi);
-  const float err = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(x, bb));
-  a.hi = s;
-  a.lo = __fadd_rn(a.lo, err);
-}
 
 // ---------------------------------------------------------------------------
 // The normal-equation system of one mode and columns of its inverse.
@@ -967,7 +952,8 @@ struct TcGramShape {
   static constexpr int SLICE = GT_ROWS / NQ;         // rows per slice (multiple of 8)
   static constexpr int Z_BYTES = GT_ROWS * R * 4;
   static constexpr int A_BYTES = 128 * GT_ROWS * 2;  // one digit tile
-  static constexpr int RED_BYTES = NDIG * R * R * 8; // the final per-digit Gram parts
+  static constexpr int RED_LD = R + 1;               // row stride of the final per-digit parts
+  static constexpr int RED_BYTES = 128 * RED_LD * 8;
   static_assert(RED_BYTES <= 2 * A_BYTES, "final reduction fits in the digit tiles");
   static_assert(SLICE % 8 == 0, "digit groups of 8 rows");
   static constexpr size_t SMEM = (size_t)GT_STAGES * Z_BYTES + 2 * A_BYTES;
@@ -983,7 +969,7 @@ inline int tc_gram_blocks(int64_t I, int cap) {
 
 // The pass over tiles vb, vb + nvb, ... of Z (see above).  `lam` holds
 // lambda (R values) then the column scale exponents g_r (R values, from
-// lambda_body).  Writes Y, gram_part[vb] (R x R) and, when M is non-null,
+// lambda_body).  Writes Y, gram_part[vb] (R x R, lower triangle) and, when M is non-null,
 // inner_part[vb] (R).  Rows without nonzeros (bit clear in `mask`) get Y = 0.
 template <typename FT, int R>
 __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
@@ -999,6 +985,7 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
   __shared__ __align__(8) uint64_t bars[GT_STAGES + 2];  // Z stages; MMAs of digit tile 0 / 1
   __shared__ double red_in[TC_THREADS];
   __shared__ int gx[R];
+  __shared__ float linv[R];
   if (*(volatile const int*)err) return;
 
   float* sZ = reinterpret_cast<float*>(smem_tc);
@@ -1010,12 +997,11 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
   const int64_t ntiles = (I + GT_ROWS - 1) / GT_ROWS;
   const int nloc = vb < ntiles ? (int)((ntiles - 1 - vb) / nvb + 1) : 0;
 
-  const double lr = lam[r];
-  const float inv = lr > 0.0 ? (float)(1.0 / lr) : 1.f;
-  const int g = (int)lam[R + r];
-  const bool gfast = g >= -125 && g <= 126;
-  const float gs = gfast ? pow2f(-g) : 1.f;
-  if (t < R) gx[t] = (int)lam[R + t];
+  if (t < R) {  // one FP64 division per column, not per thread
+    const double lr = lam[t];
+    linv[t] = lr > 0.0 ? (float)(1.0 / lr) : 1.f;
+    gx[t] = (int)lam[R + t];
+  }
   if (warp == 0) tc::tmem_alloc(&tmem_slot, 128);
   if (t == 0) {
     for (int b = 0; b < GT_STAGES + 2; ++b) mbar_init(&bars[b], 1);
@@ -1025,6 +1011,10 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_slot;
+  const float inv = linv[r];  // 1 for a column of zeros: z * 1 = z
+  const int g = gx[r];
+  const bool gfast = g >= -125 && g <= 126;
+  const float gs = gfast ? pow2f(-g) : 1.f;
 
   auto fetch = [&](int j) {  // local tile j into stage j % GT_STAGES (thread 0)
     fence_proxy_async_smem();
@@ -1065,7 +1055,7 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
         if (row < I) {
           const bool lv = (live8 >> jj) & 1u;
           const float z = lv ? zs[(k0 + jj) * R + r] : 0.f;
-          const FT ys = store_cvt<FT>(lr > 0.0 ? __fmul_rn(z, inv) : z);
+          const FT ys = store_cvt<FT>(__fmul_rn(z, inv));
           Y[row * R + r] = ys;
           y = load_f<FT>(&ys, 0);
           if (M && lv) df_add_prod(inn, M[row * R + r], y);
@@ -1145,30 +1135,39 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
   }
   tc::fence_before_sync();
   __syncthreads();
-  // per-digit parts of the Gram into the digit tiles (all MMAs have completed)
-  double* red = reinterpret_cast<double*>(sA);
-  if (t < 128)
+  // Per-digit parts of the Gram, weighted, into the digit tiles (all MMAs have
+  // completed).  They stay FP32 pairs up to the last sum: FP64 issues at 1/64
+  // of FP32's rate, and this epilogue in FP64 was most of a short tensor's
+  // pass (96 tensors: 113 and 76 us per mode at R = 32 and 16; now 64 and
+  // 54; one tile of R = 16: 12.1 -> 9.1 us).  The weights are powers of two,
+  // and the pairs' sum keeps the 2^-47 of the total that the accumulators do.
+  float2* red = reinterpret_cast<float2*>(sA);
+  if (t < 128) {
+    const uint64_t wp = f2_const(pow2f(-7 * (t / R)));
 #pragma unroll
     for (int s = 0; s < R; s += 2) {
-      df a, b;
-      f2_unpack(acc[s / 2].hi, a.hi, b.hi);
-      f2_unpack(acc[s / 2].lo, a.lo, b.lo);
-      red[t * R + s] = times_pow2(df_value(a), -7 * (t / R));
-      red[t * R + s + 1] = times_pow2(df_value(b), -7 * (t / R));
+      float2 a, b;
+      f2_unpack(f2_mul(acc[s / 2].hi, wp), a.x, b.x);
+      f2_unpack(f2_mul(acc[s / 2].lo, wp), a.y, b.y);
+      red[t * S::RED_LD + s] = a;
+      red[t * S::RED_LD + s + 1] = b;
     }
-  red_in[t] = df_value(inn);
+  }
+  if (M) red_in[t] = df_value(inn);
   __syncthreads();
   if (ok) {
-    const int RR = R * R;
-    for (int e = t; e < RR; e += TC_THREADS) {
-      const int rr = e / R, ss = e % R;
-      if (ss > rr) continue;
-      double v = 0.0;
+    // lower triangle, folded into R / 2 rows of R + 1 entries
+    for (int e = t; e < R / 2 * (R + 1); e += TC_THREADS) {
+      const int i = e / (R + 1) + R / 2, k = e % (R + 1);
+      const int rr = k <= i ? i : R - 1 - i, ss = k <= i ? k : k - i - 1;
+      df v = {0.f, 0.f};
 #pragma unroll
-      for (int p = 0; p < S::NDIG; ++p) v += red[(p * R + rr) * R + ss];
-      v = times_pow2(v, gx[rr] + gx[ss] - 14);
-      gram_part[(int64_t)vb * RR + rr * R + ss] = v;
-      gram_part[(int64_t)vb * RR + ss * R + rr] = v;
+      for (int p = S::NDIG - 1; p >= 0; --p) {
+        const float2 x = red[(p * R + rr) * S::RED_LD + ss];
+        df_add(v, x.x);
+        v.lo = __fadd_rn(v.lo, x.y);
+      }
+      gram_part[(int64_t)vb * R * R + rr * R + ss] = times_pow2(df_value(v), gx[rr] + gx[ss] - 14);
     }
     if (M && t < R) {
       double sum = 0.0;

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(ALS_THREADS, GTMAX < 4 ? 4 : 2)
 // Block (x, y): share y of the entries of tensor it[x]'s Gram.  The FP64
 // additions (R^2 per partial) spread over the SMs: with one block per tensor
 // they took 183 us for 96 tensors of R = 16 and 32 and 680 us for 10 tensors
-// up to R = 64; now 61 and 32 us.
+// up to R = 64; see gram_reduce_body for the figures since.
 __global__ void __launch_bounds__(256)
     batch_gram_reduce_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it,
                              int mode, bool init) {
