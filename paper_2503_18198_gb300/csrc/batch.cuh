@@ -48,6 +48,13 @@ struct spm_batch_s {
   // (created when the first member is added, outside any stream capture)
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // streams (the caller's besides) for the launches of a phase that do not
+  // depend on one another, as many as the members' classes need, and the events
+  // that order them; created by batch_commit
+  int n_beside = 0;
+  cudaStream_t beside[spm::KC_NONE] = {};
+  cudaEvent_t ev_beside[spm::KC_NONE] = {};
+  cudaEvent_t ev_phase = nullptr;
 };
 
 namespace spm {
