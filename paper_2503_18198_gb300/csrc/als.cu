@@ -191,7 +191,18 @@ spm_status gram(spmttkrp_plan_s* p, const void* Y, int64_t I, double* G, cudaStr
 
 spm_status ensure_als_state(spmttkrp_plan_s* p) {
   spm_als_state& A = p->als;
-  if (!A.side) SPM_CUDA_TRY(cudaStreamCreateWithFlags(&A.side, cudaStreamNonBlocking));
+  if (!A.side) {
+    // At ranks whose Gram is a pass of its own, that pass and the system go
+    // ahead of the MTTKRP where both wait for an SM: its 2048 threads per SM
+    // keep them out until it ends (R = 64, 30,000 rows: 1.95 ms with priority,
+    // 2.05 without).  Where only the small reduction and the system are on this
+    // stream it costs the MTTKRP more than it gives (R = 32, 20M nonzeros: 5.26
+    // against 5.19 ms).
+    int least = 0, greatest = 0;
+    SPM_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+    SPM_CUDA_TRY(cudaStreamCreateWithPriority(&A.side, cudaStreamNonBlocking,
+                                              tc_gram_rank(p->R) ? least : greatest));
+  }
   if (!A.ev_fork) SPM_CUDA_TRY(cudaEventCreateWithFlags(&A.ev_fork, cudaEventDisableTiming));
   if (!A.ev_join) SPM_CUDA_TRY(cudaEventCreateWithFlags(&A.ev_join, cudaEventDisableTiming));
   const int R = p->R;
@@ -247,19 +258,28 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
     }
     A.ready = true;
   }
-  for (int d = 0; d < N; ++d) {
-    const int64_t I = p->dims[d];
-    // V, its Cholesky factor and V^-1 for mode d need the other modes'
-    // Grams (final once the previous mode's Gram is reduced, i.e. at this
-    // point of `s`), not M: they are formed on the side stream beside the
-    // MTTKRP, and the solve waits for them.  The fork also orders the
-    // previous mode's solve (the last reader of V^-1) before the overwrite.
+  // The MTTKRP of a mode needs the other modes' factors, its V^-1 their Grams:
+  // once a factor is written, its Gram and the next mode's system are formed on
+  // the side stream beside the next MTTKRP, and the next solve waits for them.
+  // (R = 64, 30,000 rows: the Gram's two passes took 37 us of a mode before the
+  // MTTKRP began; request of 2 sweeps 2.10 -> 1.95 ms, 96 tensors 4.33 -> 4.16.)  The fork also orders the solve, the last reader of
+  // V^-1, before the overwrite, and the solve's wait orders the Gram partials'
+  // reader before their next writer.
+  auto fork = [&]() -> spm_status {
     SPM_CUDA_TRY(cudaEventRecord(A.ev_fork, s));
     SPM_CUDA_TRY(cudaStreamWaitEvent(A.side, A.ev_fork, 0));
-    system_kernel<<<R, SYS_THREADS, 0, A.side>>>(A.gram, N, d, R, A.winv, A.wdig,
-                                                 p->dev_err);
+    return SPM_OK;
+  };
+  auto system = [&](int d) -> spm_status {
+    system_kernel<<<R, SYS_THREADS, 0, A.side>>>(A.gram, N, d, R, A.winv, A.wdig, p->dev_err);
     SPM_CUDA_TRY(cudaGetLastError());
     SPM_CUDA_TRY(cudaEventRecord(A.ev_join, A.side));
+    return SPM_OK;
+  };
+  SPM_TRY(fork());
+  SPM_TRY(system(0));
+  for (int d = 0; d < N; ++d) {
+    const int64_t I = p->dims[d];
     SPM_TRY(run_mttkrp(p, d, factors, A.M, s, p->bf16));
     SPM_CUDA_TRY(cudaStreamWaitEvent(s, A.ev_join, 0));
     const int nb = solve_blocks(R, I, A.gram_blocks);
@@ -274,8 +294,6 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
     if (tcg) {
       nin = tc_gram_blocks(I, A.gram_blocks);
       SPM_TRY(launch_tc_scale_gram(R, p->bf16, nin, A, I, factors[d], last, p->dev_err, live, s));
-      gram_reduce_kernel<<<std::max(1, std::min(1024, R * R / 8)), 256, 0, s>>>(
-          A.gram_part, nin, R, A.gram + (size_t)d * R * R, p->dev_err);
     } else {
       nin = als_row_blocks(I, A.gram_blocks);
       if (p->bf16)
@@ -288,8 +306,16 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
                                                          last ? A.M : nullptr, A.inner_part,
                                                          p->dev_err, live);
       SPM_CUDA_TRY(cudaGetLastError());
-      SPM_TRY(gram(p, factors[d], I, A.gram + (size_t)d * R * R, s, live));
     }
+    cudaStream_t sg = last ? s : A.side;  // the fit follows the last Gram
+    if (!last) SPM_TRY(fork());
+    double* G = A.gram + (size_t)d * R * R;
+    if (tcg)
+      gram_reduce_kernel<<<std::max(1, std::min(1024, R * R / 8)), 256, 0, sg>>>(A.gram_part, nin, R, G,
+                                                                               p->dev_err);
+    else
+      SPM_TRY(gram(p, factors[d], I, G, sg, live));
+    if (!last) SPM_TRY(system(d + 1));
     if (last) {
       fit_kernel<<<1, ALS_THREADS, 0, s>>>(A.gram, N, R, A.lambda_ws, A.inner_part, nin,
                                            p->normX2, fit, lambda, p->dev_err);

@@ -577,21 +577,29 @@ spm_status batch_sweep(spm_batch_s* B, cudaStream_t s) {
   SPM_TRY(batch_commit(B, s));
   if (B->host.empty()) return SPM_OK;
   const int2* it = B->items;
-  for (int d = 0; d < B->maxN; ++d) {
+  // As in a single tensor's sweep: a mode's Grams, the fits of the members whose
+  // last mode it is and the next mode's systems on the side stream, beside the
+  // next MTTKRP.
+  const bool fork = B->side && B->ev_fork && B->ev_join;
+  cudaStream_t ss = fork ? B->side : s;
+  auto begin_side = [&]() -> spm_status {
+    if (!fork) return SPM_OK;
+    SPM_CUDA_TRY(cudaEventRecord(B->ev_fork, s));
+    SPM_CUDA_TRY(cudaStreamWaitEvent(B->side, B->ev_fork, 0));
+    return SPM_OK;
+  };
+  auto systems = [&](int d) -> spm_status {
     const spm_batch_s::ModeItems& I = B->mi[d];
-    // each member's system for mode d needs its other modes' Grams (final at
-    // this point of `s`), not its MTTKRP: formed on the side stream beside
-    // the MTTKRP launches; the fork also orders the previous mode's solve
-    // before V^-1 is overwritten
-    const bool fork = B->side && B->ev_fork && B->ev_join;
-    cudaStream_t ss = fork ? B->side : s;
-    if (fork) {
-      SPM_CUDA_TRY(cudaEventRecord(B->ev_fork, s));
-      SPM_CUDA_TRY(cudaStreamWaitEvent(B->side, B->ev_fork, 0));
-    }
-    batch_system_kernel<<<dim3(I.n_tens, ceil_div(B->maxR, SYS_COLS)), SYS_THREADS, 0, ss>>>(B->bt, it + I.tens_off, d);
+    batch_system_kernel<<<dim3(I.n_tens, ceil_div(B->maxR, SYS_COLS)), SYS_THREADS, 0, ss>>>(
+        B->bt, it + I.tens_off, d);
     SPM_CUDA_TRY(cudaGetLastError());
     if (fork) SPM_CUDA_TRY(cudaEventRecord(B->ev_join, B->side));
+    return SPM_OK;
+  };
+  SPM_TRY(begin_side());
+  SPM_TRY(systems(0));
+  for (int d = 0; d < B->maxN; ++d) {
+    const spm_batch_s::ModeItems& I = B->mi[d];
     SPM_TRY(batch_mttkrp(B, d, s));
     if (fork) SPM_CUDA_TRY(cudaStreamWaitEvent(s, B->ev_join, 0));
     Phase solve(B, s);
@@ -605,23 +613,31 @@ spm_status batch_sweep(spm_batch_s* B, cudaStream_t s) {
       }));
     SPM_TRY(solve.join());
     batch_lambda_kernel<<<dim3(I.n_tens, B->maxR), 32, 0, s>>>(B->bt, it + I.tens_off, d);
-    Phase gram(B, s);
-    SPM_TRY(gram.add(I.n_scale, [&](cudaStream_t t) {  // ranks without the fused pass
+    Phase scale(B, s);
+    SPM_TRY(scale.add(I.n_scale, [&](cudaStream_t t) {  // ranks without the fused pass
       if (B->bf16 == 1)
         batch_scale_kernel<__nv_bfloat16><<<I.n_scale, ALS_THREADS, 0, t>>>(B->bt, it + I.scale_off, d);
       else
         batch_scale_kernel<float><<<I.n_scale, ALS_THREADS, 0, t>>>(B->bt, it + I.scale_off, d);
-      return launch_batch_gram(B, it + I.gram_off, I.n_gram, d, false, t);
+      SPM_CUDA_TRY(cudaGetLastError());
+      return SPM_OK;
     }));
     for (int k = 1; k >= 0; --k)
-      SPM_TRY(gram.add(I.n_tcg[k], [&](cudaStream_t t) {
+      SPM_TRY(scale.add(I.n_tcg[k], [&](cudaStream_t t) {
         return launch_batch_tc_scale_gram(16 << k, B->bf16 == 1, B->bt, it + I.tcg_off[k],
                                           I.n_tcg[k], d, t);
       }));
-    SPM_TRY(gram.join());
-    SPM_TRY(launch_batch_gram_reduce(B, it + I.tens_off, I.n_tens, d, false, s));
-    if (I.n_fit > 0) batch_fit_kernel<<<I.n_fit, ALS_THREADS, 0, s>>>(B->bt, it + I.fit_off, d);
+    SPM_TRY(scale.join());
+    SPM_TRY(begin_side());
+    if (I.n_gram > 0) SPM_TRY(launch_batch_gram(B, it + I.gram_off, I.n_gram, d, false, ss));
+    SPM_TRY(launch_batch_gram_reduce(B, it + I.tens_off, I.n_tens, d, false, ss));
+    if (d + 1 < B->maxN) SPM_TRY(systems(d + 1));
+    if (I.n_fit > 0) batch_fit_kernel<<<I.n_fit, ALS_THREADS, 0, ss>>>(B->bt, it + I.fit_off, d);
     SPM_CUDA_TRY(cudaGetLastError());
+  }
+  if (fork) {
+    SPM_CUDA_TRY(cudaEventRecord(B->ev_join, B->side));
+    SPM_CUDA_TRY(cudaStreamWaitEvent(s, B->ev_join, 0));
   }
   return SPM_OK;
 }

@@ -58,8 +58,9 @@ struct spm_als_state {
   int* urow = nullptr;
   int* pdone = nullptr;
   int split_cap = 0;  // partitions those hold
-  // the normal-equation systems of mode d depend only on the other modes'
-  // Grams, so they are formed on a side stream while the MTTKRP of mode d runs
+  // the Gram of a mode and the normal-equation system of the next depend only on
+  // factors already written, so they are formed on a side stream while the next
+  // mode's MTTKRP runs
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
