@@ -155,7 +155,7 @@ __device__ __forceinline__ void df2_add_square(df2& a, uint64_t z) {  // a += z 
 // elimination (entry e of the triangle, row-major, belongs to thread e mod 256:
 // the entries still active at step j are a contiguous tail, spread evenly over
 // the warps), the pivot row and column go through shared memory once per step,
-// and one warp forms the reciprocal.
+// and one warp forms the reciprocal (in double-float up to R = 32, every thread).
 //
 // Bound: the chain pivot -> reciprocal -> column -> next pivot, and in FP64 its
 // throughput (2 fused multiply-adds per cycle and SM, 64 cycles each).  So the
@@ -172,8 +172,8 @@ __device__ __forceinline__ void df2_add_square(df2& a, uint64_t z) {  // a += z 
 // extended precision as with an FP64 Cholesky factor for cond(V) = 3 .. 1e8 at
 // R = 16, 32, 64 (rms 2.5e-8, the FP32 rounding of Z; the splitting's 2^-34 is
 // the rest): tests/test_gpu_system.py.
-// One system, one column per block, alone on the GPU, R = 16 / 32 / 64: 11.5 /
-// 18.5 / 51 us (the same elimination in FP64 12.3 / 25.6 / 78 us; before it, a
+// One system, one column per block, alone on the GPU, R = 16 / 32 / 64: 10 /
+// 18 / 51 us (the same elimination in FP64 12.3 / 25.6 / 78 us; before it, a
 // Cholesky factor and two substitution chains per column, 20 / 46 / 139 us).
 // ---------------------------------------------------------------------------
 constexpr int SYS_THREADS = 256;
@@ -452,6 +452,11 @@ __device__ __forceinline__ bool system_pairs_ns(SystemSmem& sm, const double* __
                                                 float* __restrict__ winv,
                                                 unsigned char* __restrict__ wdig) {
   constexpr int QG = NS % 3 == 0 ? 3 : 1;
+  // Up to three slots every thread forms the reciprocal and its rows'
+  // multipliers: one barrier per step, no wait for a warp (R = 16 / 32: 11.1 /
+  // 21.9 -> 9.7 / 21.1 us from cold caches).  With nine slots the extra issue
+  // costs more (R = 64: 63.5 -> 69 us).
+  constexpr bool OWN = NS <= 3;
   const int t = threadIdx.x, lane = t & 31;
   const int RR = R * R, T = R * (R + 1) / 2;
   int ei[NS], ek[NS], last[NS];  // last: the warp's entries' last row, so far
@@ -508,24 +513,29 @@ __device__ __forceinline__ bool system_pairs_ns(SystemSmem& sm, const double* __
 #pragma unroll
     for (int q = 0; q < NS; ++q)
       if (ei[q] >= j && (ek[q] == j || ei[q] == j)) sm.pivf[b][ek[q] == j ? ei[q] : ek[q]] = v[q];
-    __syncthreads();
-    if (t < 32) {
+    __syncthreads();  // the buffers alternate
+    float2 nr = make_float2(0.f, 0.f);
+    if (OWN || t < 32) {
       const float2 p = sm.pivf[b][j];
       const bool good = p.x >= 1.52587890625e-5f && p.x <= 16.f;  // 2^-16; false for NaN
+      if (OWN && !good) return false;
       float r0;
       asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(good ? p.x : 1.f));
       float e = fmaf(-p.x, r0, 1.f);
       e = fmaf(-p.y, r0, e);
       const float2 r = ff_norm(r0, __fmul_rn(r0, fmaf(e, e, e)));
-      const float2 nr = make_float2(-r.x, -r.y);
-      for (int i = j + 1 + t; i < R; i += 32) sm.nlf[i] = ff_mul(sm.pivf[b][i], nr);
+      nr = make_float2(-r.x, -r.y);
+      if (!OWN)
+        for (int i = j + 1 + t; i < R; i += 32) sm.nlf[i] = ff_mul(sm.pivf[b][i], nr);
       if (t == 0) {
         sm.rdf[j] = r;
         if (!good) sm.bad = 1;
       }
     }
-    __syncthreads();
-    if (sm.bad) break;
+    if (!OWN) {
+      __syncthreads();
+      if (sm.bad) break;
+    }
     // Three slots at a time while the warp has a row beyond j in them; rows up
     // to j: a zero multiplier; column j: -l = fma(-l, 1, 0).
 #pragma unroll
@@ -536,7 +546,7 @@ __device__ __forceinline__ bool system_pairs_ns(SystemSmem& sm, const double* __
       for (int u = 0; u < QG; ++u) {
         const int q = q0 + u;
         const float2 z = make_float2(0.f, 0.f);
-        l[u] = ei[q] > j ? sm.nlf[ei[q]] : z;
+        l[u] = ei[q] <= j ? z : OWN ? ff_mul(sm.pivf[b][ei[q]], nr) : sm.nlf[ei[q]];
         pv[u] = ek[q] == j ? make_float2(1.f, 0.f) : sm.pivf[b][ek[q]];
         if (ei[q] > j && ek[q] == j) v[q] = z;
       }
@@ -544,6 +554,7 @@ __device__ __forceinline__ bool system_pairs_ns(SystemSmem& sm, const double* __
       for (int u = 0; u < QG; ++u) v[q0 + u] = ff_fma(l[u], pv[u], v[q0 + u]);
     }
   }
+  if (OWN) __syncthreads();  // the last 1 / d_k
   if (sm.bad) return false;
   // X, and trace(W) = sum of X(k, c)^2 / d_k, summed in a fixed order
   float tr = 0.f;
