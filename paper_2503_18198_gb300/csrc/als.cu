@@ -72,9 +72,10 @@ __global__ void __launch_bounds__(TC_THREADS)
     tc_scale_gram_kernel(const float* __restrict__ Z, const double* __restrict__ lam, int64_t I,
                          FT* __restrict__ Y, const float* __restrict__ M,
                          double* __restrict__ gram_part, double* __restrict__ inner_part,
-                         const int* __restrict__ err, const uint32_t* __restrict__ mask) {
+                         const int* __restrict__ err, const uint32_t* __restrict__ mask,
+                         TcFuse fuse) {
   tc_scale_gram_body<FT, R>(Z, lam, I, Y, M, gram_part, inner_part, err, blockIdx.x, gridDim.x,
-                            mask);
+                            mask, fuse);
 }
 
 template <typename FT>
@@ -158,13 +159,14 @@ __attribute__((noinline)) spm_status launch_solve(int R, int nb, const spm_als_s
 
 template <typename FT, int R>
 spm_status launch_tc_scale_gram_r(int nb, const spm_als_state& A, int64_t I, void* Y, bool last,
-                                  const int* err, const uint32_t* mask, cudaStream_t s) {
+                                  const int* err, const uint32_t* mask, const TcFuse& fuse,
+                                  cudaStream_t s) {
   constexpr int smem = (int)TcGramShape<R>::SMEM;
   SPM_CUDA_TRY(cudaFuncSetAttribute(tc_scale_gram_kernel<FT, R>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   tc_scale_gram_kernel<FT, R><<<nb, TC_THREADS, smem, s>>>(A.Z, A.lambda_ws, I, static_cast<FT*>(Y),
                                                           last ? A.M : nullptr, A.gram_part,
-                                                          A.inner_part, err, mask);
+                                                          A.inner_part, err, mask, fuse);
   SPM_CUDA_TRY(cudaGetLastError());
   return SPM_OK;
 }
@@ -174,12 +176,13 @@ spm_status launch_tc_scale_gram_r(int nb, const spm_als_state& A, int64_t I, voi
 __attribute__((noinline)) spm_status launch_tc_scale_gram(int R, bool bf16, int nb,
                                                           const spm_als_state& A, int64_t I,
                                                           void* Y, bool last, const int* err,
-                                                          const uint32_t* mask, cudaStream_t s) {
+                                                          const uint32_t* mask, const TcFuse& fuse,
+                                                          cudaStream_t s) {
   switch ((R == 32 ? 1 : 0) + (bf16 ? 2 : 0)) {
-    case 0: return launch_tc_scale_gram_r<float, 16>(nb, A, I, Y, last, err, mask, s);
-    case 1: return launch_tc_scale_gram_r<float, 32>(nb, A, I, Y, last, err, mask, s);
-    case 2: return launch_tc_scale_gram_r<__nv_bfloat16, 16>(nb, A, I, Y, last, err, mask, s);
-    default: return launch_tc_scale_gram_r<__nv_bfloat16, 32>(nb, A, I, Y, last, err, mask, s);
+    case 0: return launch_tc_scale_gram_r<float, 16>(nb, A, I, Y, last, err, mask, fuse, s);
+    case 1: return launch_tc_scale_gram_r<float, 32>(nb, A, I, Y, last, err, mask, fuse, s);
+    case 2: return launch_tc_scale_gram_r<__nv_bfloat16, 16>(nb, A, I, Y, last, err, mask, fuse, s);
+    default: return launch_tc_scale_gram_r<__nv_bfloat16, 32>(nb, A, I, Y, last, err, mask, fuse, s);
   }
 }
 
@@ -287,13 +290,19 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
     const uint32_t* live = p->mode[d].empty_rows > 0 ? p->mode[d].rowmask : nullptr;
     SPM_TRY(launch_solve(R, nb, A, I, p->dev_err, live, s));
     const bool tcg = tc_gram_rank(R);
-    lambda_kernel<<<R, 32, 0, s>>>(A.colsq_part, tcg ? A.colmax_part : nullptr, nb, R,
-                                    A.lambda_ws, p->dev_err);
+    double* G = A.gram + (size_t)d * R * R;
+    TcFuse fuse;
+    if (tcg && nb <= TC_FUSE_PARTS)
+      fuse = {nb, A.colsq_part, A.colmax_part, A.lambda_ws, nullptr};
+    else
+      lambda_kernel<<<R, 32, 0, s>>>(A.colsq_part, tcg ? A.colmax_part : nullptr, nb, R,
+                                      A.lambda_ws, p->dev_err);
     const bool last = d == N - 1;
     int nin;  // inner-product partials of the last mode
     if (tcg) {
       nin = tc_gram_blocks(I, A.gram_blocks);
-      SPM_TRY(launch_tc_scale_gram(R, p->bf16, nin, A, I, factors[d], last, p->dev_err, live, s));
+      if (nin == 1) fuse.G = G;
+      SPM_TRY(launch_tc_scale_gram(R, p->bf16, nin, A, I, factors[d], last, p->dev_err, live, fuse, s));
     } else {
       nin = als_row_blocks(I, A.gram_blocks);
       if (p->bf16)
@@ -309,8 +318,9 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
     }
     cudaStream_t sg = last ? s : A.side;  // the fit follows the last Gram
     if (!last) SPM_TRY(fork());
-    double* G = A.gram + (size_t)d * R * R;
-    if (tcg)
+    if (fuse.G)
+      ;  // whole already
+    else if (tcg)
       gram_reduce_kernel<<<std::max(1, std::min(1024, R * R / 8)), 256, 0, sg>>>(A.gram_part, nin, R, G,
                                                                                p->dev_err);
     else
@@ -372,7 +382,7 @@ extern "C" spm_status spm_selftest_tc_rowpass(int R, int64_t I, const float* M, 
       lambda_kernel<<<R, 32, 0, s>>>(A.colsq_part, A.colmax_part, nb, R, A.lambda_ws, err);
       if (tcg) {
         const int nbg = tc_gram_blocks(I, cap);
-        SPM_TRY(launch_tc_scale_gram(R, false, nbg, A, I, Y, false, err, nullptr, s));
+        SPM_TRY(launch_tc_scale_gram(R, false, nbg, A, I, Y, false, err, nullptr, TcFuse{}, s));
         gram_reduce_kernel<<<std::max(1, std::min(1024, R * R / 8)), 256, 0, s>>>(A.gram_part, nbg, R,
                                                                                  G, err);
       } else {

@@ -978,6 +978,22 @@ inline int tc_gram_blocks(int64_t I, int cap) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, cap / 2));
 }
 
+// What a short mode's pass takes over from the kernels beside it: the column
+// norms (lambda_body) from `nb` > 0 partials of the solve, every block for
+// itself and block 0 for `lam`; the whole Gram in place of a partial, when there
+// is one block.  Such a launch costs more than its work: three modes of up to
+// 128 rows at R = 16, 137 -> 107 us per sweep.  A longer mode has too many
+// partials for every block to sum them.
+struct TcFuse {
+  int nb = 0;
+  const double* colsq = nullptr;
+  const float* colmax = nullptr;
+  double* lam = nullptr;  // as `lam` of the pass
+  double* G = nullptr;
+};
+// Up to this many partials the sum is a chain of additions shorter than a launch.
+constexpr int TC_FUSE_PARTS = 8;
+
 // The pass over tiles vb, vb + nvb, ... of Z (see above).  `lam` holds
 // lambda (R values) then the column scale exponents g_r (R values, from
 // lambda_body).  Writes Y, gram_part[vb] (R x R, lower triangle) and, when M is non-null,
@@ -989,7 +1005,8 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
                                                    double* __restrict__ gram_part,
                                                    double* __restrict__ inner_part,
                                                    const int* __restrict__ err, int vb, int nvb,
-                                                   const uint32_t* __restrict__ mask) {
+                                                   const uint32_t* __restrict__ mask,
+                                                   const TcFuse& fuse) {
   using S = TcGramShape<R>;
   extern __shared__ __align__(1024) unsigned char smem_tc[];
   __shared__ uint32_t tmem_slot;
@@ -1009,9 +1026,25 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
   const int nloc = vb < ntiles ? (int)((ntiles - 1 - vb) / nvb + 1) : 0;
 
   if (t < R) {  // one FP64 division per column, not per thread
-    const double lr = lam[t];
+    double lr;
+    if (fuse.nb > 0) {  // as lambda_body
+      double v = 0.0;
+      int mb = 0;
+      for (int b = 0; b < fuse.nb; ++b) {
+        v += fuse.colsq[b * R + t];
+        mb = max(mb, __float_as_int(fuse.colmax[b * R + t]));
+      }
+      lr = sqrt(v);
+      gx[t] = gram_scale_exp(__int_as_float(mb), lr);
+      if (vb == 0) {
+        fuse.lam[t] = lr;
+        fuse.lam[R + t] = (double)gx[t];
+      }
+    } else {
+      lr = lam[t];
+      gx[t] = (int)lam[R + t];
+    }
     linv[t] = lr > 0.0 ? (float)(1.0 / lr) : 1.f;
-    gx[t] = (int)lam[R + t];
   }
   if (warp == 0) tc::tmem_alloc(&tmem_slot, 128);
   if (t == 0) {
@@ -1178,7 +1211,13 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
         df_add(v, x.x);
         v.lo = __fadd_rn(v.lo, x.y);
       }
-      gram_part[(int64_t)vb * R * R + rr * R + ss] = times_pow2(df_value(v), gx[rr] + gx[ss] - 14);
+      const double x = times_pow2(df_value(v), gx[rr] + gx[ss] - 14);
+      if (fuse.G) {
+        fuse.G[rr * R + ss] = x;
+        fuse.G[ss * R + rr] = x;
+      } else {
+        gram_part[(int64_t)vb * R * R + rr * R + ss] = x;
+      }
     }
     if (M && t < R) {
       double sum = 0.0;

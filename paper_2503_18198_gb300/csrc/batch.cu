@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(TC_THREADS)
   if (!b.active) return;
   tc_scale_gram_body<FT, R>(b.Z, b.lambda_ws, b.dims[mode], static_cast<FT*>(b.fac[mode]),
                             mode == b.N - 1 ? b.M : nullptr, b.gram_part, b.inner_part, b.err,
-                            tv.y, b.nb_scale[mode], b.live[mode]);
+                            tv.y, b.nb_scale[mode], b.live[mode], TcFuse{});
 }
 
 template <typename FT, int R>
