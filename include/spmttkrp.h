@@ -298,7 +298,9 @@ spm_status spmttkrp_run_all_host(spmttkrp_plan_t plan, const void *const *host_f
  * for each d,
  *   M      = spMTTKRP_d(factors)                     (the plan's kernels)
  *   V      = Hadamard over w != d of (Y_w^T Y_w)     (R x R, FP64)
- *   Z      = M V^{-1}, through the FP64 Cholesky factor of V
+ *   Z      = M V^{-1}, V^{-1} from the factorisation L D L^T of V (in pairs
+ *            of FP32 values with a correction from the FP64 residual, or in
+ *            FP64 where V is ill-conditioned)
  *   lambda = column 2-norms of Z;  Y_d = Z diag(1/lambda) (columns with
  *            lambda_r = 0 are left as they are), stored as FP32 or BF16.
  * After the last mode the fit 1 - |X - Xhat|_F / |X|_F is evaluated from
@@ -320,10 +322,11 @@ spm_status spmttkrp_run_all_host(spmttkrp_plan_t plan, const void *const *host_f
  * check is device-side, so it is seen at the next synchronising call).
  * The CP-ALS state is the factors and lambda, both the caller's: a run
  * resumed from copies of them continues bitwise as the uninterrupted one.
- * Stream order: V and its inverse for mode d need no MTTKRP output, so they
- * are formed on a side stream owned by the plan, forked from `stream` with
- * an event and joined back into it before the solve of mode d; work queued
- * on `stream` after the call sees the whole sweep.  Calls on one plan from
+ * Stream order: the Gram of a mode and V and its inverse for the next need
+ * no MTTKRP output, so they are formed on a side stream owned by the plan,
+ * forked from `stream` with an event and joined back into it before the
+ * next mode's solve; work queued on `stream` after the call sees the whole
+ * sweep.  Calls on one plan from
  * different streams must not overlap (they share the plan's workspace). */
 spm_status cpd_als_step(spmttkrp_plan_t plan, void *const *factors,
                         double *lambda, double *fit, void *stream);
@@ -399,9 +402,10 @@ spm_status spm_batch_create(spm_batch_t *out, int ntensors,
 
 /* One sweep over every still-active tensor.  Launch-only (no host
  * synchronisation, no allocation): can be captured in a CUDA graph and
- * replayed.  Each mode's systems are formed on a side stream of the batch
- * (created when the first tensor is added), forked from and joined back
- * into `stream` with events, so a capture on `stream` records them too. */
+ * replayed.  Grams and systems, and launches of different (N, R) classes,
+ * run on streams of the batch (created with it or when its members change),
+ * forked from and joined back into `stream` with events, so a capture on
+ * `stream` records them too. */
 spm_status spm_batch_sweep(spm_batch_t batch, void *stream);
 
 /* Synchronise `stream`; active[t] (host) = 1 while tensor t still iterates,
@@ -536,7 +540,7 @@ spm_status spm_selftest_mttkrp_timeout(spmttkrp_plan_t plan, int mode,
  * the tensor-core arithmetic (Sec. II-A5's update; the splitting is stated in
  * the library's design notes).  Device pointers: M (I x R FP32, row-major),
  * V (R x R FP64, symmetric positive definite).  Runs the library's kernels:
- * W = V^{-1} by the FP64 Cholesky (one block per column) with W's BF16 digit
+ * W = V^{-1} column by column (one block each) with W's BF16 digit
  * stack, Z = M W on the tensor cores (Z: I x R FP32), lambda = column 2-norms
  * of Z (R doubles), Y = Z / lambda (I x R FP32) and, for R = 16 or 32,
  * G = Y^T Y on the tensor cores from the stored Y (R x R FP64; untouched for
