@@ -144,9 +144,10 @@ struct GramShape {
   static constexpr int LD = RMAX + 4;                  // row stride of the staged tile
   static constexpr int PF = GRAM_TILE_ROWS * RMAX / ALS_THREADS;  // staged values per thread
 };
-// Shared memory of a Gram block: the staged rows, then the merged sums.
+// Shared memory of a Gram block: the staged rows (read as float4), then the
+// merged sums.
 template <int GT>
-struct GramSmem {
+struct alignas(16) GramSmem {
   union {
     float tile[GRAM_TILE_ROWS * GramShape<GT>::LD];
     float2 sum[(GramShape<GT>::GROUPS + 1) / 2][GramShape<GT>::BR * 4][GramShape<GT>::TILES];
