@@ -212,7 +212,7 @@ spm_status ensure_als_state(spmttkrp_plan_s* p) {
   if (p->bf16 && A.split_cap < p->kappa && mttkrp_split(p->nnz, p->kappa, p->nu, sm_count()) > 1) {
     const size_t units = (size_t)p->kappa * p->nu;
     if (A.split_cap) {  // repartitioned since: queued work may still use the old arrays
-      SPM_CUDA_TRY(cudaDeviceSynchronize());
+      if (!dev_drain(p->device)) return SPM_ERR_CUDA;
       SPM_TRY(plan_realloc(p, (void**)&A.upart, sizeof(float) * 2 * units * R));
       SPM_TRY(plan_realloc(p, (void**)&A.urow, sizeof(int) * 2 * units));
       SPM_TRY(plan_realloc(p, (void**)&A.pdone, sizeof(int) * (size_t)p->kappa));

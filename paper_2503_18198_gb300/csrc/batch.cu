@@ -298,11 +298,11 @@ __global__ void __launch_bounds__(ALS_THREADS)
 
 
 template <typename T>
-spm_status grow(T** buf, size_t* cap, size_t need) {
+spm_status grow(int device, T** buf, size_t* cap, size_t need) {
   if (need <= *cap) return SPM_OK;
   const size_t n = std::max(need, *cap + *cap / 2);
   if (*buf) {
-    cudaDeviceSynchronize();  // queued work is done with it
+    if (!dev_drain(device)) return SPM_ERR_CUDA;  // queued work is done with it
     dev_free(*buf, sizeof(T) * *cap);
     *buf = nullptr;
     *cap = 0;
@@ -420,7 +420,7 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
   B->maxR = 1;
   for (int kc = 0; kc < KC_NONE; ++kc) B->mtt_smem[kc] = 0;
   const int queue_stride = KC_NONE + n;
-  SPM_TRY(grow(&B->queue, &B->queue_cap, (size_t)SPM_MAX_MODES * queue_stride));
+  SPM_TRY(grow(B->device, &B->queue, &B->queue_cap, (size_t)SPM_MAX_MODES * queue_stride));
   for (int t = 0; t < n; ++t) {
     spmttkrp_plan_s* p = B->plans[t];
     B->maxN = std::max(B->maxN, p->N);
@@ -499,8 +499,8 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
     per_tensor(&I.init_off, &I.n_init, [&](int t) { return B->fresh[t] ? B->host[t].nb_init[d] : 0; });
     per_tensor(&I.initt_off, &I.n_initt, [&](int t) { return B->fresh[t] ? 1 : 0; });
   }
-  SPM_TRY(grow(&B->bt, &B->bt_cap, std::max<size_t>(1, n)));
-  SPM_TRY(grow(&B->items, &B->items_cap, std::max<size_t>(1, v.size())));
+  SPM_TRY(grow(B->device, &B->bt, &B->bt_cap, std::max<size_t>(1, n)));
+  SPM_TRY(grow(B->device, &B->items, &B->items_cap, std::max<size_t>(1, v.size())));
   if (n > 0)
     SPM_CUDA_TRY(cudaMemcpyAsync(B->bt, B->host.data(), sizeof(BatchTensor) * n,
                                  cudaMemcpyHostToDevice, s));
@@ -644,10 +644,11 @@ spm_status batch_sweep(spm_batch_s* B, cudaStream_t s) {
 
 void batch_free(spm_batch_s* B) {
   if (!B) return;
-  cudaDeviceSynchronize();
-  dev_free(B->bt, sizeof(BatchTensor) * B->bt_cap);
-  dev_free(B->items, sizeof(int2) * B->items_cap);
-  dev_free(B->queue, sizeof(int) * B->queue_cap);
+  if (dev_drain(B->device)) {
+    dev_free(B->bt, sizeof(BatchTensor) * B->bt_cap);
+    dev_free(B->items, sizeof(int2) * B->items_cap);
+    dev_free(B->queue, sizeof(int) * B->queue_cap);
+  }
   if (B->ev_fork) cudaEventDestroy(B->ev_fork);
   if (B->ev_join) cudaEventDestroy(B->ev_join);
   if (B->side) cudaStreamDestroy(B->side);

@@ -27,7 +27,10 @@ spm_status plan_realloc(spmttkrp_plan_s* p, void** ptr, size_t bytes) {
   if (bytes == 0) bytes = 16;
   void* q = nullptr;
   SPM_TRY(dev_alloc(&q, bytes));
-  cudaDeviceSynchronize();
+  if (!dev_drain(p->device)) {
+    dev_free(q, bytes);
+    return SPM_ERR_CUDA;
+  }
   dev_free(*ptr, p->alloc_bytes[i]);
   p->bytes = p->bytes - p->alloc_bytes[i] + bytes;
   p->allocs[i] = q;
@@ -39,8 +42,7 @@ spm_status plan_realloc(spmttkrp_plan_s* p, void** ptr, size_t bytes) {
 void plan_free(spmttkrp_plan_s* p, void** ptr) {
   int i = 0;
   while (i < p->nallocs && p->allocs[i] != *ptr) ++i;
-  if (i == p->nallocs) return;
-  cudaDeviceSynchronize();
+  if (i == p->nallocs || !dev_drain(p->device)) return;
   dev_free(*ptr, p->alloc_bytes[i]);
   p->bytes -= p->alloc_bytes[i];
   for (int j = i + 1; j < p->nallocs; ++j) {
@@ -73,6 +75,7 @@ namespace {
 
 void free_plan(spmttkrp_plan_s* p) {
   if (!p) return;
+  const bool idle = dev_drain(p->device);
   for (cudaEvent_t e : p->ev)
     if (e) cudaEventDestroy(e);
   if (p->copy_in) cudaStreamDestroy(p->copy_in);
@@ -80,7 +83,7 @@ void free_plan(spmttkrp_plan_s* p) {
   if (p->als.ev_fork) cudaEventDestroy(p->als.ev_fork);
   if (p->als.ev_join) cudaEventDestroy(p->als.ev_join);
   if (p->als.side) cudaStreamDestroy(p->als.side);
-  for (int i = 0; i < p->nallocs; ++i) dev_free(p->allocs[i], p->alloc_bytes[i]);
+  for (int i = 0; idle && i < p->nallocs; ++i) dev_free(p->allocs[i], p->alloc_bytes[i]);
   (void)cudaGetLastError();
   delete p;
 }
@@ -187,8 +190,6 @@ spm_status spmttkrp_plan(spmttkrp_plan_t* out, int nmodes, const int64_t* dims, 
   if (st == SPM_OK && cudaMemsetAsync(p->dev_err, 0, 2 * sizeof(int), s) != cudaSuccess) st = SPM_ERR_CUDA;
   if (st == SPM_OK) st = build_copies(p, idx, vals, s);
   if (st != SPM_OK) {
-    cudaDeviceSynchronize();
-    (void)cudaGetLastError();
     free_plan(p);
     return st;
   }
@@ -332,8 +333,6 @@ spm_status spmttkrp_plan_autotune(spmttkrp_plan_t plan, const void* const* facto
 }
 
 void spmttkrp_plan_destroy(spmttkrp_plan_t plan) {
-  if (!plan) return;
-  cudaDeviceSynchronize();
   free_plan(plan);
 }
 

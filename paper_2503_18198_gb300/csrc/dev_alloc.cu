@@ -11,9 +11,11 @@
 // of a device go through one stream of the library that runs nothing else and
 // is drained before an allocation is handed out, so a buffer may be used from
 // any stream; a buffer is freed only when no queued work uses it (dev_free's
-// contract), from any thread.
+// contract), from any thread.  cudaFree waited for the buffer's own device; with
+// a pool the owners do (dev_drain).
 #include <mutex>
 
+#include "device_drain.h"
 #include "plan.cuh"
 
 namespace spm {
@@ -55,6 +57,13 @@ DevicePool* device_pool(int dev) {
   return &d;
 }
 
+// The pool of a device that need not be the current one, or null if it has none.
+DevicePool* known_pool(int dev) {
+  if (dev < 0 || dev >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_mutex);
+  return g_pools[dev].pool ? &g_pools[dev] : nullptr;
+}
+
 bool pooled(size_t bytes) { return bytes <= POOL_MAX_BYTES; }
 
 cudaError_t try_alloc(void** ptr, size_t bytes, DevicePool* d) {
@@ -87,10 +96,21 @@ void dev_free(void* ptr, size_t bytes) {
   if (!ptr) return;
   cudaPointerAttributes at{};
   DevicePool* d = nullptr;
-  if (pooled(bytes) && cudaPointerGetAttributes(&at, ptr) == cudaSuccess) d = device_pool(at.device);
+  if (pooled(bytes) && cudaPointerGetAttributes(&at, ptr) == cudaSuccess) d = known_pool(at.device);
   if (d) cudaFreeAsync(ptr, d->stream);
   else cudaFree(ptr);
   (void)cudaGetLastError();
+}
+
+bool dev_drain(int device) {
+  struct Runtime {
+    bool get(int* d) { return cudaGetDevice(d) == cudaSuccess; }
+    bool set(int d) { return cudaSetDevice(d) == cudaSuccess; }
+    bool sync() { return cudaDeviceSynchronize() == cudaSuccess; }
+  } rt;
+  if (drain_device(rt, device)) return true;
+  (void)cudaGetLastError();
+  return false;
 }
 
 }  // namespace spm

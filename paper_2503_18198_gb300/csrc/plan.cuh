@@ -108,9 +108,12 @@ struct spmttkrp_plan_s {
 namespace spm {
 
 // Device memory (dev_alloc.cu).  dev_free: with the size it was allocated with,
-// once no queued work uses it.
+// once no queued work uses it; dev_drain(device) waits for all work of the
+// memory's device, which need not be the current one (false: it could not, for
+// instance during a stream capture, and the memory must not be handed back).
 spm_status dev_alloc(void** ptr, size_t bytes);
 void dev_free(void* ptr, size_t bytes);
+bool dev_drain(int device);
 
 // Allocation owned by the plan (recorded for destroy and for plan_bytes).
 spm_status plan_alloc(spmttkrp_plan_s* p, void** ptr, size_t bytes);

@@ -101,14 +101,15 @@ size_t one_factor_bytes(const spm_server_s* S, const Job* j, int w) {
 
 void release_all(spm_server_s* S, Job* j) {
   release_plan(S, j);
-  if (j->fac[0] || j->lamfit) cudaDeviceSynchronize();  // queued work is done with them
+  // queued work is done with them
+  const bool idle = (j->fac[0] || j->lamfit) && dev_drain(S->B->device);
   for (int w = 0; w < SPM_MAX_MODES; ++w)
     if (j->fac[w]) {
-      dev_free(j->fac[w], one_factor_bytes(S, j, w));
+      if (idle) dev_free(j->fac[w], one_factor_bytes(S, j, w));
       j->fac[w] = nullptr;
     }
   if (j->lamfit) {
-    dev_free(j->lamfit, sizeof(double) * (j->R + 1));
+    if (idle) dev_free(j->lamfit, sizeof(double) * (j->R + 1));
     j->lamfit = nullptr;
   }
   S->used -= std::min(S->used, j->held);
