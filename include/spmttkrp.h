@@ -536,6 +536,13 @@ spm_status spm_selftest_mttkrp_timeout(spmttkrp_plan_t plan, int mode,
                                        const void *const *factors, float *out,
                                        void *stream);
 
+/* One sweep of a batch (as spm_batch_sweep) in which the record-copy waits of
+ * tensor `member` give up at once: that tensor gets SPM_ERR_TIMEOUT (read with
+ * spmttkrp_plan_status of its plan), every other tensor either its sweep or
+ * the same status -- never a sweep from an unfinished spMTTKRP.  May allocate;
+ * synchronises `stream`.  For the failure-detection tests. */
+spm_status spm_selftest_batch_timeout(spm_batch_t batch, int member, void *stream);
+
 /* The CP-ALS row passes of one mode on caller data, for precision tests of
  * the tensor-core arithmetic (Sec. II-A5's update; the splitting is stated in
  * the library's design notes).  Device pointers: M (I x R FP32, row-major),

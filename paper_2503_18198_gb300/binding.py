@@ -70,7 +70,7 @@ SYMBOLS = ("spmttkrp_plan", "spmttkrp_plan_bytes", "spmttkrp_plan_permutation",
            "spm_server_destroy", "spm_selftest_wait_timeout", "spm_inject_alloc_failure",
            "cpd_als_reset", "spm_server_snapshot", "spm_server_resume",
            "spmttkrp_run_all_host", "spm_selftest_mttkrp_timeout", "spmttkrp_noalloc_status",
-           "spmttkrp_plan_fibre_count", "spm_selftest_tc_rowpass")
+           "spmttkrp_plan_fibre_count", "spm_selftest_tc_rowpass", "spm_selftest_batch_timeout")
 
 
 def library_path() -> str:
@@ -146,6 +146,8 @@ def load(build_if_missing: bool = False):
     lib.spm_server_destroy.restype = None
     lib.spm_selftest_wait_timeout.argtypes = [u32, P]
     lib.spm_selftest_wait_timeout.restype = i32
+    lib.spm_selftest_batch_timeout.argtypes = [P, i32, P]
+    lib.spm_selftest_batch_timeout.restype = i32
     lib.spm_selftest_mttkrp_timeout.argtypes = [P, i32, P, P, P]
     lib.spm_selftest_mttkrp_timeout.restype = i32
     lib.spmttkrp_plan_fibre_count.argtypes = [P, i32, P]
@@ -593,6 +595,13 @@ class Server:
 def spm_selftest_wait_timeout(limit: int = 4096, stream=None) -> int:
     """Status of the bounded-wait self-test (SPM_ERR_TIMEOUT expected)."""
     return int(load().spm_selftest_wait_timeout(int(limit), _stream(stream)))
+
+
+def spm_selftest_batch_timeout(batch: "Batch", member: int, stream=None):
+    """One sweep in which the record-copy waits of tensor `member` give up at
+    once (failure-detection tests).  Synchronises."""
+    _check(load().spm_selftest_batch_timeout(batch.handle, int(member), _stream(stream)),
+           "spm_selftest_batch_timeout")
 
 
 def spm_selftest_mttkrp_timeout(plan, mode: int, factors, out, stream=None) -> int:

@@ -12,16 +12,19 @@ namespace spm {
 
 // grid == 0 only sets the kernel's shared-memory attributes.
 spm_status launch_batch_mttkrp_f32(int kc, const BatchTensor* bt, const int2* items, int nitems,
-                                   int* queue, int mode, int grid, size_t smem, cudaStream_t s);
+                                   int* queue, int* left, int mode, int grid, size_t smem,
+                                   cudaStream_t s);
 spm_status launch_batch_mttkrp_bf16(int kc, const BatchTensor* bt, const int2* items, int nitems,
-                                    int* queue, int mode, int grid, size_t smem, cudaStream_t s);
+                                    int* queue, int* left, int mode, int grid, size_t smem,
+                                    cudaStream_t s);
 
 namespace {
 
 constexpr int64_t BATCH_ZERO_WORDS = 1 << 10;  // row-bitmap words per zero-fill item
 
 // Rows cut by block boundaries, for members with many of them: one warp per
-// (tensor, partition).
+// (tensor, partition).  A member with a timeout may have blocks that never ran,
+// whose boundary records are whatever the buffer held before.
 __global__ void __launch_bounds__(256)
     batch_fixup_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ it, int nitems,
                        int mode) {
@@ -29,7 +32,7 @@ __global__ void __launch_bounds__(256)
   if (i >= nitems) return;
   const int2 tz = it[i];
   const BatchTensor& b = bt[tz.x];
-  if (!b.active) return;
+  if (!b.active || (*(volatile const int*)b.err & DEV_ERR_TIMEOUT)) return;
   const MttkrpArgs& a = b.margs[mode];
   mttkrp_fixup_body(a.cta_part, a.cta_meta, a.nblocks / (a.split > 1 ? a.split : 1), b.R, b.M, tz.y,
                     threadIdx.x & 31);
@@ -419,7 +422,7 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
   B->maxN = 0;
   B->maxR = 1;
   for (int kc = 0; kc < KC_NONE; ++kc) B->mtt_smem[kc] = 0;
-  const int queue_stride = KC_NONE + n;
+  const int queue_stride = 2 * KC_NONE + n;
   SPM_TRY(grow(B->device, &B->queue, &B->queue_cap, (size_t)SPM_MAX_MODES * queue_stride));
   for (int t = 0; t < n; ++t) {
     spmttkrp_plan_s* p = B->plans[t];
@@ -431,7 +434,8 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
     for (int d = 0; d < p->N; ++d) {
       MttkrpArgs& a = B->host[t].margs[d];
       mttkrp_set_shape(p, d, p->bf16, &a);
-      a.done = mttkrp_few_parts(a) ? B->queue + d * queue_stride + KC_NONE + t : nullptr;
+      a.wait_limit = t == B->give_up ? ~0u : 0u;
+      a.done = mttkrp_few_parts(a) ? B->queue + d * queue_stride + 2 * KC_NONE + t : nullptr;
       B->mtt_smem[kc] =
           std::max(B->mtt_smem[kc], mttkrp_smem_bytes(p->R, a.nu * std::max(1, a.split), BATCH_THREADS / 32));
     }
@@ -509,9 +513,9 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
                                  cudaMemcpyHostToDevice, s));
   for (int kc = 0; kc < KC_NONE; ++kc) {
     if (B->mtt_smem[kc] == 0 || B->mtt_smem[kc] <= B->smem_set[kc]) continue;
-    SPM_TRY(B->bf16 == 1 ? launch_batch_mttkrp_bf16(kc, nullptr, nullptr, 0, nullptr, 0, 0,
+    SPM_TRY(B->bf16 == 1 ? launch_batch_mttkrp_bf16(kc, nullptr, nullptr, 0, nullptr, nullptr, 0, 0,
                                                     B->mtt_smem[kc], s)
-                         : launch_batch_mttkrp_f32(kc, nullptr, nullptr, 0, nullptr, 0, 0,
+                         : launch_batch_mttkrp_f32(kc, nullptr, nullptr, 0, nullptr, nullptr, 0, 0,
                                                    B->mtt_smem[kc], s));
     B->smem_set[kc] = B->mtt_smem[kc];
   }
@@ -550,8 +554,9 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
 spm_status batch_mttkrp(spm_batch_s* B, int d, cudaStream_t s) {
   const spm_batch_s::ModeItems& I = B->mi[d];
   if (I.n_zero > 0) batch_zero_kernel<<<I.n_zero, 256, 0, s>>>(B->bt, B->items + I.zero_off, d);
-  // the item counters of the classes and the finished-block counters of the members
-  const int stride = KC_NONE + (int)B->host.size();
+  // the classes' counters of items taken and of blocks gone early, and the members'
+  // of finished blocks
+  const int stride = 2 * KC_NONE + (int)B->host.size();
   int* q = B->queue + d * stride;
   SPM_CUDA_TRY(cudaMemsetAsync(q, 0, sizeof(int) * stride, s));
   Phase ph(B, s);
@@ -561,8 +566,10 @@ spm_status batch_mttkrp(spm_batch_s* B, int d, cudaStream_t s) {
     const int2* it = B->items + I.mtt_off[kc];
     SPM_TRY(ph.add(n, [&](cudaStream_t t) {
       return B->bf16 == 1
-                 ? launch_batch_mttkrp_bf16(kc, B->bt, it, n, q + kc, d, grid, B->mtt_smem[kc], t)
-                 : launch_batch_mttkrp_f32(kc, B->bt, it, n, q + kc, d, grid, B->mtt_smem[kc], t);
+                 ? launch_batch_mttkrp_bf16(kc, B->bt, it, n, q + kc, q + KC_NONE + kc, d, grid,
+                                            B->mtt_smem[kc], t)
+                 : launch_batch_mttkrp_f32(kc, B->bt, it, n, q + kc, q + KC_NONE + kc, d, grid,
+                                           B->mtt_smem[kc], t);
     }));
   }
   SPM_TRY(ph.join());
@@ -719,6 +726,19 @@ spm_status spm_batch_status(spm_batch_t B, int* active, int* sweeps, void* strea
 }
 
 void spm_batch_destroy(spm_batch_t B) { batch_free(B); }
+
+spm_status spm_selftest_batch_timeout(spm_batch_t B, int member, void* stream) {
+  if (!B || member < 0 || member >= (int)B->host.size()) return SPM_ERR_INVALID_ARG;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (!B->dirty) SPM_TRY(batch_pull(B, s));
+  B->give_up = member;
+  B->dirty = true;
+  spm_status st = batch_sweep(B, s);
+  B->give_up = -1;
+  if (st == SPM_OK) st = batch_pull(B, s);
+  B->dirty = true;  // the next sweep waits as usual
+  return st;
+}
 
 spm_status spm_batch_autotune(int ntensors, const spmttkrp_plan_t* plans, void* const* factors,
                               const int64_t* candidates, int ncandidates, int reps,

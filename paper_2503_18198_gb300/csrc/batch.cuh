@@ -14,6 +14,7 @@ struct spm_batch_s {
   std::vector<spm::BatchTensor> host;  // descriptors; the device copy is newer after sweeps
   std::vector<char> fresh;             // member's starting Grams still to be formed
   bool dirty = true;                   // host list changed since the last upload
+  int give_up = -1;                    // member whose record-copy waits give up at once (self-test)
   // Work-item tables of one mode, as offsets into `items`.
   struct ModeItems {
     int mtt_off[spm::KC_NONE] = {};
@@ -37,7 +38,8 @@ struct spm_batch_s {
   size_t bt_cap = 0;
   int2* items = nullptr;
   size_t items_cap = 0;
-  int* queue = nullptr;  // per mode: work-queue counters of the classes, then the
+  int* queue = nullptr;  // per mode: the classes' counters of items taken and of blocks that
+                         // left before the queue was empty, then the
                          // finished-block counters of the members
   size_t queue_cap = 0;
   int grid = 0;          // SMs

@@ -88,10 +88,11 @@ constexpr int BATCH_THREADS = 512;
 // (N, R) class: blocks take items from a work queue in order.  One kernel per
 // class keeps each instantiation's register allocation that of the
 // single-tensor kernel.
+// `left` counts the blocks that leave before the queue is empty.
 template <typename FT, int KC>
 __global__ void __launch_bounds__(BATCH_THREADS, 2)
     mttkrp_batch_kernel(const BatchTensor* __restrict__ bt, const int2* __restrict__ items,
-                        int nitems, int* __restrict__ queue, int mode) {
+                        int nitems, int* __restrict__ queue, int* __restrict__ left, int mode) {
   using C = BatchClass<KC>;
   // the lane layout the single-tensor kernel picks for this (type, rank)
   constexpr int V = (sizeof(FT) == 2 && C::N == 3 && C::R <= 32) ? 4 : 16 / (int)sizeof(FT);
@@ -106,10 +107,20 @@ __global__ void __launch_bounds__(BATCH_THREADS, 2)
     const int2 tz = items[i];
     const BatchTensor& b = bt[tz.x];
     if (b.active) mttkrp_partition<C::RI, C::N - 1, FT, V, C::R / V, 1, false, PLAN>(b.margs[mode], tz.y);
-    __syncthreads();
     // a bounded wait that gave up may leave a copy in flight into this
-    // block's ring: take no further partition into it
-    if (b.active && (*(volatile const int*)b.err & DEV_ERR_TIMEOUT)) return;
+    // block's ring: take no further partition into it (one thread reads the flag,
+    // which other blocks may be setting, for the whole block).  The items that are
+    // left once every block has gone this way were not computed: their members
+    // must not be solved from what their buffers held before.
+    if (__syncthreads_or(threadIdx.x == 0 && b.active &&
+                         (*(volatile const int*)b.err & DEV_ERR_TIMEOUT))) {
+      if (threadIdx.x == 0 && atomicAdd(left, 1) == (int)gridDim.x - 1)
+        for (int j = atomicAdd(queue, nitems); j < nitems; ++j) {
+          const BatchTensor& o = bt[items[j].x];
+          if (o.active) atomicOr(o.err, DEV_ERR_TIMEOUT);
+        }
+      return;
+    }
   }
 }
 
