@@ -7,12 +7,19 @@
 // maps large memory faster than a pool does (800 MB: 240 against 630 us).
 //
 // What the pool keeps once buffers are freed is bounded (POOL_KEEP_BYTES) and
-// is given back when an allocation would otherwise fail.  All pool operations
-// of a device go through one stream of the library that runs nothing else and
+// is given back when an allocation would otherwise fail.  Buffers are allocated
+// and freed on one stream of the library that runs nothing else and
 // is drained before an allocation is handed out, so a buffer may be used from
 // any stream; a buffer is freed only when no queued work uses it (dev_free's
 // contract), from any thread.  cudaFree waited for the buffer's own device; with
 // a pool the owners do (dev_drain).
+//
+// Scratch that one stream's work uses (scratch_alloc) is freed in the order of
+// that stream: cudaFree waits for the whole device, so that a plan built beside
+// a running sweep ended with the sweep.  Large scratch still comes from
+// cudaMalloc; freed by cudaFreeAsync, it is given back when the stream is next
+// synchronised.  (50M nonzeros, 1.2 GB of scratch: a build takes 13.6 ms so, as
+// with cudaFree, and 15.3 ms with the scratch in the pool.)
 #include <mutex>
 
 #include "device_drain.h"
@@ -90,6 +97,31 @@ spm_status dev_alloc(void** ptr, size_t bytes) {
   (void)cudaGetLastError();
   *ptr = nullptr;
   return e == cudaErrorMemoryAllocation ? SPM_ERR_OOM : SPM_ERR_CUDA;
+}
+
+spm_status scratch_alloc(void** ptr, size_t bytes, cudaStream_t s) {
+  *ptr = nullptr;
+  int dev = 0;
+  SPM_CUDA_TRY(cudaGetDevice(&dev));
+  DevicePool* d = device_pool(dev);
+  auto get = [&]() {
+    return d && pooled(bytes) ? cudaMallocFromPoolAsync(ptr, bytes, d->pool, s)
+                              : cudaMalloc(ptr, bytes);
+  };
+  cudaError_t e = get();
+  if (e == cudaErrorMemoryAllocation && d) {
+    (void)cudaGetLastError();
+    (void)cudaMemPoolTrimTo(d->pool, 0);
+    e = get();
+  }
+  if (e == cudaSuccess) return SPM_OK;
+  (void)cudaGetLastError();
+  *ptr = nullptr;
+  return e == cudaErrorMemoryAllocation ? SPM_ERR_OOM : SPM_ERR_CUDA;
+}
+
+void scratch_free(void* ptr, cudaStream_t s) {
+  if (ptr && cudaFreeAsync(ptr, s) != cudaSuccess) (void)cudaGetLastError();
 }
 
 void dev_free(void* ptr, size_t bytes) {

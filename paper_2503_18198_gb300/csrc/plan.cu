@@ -971,19 +971,23 @@ struct BuildScratch {
     }
     return at;
   }
-  size_t bytes = 0;
-  spm_status alloc(int64_t cap) {
+  cudaStream_t stream = nullptr;
+  spm_status alloc(int64_t cap, cudaStream_t s) {
     void* p = nullptr;
-    bytes = layout(cap, nullptr, nullptr);
-    SPM_TRY(dev_alloc(&p, bytes));
+    stream = s;
+    SPM_TRY(scratch_alloc(&p, layout(cap, nullptr, nullptr), s));
     layout(cap, static_cast<unsigned char*>(p), this);
     return SPM_OK;
   }
-  // Freed by the owner's scope, after the build's stream is drained.
   BuildScratch() = default;
   BuildScratch(const BuildScratch&) = delete;
   BuildScratch& operator=(const BuildScratch&) = delete;
-  ~BuildScratch() { dev_free(base, bytes); }
+  ~BuildScratch() { release(); }
+  // Stream-ordered; a synchronisation after it gives large scratch back.
+  void release() {
+    scratch_free(base, stream);
+    base = nullptr;
+  }
 };
 
 template <int RI>
@@ -1001,11 +1005,7 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
   // Scheme 1 sorts the rows of a mode by degree
   const int64_t cap = sort_capacity(N, p->dims, nn, p->policy, p->kappa);
   BuildScratch b;
-  struct Drain {  // runs before the scratch is freed, on every way out
-    cudaStream_t s;
-    ~Drain() { cudaStreamSynchronize(s); }
-  } drain{s};
-  SPM_TRY(b.alloc(cap));
+  SPM_TRY(b.alloc(cap, s));
   const SortScratch& sc = b.sort;
 
   // modes grouped into <=64-bit key words from the last mode backwards
@@ -1217,6 +1217,7 @@ spm_status build_copies_t(spmttkrp_plan_s* p, const int32_t* const* idx_in, cons
     SPM_CUDA_TRY(cudaMemcpyAsync(h_cnt, b.count, sizeof(unsigned) * SPM_MAX_MODES,
                                  cudaMemcpyDeviceToHost, s));
   SPM_CUDA_TRY(cudaGetLastError());
+  b.release();
   SPM_CUDA_TRY(cudaStreamSynchronize(s));
   for (int d = 0; d < N; ++d) p->mode[d].empty_rows = p->dims[d] - (int64_t)h_cnt[d];
   return st;
