@@ -30,12 +30,24 @@ MttkrpKernelFn pick_mttkrp_f32_between5(int R);
 MttkrpKernelFn pick_mttkrp_bf16_between3(int R);
 MttkrpKernelFn pick_mttkrp_bf16_between4(int R);
 MttkrpKernelFn pick_mttkrp_bf16_between5(int R);
+MttkrpKernelFn pick_mttkrp_f32_lean_between3(int R);
+MttkrpKernelFn pick_mttkrp_f32_lean_between4(int R);
+MttkrpKernelFn pick_mttkrp_f32_lean_between5(int R);
+MttkrpKernelFn pick_mttkrp_bf16_lean_between3(int R);
+MttkrpKernelFn pick_mttkrp_bf16_lean_between4(int R);
+MttkrpKernelFn pick_mttkrp_bf16_lean_between5(int R);
 
 // 3 to 5 modes and a rank without a fast shape: the shape between, or null.
-static MttkrpKernelFn pick_mttkrp_between(bool bf16, int nin, int R) {
+static MttkrpKernelFn pick_mttkrp_between(bool bf16, bool lean, int nin, int R) {
   const int W = bf16 ? 8 : 4, l = R / W;
   const bool fast = (R % W == 0 && l <= 64 && (l & (l - 1)) == 0) || (bf16 && nin == 2 && R == 4);
   if (fast) return nullptr;
+  if (lean) switch (nin) {
+    case 2: return bf16 ? pick_mttkrp_bf16_lean_between3(R) : pick_mttkrp_f32_lean_between3(R);
+    case 3: return bf16 ? pick_mttkrp_bf16_lean_between4(R) : pick_mttkrp_f32_lean_between4(R);
+    case 4: return bf16 ? pick_mttkrp_bf16_lean_between5(R) : pick_mttkrp_f32_lean_between5(R);
+    default: return nullptr;
+  }
   switch (nin) {
     case 2: return bf16 ? pick_mttkrp_bf16_between3(R) : pick_mttkrp_f32_between3(R);
     case 3: return bf16 ? pick_mttkrp_bf16_between4(R) : pick_mttkrp_f32_between4(R);
@@ -45,7 +57,7 @@ static MttkrpKernelFn pick_mttkrp_between(bool bf16, int nin, int R) {
 }
 
 MttkrpKernelFn pick_mttkrp(bool bf16, int nin, int R) {
-  if (MttkrpKernelFn fn = pick_mttkrp_between(bf16, nin, R)) return fn;
+  if (MttkrpKernelFn fn = pick_mttkrp_between(bf16, false, nin, R)) return fn;
   if (nin == 4) return bf16 ? pick_mttkrp_bf16_c(R) : pick_mttkrp_f32_c(R);
   if (bf16) return nin <= 2 ? pick_mttkrp_bf16_a(nin, R) : pick_mttkrp_bf16_b(nin, R);
   return nin <= 2 ? pick_mttkrp_f32_a(nin, R) : pick_mttkrp_f32_b(nin, R);
@@ -156,9 +168,10 @@ spm_status run_mttkrp(spmttkrp_plan_s* p, int mode, const void* const* factors, 
   if (a.split > 0)  // BF16 (run_mttkrp's plan order)
     fn = lean ? pick_mttkrp_bf16_plan_lean(nin, R)
               : (nin <= 2 ? pick_mttkrp_bf16_plan_a(nin, R) : pick_mttkrp_bf16_plan_b(nin, R));
-  else if (lean)
-    fn = p->bf16 ? pick_mttkrp_bf16_lean(nin, R) : pick_mttkrp_f32_lean(nin, R);
-  else
+  else if (lean) {
+    fn = pick_mttkrp_between(p->bf16, true, nin, R);  // the full plan's lanes: the same sums
+    if (!fn) fn = p->bf16 ? pick_mttkrp_bf16_lean(nin, R) : pick_mttkrp_f32_lean(nin, R);
+  } else
     fn = pick_mttkrp(p->bf16, nin, R);
   if (!fn) return SPM_ERR_UNSUPPORTED;
   // a block that is full of short units leaves room for a second one

@@ -18,30 +18,31 @@ using MttkrpKernelFn = void (*)(const MttkrpArgs);
 // that a warp step still holds 32 / LPN nonzeros.  Odd ranks take one rank per
 // lane.  (2M nonzeros, R = 24, FP32, three modes: 652 us with one nonzero per
 // step and eight chunks of 32 ranks, 158 us so; R = 10, 48, 100 with 3 modes: 253,
-// 280, 335 us per mode against 43, 72, 112.)
-template <typename FT, int NIN>
+// 280, 335 us per mode against 43, 72, 112.)  Lean plans take the same shapes, so
+// that their sums are the full plan's bit for bit (same 2M nonzeros, R = 24, all modes: 619 -> 170 us).
+template <typename FT, int NIN, bool LEAN = false>
 MttkrpKernelFn pick_mttkrp_between_t(int R) {
   constexpr int RI = record_int4s(NIN + 1);
   if constexpr (sizeof(FT) == 2) {
     if (R % 8 == 0 && R > 32) {
-      if (R <= 64) return &mttkrp_kernel<RI, NIN, FT, 8, 8, 1, false, false, true>;
-      if (R <= 128) return &mttkrp_kernel<RI, NIN, FT, 8, 16, 1, false, false, true>;
-      return &mttkrp_kernel<RI, NIN, FT, 8, 32, 1, false, false, true>;
+      if (R <= 64) return &mttkrp_kernel<RI, NIN, FT, 8, 8, 1, LEAN, false, true>;
+      if (R <= 128) return &mttkrp_kernel<RI, NIN, FT, 8, 16, 1, LEAN, false, true>;
+      return &mttkrp_kernel<RI, NIN, FT, 8, 32, 1, LEAN, false, true>;
     }
   }
   if (R % 4 == 0 && R <= 128) {
-    if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 4, 8, 1, false, false, true>;
-    if (R <= 64) return &mttkrp_kernel<RI, NIN, FT, 4, 16, 1, false, false, true>;
-    return &mttkrp_kernel<RI, NIN, FT, 4, 32, 1, false, false, true>;
+    if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 4, 8, 1, LEAN, false, true>;
+    if (R <= 64) return &mttkrp_kernel<RI, NIN, FT, 4, 16, 1, LEAN, false, true>;
+    return &mttkrp_kernel<RI, NIN, FT, 4, 32, 1, LEAN, false, true>;
   }
   if (R % 2 == 0 && R <= 64) {
-    if (R <= 16) return &mttkrp_kernel<RI, NIN, FT, 2, 8, 1, false, false, true>;
-    if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 2, 16, 1, false, false, true>;
-    return &mttkrp_kernel<RI, NIN, FT, 2, 32, 1, false, false, true>;
+    if (R <= 16) return &mttkrp_kernel<RI, NIN, FT, 2, 8, 1, LEAN, false, true>;
+    if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 2, 16, 1, LEAN, false, true>;
+    return &mttkrp_kernel<RI, NIN, FT, 2, 32, 1, LEAN, false, true>;
   }
-  if (R <= 16) return &mttkrp_kernel<RI, NIN, FT, 1, 16, 1>;
-  if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 1, 32, 1>;
-  if (R <= 64) return &mttkrp_kernel<RI, NIN, FT, 1, 32, 2>;
+  if (R <= 16) return &mttkrp_kernel<RI, NIN, FT, 1, 16, 1, LEAN>;
+  if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 1, 32, 1, LEAN>;
+  if (R <= 64) return &mttkrp_kernel<RI, NIN, FT, 1, 32, 2, LEAN>;
   return nullptr;
 }
 

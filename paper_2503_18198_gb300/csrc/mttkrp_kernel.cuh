@@ -675,7 +675,7 @@ __device__ __forceinline__ void mttkrp_partition(const MttkrpArgs& a, const int 
   auto rank0 = [&](int c) -> int { return (c * LPN + sub) * VEC; };
   // MASK: R < VEC * LPN is a multiple of VEC; the lanes beyond it repeat the
   // last lane's ranks and store nothing.
-  static_assert(!MASK || (CPL == 1 && !LEAN && !PLAN), "masked ranks: one chunk");
+  static_assert(!MASK || (CPL == 1 && !PLAN), "masked ranks: one chunk");
   const bool store_lane = !MASK || rank0(0) < R;
   auto load_rank = [&](int c) -> int { return MASK ? min(rank0(c), R - VEC) : rank0(c); };
   // Vector path with the rank fixed at compile time (R == VEC * LPN * CPL):
