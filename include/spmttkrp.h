@@ -129,7 +129,11 @@ typedef enum {
  * multiprocessor (Sec. III-B); on GB300 two resident waves of partition
  * blocks per SM balance the per-partition time variance (the block
  * scheduler gives a free SM the next partition).  Any value 1..65535 may be
- * forced, e.g. SPM_KAPPA(sm count) for the paper's one-per-SM layout. */
+ * forced, e.g. SPM_KAPPA(sm count) for the paper's one-per-SM layout.  A run
+ * takes one thread block per partition where the count is a whole number per SM
+ * (or larger than the device needs) and a partition holds 4096 nonzeros;
+ * otherwise the partitions are cut or merged for the launch.  What the plan
+ * reports (partitions, work units) does not change with that. */
 #define SPM_PARTITIONS_PER_SM 2
 #define SPM_KAPPA(k) (((uint32_t)(k) & 0xFFFFu) << 16)
 #define SPM_KAPPA_OF(flags) (((uint32_t)(flags) >> 16) & 0xFFFFu)
@@ -357,14 +361,19 @@ spm_status spmttkrp_plan_repartition(spmttkrp_plan_t plan, int kappa, void *stre
 
 /* Autotune the partition count of one plan: for each candidate kappa
  * (kappas[0..nkappas-1]; NULL = {SM count, 2 x SM count}) the plan is
- * repartitioned and spmttkrp_run of every mode is timed with CUDA events on
+ * repartitioned and the spMTTKRP of every mode, as a CP-ALS sweep of the plan
+ * runs it, is timed with CUDA events on
  * `stream` (best of `reps` after one warm-up, outputs written to the plan's
- * CP-ALS workspace, which is allocated if absent).  The plan is left at the
+ * CP-ALS workspace, which is allocated if absent).  Candidates that are run in
+ * the same launch (a small tensor is cut for the device whatever kappa is) are
+ * timed once and share the time; among them the count that the plan had is
+ * kept, else the first.  The plan is left at the
  * fastest candidate, *chosen receives it and ms[c] (host, may be NULL) each
  * candidate's time for all modes.  Factors as for spmttkrp_run (read only).
  * BALANCED and SCHEME2 policies only.  Synchronises `stream`.  The paper fixes
  * one partition per SM (Sec. III-B); which count is fastest on GB300 depends
- * on the tensor's skew, hence the measurement. */
+ * on the tensor's skew, hence the measurement (from 4096 nonzeros per partition
+ * on, about 1.2M, one and two per SM are launches of their own). */
 spm_status spmttkrp_plan_autotune(spmttkrp_plan_t plan, const void *const *factors,
                                   const int *kappas, int nkappas, int reps, int *chosen,
                                   float *ms, void *stream);

@@ -3,6 +3,7 @@
 #include <cstring>
 #include <algorithm>
 #include <new>
+#include <vector>
 
 #include "plan.cuh"
 
@@ -299,15 +300,38 @@ spm_status spmttkrp_plan_autotune(spmttkrp_plan_t plan, const void* const* facto
     return SPM_ERR_CUDA;
   }
   spm_status st = SPM_OK;
+  const int had = plan->kappa;
+  // the launches that a CP-ALS sweep of the plan makes (BF16: the plan's order)
+  const bool sweep_order = plan->bf16 && plan->R <= ALS_MAX_RANK;
+  // Candidates that the kernel runs in the same blocks and units are one launch,
+  // timed once: a choice between two times of it would be noise.
+  auto same = [&](int a, int b) {
+    if (a == b) return true;
+    if (sweep_order) return false;
+    const MttkrpShape x = mttkrp_shape(plan->mode[0].scheme, plan->nnz, a, plan->nu, sms);
+    const MttkrpShape y = mttkrp_shape(plan->mode[0].scheme, plan->nnz, b, plan->nu, sms);
+    return x.kx == y.kx && x.nx == y.nx;
+  };
+  std::vector<float> took(nkappas);
   int best = -1;
   float best_ms = 0.f;
   for (int c = 0; c < nkappas && st == SPM_OK; ++c) {
+    int twin = 0;
+    while (twin < c && !same(kappas[twin], kappas[c])) ++twin;
+    if (twin < c) {
+      took[c] = took[twin];
+      if (ms) ms[c] = took[c];
+      // among equals, the count that the plan had
+      if (best >= 0 && same(kappas[best], kappas[c]) && kappas[c] == had) best = c;
+      continue;
+    }
     st = plan_repartition(plan, kappas[c], s);
+    if (st == SPM_OK) st = ensure_als_state(plan);  // sized for these partitions
     float t_min = 0.f;
     for (int r = 0; r <= reps && st == SPM_OK; ++r) {  // r == 0 warms up
       cudaEventRecord(e0, s);
       for (int d = 0; d < plan->N && st == SPM_OK; ++d)
-        st = run_mttkrp(plan, d, factors, plan->als.M, s);
+        st = run_mttkrp(plan, d, factors, plan->als.M, s, sweep_order);
       cudaEventRecord(e1, s);
       if (st == SPM_OK && cudaEventSynchronize(e1) != cudaSuccess) st = SPM_ERR_CUDA;
       float t = 0.f;
@@ -315,6 +339,7 @@ spm_status spmttkrp_plan_autotune(spmttkrp_plan_t plan, const void* const* facto
       if (r == 1 || (r > 1 && t < t_min)) t_min = t;
     }
     if (st != SPM_OK) break;
+    took[c] = t_min;
     if (ms) ms[c] = t_min;
     if (best < 0 || t_min < best_ms) {
       best = c;

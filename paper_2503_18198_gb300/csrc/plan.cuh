@@ -38,6 +38,8 @@ inline constexpr size_t als_wdig_bytes(int R) {
   return (R == 16 || R == 32 || R == 64) ? (size_t)7 * 2 * R * R + 4 * (size_t)R : 0;
 }
 
+constexpr int ALS_MAX_RANK = 64;  // of CP-ALS sweeps
+
 struct spm_als_state {
   bool ready = false;                 // Gram cache valid for `fac_ptr`
   const void* fac_ptr[SPM_MAX_MODES] = {};
@@ -151,8 +153,9 @@ void plan_bytes_estimate(int N, const int64_t* dims, int64_t nnz, int R, int kap
 
 // Thread blocks and work units per block with which a record copy of nnz
 // nonzeros is run.  The partitions B_{d,z} that the caller sees (kappa, nu)
-// are kept where they are large enough to fill a block of 32 warps; otherwise
-// the copy is cut for the device:
+// are kept, one block of 32 warps each, where there are enough of them for the
+// device -- or a whole number per SM was asked for, as in the paper -- and each
+// holds 4096 nonzeros; otherwise the copy is cut for the device:
 //  * a block per 1024 nonzeros up to two per SM.  One tensor of 4,096
 //    nonzeros on the default 304 partitions of 128 units ran 31 us per mode
 //    (cold caches), 300,000 nonzeros 50 us; in this shape 14 and 11 us;
@@ -160,6 +163,8 @@ void plan_bytes_estimate(int N, const int64_t* dims, int64_t nnz, int R, int kap
 // The kernel reads its unit boundaries off the plan's: unit j of kx * nx begins
 // j / (kx * nx) of the way through the plan's units, inside one by its length.
 // Scheme 1 keeps its partitions: their rows are not in order across them.
+// (One per SM: 20M uniform nonzeros, three modes 0.80 ms, two per SM 0.83; on
+// skewed tensors two are faster, which the autotuner finds out.)
 // A plan with fewer partitions than that was asked for few (the batch's autotuner
 // and the server choose about 131,072 nonzeros each, to share the device among
 // many tensors): MTTKRP_CUT blocks per partition.  96 FP32 tensors up to 2M
@@ -170,14 +175,15 @@ constexpr int MTTKRP_CUT = 16;
 struct MttkrpShape {
   int kx, nx;
 };
-inline int mttkrp_fine_blocks(int64_t nnz, int sms) {
+inline constexpr int mttkrp_fine_blocks(int64_t nnz, int sms) {
   const int64_t b = (nnz + 1023) / 1024;
   return (int)(b < 1 ? 1 : b > 2 * sms ? 2 * sms : b);
 }
-inline MttkrpShape mttkrp_shape(int scheme, int64_t nnz, int kappa, int nu, int sms) {
+inline constexpr MttkrpShape mttkrp_shape(int scheme, int64_t nnz, int kappa, int nu, int sms) {
   if (scheme == 1) return {kappa, nu};
   const int fine = mttkrp_fine_blocks(nnz, sms);
-  const int kx = kappa < fine ? std::min(fine, MTTKRP_CUT * kappa) : nnz / kappa >= 4096 ? kappa : fine;
+  const bool keep = kappa >= fine || kappa % sms == 0;
+  const int kx = !keep ? std::min(fine, MTTKRP_CUT * kappa) : nnz / kappa >= 4096 ? kappa : fine;
   int nx = 16;
   while (2 * nx <= nu && nnz / kx >= (int64_t)nx * 256) nx *= 2;
   return {kx, nx};
@@ -185,7 +191,7 @@ inline MttkrpShape mttkrp_shape(int scheme, int64_t nnz, int kappa, int nu, int 
 // Blocks per partition of a run in plan order (BF16 CP-ALS, see run_mttkrp): a
 // partition's units are shared by up to nu / 16 blocks (16 warps take one each)
 // while there are fewer than two blocks per SM and 1024 nonzeros for each.
-inline int mttkrp_split(int64_t nnz, int kappa, int nu, int sms) {
+inline constexpr int mttkrp_split(int64_t nnz, int kappa, int nu, int sms) {
   int s = 1;
   while (32 * s <= nu && nu % (2 * s) == 0 && kappa * s < 2 * sms && nnz / kappa >= 2048 * (int64_t)s) s *= 2;
   return s;

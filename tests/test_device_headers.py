@@ -31,3 +31,23 @@ def test_staged_gram_rows_take_16_byte_loads(nvcc, tmp_path):
     check(nvcc, tmp_path, "\n".join(
         f"static_assert(alignof(GramSmem<{g}>) % 16 == 0 && GramShape<{g}>::LD % 4 == 0, \"\");"
         for g in (1, 2, 4)))
+
+
+def test_partitions_asked_for_per_sm_are_what_a_run_takes(nvcc, tmp_path):
+    """One and two partitions per SM are different launches from 4096 nonzeros
+    per partition on (one block each), so that the autotuner's default
+    candidates are a choice; below, and at counts that leave SMs idle, the copy
+    is cut for the device."""
+    kx = "mttkrp_shape(0, {nnz}LL, {kappa}, 128, {sms}).kx"
+    cases = []
+    for sms in (148, 152):
+        for per in (1, 2, 3):
+            k = per * sms
+            cases += [(4096 * k, k, sms, k), (50_000_000, k, sms, k), (4096 * k - 1, k, sms, 2 * sms)]
+        cases += [(50_000_000, sms - 1, sms, 2 * sms), (50_000_000, 1, sms, 16), (50_000_000, 3, sms, 48),
+                  (50_000_000, sms + 1, sms, 2 * sms), (50_000_000, 2 * sms + 1, sms, 2 * sms + 1),
+                  (1, 1, sms, 1), (20_000, sms, sms, 20), (20_000, 2 * sms, sms, 20), (33_000, 2, sms, 32),
+                  (33_000, 3, sms, 33)]
+    check(nvcc, tmp_path, "\n".join(
+        f"static_assert({kx.format(nnz=n, kappa=k, sms=s)} == {want}, \"{n} {k} {s}\");"
+        for n, k, s, want in cases))
