@@ -361,7 +361,7 @@ extern "C" spm_status spm_selftest_tc_rowpass(int R, int64_t I, const float* M, 
   alloc((void**)&grams, sizeof(double) * 2 * RR);
   alloc((void**)&err, sizeof(int));
   alloc((void**)&A.winv, sizeof(float) * 2 * RR);
-  alloc((void**)&A.wdig, als_wdig_bytes(R));
+  if (als_wdig_bytes(R)) alloc((void**)&A.wdig, als_wdig_bytes(R));
   alloc((void**)&A.colsq_part, sizeof(double) * R * cap);
   alloc((void**)&A.colmax_part, sizeof(float) * R * cap);
   alloc((void**)&A.lambda_ws, sizeof(double) * 2 * R);

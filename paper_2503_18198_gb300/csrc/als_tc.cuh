@@ -45,12 +45,6 @@ constexpr int SW_DIG = 7;      // digits of a column of W (49 bits)
 constexpr int TC_LMAX = 6;     // highest digit level kept
 static_assert(TC_LMAX + 1 == SW_DIG, "W's digit stack covers every kept level");
 
-#ifndef SPM_ALS_TC
-#define SPM_ALS_TC 1  // 0: every rank takes the CUDA-core (double-float) row solve
-#endif
-__host__ __device__ constexpr bool tc_solve_rank(int R) {
-  return SPM_ALS_TC && (R == 16 || R == 32 || R == 64);
-}
 
 // Virtual blocks of the row solve over I rows: one tile of the tensor-core
 // solve each while the partial buffers last.
@@ -84,8 +78,9 @@ __host__ __device__ constexpr int tc_wdig_bytes(int R) {
          : R == 64 ? TcSolveShape<64>::WD_BYTES : 0;
 }
 
-static_assert(tc_wdig_bytes(16) == als_wdig_bytes(16) && tc_wdig_bytes(32) == als_wdig_bytes(32) &&
-                  tc_wdig_bytes(64) == als_wdig_bytes(64),
+static_assert(!SPM_ALS_TC || (tc_wdig_bytes(16) == als_wdig_bytes(16) &&
+                              tc_wdig_bytes(32) == als_wdig_bytes(32) &&
+                              tc_wdig_bytes(64) == als_wdig_bytes(64)),
               "plan accounting of the W digit tiles");
 
 // 2^k as a float for -126 <= k <= 127 (exact).

@@ -31,11 +31,18 @@ struct spm_mode_copy {
   int scheme = 0;            // 0 cost-balanced, 1 or 2 (Sec. III-B)
 };
 
-// Bytes of the W digit tiles of the tensor-core row solve for rank R: the
-// BF16 digit stack (7 digits x R x R) and R column exponents; ranks 16, 32
-// and 64 only.
+// Ranks of the tensor-core row solve.
+#ifndef SPM_ALS_TC
+#define SPM_ALS_TC 1  // 0: every rank takes the CUDA-core (double-float) row solve
+#endif
+__host__ __device__ constexpr bool tc_solve_rank(int R) {
+  return SPM_ALS_TC && (R == 16 || R == 32 || R == 64);
+}
+// Bytes of the solve's W digit tiles: the BF16 digit stack (7 digits x R x R) and
+// R column exponents.  Where there is none the system kernel writes V^{-1} for
+// the CUDA-core solve in its place.
 inline constexpr size_t als_wdig_bytes(int R) {
-  return (R == 16 || R == 32 || R == 64) ? (size_t)7 * 2 * R * R + 4 * (size_t)R : 0;
+  return tc_solve_rank(R) ? (size_t)7 * 2 * R * R + 4 * (size_t)R : 0;
 }
 
 constexpr int ALS_MAX_RANK = 64;  // of CP-ALS sweeps

@@ -51,3 +51,12 @@ def test_partitions_asked_for_per_sm_are_what_a_run_takes(nvcc, tmp_path):
     check(nvcc, tmp_path, "\n".join(
         f"static_assert({kx.format(nnz=n, kappa=k, sms=s)} == {want}, \"{n} {k} {s}\");"
         for n, k, s, want in cases))
+
+
+@pytest.mark.parametrize("tc", [1, 0])
+def test_the_digit_tile_exists_for_the_ranks_of_the_tensor_core_solve_only(nvcc, tmp_path, tc):
+    """The system kernel writes either the digit tile or V^-1 itself: a tile held
+    for a rank whose solve is on the CUDA cores would leave that solve nothing."""
+    check(nvcc, tmp_path, "\n".join(
+        f"static_assert((als_wdig_bytes({r}) != 0) == tc_solve_rank({r}), \"rank {r}\");"
+        for r in (8, 16, 24, 32, 64)), f"-DSPM_ALS_TC={tc}")
