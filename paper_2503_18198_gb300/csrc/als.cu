@@ -209,7 +209,7 @@ spm_status ensure_als_state(spmttkrp_plan_s* p) {
   if (!A.ev_fork) SPM_CUDA_TRY(cudaEventCreateWithFlags(&A.ev_fork, cudaEventDisableTiming));
   if (!A.ev_join) SPM_CUDA_TRY(cudaEventCreateWithFlags(&A.ev_join, cudaEventDisableTiming));
   const int R = p->R;
-  if (p->bf16 && A.split_cap < p->kappa && mttkrp_split(p->nnz, p->kappa, p->nu, sm_count()) > 1) {
+  if (als_splits(p->bf16, p->fibre, p->nnz, p->kappa, p->nu, sm_count()) && A.split_cap < p->kappa) {
     const size_t units = (size_t)p->kappa * p->nu;
     if (A.split_cap) {  // repartitioned since: queued work may still use the old arrays
       if (!dev_drain(p->device)) return SPM_ERR_CUDA;

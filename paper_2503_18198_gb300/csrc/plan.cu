@@ -1272,7 +1272,7 @@ void plan_bytes_estimate(int N, const int64_t* dims, int64_t nnz, int R, int kap
     b += sizeof(float) * 2 * RR + sizeof(double) * R * gb * 2 + sizeof(double) * 2 * R;
     b += sizeof(float) * R * gb + als_wdig_bytes(R);  // column maxima of Z, W digit tiles
     b += sizeof(float) * (size_t)Imax * R * 2;
-    if (bf16 && mttkrp_split(nnz, kappa, nu, sm_count()) > 1)
+    if (als_splits(bf16, fibre, nnz, kappa, nu, sm_count()))
       b += (sizeof(float) * R + sizeof(int)) * 2 * (size_t)kappa * nu + sizeof(int) * (size_t)kappa;
   }
   *resident = b;

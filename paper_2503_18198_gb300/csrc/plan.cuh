@@ -204,6 +204,12 @@ inline constexpr int mttkrp_split(int64_t nnz, int kappa, int nu, int sms) {
   return s;
 }
 
+// Whether a plan's CP-ALS keeps the buffers of such a run (fibre copies have their
+// own kernel).
+inline constexpr bool als_splits(bool bf16, bool fibre, int64_t nnz, int kappa, int nu, int sms) {
+  return bf16 && !fibre && mttkrp_split(nnz, kappa, nu, sms) > 1;
+}
+
 // Warps of a block: short unit lists leave half of the SM to a second block,
 // whose start and merge overlap the first one's gathers.
 inline int mttkrp_warps(int nx) { return nx >= 32 ? 32 : 16; }
