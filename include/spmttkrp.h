@@ -355,7 +355,9 @@ spm_status spmttkrp_plan_bytes_estimate(int nmodes, const int64_t *dims, int64_t
  * else 1..65535); the mode copies are kept.  Only for the BALANCED and
  * SCHEME2 policies (else SPM_ERR_UNSUPPORTED).  Growing kappa beyond the
  * largest value the plan has had synchronises `stream` and reallocates the
- * partition arrays.  Results of spmttkrp_run do not depend on kappa beyond
+ * partition arrays; where the plan has run CP-ALS with BF16 factors, it may also
+ * (re)allocate the buffers of its sweep, so that a sweep captured afterwards
+ * does not.  Results of spmttkrp_run do not depend on kappa beyond
  * FP32 summation order.  Must not be called while a batch holds the plan. */
 spm_status spmttkrp_plan_repartition(spmttkrp_plan_t plan, int kappa, void *stream);
 

@@ -192,7 +192,17 @@ spm_status gram(spmttkrp_plan_s* p, const void* Y, int64_t I, double* G, cudaStr
                  : launch_gram<float>(p, Y, I, G, s, mask);
 }
 
-spm_status ensure_als_state(spmttkrp_plan_s* p) {
+// Whether work on `s` is being captured (or cannot be told not to be).
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &c) == cudaSuccess) return c != cudaStreamCaptureStatusNone;
+  (void)cudaGetLastError();
+  return true;
+}
+
+// The plan-order buffers grow with the partition count, but not under a capture:
+// the sweep then takes one block per partition, with the same sums.
+spm_status ensure_als_state(spmttkrp_plan_s* p, cudaStream_t s) {
   spm_als_state& A = p->als;
   if (!A.side) {
     // At ranks whose Gram is a pass of its own, that pass and the system go
@@ -209,18 +219,15 @@ spm_status ensure_als_state(spmttkrp_plan_s* p) {
   if (!A.ev_fork) SPM_CUDA_TRY(cudaEventCreateWithFlags(&A.ev_fork, cudaEventDisableTiming));
   if (!A.ev_join) SPM_CUDA_TRY(cudaEventCreateWithFlags(&A.ev_join, cudaEventDisableTiming));
   const int R = p->R;
-  if (als_splits(p->bf16, p->fibre, p->nnz, p->kappa, p->nu, sm_count()) && A.split_cap < p->kappa) {
+  if (als_splits(p->bf16, p->fibre, p->nnz, p->kappa, p->nu, sm_count()) &&
+      A.split_cap < p->kappa && !capturing(s)) {
     const size_t units = (size_t)p->kappa * p->nu;
-    if (A.split_cap) {  // repartitioned since: queued work may still use the old arrays
-      if (!dev_drain(p->device)) return SPM_ERR_CUDA;
-      SPM_TRY(plan_realloc(p, (void**)&A.upart, sizeof(float) * 2 * units * R));
-      SPM_TRY(plan_realloc(p, (void**)&A.urow, sizeof(int) * 2 * units));
-      SPM_TRY(plan_realloc(p, (void**)&A.pdone, sizeof(int) * (size_t)p->kappa));
-    } else {
-      SPM_TRY(plan_alloc(p, (void**)&A.upart, sizeof(float) * 2 * units * R));
-      SPM_TRY(plan_alloc(p, (void**)&A.urow, sizeof(int) * 2 * units));
-      SPM_TRY(plan_alloc(p, (void**)&A.pdone, sizeof(int) * (size_t)p->kappa));
-    }
+    auto hold = [&](void** ptr, size_t bytes) {  // also after a call that failed halfway
+      return *ptr ? plan_realloc(p, ptr, bytes) : plan_alloc(p, ptr, bytes);
+    };
+    SPM_TRY(hold((void**)&A.upart, sizeof(float) * 2 * units * R));
+    SPM_TRY(hold((void**)&A.urow, sizeof(int) * 2 * units));
+    SPM_TRY(hold((void**)&A.pdone, sizeof(int) * (size_t)p->kappa));
     SPM_CUDA_TRY(cudaMemsetAsync(A.pdone, 0, sizeof(int) * (size_t)p->kappa, A.side));
     SPM_CUDA_TRY(cudaStreamSynchronize(A.side));
     A.split_cap = p->kappa;
@@ -250,7 +257,7 @@ spm_status als_sweep(spmttkrp_plan_s* p, void* const* factors, double* lambda, d
   if (gram_tile(R) == 0 || R > ALS_THREADS) return SPM_ERR_UNSUPPORTED;
   for (int w = 0; w < N; ++w)
     if (!factors[w] || (reinterpret_cast<uintptr_t>(factors[w]) & 15u)) return SPM_ERR_INVALID_ARG;
-  SPM_TRY(ensure_als_state(p));
+  SPM_TRY(ensure_als_state(p, s));
   spm_als_state& A = p->als;
   bool same = A.ready;
   for (int w = 0; w < N; ++w) same = same && A.fac_ptr[w] == factors[w];

@@ -337,7 +337,7 @@ spm_status batch_add(spm_batch_s* B, spmttkrp_plan_s* p, void* const* factors, d
     if (q == p) return SPM_ERR_INVALID_ARG;  // one batch slot per plan (shared workspace)
   // the members' convergence state lives on the device between sweeps
   if (!B->dirty) SPM_TRY(batch_pull(B, s));
-  SPM_TRY(ensure_als_state(p));
+  SPM_TRY(ensure_als_state(p, s));
   spm_als_state& A = p->als;
   A.ready = false;  // the batch keeps the Grams from now on
   BatchTensor b{};
@@ -427,7 +427,7 @@ spm_status batch_commit(spm_batch_s* B, cudaStream_t s) {
   for (int t = 0; t < n; ++t) {
     spmttkrp_plan_s* p = B->plans[t];
     B->maxN = std::max(B->maxN, p->N);
-    SPM_TRY(ensure_als_state(p));  // sized for its present partitions
+    SPM_TRY(ensure_als_state(p, s));  // sized for its present partitions
     B->maxR = std::max(B->maxR, p->R);
     // partitions may have changed since the tensor was added (autotuning)
     const int kc = B->host[t].kclass;

@@ -292,7 +292,7 @@ spm_status spmttkrp_plan_autotune(spmttkrp_plan_t plan, const void* const* facto
   for (int c = 0; c < nkappas; ++c)
     if (kappas[c] < 1 || kappas[c] > 0xFFFF) return SPM_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  SPM_TRY(ensure_als_state(plan));  // its M buffer (I_max x R) takes the outputs
+  SPM_TRY(ensure_als_state(plan, s));  // its M buffer (I_max x R) takes the outputs
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     (void)cudaGetLastError();
@@ -326,7 +326,6 @@ spm_status spmttkrp_plan_autotune(spmttkrp_plan_t plan, const void* const* facto
       continue;
     }
     st = plan_repartition(plan, kappas[c], s);
-    if (st == SPM_OK) st = ensure_als_state(plan);  // sized for these partitions
     float t_min = 0.f;
     for (int r = 0; r <= reps && st == SPM_OK; ++r) {  // r == 0 warms up
       cudaEventRecord(e0, s);

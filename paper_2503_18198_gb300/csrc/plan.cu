@@ -1320,7 +1320,8 @@ spm_status plan_repartition(spmttkrp_plan_s* p, int kappa, cudaStream_t s) {
   SPM_CUDA_TRY(cudaGetLastError());
   SPM_CUDA_TRY(cudaFreeAsync(seg, s));
   if (rows_tmp) SPM_CUDA_TRY(cudaFreeAsync(rows_tmp, s));
-  return SPM_OK;
+  // a sweep that is captured next must not have to allocate
+  return p->als.M ? ensure_als_state(p, s) : SPM_OK;
 }
 
 spm_status build_fibre_copies(spmttkrp_plan_s* p, cudaStream_t s);  // fibre_plan.cu

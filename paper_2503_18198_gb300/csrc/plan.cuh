@@ -252,7 +252,7 @@ spm_status gram(spmttkrp_plan_s* p, const void* Y, int64_t I, double* G, cudaStr
                 const uint32_t* mask = nullptr);
 
 // Allocate the plan's CP-ALS workspace on first use (als.cu).
-spm_status ensure_als_state(spmttkrp_plan_s* p);
+spm_status ensure_als_state(spmttkrp_plan_s* p, cudaStream_t s);
 
 int sm_count();
 
