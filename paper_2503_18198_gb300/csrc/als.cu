@@ -233,20 +233,23 @@ spm_status ensure_als_state(spmttkrp_plan_s* p, cudaStream_t s) {
     A.split_cap = p->kappa;
   }
   if (A.M) return SPM_OK;
+  auto need = [&](void** ptr, size_t bytes) {  // what a call that ran out of memory made is kept
+    return *ptr ? SPM_OK : plan_alloc(p, ptr, bytes);
+  };
   int64_t Imax = 1;
   for (int w = 0; w < p->N; ++w) Imax = std::max(Imax, p->dims[w]);
   A.gram_blocks = std::max(1, sm_count()) * 4;
   const size_t RR = (size_t)R * R;
-  SPM_TRY(plan_alloc(p, (void**)&A.gram, sizeof(double) * RR * p->N));
-  SPM_TRY(plan_alloc(p, (void**)&A.gram_part, sizeof(double) * RR * A.gram_blocks));
-  SPM_TRY(plan_alloc(p, (void**)&A.winv, sizeof(float) * 2 * RR));
-  SPM_TRY(plan_alloc(p, (void**)&A.colsq_part, sizeof(double) * R * A.gram_blocks));
-  SPM_TRY(plan_alloc(p, (void**)&A.colmax_part, sizeof(float) * R * A.gram_blocks));
-  if (als_wdig_bytes(R)) SPM_TRY(plan_alloc(p, (void**)&A.wdig, als_wdig_bytes(R)));
-  SPM_TRY(plan_alloc(p, (void**)&A.inner_part, sizeof(double) * R * A.gram_blocks));
-  SPM_TRY(plan_alloc(p, (void**)&A.lambda_ws, sizeof(double) * 2 * R));  // lambda, Gram scales
-  SPM_TRY(plan_alloc(p, (void**)&A.Z, sizeof(float) * (size_t)Imax * R));
-  SPM_TRY(plan_alloc(p, (void**)&A.M, sizeof(float) * (size_t)Imax * R));
+  SPM_TRY(need((void**)&A.gram, sizeof(double) * RR * p->N));
+  SPM_TRY(need((void**)&A.gram_part, sizeof(double) * RR * A.gram_blocks));
+  SPM_TRY(need((void**)&A.winv, sizeof(float) * 2 * RR));
+  SPM_TRY(need((void**)&A.colsq_part, sizeof(double) * R * A.gram_blocks));
+  SPM_TRY(need((void**)&A.colmax_part, sizeof(float) * R * A.gram_blocks));
+  if (als_wdig_bytes(R)) SPM_TRY(need((void**)&A.wdig, als_wdig_bytes(R)));
+  SPM_TRY(need((void**)&A.inner_part, sizeof(double) * R * A.gram_blocks));
+  SPM_TRY(need((void**)&A.lambda_ws, sizeof(double) * 2 * R));  // lambda, Gram scales
+  SPM_TRY(need((void**)&A.Z, sizeof(float) * (size_t)Imax * R));
+  SPM_TRY(need((void**)&A.M, sizeof(float) * (size_t)Imax * R));
   return SPM_OK;
 }
 
