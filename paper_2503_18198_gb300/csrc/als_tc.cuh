@@ -1178,8 +1178,10 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
   // completed).  They stay FP32 pairs up to the last sum: FP64 issues at 1/64
   // of FP32's rate, and this epilogue in FP64 was most of a short tensor's
   // pass (96 tensors: 113 and 76 us per mode at R = 32 and 16; now 64 and
-  // 54; one tile of R = 16: 12.1 -> 9.1 us).  The weights are powers of two,
-  // and the pairs' sum keeps the 2^-47 of the total that the accumulators do.
+  // 54; one tile of R = 16: 12.1 -> 9.1 us).  The weights are powers of two.
+  // The sum over the digits is kept in three parts, of which the last pair
+  // collects what the first loses: at R = 16, where the digits hold every bit,
+  // a sum in one pair was 20 times as far from the exact Gram as one in FP64.
   float2* red = reinterpret_cast<float2*>(sA);
   if (t < 128) {
     const uint64_t wp = f2_const(pow2f(-7 * (t / R)));
@@ -1199,14 +1201,20 @@ __device__ __forceinline__ void tc_scale_gram_body(const float* __restrict__ Z,
     for (int e = t; e < R / 2 * (R + 1); e += TC_THREADS) {
       const int i = e / (R + 1) + R / 2, k = e % (R + 1);
       const int rr = k <= i ? i : R - 1 - i, ss = k <= i ? k : k - i - 1;
-      df v = {0.f, 0.f};
+      float h = 0.f;
+      df lost = {0.f, 0.f}, low = {0.f, 0.f};  // two chains side by side
 #pragma unroll
       for (int p = S::NDIG - 1; p >= 0; --p) {
         const float2 x = red[(p * R + rr) * S::RED_LD + ss];
-        df_add(v, x.x);
-        v.lo = __fadd_rn(v.lo, x.y);
+        const float s = __fadd_rn(h, x.x);
+        const float bb = __fsub_rn(s, h);
+        df_add(lost, __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(x.x, bb)));
+        df_add(low, x.y);
+        h = s;
       }
-      const double x = times_pow2(df_value(v), gx[rr] + gx[ss] - 14);
+      df_add(low, lost.hi);
+      low.lo = __fadd_rn(low.lo, lost.lo);
+      const double x = times_pow2(__dadd_rn((double)h, df_value(low)), gx[rr] + gx[ss] - 14);
       if (fuse.G) {
         fuse.G[rr * R + ss] = x;
         fuse.G[ss * R + rr] = x;
