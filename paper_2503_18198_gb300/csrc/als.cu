@@ -219,8 +219,8 @@ spm_status ensure_als_state(spmttkrp_plan_s* p, cudaStream_t s) {
   if (!A.ev_fork) SPM_CUDA_TRY(cudaEventCreateWithFlags(&A.ev_fork, cudaEventDisableTiming));
   if (!A.ev_join) SPM_CUDA_TRY(cudaEventCreateWithFlags(&A.ev_join, cudaEventDisableTiming));
   const int R = p->R;
-  if (als_splits(p->bf16, p->fibre, p->nnz, p->kappa, p->nu, sm_count()) &&
-      A.split_cap < p->kappa && !capturing(s)) {
+  if (p->bf16 && A.split_cap < p->kappa &&
+      als_splits(p->bf16, p->fibre, p->nnz, p->kappa, p->nu, sm_count()) && !capturing(s)) {
     const size_t units = (size_t)p->kappa * p->nu;
     auto hold = [&](void** ptr, size_t bytes) {  // also after a call that failed halfway
       return *ptr ? plan_realloc(p, ptr, bytes) : plan_alloc(p, ptr, bytes);
