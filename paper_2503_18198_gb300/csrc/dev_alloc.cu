@@ -14,12 +14,12 @@
 // contract), from any thread.  cudaFree waited for the buffer's own device; with
 // a pool the owners do (dev_drain).
 //
-// Scratch that one stream's work uses (scratch_alloc) is freed in the order of
-// that stream: cudaFree waits for the whole device, so that a plan built beside
-// a running sweep ended with the sweep.  Large scratch still comes from
-// cudaMalloc; freed by cudaFreeAsync, it is given back when the stream is next
-// synchronised.  (50M nonzeros, 1.2 GB of scratch: a build takes 13.6 ms so, as
-// with cudaFree, and 15.3 ms with the scratch in the pool.)
+// Scratch that one stream's work uses waits for that stream alone when it is
+// freed (scratch_free): cudaFree waits for the whole device, so that a plan built
+// beside a running sweep ended with the sweep.  Scratch from cudaMalloc is freed
+// with cudaFreeAsync, and given back when the stream is next synchronised.  (50M
+// nonzeros, 1.2 GB of scratch: a build takes 13.7 ms so, as with cudaFree, and
+// 15.3 ms with the scratch in the pool.)
 #include <mutex>
 
 #include "device_drain.h"
@@ -99,29 +99,15 @@ spm_status dev_alloc(void** ptr, size_t bytes) {
   return e == cudaErrorMemoryAllocation ? SPM_ERR_OOM : SPM_ERR_CUDA;
 }
 
-spm_status scratch_alloc(void** ptr, size_t bytes, cudaStream_t s) {
-  *ptr = nullptr;
-  int dev = 0;
-  SPM_CUDA_TRY(cudaGetDevice(&dev));
-  DevicePool* d = device_pool(dev);
-  auto get = [&]() {
-    return d && pooled(bytes) ? cudaMallocFromPoolAsync(ptr, bytes, d->pool, s)
-                              : cudaMalloc(ptr, bytes);
-  };
-  cudaError_t e = get();
-  if (e == cudaErrorMemoryAllocation && d) {
-    (void)cudaGetLastError();
-    (void)cudaMemPoolTrimTo(d->pool, 0);
-    e = get();
+void scratch_free(void* ptr, size_t bytes, cudaStream_t s) {
+  if (!ptr) return;
+  if (pooled(bytes)) {
+    cudaStreamSynchronize(s);
+    dev_free(ptr, bytes);
+  } else {
+    cudaFreeAsync(ptr, s);
   }
-  if (e == cudaSuccess) return SPM_OK;
   (void)cudaGetLastError();
-  *ptr = nullptr;
-  return e == cudaErrorMemoryAllocation ? SPM_ERR_OOM : SPM_ERR_CUDA;
-}
-
-void scratch_free(void* ptr, cudaStream_t s) {
-  if (ptr && cudaFreeAsync(ptr, s) != cudaSuccess) (void)cudaGetLastError();
 }
 
 void dev_free(void* ptr, size_t bytes) {

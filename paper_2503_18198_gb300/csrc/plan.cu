@@ -972,10 +972,12 @@ struct BuildScratch {
     return at;
   }
   cudaStream_t stream = nullptr;
+  size_t bytes = 0;
   spm_status alloc(int64_t cap, cudaStream_t s) {
     void* p = nullptr;
     stream = s;
-    SPM_TRY(scratch_alloc(&p, layout(cap, nullptr, nullptr), s));
+    bytes = layout(cap, nullptr, nullptr);
+    SPM_TRY(dev_alloc(&p, bytes));
     layout(cap, static_cast<unsigned char*>(p), this);
     return SPM_OK;
   }
@@ -983,9 +985,9 @@ struct BuildScratch {
   BuildScratch(const BuildScratch&) = delete;
   BuildScratch& operator=(const BuildScratch&) = delete;
   ~BuildScratch() { release(); }
-  // Stream-ordered; a synchronisation after it gives large scratch back.
+  // A synchronisation of the stream after it gives large scratch back.
   void release() {
-    scratch_free(base, stream);
+    scratch_free(base, bytes, stream);
     base = nullptr;
   }
 };

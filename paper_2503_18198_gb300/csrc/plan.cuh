@@ -123,9 +123,8 @@ namespace spm {
 spm_status dev_alloc(void** ptr, size_t bytes);
 void dev_free(void* ptr, size_t bytes);
 bool dev_drain(int device);
-// Scratch for work on `s`, ordered on it: freed without waiting for anything.
-spm_status scratch_alloc(void** ptr, size_t bytes, cudaStream_t s);
-void scratch_free(void* ptr, cudaStream_t s);
+// dev_free of scratch that only work on `s` uses, whatever else is queued.
+void scratch_free(void* ptr, size_t bytes, cudaStream_t s);
 
 // Allocation owned by the plan (recorded for destroy and for plan_bytes).
 spm_status plan_alloc(spmttkrp_plan_s* p, void** ptr, size_t bytes);
