@@ -158,15 +158,16 @@ __device__ __forceinline__ void df2_add_square(df2& a, uint64_t z) {  // a += z 
 // V scaled by powers of two to a diagonal in [1, 4), and each column then takes
 // one step of iterative refinement: its residual e_c - V w in FP64 (R^2
 // multiply-adds), the correction X^T D^{-1} X r in FP32.  That leaves an error
-// below that of an FP64 factorisation while cond(V) is moderate: it is taken
-// when every pivot is at least 2^-16 and trace(V^{-1}) of the scaled system at
-// most 2^12, which bounds cond(V) by 2^12 * 4 R (the error of the pairs,
-// 2^-46 cond, times the error of the FP32 correction, 2^-24 cond, is then below
-// 2^-53 cond * R); otherwise the same elimination runs in FP64, which also
-// decides whether V is positive definite.  Rows solved with it are as far from
-// extended precision as with an FP64 Cholesky factor for cond(V) = 3 .. 1e8 at
-// R = 16, 32, 64 (rms 2.5e-8, the FP32 rounding of Z; the splitting's 2^-34 is
-// the rest): tests/test_gpu_system.py.
+// no larger than that of an FP64 factorisation while cond(V) is moderate: it is
+// taken when every pivot is at least 2^-16 and trace(V^{-1}) of the scaled system
+// at most 2^7 + 2 R (systems of the timed decompositions, R = 8 to 64: 5 to 57);
+// otherwise the same elimination runs in FP64, which also decides whether V is
+// positive definite.  Error of W against extended precision, relative to that of
+// an FP64 Cholesky factor with two substitutions (geometric means over nine ranks
+// from 3 to 64): cond(V) = 3 .. 300 0.90 - 0.96, 1e3 .. 4e3 0.92 - 0.96, 1e4 ..
+// 1e8 0.95 - 1.02.  (With a limit of 2^12 the pairs served conditions up to 1e4,
+// at 1.04 - 1.08 from 2e3 on.)  Rows solved with it: tests/test_gpu_system.py and
+// tests/test_gpu_system_ranks.py.
 // One system, one column per block, alone on the GPU, R = 16 / 32 / 64: 10 /
 // 18 / 51 us (the same elimination in FP64 12.3 / 25.6 / 78 us; before it, a
 // Cholesky factor and two substitution chains per column, 20 / 46 / 139 us).
@@ -567,7 +568,7 @@ __device__ __forceinline__ bool system_pairs_ns(SystemSmem& sm, const double* __
   float trace = 0.f;
 #pragma unroll
   for (int w = 0; w < SYS_THREADS / 32; ++w) trace += sm.red[w];
-  if (!(trace <= 4096.f)) return false;
+  if (!(trace <= (float)(128 + 2 * R))) return false;
   auto X = [&](int k, int c) -> float2 { return sm.XF[k * (k + 1) / 2 + c]; };
   const int nc = c1 - c0;
   const unsigned rinv = (65535u + R) / R;  // x / R = x rinv >> 16 for x < 1024
