@@ -483,7 +483,9 @@ typedef struct {
 } spm_job_info;
 
 /* hbm_budget: device bytes the server's jobs may hold at once (plans,
- * factors, and the transient sort scratch of a build); max_active: running
+ * factors, and the transient sort scratch of a build; memory that the library
+ * keeps for reuse is given back where it would not fit beside them, see
+ * spm_memory_trim); max_active: running
  * jobs at most; flags: SPM_FACTOR_FP32 or SPM_FACTOR_BF16;
  * nnz_per_partition: partitions per job = ceil(nnz / this), 1..65535
  * (0 = the plan default, SPM_KAPPA(0)). */
@@ -582,6 +584,14 @@ spm_status spmttkrp_plan_status(spmttkrp_plan_t plan, void *stream);
 
 /* Static, never-NULL description of a status code. */
 const char *spm_status_string(spm_status s);
+
+/* Buffers up to 32 MB that plans, batches and servers release are kept for the
+ * next ones (64 MB per device at most once the device has been synchronised).
+ * If more than `keep` bytes of the current device are kept, they go back to the
+ * driver, but for the rest of a block (32 MB) in which a live buffer lies;
+ * *held (may be NULL) = bytes still kept.  May be called at any time, from any
+ * thread. */
+spm_status spm_memory_trim(size_t keep, size_t *held);
 
 /* Number of SMs of the current device (the default kappa), or -1. */
 int spm_device_sm_count(void);

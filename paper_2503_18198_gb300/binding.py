@@ -70,7 +70,8 @@ SYMBOLS = ("spmttkrp_plan", "spmttkrp_plan_bytes", "spmttkrp_plan_permutation",
            "spm_server_destroy", "spm_selftest_wait_timeout", "spm_inject_alloc_failure",
            "cpd_als_reset", "spm_server_snapshot", "spm_server_resume",
            "spmttkrp_run_all_host", "spm_selftest_mttkrp_timeout", "spmttkrp_noalloc_status",
-           "spmttkrp_plan_fibre_count", "spm_selftest_tc_rowpass", "spm_selftest_batch_timeout")
+           "spmttkrp_plan_fibre_count", "spm_selftest_tc_rowpass", "spm_selftest_batch_timeout",
+           "spm_memory_trim")
 
 
 def library_path() -> str:
@@ -168,6 +169,8 @@ def load(build_if_missing: bool = False):
     lib.spm_server_resume.restype = i32
     lib.spm_batch_destroy.argtypes = [P]
     lib.spm_batch_destroy.restype = None
+    lib.spm_memory_trim.argtypes = [ctypes.c_size_t, P]
+    lib.spm_memory_trim.restype = i32
     lib.spm_device_sm_count.argtypes = []
     lib.spm_device_sm_count.restype = i32
     _lib = lib
@@ -218,6 +221,14 @@ class Plan:
             self.destroy()
         except Exception:
             pass
+
+
+def spm_memory_trim(keep: int = 0) -> int:
+    """Give device memory kept for reuse back if it is more than `keep` bytes;
+    returns the bytes still kept."""
+    held = ctypes.c_size_t()
+    _check(load().spm_memory_trim(int(keep), ctypes.byref(held)), "spm_memory_trim")
+    return int(held.value)
 
 
 def spm_device_sm_count() -> int:

@@ -356,6 +356,14 @@ spm_status spmttkrp_plan_autotune(spmttkrp_plan_t plan, const void* const* facto
   return st;
 }
 
+spm_status spm_memory_trim(size_t keep, size_t* held) {
+  int device = 0;
+  SPM_CUDA_TRY(cudaGetDevice(&device));
+  dev_trim(device, keep);
+  if (held) *held = dev_held(device);
+  return SPM_OK;
+}
+
 void spmttkrp_plan_destroy(spmttkrp_plan_t plan) {
   free_plan(plan);
 }

@@ -120,6 +120,26 @@ void dev_free(void* ptr, size_t bytes) {
   (void)cudaGetLastError();
 }
 
+size_t dev_held(int device) {
+  DevicePool* d = known_pool(device);
+  if (!d) return 0;
+  unsigned long long reserved = 0, used = 0;
+  if (cudaStreamSynchronize(d->stream) != cudaSuccess ||  // the frees so far
+      cudaMemPoolGetAttribute(d->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+      cudaMemPoolGetAttribute(d->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  return reserved > used ? (size_t)(reserved - used) : 0;
+}
+
+void dev_trim(int device, size_t keep) {
+  DevicePool* d = known_pool(device);
+  if (!d || dev_held(device) <= keep) return;
+  (void)cudaMemPoolTrimTo(d->pool, 0);
+  (void)cudaGetLastError();
+}
+
 bool dev_drain(int device) {
   struct Runtime {
     bool get(int* d) { return cudaGetDevice(d) == cudaSuccess; }

@@ -123,6 +123,10 @@ namespace spm {
 spm_status dev_alloc(void** ptr, size_t bytes);
 void dev_free(void* ptr, size_t bytes);
 bool dev_drain(int device);
+// Bytes that are kept for reuse on `device` and belong to no buffer, and giving
+// them back if they are more than `keep`.
+size_t dev_held(int device);
+void dev_trim(int device, size_t keep);
 // dev_free of scratch that only work on `s` uses, whatever else is queued.
 void scratch_free(void* ptr, size_t bytes, cudaStream_t s);
 

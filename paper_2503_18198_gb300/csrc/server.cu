@@ -153,6 +153,13 @@ spm_status admit(spm_server_s* S, Job* j) {
   return SPM_OK;
 }
 
+// Memory kept for reuse goes back where it does not fit the budget beside the
+// jobs' bytes and `more`.
+void trim_to_budget(spm_server_s* S, size_t more) {
+  const size_t bytes = S->used + more;
+  dev_trim(S->B->device, S->budget > bytes ? S->budget - bytes : 0);
+}
+
 void fail(spm_server_s* S, Job* j, spm_status st) {
   j->state = SPM_JOB_FAILED;
   j->status = st;
@@ -258,6 +265,7 @@ spm_status spm_server_step(spm_server_t S, int* running, int* queued) {
     }
     if (S->used + need + j->transient > S->budget) break;  // wait for memory
     S->queue.pop_front();
+    trim_to_budget(S, need + j->transient);
     j->t_admit = now_ms();
     const spm_status st = admit(S, j);
     if (st != SPM_OK) {
@@ -300,6 +308,7 @@ spm_status spm_server_step(spm_server_t S, int* running, int* queued) {
     j->state = SPM_JOB_RUNNING;
     S->running.push_back(j);
   }
+  trim_to_budget(S, 0);
   if (running) *running = (int)S->running.size();
   if (queued) *queued = (int)S->queue.size();
   return SPM_OK;
