@@ -536,9 +536,7 @@ def main():
     torch.cuda.synchronize()
     als_ms = a0.elapsed_time(a1)
 
-    # the record kernel (it clears empty rows itself) and, beyond 32 boundary
-    # parts, the fix-up
-    launches_per_step = N * (1 + (1 if plan_kappa(spm, plan) > 32 else 0))
+    launches_per_step = sum(spm.spmttkrp_plan_launches(plan, d)[0] for d in range(N))
 
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu:
@@ -1336,12 +1334,6 @@ def kernel_digest():
         with open(os.path.join(ROOT, "paper_2503_18198_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
-
-
-def plan_kappa(spm, plan):
-    import torch
-    off = torch.empty(65536 + 1, dtype=torch.int64, device="cuda")
-    return spm.spmttkrp_plan_partition(plan, 0, off)
 
 
 if __name__ == "__main__":

@@ -207,6 +207,14 @@ spm_status spmttkrp_plan_scheme(spmttkrp_plan_t plan, int mode, int *scheme);
 spm_status spmttkrp_plan_work_units(spmttkrp_plan_t plan, int mode, int64_t *off,
                                     void *stream);
 
+/* *kernels = kernel launches of one spmttkrp_run along `mode` (the spMTTKRP,
+ * the zeroing of empty rows and the boundary fix-up where they are launches of
+ * their own; clearing the output of a SCHEME1 copy or of an empty tensor is a
+ * memset), *blocks (may be NULL) = thread blocks of the spMTTKRP kernel.  Host
+ * only. */
+spm_status spmttkrp_plan_launches(spmttkrp_plan_t plan, int mode, int *kernels,
+                                  int *blocks);
+
 /* Release the plan and all its device memory (stream-ordered frees after a
  * device synchronisation).  NULL is ignored. */
 void spmttkrp_plan_destroy(spmttkrp_plan_t plan);

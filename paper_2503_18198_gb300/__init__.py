@@ -14,7 +14,7 @@ from .binding import (SPM_FACTOR_BF16, SPM_FACTOR_FP32, SPM_KAPPA,  # noqa: F401
                       spm_batch_sweep,
                       spm_device_sm_count, spm_memory_trim, spm_selftest_tc_rowpass, spm_status_string, spmttkrp_plan,
                       spmttkrp_plan_bytes, spmttkrp_plan_bytes_estimate,
-                      spmttkrp_plan_destroy, spmttkrp_plan_fibre_count,
+                      spmttkrp_plan_destroy, spmttkrp_plan_fibre_count, spmttkrp_plan_launches,
                       spmttkrp_plan_partition, spmttkrp_plan_permutation,
                       spmttkrp_plan_autotune, spmttkrp_plan_repartition,
                       spmttkrp_plan_scheme,

@@ -71,7 +71,7 @@ SYMBOLS = ("spmttkrp_plan", "spmttkrp_plan_bytes", "spmttkrp_plan_permutation",
            "cpd_als_reset", "spm_server_snapshot", "spm_server_resume",
            "spmttkrp_run_all_host", "spm_selftest_mttkrp_timeout", "spmttkrp_noalloc_status",
            "spmttkrp_plan_fibre_count", "spm_selftest_tc_rowpass", "spm_selftest_batch_timeout",
-           "spm_memory_trim")
+           "spm_memory_trim", "spmttkrp_plan_launches")
 
 
 def library_path() -> str:
@@ -169,6 +169,8 @@ def load(build_if_missing: bool = False):
     lib.spm_server_resume.restype = i32
     lib.spm_batch_destroy.argtypes = [P]
     lib.spm_batch_destroy.restype = None
+    lib.spmttkrp_plan_launches.argtypes = [P, i32, P, P]
+    lib.spmttkrp_plan_launches.restype = i32
     lib.spm_memory_trim.argtypes = [ctypes.c_size_t, P]
     lib.spm_memory_trim.restype = i32
     lib.spm_device_sm_count.argtypes = []
@@ -319,6 +321,14 @@ def spmttkrp_plan_fibre_count(plan: Plan, mode: int) -> int:
     _check(load().spmttkrp_plan_fibre_count(plan.handle, int(mode), ctypes.byref(n)),
            "spmttkrp_plan_fibre_count")
     return int(n.value)
+
+
+def spmttkrp_plan_launches(plan: Plan, mode: int):
+    """(kernel launches, blocks of the spMTTKRP kernel) of spmttkrp_run along `mode`."""
+    k, b = ctypes.c_int(), ctypes.c_int()
+    _check(load().spmttkrp_plan_launches(plan.handle, int(mode), ctypes.byref(k), ctypes.byref(b)),
+           "spmttkrp_plan_launches")
+    return int(k.value), int(b.value)
 
 
 def spmttkrp_plan_destroy(plan: Plan):

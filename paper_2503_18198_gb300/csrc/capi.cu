@@ -244,6 +244,14 @@ spm_status spmttkrp_plan_scheme(spmttkrp_plan_t plan, int mode, int* scheme) {
   return SPM_OK;
 }
 
+spm_status spmttkrp_plan_launches(spmttkrp_plan_t plan, int mode, int* kernels, int* blocks) {
+  if (!plan || mode < 0 || mode >= plan->N || !kernels) return SPM_ERR_INVALID_ARG;
+  int nb = 0;
+  *kernels = mttkrp_launches(plan, mode, &nb);
+  if (blocks) *blocks = nb;
+  return SPM_OK;
+}
+
 spm_status spmttkrp_plan_bytes_estimate(int nmodes, const int64_t* dims, int64_t nnz, int rank,
                                         uint32_t flags, size_t* resident, size_t* transient) {
   if (nmodes < 2 || nmodes > SPM_MAX_MODES || !dims || nnz < 0 || rank < 1 ||

@@ -116,6 +116,16 @@ void mttkrp_set_shape(const spmttkrp_plan_s* p, int d, bool plan_order, MttkrpAr
   a->nblocks = p->kappa * a->split;
 }
 
+int mttkrp_launches(const spmttkrp_plan_s* p, int mode, int* blocks) {
+  const spm_mode_copy& c = p->mode[mode];
+  MttkrpArgs a{};
+  mttkrp_set_shape(p, mode, false, &a);
+  *blocks = p->nnz == 0 ? 0 : c.fstream ? p->kappa : a.nblocks;
+  if (p->nnz == 0) return 0;
+  if (c.fstream) return (c.empty_rows > 0 ? 1 : 0) + 1 + (p->kappa > 1 ? 1 : 0);
+  return 1 + (c.scheme != 1 && !mttkrp_few_parts(a) ? 1 : 0);
+}
+
 spm_status run_mttkrp(spmttkrp_plan_s* p, int mode, const void* const* factors, float* out,
                       cudaStream_t s, bool plan_order) {
   if (!p || mode < 0 || mode >= p->N || !factors || !out) return SPM_ERR_INVALID_ARG;

@@ -241,6 +241,10 @@ spm_status build_copies(spmttkrp_plan_s* p, const int32_t* const* idx,
 spm_status run_mttkrp(spmttkrp_plan_s* p, int mode, const void* const* factors,
                       float* out, cudaStream_t s, bool plan_order = false);
 
+// Kernels that run_mttkrp launches (any order), and the blocks of the spMTTKRP
+// kernel among them; the same conditions as there.
+int mttkrp_launches(const spmttkrp_plan_s* p, int mode, int* blocks);
+
 // The launch shape and plan-order fields of `a` for mode d of plan p.
 struct MttkrpArgs;
 void mttkrp_set_shape(const spmttkrp_plan_s* p, int d, bool plan_order, MttkrpArgs* a);
