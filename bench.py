@@ -1216,7 +1216,8 @@ def run_precision(args, rank, world):
         torch.cuda.synchronize()
         plan_ms = (time.perf_counter() - t0) * 1e3
         fac = [y.to(dtype).clone() for y in Y]  # never alias the preset factors
-        kappa, kappa_ms = spm.spmttkrp_plan_autotune(plan, fac)  # 1 or 2 partitions per SM
+        # 1 or 2 partitions per SM, timed as this arm's sweeps run the spMTTKRP
+        kappa, kappa_ms = spm.spmttkrp_plan_autotune(plan, fac)
         outs = [torch.empty(dims[d], R, device="cuda") for d in range(N)]
         B = algorithmic_bytes(dims, nnz, R, distinct, s_f)
         ms = []

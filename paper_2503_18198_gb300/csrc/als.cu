@@ -3,7 +3,7 @@
 // Per mode d (Gauss-Seidel over d = 0..N-1, Algorithm 1's mode loop):
 //   M      = spMTTKRP_d(Y)                                   (mttkrp.cu)
 //   V      = Hadamard over w != d of G_w,  G_w = Y_w^T Y_w    (R x R, FP64)
-//   W      = V^{-1} from V = L D L^T                          (FP64, als_tc.cuh)
+//   W      = V^{-1} from V = L D L^T      (FP32 pairs and an FP64 residual, or FP64: als_tc.cuh)
 //   Z      = M W, accumulated in double-float (FP32 pairs)    (all SMs)
 //   lambda = column 2-norms of Z;  Y_d = Z / lambda stored as FP32 or BF16
 //   G_d    = Gram of the stored Y_d, exact FP32 products summed in

@@ -1,9 +1,9 @@
 // als_tc.cuh -- the CP-ALS row passes on the tensor cores, with FP64-level
 // accuracy from BF16 x BF16 -> FP32 MMAs (exact operand splitting).
 //
-// Row solve Z = M V^{-1}.  The R x R system comes from the FP64 Cholesky of
-// the Hadamard product of the Grams (Sec. II-A5; system_body), W = V^{-1} in
-// FP64.  Splitting:
+// Row solve Z = M V^{-1}.  V is the Hadamard product of the Grams (Sec. II-A5) in
+// FP64; W = V^{-1} comes from L D L^T in FP32 pairs with a correction from the
+// FP64 residual, or in FP64 where V is ill-conditioned (system_body).  Splitting:
 //  * each row i of M (FP32) is scaled by 2^-e_i (e_i the exponent of its
 //    largest magnitude) and cut into SM_DIG integer digits of 7 bits,
 //    m_i = 2^e_i * sum_p k_p(i) 2^{-7(p+1)}, |k_p| <= 128;

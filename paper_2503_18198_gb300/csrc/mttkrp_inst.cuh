@@ -91,7 +91,9 @@ MttkrpKernelFn pick_mttkrp_t(int R) {
       }
     }
   }
-  if constexpr (PLAN) {  // the scalar variant's order with the chunks that R fills
+  // Plan order at other ranks: the scalar variant's order (one nonzero per warp
+  // step, which the masked shapes would change) with the chunks that R fills
+  if constexpr (PLAN) {
     if (R <= 32) return &mttkrp_kernel<RI, NIN, FT, 1, 32, 1, LEAN, PLAN>;
     return &mttkrp_kernel<RI, NIN, FT, 1, 32, 2, LEAN, PLAN>;
   }

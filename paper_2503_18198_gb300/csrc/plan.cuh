@@ -235,9 +235,12 @@ spm_status build_copies(spmttkrp_plan_s* p, const int32_t* const* idx,
 
 // P3 + P4: one MTTKRP launch sequence for mode d (mttkrp.cu).
 // plan_order (BF16 factors, R <= 64): sum in the order that the plan's
-// partitions define, whatever the launch shape.  A decomposition with BF16 factors asks for it: each update is
-// rounded to 8 bits, so one flipped last bit of M becomes another factor, and a
-// result would depend on how the device is filled.
+// partitions define, whatever the launch shape.  A decomposition with BF16
+// factors asks for it: each update is rounded to 8 bits, so one flipped last bit
+// of M becomes another factor, and its result would depend on how the device is
+// filled.  (Any fixed order is as near to the exact sums: this is about results
+// that stay the same, not about accuracy.  It bounds the launch shapes, see
+// mttkrp_split.)
 spm_status run_mttkrp(spmttkrp_plan_s* p, int mode, const void* const* factors,
                       float* out, cudaStream_t s, bool plan_order = false);
 
