@@ -17,6 +17,8 @@ def _lib():
         pytest.skip("no CUDA device")
     spm.load(build_if_missing=True)
     profiled(lambda: torch.ones(8, device="cuda") + 1)  # the first session sees no events
+    if not profiled(lambda: torch.ones(8, device="cuda") + 1):
+        pytest.skip("the profiler sees no kernels here")
 
 
 def profiled(call):
